@@ -167,6 +167,24 @@ void keep_pool_memory() {
     });
 }
 
+// Scratch of one call from the current device's stream-ordered pool, given back (stream-ordered) on scope exit.
+struct PoolScratch {
+    cudaStream_t stream;
+    void* ptr = nullptr;
+    explicit PoolScratch(cudaStream_t s) : stream(s) {}
+    void* get(size_t bytes) {
+        keep_pool_memory();
+        if (cudaMallocAsync(&ptr, bytes, stream) != cudaSuccess) {
+            (void)cudaGetLastError();
+            ptr = nullptr;
+        }
+        return ptr;
+    }
+    ~PoolScratch() {
+        if (ptr) (void)cudaFreeAsync(ptr, stream);
+    }
+};
+
 }  // namespace
 
 extern "C" {
@@ -277,11 +295,13 @@ int lla_decode_ex(const lla_decode_params* p) {
         const size_t need = lla::decode_workspace_bytes(a.B, a.H, a.d, a.dv, a.splits);
         if (!p->workspace || p->workspace_bytes < need) a.splits = 1;
     }
-    if (a.splits > 1 && ((uintptr_t)p->workspace & 255u)) return LLA_ERR_WORKSPACE;
+    if (a.splits > 1 && (((uintptr_t)p->workspace & 255u) || !p->workspace ||
+                         p->workspace_bytes < lla::decode_workspace_bytes(a.B, a.H, p->d, p->dv, a.splits)))
+        return LLA_ERR_WORKSPACE;
+    a.workspace = p->workspace; a.workspace_bytes = p->workspace_bytes;
     a.head_rows = 2 * p->d;
     a.impl = p->impl;
     a.status = p->device_status;
-    a.workspace = p->workspace; a.workspace_bytes = p->workspace_bytes;
     a.stream = (cudaStream_t)p->stream;
     a.lambda_units = p->lambda_units;
     a.ridge_mode = p->ridge_mode;
@@ -298,26 +318,26 @@ int lla_decode_ex(const lla_decode_params* p) {
     if (p->debug_wait_clocks < 0 || (p->debug_flags & ~LLA_DEBUG_NO_LOADS)) return LLA_ERR_INVALID_ARG;
     a.wait_clocks = p->debug_wait_clocks;
     a.no_loads = (p->debug_flags & LLA_DEBUG_NO_LOADS) ? 1 : 0;
-    if (a.status) LLA_CUDA_TRY(cudaMemsetAsync(a.status, 0, sizeof(int) * LLA_STATUS_WORDS, a.stream));
-    // The units with short caches go to the direct kernel, which writes rows of `out` nobody else writes and
-    // returns at once for every other unit: it runs on the side stream beside the streaming kernel instead of
-    // behind the solve (its launch alone is 2-3 us of a 300 us step).
-    SideStream* side = side_stream();
-    if (side) {
-        std::lock_guard<std::mutex> lock(side->use);
-        LLA_CUDA_TRY(cudaEventRecord(side->fork, a.stream));
-        LLA_CUDA_TRY(cudaStreamWaitEvent(side->stream, side->fork, 0));
-        DecodeArgs h = a;
-        h.stream = side->stream;
-        const int rc_head = lla::launch_head_rows_decode(h);
-        LLA_CUDA_TRY(cudaEventRecord(side->join, side->stream));
-        const int st = lla::launch_decode(a);
-        LLA_CUDA_TRY(cudaStreamWaitEvent(a.stream, side->join, 0));
-        return st != LLA_OK ? st : rc_head;
+    // d = 128: the tensor-core path needs a buffer for the moment records.  An unsplit call without one takes it from
+    // the stream-ordered pool (the CUDA-core kernels, 30 times slower, run only if that fails).
+    PoolScratch records(a.stream);
+    if (p->splits <= 1 && p->d == 128 && p->in_dtype == LLA_BF16 && p->impl != LLA_IMPL_SIMT &&
+        p->ridge_mode == LLA_RIDGE_DEFINITION && !lla::decode_records_fit(a)) {
+        const int parts = p->splits == 1 ? 1 : lla_decode_default_splits(p->B, p->H, p->Lmax);
+        const size_t need = lla::decode_record_bytes(p->B, p->H, p->d, p->dv, parts);
+        if (void* mem = records.get(need)) {
+            a.splits = parts;
+            a.workspace = mem; a.workspace_bytes = need;
+        }
     }
-    const int st = lla::launch_decode(a);
-    if (st != LLA_OK) return st;
-    return lla::launch_head_rows_decode(a);
+    if (a.status) LLA_CUDA_TRY(cudaMemsetAsync(a.status, 0, sizeof(int) * LLA_STATUS_WORDS, a.stream));
+    // The units with short caches go to the direct kernel, which writes rows of `out` nobody else writes and returns
+    // at once for every other unit.  It goes first and the streaming kernel is its programmatic dependent, so the two
+    // overlap without a second stream (whose fork and join cost a small call several microseconds).
+    const int rc_head = lla::launch_head_rows_decode(a);
+    if (rc_head != LLA_OK) return rc_head;
+    a.behind_direct = true;
+    return lla::launch_decode(a);
 }
 
 int lla_decode(const void* q, const void* kcache, const void* vcache, const int* lens, void* out, int B,
@@ -329,16 +349,17 @@ int lla_decode(const void* q, const void* kcache, const void* vcache, const int*
     p.scale = scale; p.lambda = lambda;
     p.stream = stream;
     // scratch for the moment records comes from the stream-ordered pool (kept warm between calls)
-    p.splits = 1;
-    const size_t ws = lla_decode_workspace_bytes(B, H, Lmax, d, dv, LLA_BF16, 1);
+    p.splits = lla_decode_default_splits(B, H, Lmax);
+    const size_t ws = lla_decode_workspace_bytes(B, H, Lmax, d, dv, LLA_BF16, p.splits);
     void* scratch = nullptr;
     if (ws > 0 && B > 0 && H > 0) {
         keep_pool_memory();
         if (cudaMallocAsync(&scratch, ws, (cudaStream_t)stream) != cudaSuccess) {
             (void)cudaGetLastError();
-            scratch = nullptr;          // fall back to the fused epilogue
+            scratch = nullptr;          // fall back to one part and the fused epilogue
         }
     }
+    if (!scratch) p.splits = 1;
     p.workspace = scratch;
     p.workspace_bytes = scratch ? ws : 0;
     const int rc = lla_decode_ex(&p);

@@ -144,6 +144,7 @@ struct DecodeArgs {
     int ridge_mode;             // lla_ridge_mode
     int kv_group = 1;           // query heads per key/value head: caches are [B, H / kv_group, Lmax, d]
     PagedKv paged = {nullptr, 0, 0, 0};
+    bool behind_direct = false; // the direct kernel of the short caches is the launch before this one on `stream`
     int window = 0;             // sliding window: only the last `window` cached keys are visible (0: all)
     long long wait_clocks = 0;  // tensor-core kernel: cap of its bounded waits in SM clocks (0: default) and a test aid:
     int no_loads = 0;           // issue no copy at all (lla_decode_params.debug_*)
@@ -238,6 +239,7 @@ int launch_precond(const void* k, int B, int Hk, Strides sk, int n, int d, float
                    cudaStream_t st);
 int launch_decode(const DecodeArgs& a);
 int launch_head_rows_decode(const DecodeArgs& a);
+bool decode_records_fit(const DecodeArgs& a);
 bool decode_tensor_supported(const DecodeArgs& a);
 int launch_decode_tensor_moments(const DecodeArgs& a);
 size_t decode_workspace_bytes(int B, int H, int d, int dv, int splits);   // required bytes (0 when unsplit)

@@ -405,7 +405,8 @@ extern "C" int lla_decode_noalloc(const void* q, const void* kcache, const void*
         a.workspace = scratch;
         a.workspace_bytes = LLA_NOALLOC_SCRATCH_BYTES;
     }
-    const int st = lla::launch_decode(a);
+    const int st = lla::launch_head_rows_decode(a);
     if (st != LLA_OK) return st;
-    return lla::launch_head_rows_decode(a);
+    a.behind_direct = true;
+    return lla::launch_decode(a);
 }

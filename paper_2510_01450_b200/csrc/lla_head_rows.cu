@@ -114,6 +114,8 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
     double* zc = S;                         // HR_CHUNK * D  centred keys of the current chunk (over S)
 
     const int tid = threadIdx.x;
+    // decode: the streaming kernel launched behind this one as its programmatic dependent need not wait for it
+    if (lens) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // blockIdx.x (fastest in launch order) is the head, blockIdx.y counts rows from the last one down:
     // rows with the most keys are the longest blocks and start first, so the tail of the launch is short
     const int bh = blockIdx.x;

@@ -1,0 +1,83 @@
+"""The decode's tensor-core streaming kernel (bf16, d = 64 and 128) at the edges of its tiles of 64 keys, with the options
+that change which rows a tile reads, with short caches beside long ones, and with a first tile whose maximum is useless
+as the reference of the weights.  Tolerances are those of the other bf16 parity tests on an fp32 output buffer."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2510_01450_b200 import binding as L, inputs
+from tests.gpu_util import dev, row_err, stream_ptr
+from tests.test_parity_gpu import TOL_BF16, _to_pages
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,mode,splits", [(64, "plain", 1), (64, "late_max", 1), (64, "late_max", 2), (64, "short", 1), (128, "plain", 1),
+                                           (128, "plain", 3), (128, "late_max", 1), (128, "late_max", 2), (128, "short", 1),
+                                           (128, "paged_gqa", 1), (128, "paged_gqa", 2), (128, "window", 1)])
+def test_tile_edges_and_options(oracle, d, mode, splits):
+    H, Hkv = 4, 2 if mode == "paged_gqa" else 4
+    w = inputs.CONFIGS[5].shrink(B=6, H=H, n=1100, d=d, dv=d, len_min=10, len_max=1100, seed=400 + d)
+    q, _, _, _ = inputs.make_decode(w)
+    _, kc, vc, _ = inputs.make_decode(w.shrink(H=Hkv))
+    lens = np.array([2 * d, 2 * d + 1, 319, 384, 385, 1100], dtype=np.int32)
+    if mode == "short":
+        lens[:3] = [1, 17, 2 * d - 1]           # solved directly
+    kw = {}
+    if mode == "late_max":
+        # the first 64 keys score about 2^100 below the rest
+        qn = q / (np.linalg.norm(q, axis=-1, keepdims=True) ** 2)
+        kc[:, :, :64] += (-70.0 / w.scale) * qn[:, :, None, :]
+        kc = inputs.round_to_bf16(kc)
+    if mode == "window":
+        kw["window"] = 2 * d + 17
+        cnt = np.minimum(lens, kw["window"]).astype(np.int32)
+        kr, vr = np.zeros_like(kc), np.zeros_like(vc)
+        for b in range(w.B):
+            kr[b, :, : cnt[b]], vr[b, :, : cnt[b]] = (x[b, :, lens[b] - cnt[b]: lens[b]] for x in (kc, vc))
+        ref = oracle.decode(q, kr, vr, cnt, w.scale, w.lam)
+    else:
+        ref = oracle.decode(q, np.repeat(kc, H // Hkv, axis=1), np.repeat(vc, H // Hkv, axis=1), lens, w.scale, w.lam)
+    for b in range(w.B):                      # slots past the end may hold anything
+        kc[b, :, lens[b]:] = np.nan
+        vc[b, :, lens[b]:] = np.nan
+    if mode == "paged_gqa":
+        kc, table, max_pages, num_pages = _to_pages(kc, lens, 128, np.random.default_rng(401))
+        vc, _, _, _ = _to_pages(vc, lens, 128, np.random.default_rng(401))
+        kw.update(kv_heads=Hkv, block_table=torch.from_numpy(table).cuda(), page_size=128, max_pages=max_pages, num_pages=num_pages)
+    dq, dk, dv_, dl = dev(q, "bf16"), dev(kc, "bf16"), dev(vc, "bf16"), torch.from_numpy(lens).cuda()
+    nbytes = 4 * w.B * H * splits * (2 * d * d + 2 * d + 4)
+    # with room for the moment records in the workspace, and (one part) without a workspace
+    for ws in [torch.empty(nbytes, dtype=torch.uint8, device="cuda")] + ([None] if splits == 1 else []):
+        status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+        out = torch.full((w.B, H, d), float("nan"), dtype=torch.float32, device="cuda")
+        L.lla_decode_ex(dq, dk, dv_, dl, out, w.B, H, w.n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, splits=splits,
+                        device_status=status, workspace=ws, workspace_bytes=nbytes if ws is not None else 0, stream=stream_ptr(), **kw)
+        torch.cuda.synchronize()
+        err = row_err(out.cpu().numpy(), ref)
+        assert np.isfinite(err).all() and err.max() <= TOL_BF16, (float(err.max()), int(err.argmax()))
+        assert status.cpu().numpy()[L.STATUS_TIMEOUT] == 0
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_solve_falls_back_to_elimination(oracle, d):
+    """Keys on which the conjugate gradients of the solve do not converge within their cap (features scaled over six
+    decades, a tiny ridge): the elimination must take over.  The reference is the oracle's own direct solve; fp32 moments
+    bound what can be asked: the output is an affine fit, so it reproduces values that are affine in the keys."""
+    B, H, n = 2, 2, 700
+    rng = np.random.default_rng(410 + d)
+    sc = np.logspace(0, -3, d).astype(np.float32)
+    kc = inputs.round_to_bf16(rng.standard_normal((B, H, n, d)).astype(np.float32) * sc)
+    q = inputs.round_to_bf16(rng.standard_normal((B, H, d)).astype(np.float32) * sc * 0.5)
+    vc = inputs.round_to_bf16(np.einsum("bhjc,ec->bhje", kc, rng.standard_normal((d, d)).astype(np.float32)) + 1.0)
+    lens = np.array([n, 520], dtype=np.int32)
+    lam = 1e-9
+    ref = oracle.decode(q, kc, vc, lens, 0.1, lam)
+    out = torch.full((B, H, d), float("nan"), dtype=torch.float32, device="cuda")
+    ws = torch.empty(4 * B * H * (2 * d * d + 2 * d + 4), dtype=torch.uint8, device="cuda")
+    L.lla_decode_ex(dev(q, "bf16"), dev(kc, "bf16"), dev(vc, "bf16"), torch.from_numpy(lens).cuda(), out, B, H, n, d, d, 0.1, lam,
+                    out_dtype=L.LLA_F32, splits=1, workspace=ws, workspace_bytes=ws.numel(), stream=stream_ptr())
+    torch.cuda.synchronize()
+    # bf16 operand pairs of w k carry 2^-17 relative error per key, features at 1e-3 of the largest: 1e-2 covers it
+    assert row_err(out.cpu().numpy(), ref).max() <= 1e-2
