@@ -111,7 +111,6 @@ struct alignas(16) SolveSmem {
     float red[2][2 * SvCfg<D>::NW];
     double dred[2 * SvCfg<D>::NW];
     double a[D], c[D], x[D];                 // kbar, vbar, solution
-    double f[DS_MAX_SPLITS];                 // exp(m_p - m) / omega per part
 };
 template <int D>
 __device__ __forceinline__ void sv_sync() { asm volatile("bar.sync 2, %0;" ::"n"(D) : "memory"); }
@@ -130,22 +129,13 @@ __device__ __forceinline__ double sv_sum(double v, SolveSmem<D>& sm) {
     return s;
 }
 
-// entry (j, r) of the centred matrix
-template <int D>
-__device__ __forceinline__ double sv_entry(const float* __restrict__ src, int splits, int j, int r, double ar, double ridge, const SolveSmem<D>& sm) {
-    constexpr int PF = DtCfg<D>::REC;
-    double s = 0.0;
-    for (int p = 0; p < splits; ++p) s += sm.f[p] * (double)src[(size_t)p * PF + j * D + r];
-    return s - sm.a[j] * ar + (j == r ? ridge : 0.0);
-}
-
 // Gaussian elimination without pivoting in fp64 (the matrix is symmetric positive definite), thread r on row r; only
 // for systems on which the conjugate gradients gave up.  Returns false if a pivot was not positive.
 template <int D>
-__device__ __noinline__ bool sv_eliminate(const float* src, int splits, double ridge, double b, SolveSmem<D>& sm, double* prow) {
+__device__ __noinline__ bool sv_eliminate(const float* src, double inv, double ridge, double b, SolveSmem<D>& sm, double* prow) {
     const int r = threadIdx.x;
     double row[D];
-    for (int j = 0; j < D; ++j) row[j] = sv_entry<D>(src, splits, j, r, sm.a[r], ridge, sm);
+    for (int j = 0; j < D; ++j) row[j] = (double)src[j * D + r] * inv - sm.a[j] * sm.a[r] + (j == r ? ridge : 0.0);
     bool ok = true;
     for (int k = 0; k < D; ++k) {
         sv_sync<D>();
@@ -171,8 +161,9 @@ __device__ __noinline__ bool sv_eliminate(const float* src, int splits, double r
     return ok;
 }
 
-// Merge the moment records of one unit's parts at src (global or shared memory), centre, solve and emit the output
-// row.  Called by threads 0 .. D - 1 of a block.
+// Centre the moments of one unit at src (global or shared memory), solve and emit the output row.  With several parts
+// the matrices and first moments at src are already the sums over the parts (decode_merge_kernel), relative to the
+// largest of the parts' maxima; weight and maximum are still those of each part.  Called by threads 0 .. D - 1 of a block.
 template <int D, typename TOut>
 __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qrow, const float* __restrict__ src, int splits, float lambda_u,
                                            int ridge_mode, TOut* __restrict__ orow, int* __restrict__ status, SolveSmem<D>& sm, double* prow) {
@@ -185,50 +176,30 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
     double omega = 0.0;
-    bool bad = false;
-    for (int p = lane; p < splits; p += 32) {
-        const float mp = src[(size_t)p * PF + 2 * D * D + 2 * D + 1];
-        const double f = splits == 1 ? 1.0 : exp((double)mp - (double)m);       // 0 for empty parts
-        bad |= mp != mp;                                                        // poisoned record of an aborted block
-        omega += f * (double)src[(size_t)p * PF + 2 * D * D + 2 * D];
-        if (wp == 0) sm.f[p] = f;
-    }
+    for (int p = lane; p < splits; p += 32)       // (NaN in the record of an aborted block)
+        omega += (double)expf(src[(size_t)p * PF + 2 * D * D + 2 * D + 1] - m) * (double)src[(size_t)p * PF + 2 * D * D + 2 * D];
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) omega += __shfl_xor_sync(0xffffffffu, omega, off);
-    if (__any_sync(0xffffffffu, bad)) omega = __longlong_as_double(0x7ff8000000000000ll);
     const double inv = 1.0 / omega;
     const double lam_u = (double)lambda_u;
     const double ridge = (ridge_mode == LLA_RIDGE_PRINTED ? lam_u : lam_u * exp(-(double)m)) * inv;
-    __syncwarp();
-    if (wp == 0)
-        for (int p = lane; p < splits; p += 32) sm.f[p] *= inv;
-    sv_sync<D>();
-    double ar = 0.0, cb = 0.0;
-    for (int p = 0; p < splits; ++p) {
-        ar += sm.f[p] * (double)src[(size_t)p * PF + 2 * D * D + r];
-        cb += sm.f[p] * (double)src[(size_t)p * PF + 2 * D * D + D + r];
-    }
+    const double ar = (double)src[2 * D * D + r] * inv, cb = (double)src[2 * D * D + D + r] * inv;
     sm.a[r] = ar;
     sv_sync<D>();
     // row r of the centred matrix (column r: M is symmetric up to fp32 rounding and the loads are coalesced)
     uint64_t row[D / 2];
 #pragma unroll
     for (int j = 0; j < D; j += 8) {
-        double s[8];
+        float v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) s[e] = 0.0;
-        for (int p = 0; p < splits; ++p) {
-            const double f = sm.f[p];
+        for (int e = 0; e < 8; ++e) v[e] = src[(j + e) * D + r];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) s[e] += f * (double)src[(size_t)p * PF + (j + e) * D + r];
+        for (int e = 0; e < 8; e += 2) {
+            double s0 = (double)v[e] * inv - sm.a[j + e] * ar, s1 = (double)v[e + 1] * inv - sm.a[j + e + 1] * ar;
+            if (j + e == r) s0 += ridge;
+            if (j + e + 1 == r) s1 += ridge;
+            row[(j + e) / 2] = pk2((float)s0, (float)s1);
         }
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            s[e] -= sm.a[j + e] * ar;
-            if (j + e == r) s[e] += ridge;
-        }
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) row[(j + e) / 2] = pk2((float)s[e], (float)s[e + 1]);
     }
     const double b = (double)to_f32(qrow[r]) - ar;
     double x = 0.0, res = b;
@@ -290,41 +261,30 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
         sm.x[r] = x;
         sv_sync<D>();
         double s0 = 0.0, s1 = 0.0;
-        for (int p = 0; p < splits; ++p) {
-            const double f = sm.f[p];
-            double t0 = 0.0, t1 = 0.0;
-#pragma unroll 8
-            for (int j = 0; j < D; j += 2) {
-                t0 += (double)src[(size_t)p * PF + j * D + r] * sm.x[j];
-                t1 += (double)src[(size_t)p * PF + (j + 1) * D + r] * sm.x[j + 1];
-            }
-            s0 += f * t0;
-            s1 += f * t1;
+#pragma unroll 4
+        for (int j = 0; j < D; j += 2) {
+            s0 += (double)src[j * D + r] * sm.x[j];
+            s1 += (double)src[(j + 1) * D + r] * sm.x[j + 1];
         }
         const double ax = sv_sum<D>(ar * x, sm);
-        res = b - ((s0 + s1) - ar * ax + ridge * x);
+        res = b - ((s0 + s1) * inv - ar * ax + ridge * x);
         const double rr2 = sv_sum<D>(res * res, sm);
         done = rr2 <= stop_all;
         if (!conv || !(rr2 < 0.25 * rr)) break;      // no progress
         rr = rr2;
     }
     bool solved = true;
-    if (!done) solved = sv_eliminate<D>(src, splits, ridge, b, sm, prow);      // uniform: the decision comes from block-wide sums
+    if (!done) solved = sv_eliminate<D>(src, inv, ridge, b, sm, prow);      // uniform: the decision comes from block-wide sums
     // o_e = vbar_e + sum_f (N[e][f] / omega - vbar_e kbar_f) y_f
     const double yv = done ? x : sm.x[r];
-    if (done) sm.x[r] = x;
     const double ky = sv_sum<D>(ar * yv, sm);
-    double o = 0.0;
-    for (int p = 0; p < splits; ++p) {
-        double t0 = 0.0, t1 = 0.0;
+    double o0 = 0.0, o1 = 0.0;
 #pragma unroll 8
-        for (int j = 0; j < D; j += 2) {
-            t0 += (double)src[(size_t)p * PF + D * D + j * D + r] * sm.x[j];
-            t1 += (double)src[(size_t)p * PF + D * D + (j + 1) * D + r] * sm.x[j + 1];
-        }
-        o += sm.f[p] * (t0 + t1);
+    for (int j = 0; j < D; j += 2) {
+        o0 += (double)src[D * D + j * D + r] * sm.x[j];
+        o1 += (double)src[D * D + (j + 1) * D + r] * sm.x[j + 1];
     }
-    store_out(orow + r, (float)(o + cb * (1.0 - ky)));
+    store_out(orow + r, (float)((o0 + o1) * inv + cb * (1.0 - ky)));
     if (r == 0 && status) {
         atomicAdd(status + LLA_STATUS_ITER_SUM, its);
         if (!solved) atomicAdd(status + LLA_STATUS_BAD_PIVOT, 1);
@@ -804,7 +764,41 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
 }
 
-// Second kernel of the two-kernel decode.  Several blocks share an SM; the solve is latency-bound (barriers and
+// Sum of the parts' moments of one unit into the record of its first part, each scaled to the largest of their maxima
+// (the parts' weights and maxima stay as they are).  Split calls are small ones, which leave most of the chip idle:
+// merging in the solve kernel, whose few blocks would read every part through 64 threads, made that kernel 42 us long
+// at one sequence x 16 heads, d = 64, 8 parts; now 4 us here and 10 us there.
+constexpr int DM_THREADS = 256;
+template <int D>
+__global__ void __launch_bounds__(DM_THREADS)
+decode_merge_kernel(float* __restrict__ parts, const int* __restrict__ lens, int H, int Lmax, int head_rows, int splits, int window) {
+    constexpr int PF = DtCfg<D>::REC;
+    __shared__ float s_f[DS_MAX_SPLITS];
+    const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");      // a programmatic dependent of the streaming kernel
+    if (visible_keys(lens[bh / H], Lmax, window) < head_rows) return;
+    float* src = parts + (size_t)bh * splits * PF;
+    if (tid < 32) {
+        float m = -INFINITY;
+        for (int p = lane; p < splits; p += 32) m = fmaxf(m, src[(size_t)p * PF + 2 * D * D + 2 * D + 1]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, off));
+        for (int p = lane; p < splits; p += 32) s_f[p] = expf(src[(size_t)p * PF + 2 * D * D + 2 * D + 1] - m);      // 0 for empty parts
+    }
+    __syncthreads();
+    const int e = blockIdx.x * DM_THREADS + tid;
+    if (e >= (2 * D * D + 2 * D) / 4) return;
+    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+#pragma unroll 8
+    for (int p = 0; p < splits; ++p) {
+        const float4 v = reinterpret_cast<const float4*>(src + (size_t)p * PF)[e];
+        const double f = (double)s_f[p];
+        a0 += f * (double)v.x; a1 += f * (double)v.y; a2 += f * (double)v.z; a3 += f * (double)v.w;
+    }
+    reinterpret_cast<float4*>(src)[e] = make_float4((float)a0, (float)a1, (float)a2, (float)a3);
+}
+
+// Last kernel of the decode with a record buffer.  Several blocks share an SM; the solve is latency-bound (barriers and
 // shuffles), which is why it is kept out of the streaming kernel whenever there is a record buffer.
 template <int D, typename TOut>
 __global__ void __launch_bounds__(D, D == 64 ? 8 : 2)
@@ -860,6 +854,15 @@ int launch_t(const DecodeArgs& a) {
     cfg.attrs = attr;
     cfg.numAttrs = a.behind_direct ? 1 : 0;
     LLA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mk, mv, (const __nv_bfloat16*)a.q, (TOut*)a.out, prm));
+    if (splits > 1) {
+        cudaLaunchConfig_t cm = {};
+        cm.gridDim = dim3(((2 * D * D + 2 * D) / 4 + DM_THREADS - 1) / DM_THREADS, BH);
+        cm.blockDim = dim3(DM_THREADS);
+        cm.stream = a.stream;
+        cm.attrs = attr;
+        cm.numAttrs = 1;
+        LLA_CUDA_TRY(cudaLaunchKernelEx(&cm, decode_merge_kernel<D>, (float*)a.workspace, a.lens, a.H, a.Lmax, a.head_rows, splits, a.window));
+    }
     if (have_ws) {
         cudaLaunchConfig_t cs = {};
         cs.gridDim = dim3(BH);
