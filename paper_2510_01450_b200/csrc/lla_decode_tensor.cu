@@ -7,13 +7,13 @@
 // Per tile of 64 keys, each role at its own pace, coupled by mbarriers only:
 //   TMA         K and V tiles -> 128B-swizzled shared memory, where they are the MN-major B operand as they arrive:
 //               nothing is written to shared memory by a thread except the weights.
-//   4 warps     scores and weights (d / 32 lanes per key), weights to shared memory; omega
+//   4 or 8 warps  scores and weights (d / 32 lanes per key), weights to shared memory; omega (and c at d = 128)
 //   4 or 8 warps  the A operand: a key (or value) tile is read transposed (ldmatrix.trans), scaled by the weights and
-//               stored to TMEM as bf16 hi + lo (hi truncated, lo rounded: 16 to 17 mantissa bits).  The fragment that
-//               ldmatrix.trans leaves in a thread -- feature lane / 4, keys 2 (lane % 4), + 1 -- is the one that
-//               tcgen05.st.16x128b stores.  Row sums of the operand are the first moments.
-//   MMA (TS)    d = 64 : A = [wK ; wV]^T (128 rows), B = K (N = 64):        D = [M ; N]
-//               d = 128: A = [wK]^T,                 B = [K | V] (N = 256): D = [M | N^T]; c on the score warps
+//               stored to TMEM as bf16 hi + lo (16 to 17 mantissa bits).  The fragment that ldmatrix.trans leaves in a
+//               thread -- feature lane / 4, keys 2 (lane % 4), + 1 -- is the one that tcgen05.st.16x128b stores, and the
+//               products are formed on those packed pairs.
+//   MMA (TS)    d = 64 : A = [wK ; wV]^T (128 rows), B = [K | 1] (N = 80):  D = [M a ; N c]
+//               d = 128: A = [wK]^T,                 B = [K | V] (N = 256): D = [M | N^T]; a, c on the CUDA cores
 //
 // Why this form: the earlier kernel had [K^T ; V^T] as A and the weighted keys as B, written to shared memory by the
 // threads: 80 KB of shared-memory traffic per 16 KB of cache, and one chain of dependent phases per tile.  Here it is
@@ -39,38 +39,45 @@ struct DtCfg {
     static constexpr int NSUB = D / 64;                    // 64-column sub-tiles of K (and of V) in a stage
     static constexpr int SUB = DT_BK * 128;                // bytes of a sub-tile
     static constexpr int STAGE = 2 * NSUB * SUB;           // K tile, V tile
-    static constexpr int NST = 6;                          // ring stages: 96 KB and two blocks per SM at d = 64, 192 KB and one at d = 128
-    static constexpr int TC_A = D == 64 ? 64 : 256;        // first TMEM column behind the accumulator
-    static constexpr int NAB = D == 64 ? 3 : 4;            // A operand buffers, 64 columns each (hi 32, lo 32)
-    static constexpr int TMEM = TC_A + 64 * NAB;
-    static constexpr uint32_t IDESC = make_idesc(128, TC_A, 0, 1);
+    static constexpr int NST = D == 64 ? 5 : 6;            // ring stages: 80 KB and two blocks per SM at d = 64, 192 KB and one at d = 128
+    static constexpr int NMMA = D == 64 ? 80 : 256;        // accumulator columns (d = 64: a ones column at 64, padded to 16)
+    static constexpr int TC_A = D == 64 ? 96 : 256;        // first TMEM column of the A operand buffers
+    static constexpr int NAB = D == 64 ? 2 : 4;            // these buffers, 64 columns each (hi 32, lo 32)
+    static constexpr int TMEM = D == 64 ? 256 : 512;
+    static_assert(TC_A + 64 * NAB <= TMEM, "TMEM");
+    static constexpr uint32_t IDESC = make_idesc(128, NMMA, 0, 1);
+    static constexpr int NSW = D / 16;                     // score warps: 16 keys of the tile each at d = 64, 8 at d = 128
+    static constexpr int KPW = DT_BK / NSW;                // (d / 32 lanes per key)
     static constexpr int NBG = D / 64;                     // groups of four operand warps; they take the tiles in turn
-    static constexpr int W_TMA = 4 + 4 * NBG;              // warps 0..3: scores; 4 .. W_TMA - 1: operand; then TMA, MMA
+    static constexpr int W_TMA = NSW + 4 * NBG;            // warps: scores, operand, TMA, MMA
     static constexpr int THREADS = 32 * (W_TMA + 2);
-    static constexpr int KPP = 1024 / D;                   // keys per warp and score pass (d / 32 lanes per key)
-    static constexpr int PASSES = DT_BK / (4 * KPP);       // score passes of a warp per tile
     static constexpr int REC = 2 * D * D + 2 * D + 4;      // floats of a moment record: M, N^T, a, c, omega, m, 2 pad
-    static constexpr int SM_BAR = NST * STAGE;
+    static constexpr int SM_ONES = NST * STAGE;            // d = 64: a tile of 64 rows whose column 0 is 1 and the rest 0
+    static constexpr int SM_BAR = SM_ONES + (D == 64 ? SUB : 0);
     static constexpr int SM_MISC = SM_BAR + 256;           // tmem base, abort, repeat flag, warp maxima
-    static constexpr int SM_W = SM_MISC + 128;             // NST x 64 weights
-    static constexpr int SM_TOTAL = SM_W + NST * DT_BK * 4;
+    static constexpr int SM_W = SM_MISC + 128;             // NST x 64 weights as bf16 pairs: per two keys hi, hi, lo, lo
+    static constexpr int SM_WF = SM_W + NST * DT_BK * 4;   // NST x 64 weights, fp32
+    static constexpr int SM_TOTAL = SM_WF + (D == 128 ? NST * DT_BK * 4 : 0);
     static constexpr int SM_ALLOC = SM_TOTAL + 1024;
     enum { KVFULL = 0, KVEMPTY = KVFULL + NST, WFULL = KVEMPTY + NST, AFULL = WFULL + NST, AFREE = AFULL + NAB,
            DFULL = AFREE + NAB, PASS = DFULL + 2, EXIT = PASS + 1, NBAR = EXIT + 1 };
     static_assert(NBAR * 8 <= 256, "barrier area too small");
-    static_assert((TMEM & (TMEM - 1)) == 0, "TMEM allocations are powers of two");
 };
 
 // D += A_hi B, D += A_lo B over 64 keys.  B is MN-major, 128B swizzle: 64-column groups one sub-tile apart (leading
 // byte offset), 8-key groups 1024 bytes apart; a 16-key step is 2048 bytes (128 descriptor units) and 8 columns of A.
+// At d = 64 the second column group is the ones tile, so that column 64 of D is the row sum of the operand.
 template <int D>
-__device__ __forceinline__ void mma_tile(uint32_t el, uint32_t d, uint32_t a, uint32_t kv_smem, bool first) {
+__device__ __forceinline__ void mma_tile(uint32_t el, uint32_t d, uint32_t a, uint32_t kv_smem, uint32_t ones, bool first) {
     using C = DtCfg<D>;
-    const uint64_t b = make_desc(kv_smem, C::SUB);
+    const uint64_t b = make_desc(kv_smem, D == 64 ? ones - kv_smem : (uint32_t)C::SUB);
     mma_ts_k64c(el, d, a, b, C::IDESC, first ? 0u : 1u);
     mma_ts_k64c(el, d, a + 32, b, C::IDESC, 1u);
 }
 
+// packed bf16 arithmetic
+__device__ __forceinline__ uint32_t mul_bf2(uint32_t a, uint32_t b) { uint32_t r; asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b)); return r; }
+__device__ __forceinline__ uint32_t fma_bf2(uint32_t a, uint32_t b, uint32_t c) { uint32_t r; asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(c)); return r; }
 // four 8 x 8 blocks of 16-bit elements, each transposed: lane l gets row l / 4, columns 2 (l % 4) and + 1 of every block
 __device__ __forceinline__ void ldsm4_t(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -318,7 +325,7 @@ __global__ void __launch_bounds__(DtCfg<D>::THREADS, D == 64 ? 2 : 1)
 decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                  const __nv_bfloat16* __restrict__ q, TOut* __restrict__ out, const DtParams prm) {
     using C = DtCfg<D>;
-    constexpr int BK = DT_BK, NST = C::NST, NAB = C::NAB, NBG = C::NBG, W_TMA = C::W_TMA, W_MMA = W_TMA + 1;
+    constexpr int BK = DT_BK, NST = C::NST, NAB = C::NAB, NBG = C::NBG, NSW = C::NSW, W_TMA = C::W_TMA, W_MMA = W_TMA + 1;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = smem_u32(smem);
@@ -326,8 +333,9 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     auto bar = [&](int i) { return bars + 8u * i; };
     volatile int* misc = reinterpret_cast<volatile int*>(smem + C::SM_MISC);   // [0] tmem base, [1] abort, [2] repeat the pass
     volatile int* abort_flag = misc + 1;
-    volatile float* tmax = reinterpret_cast<volatile float*>(smem + C::SM_MISC + 16);   // 2 x 4 warp maxima
-    float* wbuf = reinterpret_cast<float*>(smem + C::SM_W);
+    volatile float* tmax = reinterpret_cast<volatile float*>(smem + C::SM_MISC + 16);   // 2 x 8 warp maxima
+    uint8_t* wbuf = smem + C::SM_W;
+    float* wfbuf = reinterpret_cast<float*>(smem + C::SM_WF);
     const long long wcap = prm.wait_clocks;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -365,17 +373,25 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             mbar_init(bar(C::KVFULL + s), 1);
-            mbar_init(bar(C::KVEMPTY + s), D == 64 ? 1 : 5);      // d = 128: the score warps read V after the weights
-            mbar_init(bar(C::WFULL + s), 4);
+            mbar_init(bar(C::KVEMPTY + s), D == 64 ? 1 : 1 + NSW);      // d = 128: the score warps read V after the weights
+            mbar_init(bar(C::WFULL + s), NSW);
         }
         for (int b = 0; b < NAB; ++b) { mbar_init(bar(C::AFULL + b), 4); mbar_init(bar(C::AFREE + b), 1); }
         mbar_init(bar(C::DFULL), 1);              // the accumulator is complete: one barrier per pass
         mbar_init(bar(C::DFULL + 1), 1);
-        mbar_init(bar(C::PASS), 4);
+        mbar_init(bar(C::PASS), NSW);
         mbar_init(bar(C::EXIT), 1);
         misc[1] = 0;
         misc[2] = 0;      // set by the score warps when the pass has to be repeated
         fence_barrier_init();
+    }
+    if (D == 64) {
+        // (column 0 of row r is the first element of its chunk 0, which the 128-byte swizzle puts at chunk r % 8)
+        for (int e = tid; e < C::SUB / 16; e += C::THREADS) {
+            const int row = e >> 3;
+            *reinterpret_cast<uint4*>(smem + C::SM_ONES + 16 * e) = make_uint4((e & 7) == (row & 7) ? 0x3F80u : 0u, 0u, 0u, 0u);
+        }
+        fence_proxy_async();
     }
     if (warp == W_TMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -388,9 +404,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     const uint32_t tmem = (uint32_t)misc[0];
 
     float omega = 0.f, m_ref = -INFINITY;     // score warps; m_ref in log2 units
-    // operand warps: sums of w x over the keys for the features 16 g + lane / 4 (+ 8) of this warp's lanes, even and odd
-    // keys apart (x = k, at d = 64 in warps 2 and 3 of a group v); score warps at d = 128: w v for the eight features of
-    // this thread's chunk
+    // d = 128 only.  Operand warps: sum of w k for the features 16 g + lane / 4 (+ 8) of this warp's lanes, even and odd
+    // keys apart; score warps: sum of w v for the eight features of this thread's chunk
     uint64_t sums[2][2] = {{0ull, 0ull}, {0ull, 0ull}};
 
     if (warp == W_TMA) {
@@ -440,7 +455,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (!mbar_wait(bar(C::KVFULL + s), (g / NST) & 1, abort_flag, wcap)) { okp = false; break; }
                 if (!mbar_wait(bar(C::AFULL + b), (g / NAB) & 1, abort_flag, wcap)) { okp = false; break; }
                 tc_fence_after();
-                mma_tile<D>(el, tmem, tmem + C::TC_A + 64 * b, sbase + s * C::STAGE, t == 0);     // t == 0 overwrites
+                mma_tile<D>(el, tmem, tmem + C::TC_A + 64 * b, sbase + s * C::STAGE, sbase + C::SM_ONES, t == 0);     // t == 0 overwrites
                 tc_commit_el(el, bar(C::KVEMPTY + s));
                 tc_commit_el(el, bar(C::AFREE + b));
                 if (t == ntile - 1) tc_commit_el(el, bar(C::DFULL + pass));
@@ -451,14 +466,23 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             tc_commit_el(el, bar(C::EXIT));
             (void)mbar_wait_landed(bar(C::EXIT), 0, wcap);
         }
-    } else if (warp < 4) {
+    } else if (warp < NSW) {
         // ================================ score warps ================================
-        // A warp takes 16 keys of the tile, KPP in a pass: key j0 + KPP * u, features 32 h .. 32 h + 31.  The eight lanes
-        // that share a 128-byte shared-memory wavefront have the same h and neighbouring keys, so the swizzled chunks
-        // never collide.
-        constexpr int KPP = C::KPP, PASSES = C::PASSES, CH = D / 8;
-        const int h = lane / KPP, j0 = warp * 16 + lane % KPP;
-        const uint32_t krow = (h >> 1) * C::SUB + j0 * 128;
+        // Key j of the tile, features 32 h .. 32 h + 31.  The eight lanes that share a 128-byte shared-memory wavefront have
+        // the same h and neighbouring keys, so the swizzled chunks never collide.
+        constexpr int KPW = C::KPW, CH = D / 8;
+        const int h = lane / KPW, j = warp * KPW + lane % KPW;
+        auto max_over_warps = [&](volatile float* tm, float v) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+            if (lane == 0) tm[warp] = v;
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * NSW) : "memory");
+            v = tm[0];
+#pragma unroll
+            for (int i = 1; i < NSW; ++i) v = fmaxf(v, tm[i]);
+            return v;
+        };
+        const uint32_t krow = (h >> 1) * C::SUB + j * 128;
         const float c1 = prm.scale * 1.4426950408889634f;
         uint64_t qv[16];
         {
@@ -488,62 +512,49 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 const int g = g0 + t, sl = g % NST;
                 ok = mbar_wait(bar(C::KVFULL + sl), (g / NST) & 1, abort_flag, wcap);
                 ok = __all_sync(0xffffffffu, ok);              // what follows is warp-wide
-                if (t == 0) ok = !bar_or(1, 128, !ok);         // and for the first tile takes all four warps
+                if (t == 0) ok = !bar_or(1, 32 * NSW, !ok);    // and for the first tile takes all score warps
                 if (!ok) break;
                 uint8_t* stage = smem + sl * C::STAGE;
-                float s2[PASSES];
-                bool valid[PASSES];
+                uint8_t* ks = stage + krow;
+                uint64_t sd[4] = {0ull, 0ull, 0ull, 0ull};      // four independent chains of pairs
 #pragma unroll
-                for (int u = 0; u < PASSES; ++u) {
-                    uint8_t* ks = stage + krow + u * KPP * 128;
-                    uint64_t sd[4] = {0ull, 0ull, 0ull, 0ull};      // four independent chains of pairs
+                for (int i = 0; i < 4; ++i) {
+                    const uint4 raw = *reinterpret_cast<const uint4*>(ks + (((4 * (h & 1) + i) ^ (j & 7)) << 4));
+                    const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        sd[e] = fma2(qv[4 * i + e], pk2(__uint_as_float(wds[e] << 16), __uint_as_float(wds[e] & 0xFFFF0000u)), sd[e]);
+                }
+                float a0, a1;
+                upk2(add2(add2(sd[0], sd[1]), add2(sd[2], sd[3])), a0, a1);
+                float s2 = a0 + a1;
+#pragma unroll
+                for (int off = KPW; off < 32; off <<= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
+                const bool valid = jbeg + t * BK + j < jend;
+                if (!valid) {
+                    // ragged last tile: rows past the end may hold anything (unused cache slots).  They are
+                    // operands, so clear them (0 x NaN would poison the accumulator).
+                    s2 = -INFINITY;
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const uint4 raw = *reinterpret_cast<const uint4*>(ks + (((4 * (h & 1) + i) ^ (j0 & 7)) << 4));
-                        const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            sd[e] = fma2(qv[4 * i + e], pk2(__uint_as_float(wds[e] << 16), __uint_as_float(wds[e] & 0xFFFF0000u)), sd[e]);
+                        const uint32_t off = ((4 * (h & 1) + i) ^ (j & 7)) << 4;
+                        *reinterpret_cast<uint4*>(ks + off) = make_uint4(0, 0, 0, 0);
+                        *reinterpret_cast<uint4*>(ks + C::NSUB * C::SUB + off) = make_uint4(0, 0, 0, 0);
                     }
-                    float a0, a1;
-                    upk2(add2(add2(sd[0], sd[1]), add2(sd[2], sd[3])), a0, a1);
-                    s2[u] = a0 + a1;
-#pragma unroll
-                    for (int off = KPP; off < 32; off <<= 1) s2[u] += __shfl_xor_sync(0xffffffffu, s2[u], off);
-                    valid[u] = jbeg + t * BK + j0 + u * KPP < jend;
-                    if (!valid[u]) {
-                        // ragged last tile: rows past the end may hold anything (unused cache slots).  They are
-                        // operands, so clear them (0 x NaN would poison the accumulator).
-                        s2[u] = -INFINITY;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const uint32_t off = ((4 * (h & 1) + i) ^ (j0 & 7)) << 4;
-                            *reinterpret_cast<uint4*>(ks + off) = make_uint4(0, 0, 0, 0);
-                            *reinterpret_cast<uint4*>(ks + C::NSUB * C::SUB + off) = make_uint4(0, 0, 0, 0);
-                        }
-                        fence_proxy_async();
-                    }
+                    fence_proxy_async();
                 }
-                if (t == 0 && pass == 0) {
-                    float wm = s2[0];
-#pragma unroll
-                    for (int u = 1; u < PASSES; ++u) wm = fmaxf(wm, s2[u]);
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, off));
-                    if (lane == 0) tmax[warp] = wm;
-                    asm volatile("bar.sync 1, 128;" ::: "memory");
-                    m_ref = fmaxf(fmaxf(tmax[0], tmax[1]), fmaxf(tmax[2], tmax[3]));
-                }
-                float* wt = wbuf + sl * BK;
-#pragma unroll
-                for (int u = 0; u < PASSES; ++u) {
-                    run_max = fmaxf(run_max, s2[u]);
-                    over |= s2[u] > m_ref + 90.f;
-                    const float w = valid[u] ? ex2f(fminf(s2[u] - m_ref, 100.f)) : 0.f;
-                    if (h == 0) {
-                        omega += w;
-                        wt[j0 + u * KPP] = w;
-                    }
+                if (t == 0 && pass == 0) m_ref = max_over_warps(tmax, s2);
+                run_max = fmaxf(run_max, s2);
+                over |= s2 > m_ref + 90.f;
+                const float w = valid ? ex2f(fminf(s2 - m_ref, 100.f)) : 0.f;
+                if (h == 0) {
+                    omega += w;
+                    const __nv_bfloat16 whi = __float2bfloat16_rn(w);
+                    const __nv_bfloat16 wlo = __float2bfloat16_rn(w - __bfloat162float(whi));
+                    __nv_bfloat16* wj = reinterpret_cast<__nv_bfloat16*>(wbuf + sl * BK * 4 + (j >> 1) * 8) + (j & 1);
+                    wj[0] = whi;
+                    wj[2] = wlo;
+                    if (D == 128) wfbuf[sl * BK + j] = w;
                 }
                 // one arrival per warp: 32 lanes arriving on one mbarrier are 32 serialised shared-memory atomics
                 __syncwarp();
@@ -551,12 +562,12 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if constexpr (D == 128) {
                     const int vchunk = lane % CH;
                     const uint8_t* vs = stage + (C::NSUB + (vchunk >> 3)) * C::SUB;
+                    const float* wt = wfbuf + sl * BK;
 #pragma unroll
-                    for (int i = 0; i < 16 * CH / 32; ++i) {
-                        const int key = warp * 16 + lane / CH + 32 / CH * i;
+                    for (int i = 0; i < KPW * CH / 32; ++i) {
+                        const int key = warp * KPW + lane / CH + 32 / CH * i;
                         const uint4 x = *reinterpret_cast<const uint4*>(vs + key * 128 + (((vchunk & 7) ^ (key & 7)) << 4));
-                        const float w = wt[key];
-                        const uint64_t w2 = pk2(w, w);
+                        const uint64_t w2 = pk2(wt[key], wt[key]);
                         sums[0][0] = fma2(w2, pk2(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xFFFF0000u)), sums[0][0]);
                         sums[0][1] = fma2(w2, pk2(__uint_as_float(x.y << 16), __uint_as_float(x.y & 0xFFFF0000u)), sums[0][1]);
                         sums[1][0] = fma2(w2, pk2(__uint_as_float(x.z << 16), __uint_as_float(x.z & 0xFFFF0000u)), sums[1][0]);
@@ -567,21 +578,15 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 }
             }
             // end of a pass.  (A warp whose wait failed still takes part in the barriers; all warps leave together.)
-            if (bar_or(1, 128, !ok) || pass == 1) break;
+            if (bar_or(1, 32 * NSW, !ok) || pass == 1) break;
             // did any score leave the range of the reference?  (one barrier per pass)
-            const bool any = bar_or(1, 128, over);
-            if (any) {
-                float wm = run_max;
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, off));
-                if (lane == 0) tmax[4 + warp] = wm;
-            }
+            const bool any = bar_or(1, 32 * NSW, over);
             if (tid == 0) misc[2] = (int)any;
-            asm volatile("bar.sync 1, 128;" ::: "memory");
             if (any) {
-                m_ref = fmaxf(fmaxf(tmax[4], tmax[5]), fmaxf(tmax[6], tmax[7]));
+                m_ref = max_over_warps(tmax + 8, run_max);
                 over = false;
             }
+            asm volatile("bar.sync 1, %0;" ::"n"(32 * NSW) : "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(C::PASS));      // the other warps read misc[2] after this
             if (!any) break;
@@ -593,7 +598,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         // ================================ operand warps ================================
         // Warp w stores to TMEM lanes 32 (w % 4) .. + 31.  d = 128: the features of that number of the keys; d = 64: lanes
         // 0 .. 63 the keys' features, 64 .. 127 the values'.  The groups of four warps take the tiles in turn.
-        const int quad = warp & 3, grp = (warp >> 2) - 1;
+        const int quad = warp & 3, grp = (warp - NSW) >> 2;
         const uint32_t src0 = D == 64 ? (quad >> 1) * C::NSUB * C::SUB : (quad >> 1) * C::SUB;
         // ldmatrix: lanes 8 m .. 8 m + 7 address matrix m; matrices (key group, chunk), (same, chunk + 1), (next, ..)
         const uint32_t lrow = 8 * (lane >> 4) + (lane & 7);
@@ -613,25 +618,30 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t tile = sbase + sl * C::STAGE + src0 + lrow * 128;
-                const float* wt = wbuf + sl * BK;
-                uint64_t ww[8];
+                const uint8_t* wp = wbuf + sl * BK * 4 + 8 * (lane & 3);
+                uint2 ww[8];                                 // the weights of keys 8 kg + 2 (lane % 4), + 1: hi pair, lo pair
 #pragma unroll
-                for (int kg = 0; kg < 8; ++kg) ww[kg] = *reinterpret_cast<const uint64_t*>(wt + 8 * kg + 2 * (lane & 3));
+                for (int kg = 0; kg < 8; ++kg) ww[kg] = *reinterpret_cast<const uint2*>(wp + 32 * kg);
 #pragma unroll
                 for (int fg = 0; fg < 2; ++fg) {             // 16 features at a time
                     const uint32_t base = tile + (((lchunk + 2 * fg) ^ (lane & 7)) << 4);
                     uint32_t r[16], lo[16];
 #pragma unroll
                     for (int kg = 0; kg < 8; kg += 2) ldsm4_t(base + kg * 1024, r[2 * kg], r[2 * kg + 1], r[2 * kg + 2], r[2 * kg + 3]);
+                    if constexpr (D == 128) {
+                    const float* wt = wfbuf + sl * BK + 2 * (lane & 3);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        sums[fg][i & 1] = fma2(*reinterpret_cast<const uint64_t*>(wt + 8 * (i >> 1)),
+                                               pk2(__uint_as_float(r[i] << 16), __uint_as_float(r[i] & 0xFFFF0000u)), sums[fg][i & 1]);
+                    }
+                    // w k = (w_hi + w_lo) k with bf16 w_hi, w_lo: hi = round(w_hi k); w_hi k - hi fits bf16 exactly;
+                    // lo = round(w_lo k + that).  Relative error of hi + lo about 2^-17, three instructions per two keys.
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
-                        const uint64_t p = mul2(ww[i >> 1], pk2(__uint_as_float(r[i] << 16), __uint_as_float(r[i] & 0xFFFF0000u)));
-                        sums[fg][i & 1] = add2(sums[fg][i & 1], p);
-                        float p0, p1, l0, l1;
-                        upk2(p, p0, p1);
-                        r[i] = __byte_perm(__float_as_uint(p0), __float_as_uint(p1), 0x7632);
-                        upk2(sub2(p, pk2(__uint_as_float(__float_as_uint(p0) & 0xFFFF0000u), __uint_as_float(__float_as_uint(p1) & 0xFFFF0000u))), l0, l1);
-                        lo[i] = pack_bf16(l1, l0);
+                        const uint32_t hi = mul_bf2(ww[i >> 1].x, r[i]);
+                        lo[i] = fma_bf2(ww[i >> 1].y, r[i], fma_bf2(ww[i >> 1].x, r[i], hi ^ 0x80008000u));
+                        r[i] = hi;
                     }
                     const uint32_t at = lane_addr + ((uint32_t)(16 * fg) << 16) + 64 * b;
                     tmem_st_16x128(at, r);
@@ -647,13 +657,13 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
 
     // ================================ epilogue ================================
-    if (warp < 8 && ntile > 0) {
+    if (warp < W_TMA && ntile > 0) {
         (void)mbar_wait(bar(C::DFULL + (misc[2] ? 1 : 0)), 0, abort_flag, wcap);
         tc_fence_after();
     }
-    __shared__ float s_omega[4];
+    __shared__ float s_omega[8];
     __shared__ float s_mref;
-    if (warp < 4 && lane == 0) s_omega[warp] = omega;
+    if (warp < NSW && lane == 0) s_omega[warp] = omega;
     if (tid == 0) s_mref = m_ref;
     __syncthreads();       // every pipeline stage is drained: shared memory can be re-carved
     const bool aborted = *abort_flag != 0;
@@ -678,9 +688,9 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     }
     // shared memory now: partial first moments, then (without a workspace) the record
     float* s_fa = reinterpret_cast<float*>(smem);                        // [NBG][128]
-    float* s_fc = s_fa + NBG * 128;                                      // [4][D]  (d = 128)
+    float* s_fc = s_fa + NBG * 128;                                      // [NSW][D]  (d = 128)
     float* s_rec = reinterpret_cast<float*>(smem + 8192);                // REC floats
-    if (warp < 4) {
+    if (warp < NSW) {
         if constexpr (D == 128) {
             float cs[8];
 #pragma unroll
@@ -691,7 +701,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 if (lane < 16) s_fc[warp * D + 8 * lane + i] = cs[i];
             }
         }
-    } else if (warp < W_TMA) {
+    } else if (D == 128 && warp < W_TMA) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             float e0, e1;
@@ -699,22 +709,24 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             float s = e0 + e1;
             s += __shfl_xor_sync(0xffffffffu, s, 1);
             s += __shfl_xor_sync(0xffffffffu, s, 2);
-            if ((lane & 3) == 0) s_fa[((warp >> 2) - 1) * 128 + 32 * (warp & 3) + 16 * (i >> 1) + 8 * (i & 1) + (lane >> 2)] = s;
+            if ((lane & 3) == 0) s_fa[((warp - NSW) >> 2) * 128 + 32 * (warp & 3) + 16 * (i >> 1) + 8 * (i & 1) + (lane >> 2)] = s;
         }
     }
     __syncthreads();
-    const float omega_tot = (s_omega[0] + s_omega[1]) + (s_omega[2] + s_omega[3]);
+    float omega_tot = 0.f;
+#pragma unroll
+    for (int i = 0; i < NSW; ++i) omega_tot += s_omega[i];
     const float mref_ln = s_mref * 0.6931471805599453f;          // back to natural-log units
     const bool rec_ok = LLA_IN_BOUNDS((size_t)bh * prm.splits + part, (size_t)gridDim.y * prm.splits, prm.status, 501);
     float* dst = prm.parts ? prm.parts + ((size_t)bh * prm.splits + part) * C::REC : s_rec;
-    if (warp < 8 && rec_ok) {
-        const int quad = warp & 3, half = warp >> 2;
+    if (warp < W_TMA && rec_ok) {
+        const int quad = warp & 3, cg = warp >> 2;          // TMEM lanes 32 quad .. + 31; columns in 2 or 4 groups
         const int f = 32 * quad + lane;
+        constexpr int CPG = D / 2;                            // columns of a group: 32 or 64
         // d = 64: lane f, column c: M[f][c] (f < 64) or N[f - 64][c], stored transposed: both blocks are [c][lane];
         // d = 128: columns 0 .. 127 M[f][c], stored as [c][f]; columns 128 .. 255 N[c - 128][f], stored as [f][c - 128]
 #pragma unroll 1
-        for (int cb = 0; cb < C::TC_A / 2; cb += 32) {
-            const int c0 = C::TC_A / 2 * half + cb;
+        for (int c0 = CPG * cg; c0 < CPG * cg + CPG; c0 += 32) {
             uint32_t v[32];
             if (ntile > 0) {
                 tmem_ld32(tmem + ((uint32_t)(32 * quad) << 16) + c0, v);
@@ -723,7 +735,7 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 #pragma unroll
                 for (int e = 0; e < 32; ++e) v[e] = 0u;
             }
-            if (D == 128 && half == 1) {
+            if (D == 128 && c0 >= 128) {
 #pragma unroll
                 for (int e = 0; e < 32; e += 4)
                     *reinterpret_cast<uint4*>(dst + (size_t)D * D + f * D + (c0 - 128) + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
@@ -734,12 +746,21 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             }
         }
         if (D == 64) {
-            if (tid < 128) dst[2 * D * D + tid] = s_fa[tid];      // a then c
+            if (cg == 0) {                                       // column 64: a then c
+                uint32_t v[16] = {0u};
+                if (ntile > 0) {
+                    tmem_ld16(tmem + ((uint32_t)(32 * quad) << 16) + 64, v);
+                    tc_wait_ld();
+                }
+                dst[2 * D * D + tid] = __uint_as_float(v[0]);
+            }
         } else if (tid < D) {
             dst[2 * D * D + tid] = s_fa[tid] + s_fa[(NBG - 1) * 128 + tid];
         } else if (tid < 2 * D) {
-            const int e = tid - D;
-            dst[2 * D * D + tid] = (s_fc[e] + s_fc[D + e]) + (s_fc[2 * D + e] + s_fc[3 * D + e]);
+            float c = 0.f;
+#pragma unroll
+            for (int i = 0; i < NSW; ++i) c += s_fc[i * D + tid - D];
+            dst[2 * D * D + tid] = c;
         }
         if (tid == 0) {
             dst[2 * D * D + 2 * D] = omega_tot;
