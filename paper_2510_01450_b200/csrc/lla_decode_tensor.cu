@@ -46,9 +46,10 @@ struct DtCfg {
     static constexpr int TMEM = D == 64 ? 256 : 512;
     static_assert(TC_A + 64 * NAB <= TMEM, "TMEM");
     static constexpr uint32_t IDESC = make_idesc(128, NMMA, 0, 1);
-    static constexpr int NSW = D / 16;                     // score warps: 16 keys of the tile each at d = 64, 8 at d = 128
-    static constexpr int KPW = DT_BK / NSW;                // (d / 32 lanes per key)
-    static constexpr int NBG = D / 64;                     // groups of four operand warps; they take the tiles in turn
+    static constexpr int NBG = D / 64;                     // groups of four score warps and of four operand warps, which
+    static constexpr int NSW = 4 * NBG;                    // take the tiles in turn
+    static constexpr int KPP = 1024 / D;                   // keys of a score warp and pass (d / 32 lanes per key)
+    static constexpr int PASSES = 16 / KPP;                // passes over the 16 keys of a score warp
     static constexpr int W_TMA = NSW + 4 * NBG;            // warps: scores, operand, TMA, MMA
     static constexpr int THREADS = 32 * (W_TMA + 2);
     static constexpr int REC = 2 * D * D + 2 * D + 4;      // floats of a moment record: M, N^T, a, c, omega, m, 2 pad
@@ -83,13 +84,11 @@ __device__ __forceinline__ void ldsm4_t(uint32_t addr, uint32_t& r0, uint32_t& r
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
 }
-// 16 TMEM lanes x 32 columns: r[2 g] is lane l / 4 and r[2 g + 1] lane l / 4 + 8, column 4 g + l % 4
-__device__ __forceinline__ void tmem_st_16x128(uint32_t addr, const uint32_t (&r)[16]) {
+// 16 TMEM lanes x 16 columns: r[2 g] is lane l / 4 and r[2 g + 1] lane l / 4 + 8, column 4 g + l % 4
+__device__ __forceinline__ void tmem_st_16x128(uint32_t addr, const uint32_t (&r)[8]) {
     asm volatile(
-        "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], "
-        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-        ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
-          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]) : "memory");
+        "tcgen05.st.sync.aligned.16x128b.x4.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+        ::"r"(addr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -373,8 +372,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             mbar_init(bar(C::KVFULL + s), 1);
-            mbar_init(bar(C::KVEMPTY + s), D == 64 ? 1 : 1 + NSW);      // d = 128: the score warps read V after the weights
-            mbar_init(bar(C::WFULL + s), NSW);
+            mbar_init(bar(C::KVEMPTY + s), D == 64 ? 1 : 5);      // d = 128: the score warps read V after the weights
+            mbar_init(bar(C::WFULL + s), 4);
         }
         for (int b = 0; b < NAB; ++b) { mbar_init(bar(C::AFULL + b), 4); mbar_init(bar(C::AFREE + b), 1); }
         mbar_init(bar(C::DFULL), 1);              // the accumulator is complete: one barrier per pass
@@ -468,20 +467,10 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         }
     } else if (warp < NSW) {
         // ================================ score warps ================================
-        // Key j of the tile, features 32 h .. 32 h + 31.  The eight lanes that share a 128-byte shared-memory wavefront have
-        // the same h and neighbouring keys, so the swizzled chunks never collide.
-        constexpr int KPW = C::KPW, CH = D / 8;
-        const int h = lane / KPW, j = warp * KPW + lane % KPW;
-        auto max_over_warps = [&](volatile float* tm, float v) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-            if (lane == 0) tm[warp] = v;
-            asm volatile("bar.sync 1, %0;" ::"n"(32 * NSW) : "memory");
-            v = tm[0];
-#pragma unroll
-            for (int i = 1; i < NSW; ++i) v = fmaxf(v, tm[i]);
-            return v;
-        };
+        // Keys j, j + KPP of the tile, features 32 h .. 32 h + 31.  The eight lanes that share a 128-byte shared-memory
+        // wavefront have the same h and neighbouring keys, so the swizzled chunks never collide.
+        constexpr int KPP = C::KPP, PASSES = C::PASSES, CH = D / 8;
+        const int grp = warp >> 2, h = lane / KPP, j = (warp & 3) * 16 + lane % KPP;
         const uint32_t krow = (h >> 1) * C::SUB + j * 128;
         const float c1 = prm.scale * 1.4426950408889634f;
         uint64_t qv[16];
@@ -496,78 +485,125 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             }
         }
         bool ok = true;
-        float run_max = -INFINITY;
-        bool over = false;
-        // The reference maximum is the first tile's (one reduction over the score warps per pass at most); later
-        // tiles only note, per thread and without any barrier, the largest score seen and whether one exceeded the
-        // reference by more than 2^90 -- then the weights of this pass are useless (they are clamped, so nothing
-        // overflows) and the pass is repeated with the true maximum as reference.
+        float run_max = -INFINITY, s2[PASSES];
+        bool over = false, valid[PASSES];
+        // (t: tile of the pass, it fixes the keys; g: running tile count over both passes, it fixes ring stage,
+        //  buffer and barrier phase)
+        auto score = [&](int t, int g) -> bool {
+            const int sl = g % NST;
+            const bool landed = mbar_wait(bar(C::KVFULL + sl), (g / NST) & 1, abort_flag, wcap);
+            if (!__all_sync(0xffffffffu, landed)) return false;      // what follows is warp-wide
+            uint8_t* ks = smem + sl * C::STAGE + krow;
+            uint64_t sd[PASSES][4 / PASSES];                          // four independent chains of pairs
+#pragma unroll
+            for (int u = 0; u < PASSES; ++u)
+#pragma unroll
+                for (int e = 0; e < 4 / PASSES; ++e) sd[u][e] = 0ull;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int u = 0; u < PASSES; ++u) {
+                    const uint4 raw = *reinterpret_cast<const uint4*>(ks + u * KPP * 128 + (((4 * (h & 1) + i) ^ (j & 7)) << 4));
+                    const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint64_t& d = sd[u][e % (4 / PASSES)];
+                        d = fma2(qv[4 * i + e], pk2(__uint_as_float(wds[e] << 16), __uint_as_float(wds[e] & 0xFFFF0000u)), d);
+                    }
+                }
+#pragma unroll
+            for (int u = 0; u < PASSES; ++u) {
+                uint64_t d = sd[u][0];
+#pragma unroll
+                for (int e = 1; e < 4 / PASSES; ++e) d = add2(d, sd[u][e]);
+                float a0, a1;
+                upk2(d, a0, a1);
+                s2[u] = a0 + a1;
+            }
+#pragma unroll
+            for (int off = KPP; off < 32; off <<= 1)
+#pragma unroll
+                for (int u = 0; u < PASSES; ++u) s2[u] += __shfl_xor_sync(0xffffffffu, s2[u], off);
+#pragma unroll
+            for (int u = 0; u < PASSES; ++u) {
+                valid[u] = jbeg + t * BK + j + u * KPP < jend;
+                if (!valid[u]) s2[u] = -INFINITY;
+            }
+            if (jbeg + (t + 1) * BK > jend) {
+                // ragged last tile: rows past the end may hold anything (unused cache slots).  They are
+                // operands, so clear them (0 x NaN would poison the accumulator).
+#pragma unroll
+                for (int u = 0; u < PASSES; ++u)
+                    if (!valid[u]) {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const uint32_t off = u * KPP * 128 + (((4 * (h & 1) + i) ^ (j & 7)) << 4);
+                            *reinterpret_cast<uint4*>(ks + off) = make_uint4(0, 0, 0, 0);
+                            *reinterpret_cast<uint4*>(ks + C::NSUB * C::SUB + off) = make_uint4(0, 0, 0, 0);
+                        }
+                    }
+                fence_proxy_async();
+            }
+            return true;
+        };
+        auto warp_max = [&](float v) {
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+            return v;
+        };
+        // The reference maximum is the first tile's; later tiles only note, per thread and without any barrier, the
+        // largest score seen and whether one exceeded the reference by more than 2^90 -- then the weights of this pass
+        // are useless (they are clamped, so nothing overflows) and the pass is repeated with the true maximum as
+        // reference.
+        if (ntile > 0) {
+            if (grp == 0) {
+                ok = score(0, 0);
+                float v = s2[0];
+#pragma unroll
+                for (int u = 1; u < PASSES; ++u) v = fmaxf(v, s2[u]);
+                v = warp_max(v);
+                if (lane == 0) tmax[warp] = v;
+            }
+            ok = !bar_or(1, 32 * NSW, !ok);
+            m_ref = fmaxf(fmaxf(tmax[0], tmax[1]), fmaxf(tmax[2], tmax[3]));
+        }
         for (int pass = 0, g0 = 0; pass < 2 && ntile > 0; ++pass, g0 += ntile) {
             omega = 0.f;
 #pragma unroll
             for (int i = 0; i < 4; ++i) sums[i >> 1][i & 1] = 0ull;
-            // (t: tile of the pass, it fixes the keys; g: running tile count over both passes, it fixes ring stage,
-            //  buffer and barrier phase)
-            for (int t = 0; t < ntile; ++t) {
+            for (int t = grp; t < ntile && ok; t += NBG) {
                 const int g = g0 + t, sl = g % NST;
-                ok = mbar_wait(bar(C::KVFULL + sl), (g / NST) & 1, abort_flag, wcap);
-                ok = __all_sync(0xffffffffu, ok);              // what follows is warp-wide
-                if (t == 0) ok = !bar_or(1, 32 * NSW, !ok);    // and for the first tile takes all score warps
+                ok = score(t, g);
                 if (!ok) break;
-                uint8_t* stage = smem + sl * C::STAGE;
-                uint8_t* ks = stage + krow;
-                uint64_t sd[4] = {0ull, 0ull, 0ull, 0ull};      // four independent chains of pairs
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint4 raw = *reinterpret_cast<const uint4*>(ks + (((4 * (h & 1) + i) ^ (j & 7)) << 4));
-                    const uint32_t wds[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        sd[e] = fma2(qv[4 * i + e], pk2(__uint_as_float(wds[e] << 16), __uint_as_float(wds[e] & 0xFFFF0000u)), sd[e]);
-                }
-                float a0, a1;
-                upk2(add2(add2(sd[0], sd[1]), add2(sd[2], sd[3])), a0, a1);
-                float s2 = a0 + a1;
-#pragma unroll
-                for (int off = KPW; off < 32; off <<= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, off);
-                const bool valid = jbeg + t * BK + j < jend;
-                if (!valid) {
-                    // ragged last tile: rows past the end may hold anything (unused cache slots).  They are
-                    // operands, so clear them (0 x NaN would poison the accumulator).
-                    s2 = -INFINITY;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint32_t off = ((4 * (h & 1) + i) ^ (j & 7)) << 4;
-                        *reinterpret_cast<uint4*>(ks + off) = make_uint4(0, 0, 0, 0);
-                        *reinterpret_cast<uint4*>(ks + C::NSUB * C::SUB + off) = make_uint4(0, 0, 0, 0);
+                for (int u = 0; u < PASSES; ++u) {
+                    run_max = fmaxf(run_max, s2[u]);
+                    over |= s2[u] > m_ref + 90.f;
+                    const float w = valid[u] ? ex2f(fminf(s2[u] - m_ref, 100.f)) : 0.f;
+                    if (h == 0) {
+                        omega += w;
+                        const int key = j + u * KPP;
+                        const __nv_bfloat16 whi = __float2bfloat16_rn(w);
+                        const __nv_bfloat16 wlo = __float2bfloat16_rn(w - __bfloat162float(whi));
+                        __nv_bfloat16* wj = reinterpret_cast<__nv_bfloat16*>(wbuf + sl * BK * 4 + (key >> 1) * 8) + (key & 1);
+                        wj[0] = whi;
+                        wj[2] = wlo;
+                        if (D == 128) wfbuf[sl * BK + key] = w;
                     }
-                    fence_proxy_async();
-                }
-                if (t == 0 && pass == 0) m_ref = max_over_warps(tmax, s2);
-                run_max = fmaxf(run_max, s2);
-                over |= s2 > m_ref + 90.f;
-                const float w = valid ? ex2f(fminf(s2 - m_ref, 100.f)) : 0.f;
-                if (h == 0) {
-                    omega += w;
-                    const __nv_bfloat16 whi = __float2bfloat16_rn(w);
-                    const __nv_bfloat16 wlo = __float2bfloat16_rn(w - __bfloat162float(whi));
-                    __nv_bfloat16* wj = reinterpret_cast<__nv_bfloat16*>(wbuf + sl * BK * 4 + (j >> 1) * 8) + (j & 1);
-                    wj[0] = whi;
-                    wj[2] = wlo;
-                    if (D == 128) wfbuf[sl * BK + j] = w;
                 }
                 // one arrival per warp: 32 lanes arriving on one mbarrier are 32 serialised shared-memory atomics
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(C::WFULL + sl));
                 if constexpr (D == 128) {
                     const int vchunk = lane % CH;
-                    const uint8_t* vs = stage + (C::NSUB + (vchunk >> 3)) * C::SUB;
+                    const uint8_t* vs = smem + sl * C::STAGE + (C::NSUB + (vchunk >> 3)) * C::SUB;
                     const float* wt = wfbuf + sl * BK;
 #pragma unroll
-                    for (int i = 0; i < KPW * CH / 32; ++i) {
-                        const int key = warp * KPW + lane / CH + 32 / CH * i;
+                    for (int i = 0; i < 16 * CH / 32; ++i) {
+                        const int key = (warp & 3) * 16 + lane / CH + 32 / CH * i;
                         const uint4 x = *reinterpret_cast<const uint4*>(vs + key * 128 + (((vchunk & 7) ^ (key & 7)) << 4));
-                        const uint64_t w2 = pk2(wt[key], wt[key]);
+                        const float w = wt[key];
+                        const uint64_t w2 = pk2(w, w);
                         sums[0][0] = fma2(w2, pk2(__uint_as_float(x.x << 16), __uint_as_float(x.x & 0xFFFF0000u)), sums[0][0]);
                         sums[0][1] = fma2(w2, pk2(__uint_as_float(x.y << 16), __uint_as_float(x.y & 0xFFFF0000u)), sums[0][1]);
                         sums[1][0] = fma2(w2, pk2(__uint_as_float(x.z << 16), __uint_as_float(x.z & 0xFFFF0000u)), sums[1][0]);
@@ -583,11 +619,16 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
             const bool any = bar_or(1, 32 * NSW, over);
             if (tid == 0) misc[2] = (int)any;
             if (any) {
-                m_ref = max_over_warps(tmax + 8, run_max);
-                over = false;
+                const float v = warp_max(run_max);
+                if (lane == 0) tmax[8 + warp] = v;
             }
             asm volatile("bar.sync 1, %0;" ::"n"(32 * NSW) : "memory");
-            __syncwarp();
+            if (any) {
+                m_ref = tmax[8];
+#pragma unroll
+                for (int i = 1; i < NSW; ++i) m_ref = fmaxf(m_ref, tmax[8 + i]);
+                over = false;
+            }
             if (lane == 0) mbar_arrive(bar(C::PASS));      // the other warps read misc[2] after this
             if (!any) break;
         }
@@ -619,33 +660,36 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
                 tc_fence_after();
                 const uint32_t tile = sbase + sl * C::STAGE + src0 + lrow * 128;
                 const uint8_t* wp = wbuf + sl * BK * 4 + 8 * (lane & 3);
-                uint2 ww[8];                                 // the weights of keys 8 kg + 2 (lane % 4), + 1: hi pair, lo pair
+                const float* wt = wfbuf + sl * BK + 2 * (lane & 3);
 #pragma unroll
-                for (int kg = 0; kg < 8; ++kg) ww[kg] = *reinterpret_cast<const uint2*>(wp + 32 * kg);
+                for (int kh = 0; kh < 2; ++kh) {                 // 32 keys at a time
+                    uint2 ww[4];                                 // the weights of keys 8 kg + 2 (lane % 4), + 1: hi pair, lo pair
 #pragma unroll
-                for (int fg = 0; fg < 2; ++fg) {             // 16 features at a time
-                    const uint32_t base = tile + (((lchunk + 2 * fg) ^ (lane & 7)) << 4);
-                    uint32_t r[16], lo[16];
+                    for (int kg = 0; kg < 4; ++kg) ww[kg] = *reinterpret_cast<const uint2*>(wp + 32 * (4 * kh + kg));
 #pragma unroll
-                    for (int kg = 0; kg < 8; kg += 2) ldsm4_t(base + kg * 1024, r[2 * kg], r[2 * kg + 1], r[2 * kg + 2], r[2 * kg + 3]);
-                    if constexpr (D == 128) {
-                    const float* wt = wfbuf + sl * BK + 2 * (lane & 3);
+                    for (int fg = 0; fg < 2; ++fg) {             // 16 features at a time
+                        const uint32_t base = tile + (((lchunk + 2 * fg) ^ (lane & 7)) << 4) + 4096 * kh;
+                        uint32_t r[8], lo[8];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        sums[fg][i & 1] = fma2(*reinterpret_cast<const uint64_t*>(wt + 8 * (i >> 1)),
-                                               pk2(__uint_as_float(r[i] << 16), __uint_as_float(r[i] & 0xFFFF0000u)), sums[fg][i & 1]);
+                        for (int kg = 0; kg < 4; kg += 2) ldsm4_t(base + kg * 1024, r[2 * kg], r[2 * kg + 1], r[2 * kg + 2], r[2 * kg + 3]);
+                        if constexpr (D == 128) {
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                sums[fg][i & 1] = fma2(*reinterpret_cast<const uint64_t*>(wt + 32 * kh + 8 * (i >> 1)),
+                                                       pk2(__uint_as_float(r[i] << 16), __uint_as_float(r[i] & 0xFFFF0000u)), sums[fg][i & 1]);
+                        }
+                        // w k = (w_hi + w_lo) k with bf16 w_hi, w_lo: hi = round(w_hi k); w_hi k - hi fits bf16 exactly;
+                        // lo = round(w_lo k + that).  Relative error of hi + lo about 2^-17, four instructions per two keys.
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const uint32_t hi = mul_bf2(ww[i >> 1].x, r[i]);
+                            lo[i] = fma_bf2(ww[i >> 1].y, r[i], fma_bf2(ww[i >> 1].x, r[i], hi ^ 0x80008000u));
+                            r[i] = hi;
+                        }
+                        const uint32_t at = lane_addr + ((uint32_t)(16 * fg) << 16) + 64 * b + 16 * kh;
+                        tmem_st_16x128(at, r);
+                        tmem_st_16x128(at + 32, lo);
                     }
-                    // w k = (w_hi + w_lo) k with bf16 w_hi, w_lo: hi = round(w_hi k); w_hi k - hi fits bf16 exactly;
-                    // lo = round(w_lo k + that).  Relative error of hi + lo about 2^-17, three instructions per two keys.
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const uint32_t hi = mul_bf2(ww[i >> 1].x, r[i]);
-                        lo[i] = fma_bf2(ww[i >> 1].y, r[i], fma_bf2(ww[i >> 1].x, r[i], hi ^ 0x80008000u));
-                        r[i] = hi;
-                    }
-                    const uint32_t at = lane_addr + ((uint32_t)(16 * fg) << 16) + 64 * b;
-                    tmem_st_16x128(at, r);
-                    tmem_st_16x128(at + 32, lo);
                 }
                 tc_wait_st();
                 tc_fence_before();
