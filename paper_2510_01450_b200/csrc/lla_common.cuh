@@ -87,6 +87,7 @@ struct ForwardArgs {
     int max_iters;
     float tol;
     int head_rows;   // rows seeing fewer keys than this are solved directly (fp64)
+    bool all_direct = false;     // every row is (the problems the tensor-core kernel does not take, default solver settings)
     float* rho;      // optional
     float* stats;    // optional
     int* iters;      // optional

@@ -347,22 +347,6 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
 }
 
 template <int D, typename TIn, typename TOut>
-int launch_t(const ForwardArgs& a, int rows_per_head, int lcap) {
-    using C = HrCfg<D>;
-    const size_t smem = sizeof(double) * C::smem_doubles(lcap);
-    auto kern = head_rows_kernel<D, D, TIn, TOut>;
-    LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-    dim3 grid(a.B * a.H, rows_per_head);
-    kern<<<grid, C::THREADS, smem, a.stream>>>(
-        (const TIn*)a.q, (const TIn*)a.k, (const TIn*)a.v, (TOut*)a.out, a.n, rows_per_head, a.causal,
-        (double)a.scale, (double)a.lambda, lcap, a.rho, a.stats, a.iters, a.status, nullptr, a.H, a.lambda_rows,
-        a.ridge_mode, a.nq, a.kv_group, PagedKv{nullptr, 0, 0, 0}, 0, a.sq, a.sk, a.sv, a.so);
-    LLA_CUDA_TRY(cudaGetLastError());
-    return LLA_OK;
-}
-
-template <int D, typename TIn, typename TOut>
 int launch_decode_t(const DecodeArgs& a, int lcap) {
     using C = HrCfg<D>;
     const size_t smem = sizeof(double) * C::smem_doubles(lcap);
@@ -389,41 +373,7 @@ int launch_decode_d(const DecodeArgs& a, int lcap) {
     return LLA_ERR_UNSUPPORTED;
 }
 
-template <int D>
-int launch_d(const ForwardArgs& a, int rows_per_head, int lcap) {
-    if (a.in_dtype == LLA_BF16 && a.out_dtype == LLA_BF16)
-        return launch_t<D, __nv_bfloat16, __nv_bfloat16>(a, rows_per_head, lcap);
-    if (a.in_dtype == LLA_BF16 && a.out_dtype == LLA_F32)
-        return launch_t<D, __nv_bfloat16, float>(a, rows_per_head, lcap);
-    if (a.in_dtype == LLA_F32 && a.out_dtype == LLA_F32)
-        return launch_t<D, float, float>(a, rows_per_head, lcap);
-    return LLA_ERR_UNSUPPORTED;
-}
-
 }  // namespace
-
-// Number of leading rows per head handled directly (causal), or n / 0 (non-causal).
-int head_rows_count(const ForwardArgs& a) {
-    if (a.head_rows <= 0) return 0;
-    if (a.causal) {     // query row i sees n - nq + i + 1 keys
-        const int rows = a.head_rows - 1 - (a.n - a.nq);
-        return rows < 0 ? 0 : (rows > a.nq ? a.nq : rows);
-    }
-    return a.n < a.head_rows ? a.nq : 0;
-}
-
-int launch_head_rows(const ForwardArgs& a) {
-    const int rows = head_rows_count(a);
-    if (rows <= 0) return LLA_OK;
-    const int lcap = a.causal ? (a.n - a.nq) + rows : a.n;
-    if (a.d != a.dv) return LLA_ERR_UNSUPPORTED;
-    switch (a.d) {
-        case 16: return launch_d<16>(a, rows, lcap);
-        case 64: return launch_d<64>(a, rows, lcap);
-        case 128: return launch_d<128>(a, rows, lcap);
-        default: return LLA_ERR_UNSUPPORTED;
-    }
-}
 
 // Decode: (sequence, head) pairs whose cache holds at most head_rows - 1 keys.
 int launch_head_rows_decode(const DecodeArgs& a) {
