@@ -192,7 +192,8 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         }
         for (int j = tt; j < CH; j += 32 * NW) {
             const bool vis = j < nk && j0 + j < L && j0 + j >= jlo;
-            const double e = vis ? exp(sm.s[tm][j] * scale - m_ref) : 0.0;
+            const double sj = sm.s[tm][j], e = vis ? exp(sj * scale - m_ref) : 0.0;
+            if (dual) sm.t[tm][j] = sj;
             sm.s[tm][j] = e;
             omega += e;
         }
@@ -200,23 +201,27 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         if (!dual) {
             // keys 4 s + t4: A operand w_j k_j of this warp's block rows, B operand k_j of every block column
             const int ns = (min(nk, L - j0) + 3) / 4;
-            for (int s = 0; s < ns; ++s) {
-                const double* kr = sm.kv[4 * s + t4] + g;
-                const double wj = sm.s[tm][4 * s + t4];
-                double av[R];
+            team::with_warp<NW>(w, [&](auto wc) {
+                constexpr int W = decltype(wc)::value;
+#pragma unroll(D == 16 ? 4 : 1)
+                for (int s = 0; s < ns; ++s) {
+                    const double* kr = sm.kv[4 * s + t4] + g;
+                    const double wj = sm.s[tm][4 * s + t4];
+                    double av[R];
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    av[r] = wj * kr[8 * T::row(r, w)];
-                    asum[r] += av[r];
+                    for (int r = 0; r < R; ++r) {
+                        av[r] = wj * kr[8 * T::row(r, W)];
+                        asum[r] += av[r];
+                    }
+#pragma unroll
+                    for (int j = 0; j <= T::row(R - 1, W); ++j) {
+                        const double bv = kr[8 * j];
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            if (j <= T::row(r, W)) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
+                    }
                 }
-#pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    const double bv = kr[8 * j];
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        if (T::cols(r) > j && (j <= r * NW || j <= T::row(r, w))) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
-                }
-            }
+            });
         }
     }
     // team-wide sums (every team has run every block barrier above)
@@ -231,35 +236,48 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     if (dual) {
         // The block's keys are one chunk and still in shared memory.  Row and column index: key jlo + 8 b + ..; the
         // padding to a multiple of eight is an identity block.
+        // (z_j . z_l = k_j . k_l - k_j . q - k_l . q + q . q; rows of the chunk past the block's keys are zero)
         const int Lr = L - jlo, base = jlo - jbeg;
         nba = (Lr + 7) / 8;
-        for (int s = 0; s < D / 4; ++s) {
-            const double qc = sm.q[tm][4 * s + t4];
-            auto z = [&](int b) { return 8 * b + g < Lr ? sm.kv[base + 8 * b + g][4 * s + t4] - qc : 0.0; };
-            double av[R];
+        team::with_warp<NW>(w, [&](auto wc) {
+            constexpr int W = decltype(wc)::value;
+            for (int s = 0; s < D / 4; ++s) {
+                const double* kr = sm.kv[base + g] + 4 * s + t4;
+                double av[R];
 #pragma unroll
-            for (int r = 0; r < R; ++r) av[r] = z(T::row(r, w));
+                for (int r = 0; r < R; ++r) av[r] = kr[8 * C::LDK * T::row(r, W)];
 #pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                if (j < nba) {
-                    const double bv = z(j);
+                for (int j = 0; j <= T::row(R - 1, W); ++j) {
+                    if (j >= nba) break;
+                    const double bv = kr[8 * C::LDK * j];
 #pragma unroll
                     for (int r = 0; r < R; ++r)
-                        if (T::cols(r) > j && j <= T::row(r, w) && T::row(r, w) < nba) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
+                        if (j <= T::row(r, W)) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
                 }
             }
-        }
+        });
+        double qq = 0.0;
+        for (int e = lane; e < D; e += 32) qq += sm.q[tm][e] * sm.q[tm][e];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) qq += __shfl_xor_sync(FULL, qq, o);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            const int bi = T::row(r, w);
+            const int bi = T::row(r, w), idx = 8 * bi + g;
+            const double si = qq - sm.t[tm][base + idx];
 #pragma unroll
             for (int j = 0; j < NB; ++j)
-                if (T::cols(r) > j && j == bi && bi < nba) {
-                    const int idx = 8 * bi + g;
-                    // ridge over weight for live keys (weights kept away from zero), one for the padding
-                    const double dg = idx < Lr ? lam_m / fmax(sm.s[tm][base + idx], 1e-290) : 1.0;
-                    if (g == 2 * t4) c[T::off(r) + j][0] += dg;
-                    if (g == 2 * t4 + 1) c[T::off(r) + j][1] += dg;
+                if (T::cols(r) > j && j <= bi && bi < nba) {
+                    double* cp = c[T::off(r) + j];
+                    const int jdx = 8 * j + 2 * t4;
+                    const bool in0 = idx < Lr && jdx < Lr, in1 = idx < Lr && jdx + 1 < Lr;
+                    cp[0] = in0 ? cp[0] + (si - sm.t[tm][base + jdx]) : 0.0;
+                    cp[1] = in1 ? cp[1] + (si - sm.t[tm][base + jdx + 1]) : 0.0;
+                    if (j == bi) {
+                        // ridge over weight for live keys (weights kept away from zero), one for the padding
+                        const double dg = idx < Lr ? lam_m / fmax(sm.s[tm][base + idx], 1e-290) : 1.0;
+                        if (g == 2 * t4) cp[0] += dg;
+                        if (g == 2 * t4 + 1) cp[1] += dg;
+                    }
                 }
         }
         for (int e = tt; e < 8 * nba; e += 32 * NW) ss.b[0][e] = e < Lr ? 1.0 : 0.0;
@@ -298,7 +316,8 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     double ybar = 0.0, gfac = 1.0, csum = 0.0;
     if (live) {
         team::sync<NW>(bar_id);
-        ok = team::solve<D, NW, 1>(c, ss, nba, w, lane, bar_id);
+        if constexpr (NW <= 2) team::with_warp<NW>(w, [&](auto wc) { ok = team::solve<D, NW, 1>(c, ss, nba, decltype(wc)::value, lane, bar_id); });
+        else ok = team::solve<D, NW, 1>(c, ss, nba, w, lane, bar_id);
         team::sync<NW>(bar_id);
         if (dual) {
             // coefficients lambda' alpha_j over the chunk's keys

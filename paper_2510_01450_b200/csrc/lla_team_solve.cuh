@@ -30,10 +30,37 @@ struct Cfg {
     static constexpr int NBLK = NW * R * (R + 1) / 2;  // blocks a warp keeps (some of the last NW columns unused)
     __host__ __device__ static constexpr int off(int r) { return NW * r * (r + 1) / 2; }
     __host__ __device__ static constexpr int cols(int r) { return NW * (r + 1); }
-    __device__ static int row(int r, int w) { return r & 1 ? r * NW + NW - 1 - w : r * NW + w; }
+    __host__ __device__ static constexpr int row(int r, int w) { return r & 1 ? r * NW + NW - 1 - w : r * NW + w; }
     __host__ __device__ static constexpr int owner(int p) { return (p / NW) & 1 ? NW - 1 - p % NW : p % NW; }
     static_assert(NB % NW == 0, "block rows per warp");
 };
+
+// f(the warp's number in the team as a constant): the loops over a warp's blocks have no guards then, which a run-time
+// number would put around every instruction
+template <int V>
+struct Const {
+    static constexpr int value = V;
+};
+template <int NW, typename F>
+__device__ __forceinline__ void with_warp(int w, F&& f) {
+    static_assert(NW == 1 || NW == 2 || NW == 8, "team sizes in use");
+    if constexpr (NW == 1) {
+        f(Const<0>{});
+    } else if constexpr (NW == 2) {
+        if (w == 0) f(Const<0>{}); else f(Const<1>{});
+    } else {
+        switch (w) {
+            case 0: f(Const<0>{}); break;
+            case 1: f(Const<1>{}); break;
+            case 2: f(Const<2>{}); break;
+            case 3: f(Const<3>{}); break;
+            case 4: f(Const<4>{}); break;
+            case 5: f(Const<5>{}); break;
+            case 6: f(Const<6>{}); break;
+            default: f(Const<7>{}); break;
+        }
+    }
+}
 
 template <int D, int NW, int NRHS>
 struct alignas(16) Smem {
@@ -72,7 +99,7 @@ __device__ __forceinline__ bool solve(double (&c)[Cfg<D, NW>::NBLK][2], Smem<D, 
             const double f = __shfl_sync(FULL, col, (lane & 28) + (k >> 1));
             const double pr0 = __shfl_sync(FULL, a0, 4 * k + t4), pr1 = __shfl_sync(FULL, a1, 4 * k + t4);
             const double wr0 = __shfl_sync(FULL, w0, 4 * k + t4), wr1 = __shfl_sync(FULL, w1, 4 * k + t4);
-            const double inv = fast_rcp(piv);
+            const double inv = fast_rcp1(piv);
             const double m = n > k ? f * inv : 0.0;
             a0 -= m * pr0;
             a1 -= m * pr1;
