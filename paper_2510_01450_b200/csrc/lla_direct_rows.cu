@@ -14,14 +14,15 @@
 // dual (Gram) form: with Z the L x d matrix of k_j - q, w_j (1 - z_j . rho) = lambda' alpha_j where
 // (Z Z^T + lambda' diag(1 / w)) alpha = 1 -- a smaller system, free of the cancellation in 1 - z . rho.
 //
-// A block takes a few consecutive rows of a head (8 at d = 64), one team of warps each, and streams the keys through
+// A block takes a few consecutive rows of a head (4 at d = 64), one team of warps each, and streams the keys through
 // shared memory as doubles, a chunk at a time.  Every product is an 8 x 8 x 4 matrix instruction: scores (the block's
 // query rows against eight keys), the moments (A operand w_j k_j, B operand k_j; the lower block triangle in the
 // team's registers, where the factorisation continues in place: lla_team_solve.cuh), and in a second sweep k_j . y and
 // the output sum (coefficients against values).  The second sweep forms the weights again instead of keeping them.
 //
 // What bounds it: the matrix pipe in the moments of long rows (36 of the about 47 instructions per 4 keys and row at
-// d = 64), the chain of reciprocals in the pivot blocks for short ones; 16 warps and eight systems per SM hide the latter.
+// d = 64; measured at 89 % of its rate), the chain of reciprocals in the pivot blocks for short ones, which the eight
+// systems of two blocks on an SM hide in part.
 #include "lla_team_solve.cuh"
 
 namespace lla {
@@ -30,10 +31,11 @@ namespace {
 template <int D>
 struct DrCfg {
     static constexpr int NW = D == 16 ? 1 : D == 64 ? 2 : 8;      // warps per row: what the registers of 16 warps hold
-    static constexpr int TEAMS = D == 16 ? 4 : D == 64 ? 8 : 2;   // rows per block
+    static constexpr int TEAMS = D == 128 ? 2 : 4;                // rows per block; d = 64: two blocks per SM, so that the pivot
+                                                                  // chains of one run beside the products of the other
     static constexpr int WARPS = NW * TEAMS, THREADS = 32 * WARPS;
     // keys per chunk: the keys of a block with a dual row (at most d + TEAMS - 1, with a window d + TEAMS) are one chunk
-    static constexpr int CH = D == 128 ? 136 : D == 64 ? 128 : 64;
+    static constexpr int CH = D == 128 ? 136 : D == 64 ? 72 : 64;
     static constexpr int LDK = D + 4;                             // row stride in doubles: 4 mod 16, both operand accesses conflict-free
     static constexpr int NB = D / 8;
     static constexpr int HALVES = WARPS / NB;                     // output sum: a warp per 8 columns and part of the keys
@@ -49,6 +51,7 @@ struct DrSmem {
     double s[C::TEAMS][C::LDW];               // scores -> weights -> output coefficients of the chunk
     double t[C::TEAMS][C::LDW];               // k_j . y
     double kbar[C::TEAMS][D];
+    double gram[D <= 64 ? C::NB * (C::NB + 1) / 2 : 1][64];     // K K^T of the first d keys, 8 x 8 blocks in accumulator layout
     double osum[C::HALVES > 1 ? C::TEAMS : 1][D];   // second half of the output sum
     double red[2][C::TEAMS][C::NW];
     double den[C::TEAMS];
@@ -75,6 +78,7 @@ template <int D, typename TIn>
 __device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend) {
     using C = DrCfg<D>;
     constexpr int PER = C::CH * D / 2 / C::THREADS;
+    static_assert(PER * 2 * C::THREADS == C::CH * D, "a chunk is a whole number of rounds");
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
         const int e = threadIdx.x + C::THREADS * u, j = e / (D / 2), c = 2 * (e % (D / 2));
@@ -100,7 +104,7 @@ __device__ __forceinline__ void dots(double (*out)[DrCfg<D>::LDW], const double 
 }
 
 template <int D, typename TIn, typename TOut>
-__global__ void __launch_bounds__(DrCfg<D>::THREADS)
+__global__ void __launch_bounds__(DrCfg<D>::THREADS, D == 64 ? 2 : 1)
 direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v, TOut* __restrict__ out,
                    int n, int nq, int rows_per_head, int head_rows, int causal, double scale, double lambda, const float* __restrict__ lambda_rows,
                    int ridge_mode, float* __restrict__ rho_out, float* __restrict__ stats, int* __restrict__ iters,
@@ -161,7 +165,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     // after which everything is rescaled); m_max is the true maximum, which the outputs refer to.
     double m_ref = -INFINITY, m_max = -INFINITY, omega = 0.0, lam_m = 0.0;
     // at most d keys: the dual form.  (lambda' could only vanish if lambda does.)
-    const bool dual = live && L - jlo <= D && jend - jbeg <= CH && lam_i > 0.0;
+    const bool dual = live && L <= D && jlo == 0 && jbeg == 0 && jend <= CH && lam_i > 0.0;
 
     // ---- first sweep: weights and moments ----
     for (int j0 = jbeg; j0 < jend; j0 += CH) {
@@ -170,6 +174,17 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         stage<D>(sm.kv, kb, sk.r, j0, jend);
         __syncthreads();
         dots<D>(sm.s, sm.q, sm.kv, nk, warp, lane);
+        if (D <= 64 && jend <= CH && (causal ? off + i0 + 1 : n) <= D) {        // a row of the block may be dual
+            for (int e = warp, bi = 0; e < NB * (NB + 1) / 2; e += C::WARPS) {
+                while ((bi + 1) * (bi + 2) / 2 <= e) ++bi;
+                const int bj = e - bi * (bi + 1) / 2;
+                if (8 * bi >= nk) continue;
+                double x[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+                for (int s = 0; s < D / 4; ++s) team::dmma(x[s & 1][0], x[s & 1][1], sm.kv[8 * bi + g][4 * s + t4], sm.kv[8 * bj + g][4 * s + t4]);
+                *reinterpret_cast<double2*>(&sm.gram[e][2 * lane]) = make_double2(x[0][0] + x[1][0], x[0][1] + x[1][1]);
+            }
+        }
         __syncthreads();
         if (j0 >= L || j0 + CH <= jlo) continue;                          // (uniform over the team) no key of this row
         double cmax = -INFINITY;
@@ -234,28 +249,43 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     bool ok = true;
     int nba = NB;
     if (dual) {
-        // The block's keys are one chunk and still in shared memory.  Row and column index: key jlo + 8 b + ..; the
-        // padding to a multiple of eight is an identity block.
-        // (z_j . z_l = k_j . k_l - k_j . q - k_l . q + q . q; rows of the chunk past the block's keys are zero)
-        const int Lr = L - jlo, base = jlo - jbeg;
-        nba = (Lr + 7) / 8;
-        team::with_warp<NW>(w, [&](auto wc) {
-            constexpr int W = decltype(wc)::value;
-            for (int s = 0; s < D / 4; ++s) {
-                const double* kr = sm.kv[base + g] + 4 * s + t4;
-                double av[R];
+        // The block's keys are one chunk and still in shared memory (jlo = 0: a window is never shorter than the rows
+        // that see at most d keys).  Row and column index: the key; the padding to a multiple of eight is an identity block.
+        // z_j . z_l = k_j . k_l - k_j . q - k_l . q + q . q; the first product is the same for the block's rows (it has
+        // them in shared memory at d <= 64: 576 instead of 576 per row instructions at 64 keys).  Rows of the chunk past
+        // the block's keys are zero.
+        nba = (L + 7) / 8;
+        if constexpr (D <= 64) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) av[r] = kr[8 * C::LDK * T::row(r, W)];
+            for (int r = 0; r < R; ++r) {
+                const int bi = T::row(r, w);
 #pragma unroll
-                for (int j = 0; j <= T::row(R - 1, W); ++j) {
-                    if (j >= nba) break;
-                    const double bv = kr[8 * C::LDK * j];
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        if (j <= T::row(r, W)) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
-                }
+                for (int j = 0; j < NB; ++j)
+                    if (T::cols(r) > j && j <= bi && bi < nba) {
+                        const double2 x = *reinterpret_cast<const double2*>(&sm.gram[bi * (bi + 1) / 2 + j][2 * lane]);
+                        c[T::off(r) + j][0] = x.x;
+                        c[T::off(r) + j][1] = x.y;
+                    }
             }
-        });
+        } else {
+            team::with_warp<NW>(w, [&](auto wc) {
+                constexpr int W = decltype(wc)::value;
+                for (int s = 0; s < D / 4; ++s) {
+                    const double* kr = sm.kv[g] + 4 * s + t4;
+                    double av[R];
+#pragma unroll
+                    for (int r = 0; r < R; ++r) av[r] = kr[8 * C::LDK * T::row(r, W)];
+#pragma unroll
+                    for (int j = 0; j <= T::row(R - 1, W); ++j) {
+                        if (j >= nba) break;
+                        const double bv = kr[8 * C::LDK * j];
+#pragma unroll
+                        for (int r = 0; r < R; ++r)
+                            if (j <= T::row(r, W)) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
+                    }
+                }
+            });
+        }
         double qq = 0.0;
         for (int e = lane; e < D; e += 32) qq += sm.q[tm][e] * sm.q[tm][e];
 #pragma unroll
@@ -263,24 +293,24 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int bi = T::row(r, w), idx = 8 * bi + g;
-            const double si = qq - sm.t[tm][base + idx];
+            const double si = qq - sm.t[tm][idx];
 #pragma unroll
             for (int j = 0; j < NB; ++j)
                 if (T::cols(r) > j && j <= bi && bi < nba) {
                     double* cp = c[T::off(r) + j];
                     const int jdx = 8 * j + 2 * t4;
-                    const bool in0 = idx < Lr && jdx < Lr, in1 = idx < Lr && jdx + 1 < Lr;
-                    cp[0] = in0 ? cp[0] + (si - sm.t[tm][base + jdx]) : 0.0;
-                    cp[1] = in1 ? cp[1] + (si - sm.t[tm][base + jdx + 1]) : 0.0;
+                    const bool in0 = idx < L && jdx < L, in1 = idx < L && jdx + 1 < L;
+                    cp[0] = in0 ? cp[0] + (si - sm.t[tm][jdx]) : 0.0;
+                    cp[1] = in1 ? cp[1] + (si - sm.t[tm][jdx + 1]) : 0.0;
                     if (j == bi) {
                         // ridge over weight for live keys (weights kept away from zero), one for the padding
-                        const double dg = idx < Lr ? lam_m / fmax(sm.s[tm][base + idx], 1e-290) : 1.0;
+                        const double dg = idx < L ? lam_m / fmax(sm.s[tm][idx], 1e-290) : 1.0;
                         if (g == 2 * t4) cp[0] += dg;
                         if (g == 2 * t4 + 1) cp[1] += dg;
                     }
                 }
         }
-        for (int e = tt; e < 8 * nba; e += 32 * NW) ss.b[0][e] = e < Lr ? 1.0 : 0.0;
+        for (int e = tt; e < 8 * nba; e += 32 * NW) ss.b[0][e] = e < L ? 1.0 : 0.0;
     } else if (live) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -321,16 +351,15 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         team::sync<NW>(bar_id);
         if (dual) {
             // coefficients lambda' alpha_j over the chunk's keys
-            const int Lr = L - jlo, base = jlo - jbeg;
             for (int j = tt; j < CH; j += 32 * NW) {
-                const double cj = j >= base && j < base + Lr ? lam_m * ss.x[w][0][j - base] : 0.0;
+                const double cj = j < L ? lam_m * ss.x[w][0][j] : 0.0;
                 sm.s[tm][j] = cj;
                 csum += cj;
             }
             if (rho_out)                                                   // rho = Z^T alpha
                 for (int e = tt; e < D; e += 32 * NW) {
                     double a = 0.0;
-                    for (int j = 0; j < Lr; ++j) a += ss.x[w][0][j] * (sm.kv[base + j][e] - sm.q[tm][e]);
+                    for (int j = 0; j < L; ++j) a += ss.x[w][0][j] * (sm.kv[j][e] - sm.q[tm][e]);
                     rho_out[row * D + e] = (float)a;
                 }
         } else {
