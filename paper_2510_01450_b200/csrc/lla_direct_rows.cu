@@ -17,8 +17,8 @@
 // A block takes a few consecutive rows of a head (4 at d = 64), one team of warps each, and streams the keys through
 // shared memory as doubles, a chunk at a time.  Every product is an 8 x 8 x 4 matrix instruction: scores (the block's
 // query rows against eight keys), the moments (A operand w_j k_j, B operand k_j; the lower block triangle in the
-// team's registers, where the factorisation continues in place: lla_team_solve.cuh), and in a second sweep k_j . y and
-// the output sum (coefficients against values).  The second sweep forms the weights again instead of keeping them.
+// team's registers, then in shared memory over the keys for the factorisation: lla_team_solve.cuh), and in a second
+// sweep k_j . y and the output sum (coefficients against values).  The second sweep forms the weights again instead of keeping them.
 //
 // What bounds it: the matrix pipe in the moments of long rows (36 of the about 47 instructions per 4 keys and row at
 // d = 64; measured at 89 % of its rate), the chain of reciprocals in the pivot blocks for short ones, which the eight
@@ -36,6 +36,7 @@ struct DrCfg {
     static constexpr int WARPS = NW * TEAMS, THREADS = 32 * WARPS;
     // keys per chunk: the keys of a block with a dual row (at most d + TEAMS - 1, with a window d + TEAMS) are one chunk
     static constexpr int CH = D == 128 ? 136 : D == 64 ? 72 : 64;
+    static constexpr int STEP = D == 128 ? 128 : 64;              // .. and the others' chunks: eight keys a warp
     static constexpr int LDK = D + 4;                             // row stride in doubles: 4 mod 16, both operand accesses conflict-free
     static constexpr int NB = D / 8;
     static constexpr int HALVES = WARPS / NB;                     // output sum: a warp per 8 columns and part of the keys
@@ -45,16 +46,19 @@ struct DrCfg {
 template <int D>
 struct DrSmem {
     using C = DrCfg<D>;
-    double kv[C::CH][C::LDK];                 // the current chunk of keys (or values)
+    union {
+        double kv[C::CH][C::LDK];                                  // the current chunk of keys (or values)
+        double mat[C::TEAMS][team::Cfg<D, C::NW>::LOWER][64];      // the systems, between the sweeps
+    };
     double q[C::TEAMS][C::LDK];               // query rows, zero beyond the head's
     double y[C::TEAMS][C::LDK];                    // their solutions (second sweep)
     double s[C::TEAMS][C::LDW];               // scores -> weights -> output coefficients of the chunk
     double t[C::TEAMS][C::LDW];               // k_j . y
     double kbar[C::TEAMS][D];
-    double gram[D <= 64 ? C::NB * (C::NB + 1) / 2 : 1][64];     // K K^T of the first d keys, 8 x 8 blocks in accumulator layout
     double osum[C::HALVES > 1 ? C::TEAMS : 1][D];   // second half of the output sum
     double red[2][C::TEAMS][C::NW];
-    double den[C::TEAMS];
+    double den[C::TEAMS], lam[C::TEAMS], qq[C::TEAMS];
+    int dual[C::TEAMS];                       // visible keys of a dual row, 0 for the others
     team::Smem<D, C::NW, 1> solve[C::TEAMS];
 };
 
@@ -73,14 +77,15 @@ __device__ __forceinline__ void load_pair<float>(const float* p, double& a, doub
     b = (double)f.y;
 }
 
-// keys (or values) j0 .. j0 + CH - 1 -> shared memory; rows from jend on are zero
+// keys (or values) j0 .. j0 + ch - 1 -> shared memory; rows from jend on are zero
 template <int D, typename TIn>
-__device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend) {
+__device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch) {
     using C = DrCfg<D>;
-    constexpr int PER = C::CH * D / 2 / C::THREADS;
-    static_assert(PER * 2 * C::THREADS == C::CH * D, "a chunk is a whole number of rounds");
+    constexpr int PER = C::CH * D / 2 / C::THREADS, PER_STEP = C::STEP * D / 2 / C::THREADS;
+    static_assert(PER * 2 * C::THREADS == C::CH * D && PER_STEP * 2 * C::THREADS == C::STEP * D, "a chunk is a whole number of rounds");
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
+        if (u >= PER_STEP && ch == C::STEP) break;
         const int e = threadIdx.x + C::THREADS * u, j = e / (D / 2), c = 2 * (e % (D / 2));
         double a = 0.0, b = 0.0;
         if (j0 + j < jend) load_pair(src + (size_t)(j0 + j) * stride + c, a, b);
@@ -129,6 +134,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     const int last = min(i0 + TEAMS, rows_per_head) - 1;
     const int jend = causal ? off + last + 1 : n;                       // keys of the block
     const int jbeg = causal && window > 0 ? max(0, off + i0 + 1 - window) : 0;
+    const int ch = jend - jbeg <= CH ? CH : C::STEP;                    // keys per chunk
     const size_t row = (size_t)bh * nq + i;
     const int hk = (bh % H) / max(kv_group, 1);
     const TIn* kb = k + sk.at(bh / H, hk, 0);
@@ -168,25 +174,14 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     const bool dual = live && L <= D && jlo == 0 && jbeg == 0 && jend <= CH && lam_i > 0.0;
 
     // ---- first sweep: weights and moments ----
-    for (int j0 = jbeg; j0 < jend; j0 += CH) {
-        const int nk = min(CH, jend - j0);
+    for (int j0 = jbeg; j0 < jend; j0 += ch) {
+        const int nk = min(ch, jend - j0);
         __syncthreads();
-        stage<D>(sm.kv, kb, sk.r, j0, jend);
+        stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
         __syncthreads();
         dots<D>(sm.s, sm.q, sm.kv, nk, warp, lane);
-        if (D <= 64 && jend <= CH && (causal ? off + i0 + 1 : n) <= D) {        // a row of the block may be dual
-            for (int e = warp, bi = 0; e < NB * (NB + 1) / 2; e += C::WARPS) {
-                while ((bi + 1) * (bi + 2) / 2 <= e) ++bi;
-                const int bj = e - bi * (bi + 1) / 2;
-                if (8 * bi >= nk) continue;
-                double x[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll
-                for (int s = 0; s < D / 4; ++s) team::dmma(x[s & 1][0], x[s & 1][1], sm.kv[8 * bi + g][4 * s + t4], sm.kv[8 * bj + g][4 * s + t4]);
-                *reinterpret_cast<double2*>(&sm.gram[e][2 * lane]) = make_double2(x[0][0] + x[1][0], x[0][1] + x[1][1]);
-            }
-        }
         __syncthreads();
-        if (j0 >= L || j0 + CH <= jlo) continue;                          // (uniform over the team) no key of this row
+        if (j0 >= L || j0 + ch <= jlo) continue;                          // (uniform over the team) no key of this row
         double cmax = -INFINITY;
         for (int j = tt; j < nk; j += 32 * NW) {
             const bool vis = j0 + j < L && j0 + j >= jlo;
@@ -205,10 +200,10 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             omega *= f;
             m_ref = cmax;
         }
-        for (int j = tt; j < CH; j += 32 * NW) {
+        for (int j = tt; j < ch; j += 32 * NW) {
             const bool vis = j < nk && j0 + j < L && j0 + j >= jlo;
             const double sj = sm.s[tm][j], e = vis ? exp(sj * scale - m_ref) : 0.0;
-            if (dual) sm.t[tm][j] = sj;
+            sm.t[tm][j] = sj;                          // (kept for the dual form)
             sm.s[tm][j] = e;
             omega += e;
         }
@@ -247,71 +242,17 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     const double inv = 1.0 / omega;
     team::Smem<D, NW, 1>& ss = sm.solve[tm];
     bool ok = true;
-    int nba = NB;
-    if (dual) {
-        // The block's keys are one chunk and still in shared memory (jlo = 0: a window is never shorter than the rows
-        // that see at most d keys).  Row and column index: the key; the padding to a multiple of eight is an identity block.
-        // z_j . z_l = k_j . k_l - k_j . q - k_l . q + q . q; the first product is the same for the block's rows (it has
-        // them in shared memory at d <= 64: 576 instead of 576 per row instructions at 64 keys).  Rows of the chunk past
-        // the block's keys are zero.
-        nba = (L + 7) / 8;
-        if constexpr (D <= 64) {
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                const int bi = T::row(r, w);
-#pragma unroll
-                for (int j = 0; j < NB; ++j)
-                    if (T::cols(r) > j && j <= bi && bi < nba) {
-                        const double2 x = *reinterpret_cast<const double2*>(&sm.gram[bi * (bi + 1) / 2 + j][2 * lane]);
-                        c[T::off(r) + j][0] = x.x;
-                        c[T::off(r) + j][1] = x.y;
-                    }
-            }
-        } else {
-            team::with_warp<NW>(w, [&](auto wc) {
-                constexpr int W = decltype(wc)::value;
-                for (int s = 0; s < D / 4; ++s) {
-                    const double* kr = sm.kv[g] + 4 * s + t4;
-                    double av[R];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) av[r] = kr[8 * C::LDK * T::row(r, W)];
-#pragma unroll
-                    for (int j = 0; j <= T::row(R - 1, W); ++j) {
-                        if (j >= nba) break;
-                        const double bv = kr[8 * C::LDK * j];
-#pragma unroll
-                        for (int r = 0; r < R; ++r)
-                            if (j <= T::row(r, W)) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
-                    }
-                }
-            });
-        }
+    const int nba = dual ? (L + 7) / 8 : NB;
+    sm.dual[tm] = dual ? L : 0;
+    sm.lam[tm] = lam_m;
+    if (dual && w == 0) {
         double qq = 0.0;
         for (int e = lane; e < D; e += 32) qq += sm.q[tm][e] * sm.q[tm][e];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) qq += __shfl_xor_sync(FULL, qq, o);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const int bi = T::row(r, w), idx = 8 * bi + g;
-            const double si = qq - sm.t[tm][idx];
-#pragma unroll
-            for (int j = 0; j < NB; ++j)
-                if (T::cols(r) > j && j <= bi && bi < nba) {
-                    double* cp = c[T::off(r) + j];
-                    const int jdx = 8 * j + 2 * t4;
-                    const bool in0 = idx < L && jdx < L, in1 = idx < L && jdx + 1 < L;
-                    cp[0] = in0 ? cp[0] + (si - sm.t[tm][jdx]) : 0.0;
-                    cp[1] = in1 ? cp[1] + (si - sm.t[tm][jdx + 1]) : 0.0;
-                    if (j == bi) {
-                        // ridge over weight for live keys (weights kept away from zero), one for the padding
-                        const double dg = idx < L ? lam_m / fmax(sm.s[tm][idx], 1e-290) : 1.0;
-                        if (g == 2 * t4) cp[0] += dg;
-                        if (g == 2 * t4 + 1) cp[1] += dg;
-                    }
-                }
-        }
-        for (int e = tt; e < 8 * nba; e += 32 * NW) ss.b[0][e] = e < L ? 1.0 : 0.0;
-    } else if (live) {
+        if (lane == 0) sm.qq[tm] = qq;
+    }
+    if (live && !dual) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             double a = asum[r];
@@ -323,7 +264,60 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 ss.b[0][cc] = a * inv - sm.q[tm][cc];
             }
         }
-        team::sync<NW>(bar_id);
+    }
+    // Dual rows of the block (its first keys are one chunk, still in shared memory; jlo = 0, for a window is never
+    // shorter than the rows that see at most d keys): z_j . z_l = k_j . k_l - k_j . q - k_l . q + q . q, of which the
+    // first product is the same for all of them.  The block's warps share its blocks out, and each
+    // writes a block of K K^T, corrected, into every dual row's matrix.
+    constexpr int GB = (T::LOWER + C::WARPS - 1) / C::WARPS;
+    double gm[GB][2];
+    const bool some_dual = jbeg == 0 && jend <= CH && (causal ? off + i0 + 1 : n) <= D;
+    if (some_dual) {
+#pragma unroll
+        for (int u = 0; u < GB; ++u) {
+            const int e = warp + C::WARPS * u;
+            int bi = 0;
+            while ((bi + 1) * (bi + 2) / 2 <= e) ++bi;
+            const int bj = e - team::blk(bi, 0);
+            gm[u][0] = gm[u][1] = 0.0;
+            if (e < T::LOWER && 8 * bi < jend) {
+                double x[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll 8
+                for (int s = 0; s < D / 4; ++s) team::dmma(x[s & 1][0], x[s & 1][1], sm.kv[8 * bi + g][4 * s + t4], sm.kv[8 * bj + g][4 * s + t4]);
+                gm[u][0] = x[0][0] + x[1][0];
+                gm[u][1] = x[0][1] + x[1][1];
+            }
+        }
+    }
+    __syncthreads();               // the keys are no longer read: their place takes the matrices
+    if (some_dual) {
+#pragma unroll
+        for (int u = 0; u < GB; ++u) {
+            const int e = warp + C::WARPS * u;
+            if (e >= T::LOWER) break;
+            int bi = 0;
+            while ((bi + 1) * (bi + 2) / 2 <= e) ++bi;
+            const int bj = e - team::blk(bi, 0), idx = 8 * bi + g, jdx = 8 * bj + 2 * t4;
+            for (int t = 0; t < TEAMS; ++t) {
+                const int Lt = sm.dual[t];
+                if (8 * bi >= Lt) continue;
+                const double si = sm.qq[t] - (idx < Lt ? sm.t[t][idx] : 0.0);
+                double v0 = idx < Lt && jdx < Lt ? gm[u][0] + (si - sm.t[t][jdx]) : 0.0;
+                double v1 = idx < Lt && jdx + 1 < Lt ? gm[u][1] + (si - sm.t[t][jdx + 1]) : 0.0;
+                if (bi == bj) {
+                    // ridge over weight for live keys (weights kept away from zero); the padding to a multiple of eight
+                    // is an identity block
+                    const double dg = idx < Lt ? sm.lam[t] / fmax(sm.s[t][idx], 1e-290) : 1.0;
+                    if (g == 2 * t4) v0 += dg;
+                    if (g == 2 * t4 + 1) v1 += dg;
+                }
+                *reinterpret_cast<double2*>(&sm.mat[t][e][2 * lane]) = make_double2(v0, v1);
+            }
+        }
+    }
+    if (dual) {
+        for (int e = tt; e < 8 * nba; e += 32 * NW) ss.b[0][e] = e < L ? 1.0 : 0.0;
+    } else if (live) {
         const double ridge = lam_m * inv;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -332,23 +326,21 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
 #pragma unroll
             for (int j = 0; j < NB; ++j)
                 if (T::cols(r) > j && j <= bi) {
-                    double* cp = c[T::off(r) + j];
                     const double2 kc = *reinterpret_cast<const double2*>(&sm.kbar[tm][8 * j + 2 * t4]);
-                    cp[0] = cp[0] * inv - kr * kc.x;
-                    cp[1] = cp[1] * inv - kr * kc.y;
+                    double v0 = c[T::off(r) + j][0] * inv - kr * kc.x, v1 = c[T::off(r) + j][1] * inv - kr * kc.y;
                     if (j == bi) {
-                        if (g == 2 * t4) cp[0] += ridge;
-                        if (g == 2 * t4 + 1) cp[1] += ridge;
+                        if (g == 2 * t4) v0 += ridge;
+                        if (g == 2 * t4 + 1) v1 += ridge;
                     }
+                    *reinterpret_cast<double2*>(&sm.mat[tm][team::blk(bi, j)][2 * lane]) = make_double2(v0, v1);
                 }
         }
     }
+    if (some_dual) __syncthreads();
     double ybar = 0.0, gfac = 1.0, csum = 0.0;
     if (live) {
         team::sync<NW>(bar_id);
-        if constexpr (NW <= 2) team::with_warp<NW>(w, [&](auto wc) { ok = team::solve<D, NW, 1>(c, ss, nba, decltype(wc)::value, lane, bar_id); });
-        else ok = team::solve<D, NW, 1>(c, ss, nba, w, lane, bar_id);
-        team::sync<NW>(bar_id);
+        ok = team::solve<D, NW, 1>(sm.mat[tm], ss, nba, w, lane, bar_id);
         if (dual) {
             // coefficients lambda' alpha_j over the chunk's keys
             for (int j = tt; j < CH; j += 32 * NW) {
@@ -356,12 +348,6 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 sm.s[tm][j] = cj;
                 csum += cj;
             }
-            if (rho_out)                                                   // rho = Z^T alpha
-                for (int e = tt; e < D; e += 32 * NW) {
-                    double a = 0.0;
-                    for (int j = 0; j < L; ++j) a += ss.x[w][0][j] * (sm.kv[j][e] - sm.q[tm][e]);
-                    rho_out[row * D + e] = (float)a;
-                }
         } else {
             double yb = 0.0, yk = 0.0;
             for (int e = lane; e < D; e += 32) {
@@ -384,29 +370,39 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     // ---- second sweep: coefficients and output ----
     const int ob = warp % NB, half = warp / NB;
     double o0 = 0.0, o1 = 0.0;
-    const bool one_chunk = jend - jbeg <= CH;
-    for (int j0 = jbeg; j0 < jend; j0 += CH) {
-        const int nk = min(CH, jend - j0);
+    // (a block of dual rows needs its keys again only for rho)
+    const bool keys = !some_dual || rho_out || (causal ? off + last + 1 : n) > D || lambda_rows || lambda == 0.0;
+    for (int j0 = jbeg; j0 < jend; j0 += ch) {
+        const int nk = min(ch, jend - j0);
         __syncthreads();
-        if (!one_chunk) {
-            stage<D>(sm.kv, kb, sk.r, j0, jend);
+        if (keys) {
+            stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
             __syncthreads();
-            dots<D>(sm.s, sm.q, sm.kv, nk, warp, lane);         // (a dual row's block is one chunk)
+            if (dual) {
+                if (rho_out)                                       // rho = Z^T alpha
+                    for (int e = tt; e < D; e += 32 * NW) {
+                        double a = 0.0;
+                        for (int j = 0; j < L; ++j) a += ss.x[w][0][j] * (sm.kv[j][e] - sm.q[tm][e]);
+                        rho_out[row * D + e] = (float)a;
+                    }
+            }
+            // scores again, except in a block of one chunk, which still has the weights
+            if (jend - jbeg > CH) dots<D>(sm.s, sm.q, sm.kv, nk, warp, lane);
         }
-        dots<D>(sm.t, sm.y, sm.kv, nk, warp, lane);
+        if (keys) dots<D>(sm.t, sm.y, sm.kv, nk, warp, lane);
         __syncthreads();
         if (!dual)
-            for (int j = tt; j < CH; j += 32 * NW) {
+            for (int j = tt; j < ch; j += 32 * NW) {
                 const bool vis = j < nk && j0 + j < L && j0 + j >= jlo;
                 double cj = 0.0;
                 if (vis) {
-                    const double e = one_chunk ? sm.s[tm][j] : exp(sm.s[tm][j] * scale - m_ref);
+                    const double e = jend - jbeg <= CH ? sm.s[tm][j] : exp(sm.s[tm][j] * scale - m_ref);
                     cj = e * (1.0 - (sm.t[tm][j] - ybar));
                 }
                 sm.s[tm][j] = cj;
                 csum += cj;
             }
-        stage<D>(sm.kv, vb, sv.r, j0, jend);
+        stage<D>(sm.kv, vb, sv.r, j0, jend, ch);
         __syncthreads();
         if (half < C::HALVES) {
             const int s1 = (nk + 3) / 4;
