@@ -22,7 +22,7 @@
 //   forward_tc_kernel     in solve mode: C_i t_i = h_i by conjugate gradients           (tcgen05 tensor cores)
 //   bwd_rowprep_kernel    y_i, the per-row scalars, dL/dlambda_i; y and -t as bf16 pairs
 //   pairs                 dQ per query tile, dK and dV per key tile
-//   bwd_head_rows_kernel  rows with fewer than head_rows keys: everything in fp64 with a direct solve
+//   bwd_rows_kernel       rows with fewer than head_rows keys: everything in fp64 with a direct solve (lla_backward_rows.cu)
 // The moments and pair kernels are the tcgen05 kernels of lla_backward_tensor.cu (dQ by plain stores of the tile
 // that owns the rows; dK and dV by atomic adds, which the direct rows and grouped heads also add into).  The fp32
 // CUDA-core versions in this file (impl = LLA_IMPL_SIMT) are kept as an independent cross-check; their pair kernel
@@ -428,203 +428,6 @@ bwd_pairs_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     }
 }
 
-// ------------------------------------------------------------------------------------------------
-// Rows that see fewer than head_rows keys: C is ill-conditioned (rank-deficient up to the ridge), so the
-// whole row -- both solves and every pair term -- runs in fp64 with an explicit C and a direct LDL^T
-// solve, the same split the forward makes.  One block per row; dK and dV go out with atomic adds.
-// ------------------------------------------------------------------------------------------------
-
-constexpr int HB_THREADS = 160;   // 136 4x4 tiles of the matrix build fit one round; four blocks per SM
-// eight lanes per key: sum over the lanes of a group of eight
-__device__ __forceinline__ double group8_sum(double x) {
-#pragma unroll
-    for (int o = 4; o >= 1; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-// D / 8 consecutive bf16 of a row -> doubles
-template <int NE>
-__device__ __forceinline__ void load_bf16_run(const __nv_bfloat16* p, double (&dst)[NE]) {
-#pragma unroll
-    for (int e = 0; e < NE; e += 8) {
-        const uint4 r = *reinterpret_cast<const uint4*>(p + e);
-        const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            dst[e + 2 * x] = (double)__uint_as_float(w[x] << 16);
-            dst[e + 2 * x + 1] = (double)__uint_as_float(w[x] & 0xFFFF0000u);
-        }
-    }
-}
-template <int D>
-__global__ void __launch_bounds__(HB_THREADS, D == 64 ? 4 : 1)
-bwd_head_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                     const __nv_bfloat16* __restrict__ v, const void* __restrict__ dout, int dout_dtype,
-                     float* __restrict__ dq, float* __restrict__ dk, float* __restrict__ dv, int n, int lcap,
-                     double scale, double lambda, int* __restrict__ status, float* __restrict__ dlambda, int H, int kv_group,
-                     int nq) {
-    constexpr int LDS = D + 1;
-    extern __shared__ __align__(16) double hb_smem[];
-    double* S = hb_smem;                  // D x (D + 1)
-    double* rhs = S + D * LDS;            // [2][D]: mbar -> y, h -> t
-    double* kb = rhs + 2 * D;
-    double* mb = kb + D;
-    double* qd = mb + D;
-    double* gd = qd + D;
-    double* hp = gd + D;                  // sum_j p_j gamma_j k_j
-    double* pj = hp + D;                  // [lcap] each
-    double* gam = pj + lcap;
-    double* ee = gam + lcap;
-    double* ff = ee + lcap;
-    __nv_bfloat16* Kr = reinterpret_cast<__nv_bfloat16*>(ff + lcap);   // [lcap][D]
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int bh = blockIdx.x;
-    const int i = gridDim.y - 1 - blockIdx.y;       // rows with the most keys first
-    const int L = (n - nq) + i + 1;                 // query row i sits at position n - nq + i
-    if (!LLA_IN_BOUNDS(L, lcap + 1, status, 602)) return;      // (debug build: the keys must fit the arrays sized for lcap)
-    const size_t base = (size_t)bh * nq;            // rows of q, dout, dq, dlambda
-    const size_t kvbase = (size_t)kv_unit(bh, H, kv_group) * n;     // grouped heads: the key/value head's rows
-    for (int c = tid; c < D; c += HB_THREADS) {
-        qd[c] = (double)__bfloat162float(q[(base + i) * D + c]);
-        gd[c] = (double)ld_any(dout, dout_dtype, (base + i) * D + c);
-    }
-    for (int idx = tid; idx < L * (D / 8); idx += HB_THREADS)
-        reinterpret_cast<uint4*>(Kr)[idx] = reinterpret_cast<const uint4*>(k + kvbase * D)[idx];
-    __syncthreads();
-    // scores and gamma_j = g . v_j: eight lanes per key (D / 8 consecutive elements each), four keys per warp
-    constexpr int NE = D / 8;
-    const int l8 = lane & 7, kslot = warp * 4 + (lane >> 3);
-    for (int j0 = 0; j0 < L; j0 += 4 * (HB_THREADS / 32)) {
-        const int j = j0 + kslot;
-        double s = 0.0, gv = 0.0;
-        if (j < L) {
-            double kk[NE], vv[NE];
-            load_bf16_run<NE>(Kr + j * D + NE * l8, kk);
-            load_bf16_run<NE>(v + (kvbase + j) * D + NE * l8, vv);
-#pragma unroll
-            for (int e = 0; e < NE; ++e) {
-                s += qd[NE * l8 + e] * kk[e];
-                gv += gd[NE * l8 + e] * vv[e];
-            }
-        }
-        s = group8_sum(s);
-        gv = group8_sum(gv);
-        if (j < L && l8 == 0) { pj[j] = scale * s; gam[j] = gv; }
-    }
-    __syncthreads();
-    double m = -1e300;
-    for (int j = 0; j < L; ++j) m = fmax(m, pj[j]);
-    __syncthreads();
-    for (int j = tid; j < L; j += HB_THREADS) pj[j] = exp(pj[j] - m);
-    __syncthreads();
-    double omega = 0.0;
-    for (int j = 0; j < L; ++j) omega += pj[j];
-    const double em_om = exp(-m) / omega;     // d(ridge of C) / d(lambda)
-    const double eps = lambda * em_om;
-    __syncthreads();
-    for (int j = tid; j < L; j += HB_THREADS) pj[j] /= omega;
-    __syncthreads();
-    double gbar = 0.0;
-    for (int j = 0; j < L; ++j) gbar += pj[j] * gam[j];
-    for (int c = tid; c < 2 * D; c += HB_THREADS) {
-        const int cc = c % D;
-        double acc = 0.0;
-        if (c < D) for (int j = 0; j < L; ++j) acc += pj[j] * (double)__bfloat162float(Kr[j * D + cc]);
-        else for (int j = 0; j < L; ++j) acc += pj[j] * gam[j] * (double)__bfloat162float(Kr[j * D + cc]);
-        (c < D ? kb : hp)[cc] = acc;
-    }
-    __syncthreads();
-    for (int c = tid; c < D; c += HB_THREADS) {
-        mb[c] = kb[c] - qd[c];
-        rhs[c] = mb[c];
-        rhs[D + c] = hp[c] - gbar * kb[c];
-    }
-    // C (lower triangle) in 4 x 4 blocks
-    for (int blk = tid; blk < (D / 4) * (D / 4); blk += HB_THREADS) {
-        const int a0 = (blk / (D / 4)) * 4, b0 = (blk % (D / 4)) * 4;
-        if (b0 > a0) continue;
-        double acc[4][4] = {};
-        for (int j = 0; j < L; ++j) {
-            // four consecutive bf16 keys per 8-byte load (a0, b0 are multiples of four)
-            const uint2 ra = *reinterpret_cast<const uint2*>(Kr + j * D + a0);
-            const uint2 rb = *reinterpret_cast<const uint2*>(Kr + j * D + b0);
-            const double ka[4] = {(double)__uint_as_float(ra.x << 16), (double)__uint_as_float(ra.x & 0xFFFF0000u),
-                                  (double)__uint_as_float(ra.y << 16), (double)__uint_as_float(ra.y & 0xFFFF0000u)};
-            const double kc[4] = {(double)__uint_as_float(rb.x << 16), (double)__uint_as_float(rb.x & 0xFFFF0000u),
-                                  (double)__uint_as_float(rb.y << 16), (double)__uint_as_float(rb.y & 0xFFFF0000u)};
-            const double p = pj[j];
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-#pragma unroll
-                for (int y = 0; y < 4; ++y) acc[x][y] += p * ka[x] * kc[y];
-        }
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-            for (int y = 0; y < 4; ++y) {
-                const int a = a0 + x, b = b0 + y;
-                if (b <= a) S[a * LDS + b] = acc[x][y] - kb[a] * kb[b] + (a == b ? eps : 0.0);
-            }
-    }
-    const bool okf = block_ldlt_solve<D>(S, LDS, rhs, D, 2, D);
-    if (!okf && tid == 0 && status) atomicAdd(status + LLA_STATUS_BAD_PIVOT, 1);
-    const double* y = rhs;
-    const double* t = rhs + D;
-    // e_j = xi_j . y, f_j = xi_j . t
-    for (int j0 = 0; j0 < L; j0 += 4 * (HB_THREADS / 32)) {
-        const int j = j0 + kslot;
-        double e = 0.0, f = 0.0;
-        if (j < L) {
-            double kk[NE];
-            load_bf16_run<NE>(Kr + j * D + NE * l8, kk);
-#pragma unroll
-            for (int x = 0; x < NE; ++x) {
-                const double xi = kk[x] - kb[NE * l8 + x];
-                e += xi * y[NE * l8 + x];
-                f += xi * t[NE * l8 + x];
-            }
-        }
-        e = group8_sum(e);
-        f = group8_sum(f);
-        if (j < L && l8 == 0) { ee[j] = e; ff[j] = f; }
-    }
-    __syncthreads();
-    double kappa = 0.0;
-    for (int j = 0; j < L; ++j) kappa += pj[j] * (1.0 - ee[j]) * gam[j];      // g . o_i
-    double ty = 0.0;
-    for (int c = 0; c < D; ++c) {
-        kappa += t[c] * mb[c];
-        ty += t[c] * y[c];
-    }
-    if (dlambda && tid == 0) dlambda[base + i] = (float)(em_om * ty);     // dL = t^T dC y
-    __syncthreads();
-    // per key: a_j -> pj, scale dL/ds_ij -> gam, p (f - gamma + gbar) -> ff, p (e - 1) -> ee
-    for (int j = tid; j < L; j += HB_THREADS) {
-        const double p = pj[j], e = ee[j], f = ff[j], gmj = gam[j];
-        pj[j] = p * (1.0 - e);
-        gam[j] = scale * p * (gmj * (1.0 - e) + (gbar + f) * e - f - kappa);
-        ff[j] = p * (f - gmj + gbar);
-        ee[j] = p * (e - 1.0);
-    }
-    __syncthreads();
-    for (int c = tid; c < D; c += HB_THREADS) {
-        double acc = t[c];
-        for (int j = 0; j < L; ++j) acc += gam[j] * (double)__bfloat162float(Kr[j * D + c]);
-        dq[(base + i) * D + c] = (float)acc;
-    }
-    // (one atomic per row and output: a version that wrote the per-key coefficients out and summed the rows in
-    //  a second kernel was slower, the sum's serial loop costing more than the atomics it saved)
-    for (int idx = tid; idx < L * D; idx += HB_THREADS) {
-        const int j = idx / D, c = idx % D;
-        atomicAdd(dk + (kvbase + j) * D + c, (float)(gam[j] * qd[c] + ff[j] * y[c] + ee[j] * t[c]));
-        atomicAdd(dv + (kvbase + j) * D + c, (float)(pj[j] * gd[c]));
-    }
-}
-
-template <int D>
-size_t head_smem_bytes(int lcap) {
-    return sizeof(double) * ((size_t)D * (D + 1) + 7 * D + 4 * lcap) + sizeof(__nv_bfloat16) * (size_t)lcap * D;
-}
-
 // workspace: kbar, h, t, y as [rows][D] fp32, the scalar records, then the tensor-core kernels' bf16 operand arrays
 // (y and -t as hi and lo; the upstream gradient's hi and lo, used when it comes in fp32)
 size_t ws_floats(long long rows, int d) { return (size_t)rows * (4 * (size_t)d + BW_ROWSC); }
@@ -658,10 +461,6 @@ int launch_t(const BackwardArgs& a) {
     const auto* q = static_cast<const __nv_bfloat16*>(a.q);
     const auto* k = static_cast<const __nv_bfloat16*>(a.k);
     const auto* v = static_cast<const __nv_bfloat16*>(a.v);
-    const int lcap = first > 0 ? off + first : 0;              // most keys a directly-solved row sees
-    const size_t head_smem = head_smem_bytes<D>(lcap);
-    if (head_smem > 227u * 1024u) return LLA_ERR_UNSUPPORTED;
-    LLA_CUDA_TRY(cudaFuncSetAttribute(bwd_head_rows_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)head_smem));
     LLA_CUDA_TRY(cudaMemsetAsync(a.dk, 0, sizeof(float) * kvrows * D, a.stream));
     LLA_CUDA_TRY(cudaMemsetAsync(a.dv, 0, sizeof(float) * kvrows * D, a.stream));
     // the directly-solved rows depend on nothing the other kernels make: they run beside them on the side stream
@@ -672,10 +471,8 @@ int launch_t(const BackwardArgs& a) {
         LLA_CUDA_TRY(cudaStreamWaitEvent(hs, a.fork, 0));
     }
     if (first > 0) {
-        const dim3 gh(BH, first);
-        bwd_head_rows_kernel<D><<<gh, HB_THREADS, head_smem, hs>>>(
-            q, k, v, a.dout, a.dout_dtype, a.dq, a.dk, a.dv, a.n, lcap, (double)a.scale, (double)a.lambda, a.status, a.dlambda, a.H, kvg, nq);
-        LLA_CUDA_TRY(cudaGetLastError());
+        const int rc_rows = launch_backward_rows(a, nq, first, hs);
+        if (rc_rows != LLA_OK) return rc_rows;
         if (forked) LLA_CUDA_TRY(cudaEventRecord(a.join, hs));
     }
     if (first < nq) {

@@ -219,6 +219,7 @@ struct BwdTensorArgs {
 int launch_backward_tensor(const BwdTensorArgs& a, int which);   // which: 0 = kbar, gbar, h; 1 = dQ; 2 = dK and dV
 size_t backward_workspace_bytes(int B, int H, int n, int d);
 int launch_backward(const BackwardArgs& a);
+int launch_backward_rows(const BackwardArgs& a, int nq, int rows, cudaStream_t stream);      // the directly-solved rows
 
 // Launchers implemented in the other translation units; each returns an lla_status.
 int head_rows_count(const ForwardArgs& a);   // leading query rows per head solved directly

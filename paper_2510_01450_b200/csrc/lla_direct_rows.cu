@@ -23,25 +23,10 @@
 // What bounds it: the matrix pipe in the moments of long rows (36 of the about 47 instructions per 4 keys and row at
 // d = 64; measured at 89 % of its rate), the chain of reciprocals in the pivot blocks for short ones, which the eight
 // systems of two blocks on an SM hide in part.
-#include "lla_team_solve.cuh"
+#include "lla_rows.cuh"
 
 namespace lla {
 namespace {
-
-template <int D>
-struct DrCfg {
-    static constexpr int NW = D == 16 ? 1 : D == 64 ? 2 : 8;      // warps per row: what the registers of 16 warps hold
-    static constexpr int TEAMS = D == 128 ? 2 : 4;                // rows per block; d = 64: two blocks per SM, so that the pivot
-                                                                  // chains of one run beside the products of the other
-    static constexpr int WARPS = NW * TEAMS, THREADS = 32 * WARPS;
-    // keys per chunk: the keys of a block with a dual row (at most d + TEAMS - 1, with a window d + TEAMS) are one chunk
-    static constexpr int CH = D == 128 ? 136 : D == 64 ? 72 : 64;
-    static constexpr int STEP = D == 128 ? 128 : 64;              // .. and the others' chunks: eight keys a warp
-    static constexpr int LDK = D + 4;                             // row stride in doubles: 4 mod 16, both operand accesses conflict-free
-    static constexpr int NB = D / 8;
-    static constexpr int HALVES = WARPS / NB;                     // output sum: a warp per 8 columns and part of the keys
-    static constexpr int LDW = CH + 4;
-};
 
 template <int D>
 struct DrSmem {
@@ -62,52 +47,6 @@ struct DrSmem {
     team::Smem<D, C::NW, 1> solve[C::TEAMS];
 };
 
-template <typename TIn>
-__device__ __forceinline__ void load_pair(const TIn* p, double& a, double& b);
-template <>
-__device__ __forceinline__ void load_pair<__nv_bfloat16>(const __nv_bfloat16* p, double& a, double& b) {
-    const uint32_t raw = *reinterpret_cast<const uint32_t*>(p);
-    a = (double)__uint_as_float(raw << 16);
-    b = (double)__uint_as_float(raw & 0xFFFF0000u);
-}
-template <>
-__device__ __forceinline__ void load_pair<float>(const float* p, double& a, double& b) {
-    const float2 f = *reinterpret_cast<const float2*>(p);
-    a = (double)f.x;
-    b = (double)f.y;
-}
-
-// keys (or values) j0 .. j0 + ch - 1 -> shared memory; rows from jend on are zero
-template <int D, typename TIn>
-__device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch) {
-    using C = DrCfg<D>;
-    constexpr int PER = C::CH * D / 2 / C::THREADS, PER_STEP = C::STEP * D / 2 / C::THREADS;
-    static_assert(PER * 2 * C::THREADS == C::CH * D && PER_STEP * 2 * C::THREADS == C::STEP * D, "a chunk is a whole number of rounds");
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        if (u >= PER_STEP && ch == C::STEP) break;
-        const int e = threadIdx.x + C::THREADS * u, j = e / (D / 2), c = 2 * (e % (D / 2));
-        double a = 0.0, b = 0.0;
-        if (j0 + j < jend) load_pair(src + (size_t)(j0 + j) * stride + c, a, b);
-        *reinterpret_cast<double2*>(&dst[j][c]) = make_double2(a, b);
-    }
-}
-
-// out[TEAMS][CH] = rows . keys, eight keys per step of a warp
-template <int D>
-__device__ __forceinline__ void dots(double (*out)[DrCfg<D>::LDW], const double (*rows)[DrCfg<D>::LDK], const double (*keys)[DrCfg<D>::LDK],
-                                     int nkeys, int warp, int lane) {
-    using C = DrCfg<D>;
-    const int n = lane >> 2, t4 = lane & 3;
-    for (int kb = warp; 8 * kb < nkeys; kb += C::WARPS) {
-        double c[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll
-        for (int s = 0; s < D / 4; ++s)
-            team::dmma(c[s & 1][0], c[s & 1][1], n < C::TEAMS ? rows[n][4 * s + t4] : 0.0, keys[8 * kb + n][4 * s + t4]);
-        if (n < C::TEAMS) *reinterpret_cast<double2*>(&out[n][8 * kb + 2 * t4]) = make_double2(c[0][0] + c[1][0], c[0][1] + c[1][1]);
-    }
-}
-
 template <int D, typename TIn, typename TOut>
 __global__ void __launch_bounds__(DrCfg<D>::THREADS, D == 64 ? 2 : 1)
 direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v, TOut* __restrict__ out,
@@ -121,6 +60,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char dr_smem[];
     DrSmem<D>& sm = *reinterpret_cast<DrSmem<D>*>(dr_smem);
+    auto row_of = [](auto& rows) { return [&rows](int r) { return &rows[r][0]; }; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
     const int tm = warp / NW, w = warp % NW, tt = tid % (32 * NW);      // team, warp and thread inside the team
     const int bar_id = 1 + tm;
@@ -179,7 +119,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         __syncthreads();
         stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
         __syncthreads();
-        dots<D>(sm.s, sm.q, sm.kv, nk, warp, lane);
+        dots<D>(row_of(sm.s), row_of(sm.q), sm.kv, nk, warp, lane);
         __syncthreads();
         if (j0 >= L || j0 + ch <= jlo) continue;                          // (uniform over the team) no key of this row
         double cmax = -INFINITY;
@@ -387,9 +327,9 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                     }
             }
             // scores again, except in a block of one chunk, which still has the weights
-            if (jend - jbeg > CH) dots<D>(sm.s, sm.q, sm.kv, nk, warp, lane);
+            if (jend - jbeg > CH) dots<D>(row_of(sm.s), row_of(sm.q), sm.kv, nk, warp, lane);
         }
-        if (keys) dots<D>(sm.t, sm.y, sm.kv, nk, warp, lane);
+        if (keys) dots<D>(row_of(sm.t), row_of(sm.y), sm.kv, nk, warp, lane);
         __syncthreads();
         if (!dual)
             for (int j = tt; j < ch; j += 32 * NW) {

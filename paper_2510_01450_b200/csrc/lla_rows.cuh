@@ -1,0 +1,73 @@
+// What the kernels of the directly-solved rows share (forward: lla_direct_rows.cu, backward: lla_backward_rows.cu): block
+// shapes, staging of keys and values as doubles, and products of a block's rows with the staged keys.
+#pragma once
+
+#include "lla_team_solve.cuh"
+
+namespace lla {
+
+template <int D>
+struct DrCfg {
+    static constexpr int NW = D == 16 ? 1 : D == 64 ? 2 : 8;      // warps per row: what the registers of 16 warps hold
+    static constexpr int TEAMS = D == 128 ? 2 : 4;                // rows per block; d = 64: two blocks per SM, so that the pivot
+                                                                  // chains of one run beside the products of the other
+    static constexpr int WARPS = NW * TEAMS, THREADS = 32 * WARPS;
+    // keys per chunk: the keys of a block with a dual row (at most d + TEAMS - 1, with a window d + TEAMS) are one chunk,
+    // and at d = 64 so are those of every row solved directly for its few keys
+    static constexpr int CH = D == 128 ? 136 : D == 64 ? 128 : 64;
+    static constexpr int STEP = D == 128 ? 128 : 64;              // .. and the chunks of longer blocks: eight keys a warp
+    static constexpr int LDK = D + 4;                             // row stride in doubles: 4 mod 16, both operand accesses conflict-free
+    static constexpr int NB = D / 8;
+    static constexpr int HALVES = WARPS / NB;                     // output sum: a warp per 8 columns and part of the keys
+    static constexpr int LDW = CH + 4;
+};
+
+template <typename TIn>
+__device__ __forceinline__ void load_pair(const TIn* p, double& a, double& b);
+template <>
+__device__ __forceinline__ void load_pair<__nv_bfloat16>(const __nv_bfloat16* p, double& a, double& b) {
+    const uint32_t raw = *reinterpret_cast<const uint32_t*>(p);
+    a = (double)__uint_as_float(raw << 16);
+    b = (double)__uint_as_float(raw & 0xFFFF0000u);
+}
+template <>
+__device__ __forceinline__ void load_pair<float>(const float* p, double& a, double& b) {
+    const float2 f = *reinterpret_cast<const float2*>(p);
+    a = (double)f.x;
+    b = (double)f.y;
+}
+
+// keys (or values) j0 .. j0 + ch - 1 -> shared memory; rows from jend on are zero
+template <int D, typename TIn>
+__device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch) {
+    using C = DrCfg<D>;
+    constexpr int PER = C::CH * D / 2 / C::THREADS, PER_STEP = C::STEP * D / 2 / C::THREADS;
+    static_assert(PER * 2 * C::THREADS == C::CH * D && PER_STEP * 2 * C::THREADS == C::STEP * D, "a chunk is a whole number of rounds");
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        if (u >= PER_STEP && ch == C::STEP) break;
+        const int e = threadIdx.x + C::THREADS * u, j = e / (D / 2), c = 2 * (e % (D / 2));
+        double a = 0.0, b = 0.0;
+        if (j0 + j < jend) load_pair(src + (size_t)(j0 + j) * stride + c, a, b);
+        *reinterpret_cast<double2*>(&dst[j][c]) = make_double2(a, b);
+    }
+}
+
+// out(r)[j] = row(r) . keys[j], eight keys per step of a warp; row and out: pointers of the block's r-th row
+template <int D, typename Row, typename Out>
+__device__ __forceinline__ void dots(Out&& out, Row&& row, const double (*keys)[DrCfg<D>::LDK], int nkeys, int warp, int lane) {
+    using C = DrCfg<D>;
+    const int n = lane >> 2, t4 = lane & 3;
+    const double* rp = row(n < C::TEAMS ? n : 0);
+    for (int kb = warp; 8 * kb < nkeys; kb += C::WARPS) {
+        double c[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+        for (int s = 0; s < D / 4; ++s) {
+            const double a = rp[4 * s + t4];
+            team::dmma(c[s & 1][0], c[s & 1][1], n < C::TEAMS ? a : 0.0, keys[8 * kb + n][4 * s + t4]);
+        }
+        if (n < C::TEAMS) *reinterpret_cast<double2*>(out(n) + 8 * kb + 2 * t4) = make_double2(c[0][0] + c[1][0], c[0][1] + c[1][1]);
+    }
+}
+
+}  // namespace lla
