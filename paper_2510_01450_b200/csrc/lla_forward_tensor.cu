@@ -100,14 +100,17 @@ enum { B_QFULL = 0, B_KVFULL = 1, B_KVEMPTY = B_KVFULL + TC_NST_MAX, B_VFULL = B
        B_UFULL = B_SAFULL + TC_NBUF, B_BUFFREE = B_UFULL + TC_NBUF, B_ACCFULL = B_BUFFREE + TC_NBUF, B_CTL = B_ACCFULL + 1,
        B_EXIT = B_CTL + 1,   // two: the MMA warps' last commits on an aborted run
        B_MFULL = B_EXIT + 2, // the preconditioner matrix has landed
-       B_COUNT = B_MFULL + 1 };
+       B_XREADY = B_MFULL + 1, B_XFULL = B_XREADY + 1,   // exchange of a pair of blocks: the other's sweep is done, its sums are here
+       B_COUNT = B_XFULL + 1 };
 static_assert(B_COUNT * 8 <= 256, "barrier area too small");
 
 constexpr uint32_t IDESC_SS = make_idesc(TC_BR, TC_BC, 0, 0);   // S/A: A, B K-major; ACC uses make_idesc(128, D, 0, 1)
 constexpr uint32_t IDESC_SS16 = make_idesc(TC_BR, TC_BC, 0, 0, /*f16=*/1);   // the same products with both operands fp16
 
 struct TcParams {
-    int n, nq, causal, head_rows, max_iters, first_tile;   // n keys; nq query rows at positions n - nq .. n - 1
+    int n, nq, causal, head_rows, max_iters, first_tile;   // n keys; nq query rows of a unit
+    int nq_pos;          // query rows of a head, at positions n - nq_pos .. n - 1.  nq = nq_pos, or a multiple of it: the heads
+                         // that share a key/value head as one unit, row r being row r % nq_pos of its head r / nq_pos
     int precise_iters;   // CG iterations whose operands are bf16 hi + lo pairs; later ones use single fp16 operands
     int precise_iters_early;   // the same for the row tiles that end within the first 8 D positions
     long long wait_clocks;   // cap of every bounded wait, in SM clocks
@@ -117,7 +120,7 @@ struct TcParams {
     float scale, lambda, tol;
     float* rho;
     float* stats;
-    int H, kv_group;     // query heads per (batch), query heads per key/value head
+    int H, kv_group;     // units per batch, units per key/value head
     Strides so;          // layout of out [B, H, nq, D]
     int window;          // causal sliding window (0: none): a row sees its last `window` positions
     const float* rhs;    // solve mode: right-hand sides h_i [B, H, nq, D]; the CG then solves C_i x = h_i ...
@@ -139,7 +142,11 @@ struct TcParams {
 // PC: preconditioned CG compiled in (an instance of its own, so that the plain path carries none of its code).
 // GIVEN: solve mode with kbar and the saved row statistics supplied (fp32 output type only), likewise an instance
 // of its own: the statistics sweep is compiled out.
-template <int D, typename TOut, bool PC, bool GIVEN = false>
+// NS = 2: the blocks come in clusters of two that share a query tile, each sweeping half of its key blocks.  After a sweep
+// they add up their accumulators and row sums (through distributed shared memory, into the other block's operand tiles,
+// which nothing reads between two sweeps) and carry on with the same numbers.  For grids that leave much of the chip
+// idle; see launch_t.
+template <int D, typename TOut, bool PC, bool GIVEN = false, int NS = 1>
 __global__ void __launch_bounds__(D == 128 ? 384 : TC_THREADS, 1)
 forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK16,
@@ -180,14 +187,22 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // blockIdx.x runs fastest in launch order: all heads of one query tile start together, the tiles
     // in order of decreasing estimated cost (see tile_order on the host side)
-    const int bh = blockIdx.x;
+    const int bh = blockIdx.x / NS;
+    const uint32_t rank = NS > 1 ? cluster_rank() : 0u;
     const int tile = prm.first_tile + (prm.use_order ? (int)prm.order[blockIdx.y] : (int)(gridDim.y - 1 - blockIdx.y));
     const int r0 = tile * TC_BR;
-    const int n = prm.n, nq = prm.nq, off = n - nq;     // query row r sits at position off + r
+    const int n = prm.n, nq = prm.nq, off = n - prm.nq_pos;     // row r of a head sits at position off + r
     const int nblk_all = (n + TC_BC - 1) / TC_BC;
-    const int cend = prm.causal ? min(nblk_all, (off + r0 + TC_BR + TC_BC - 1) / TC_BC) : nblk_all;
+    // the tile's rows inside their heads: from r0p on; a tile that runs over a head's end holds rows 0 .. of the next
+    const int r0p = r0 % prm.nq_pos;
+    const bool wraps = r0p + TC_BR > prm.nq_pos && r0 - r0p + prm.nq_pos < nq;
+    int cend = prm.causal ? min(nblk_all, (off + (wraps ? prm.nq_pos : r0p + TC_BR) + TC_BC - 1) / TC_BC) : nblk_all;
     // sliding window: the tile's sweeps start at the block that holds its first row's first visible key
-    const int cbeg = (prm.causal && prm.window > 0) ? max(0, off + r0 + 1 - prm.window) / TC_BC : 0;
+    int cbeg = (prm.causal && prm.window > 0) ? max(0, off + (wraps ? 0 : r0p) + 1 - prm.window) / TC_BC : 0;
+    if (NS > 1) {
+        const int mid = cbeg + (cend - cbeg + 1) / 2;
+        if (rank == 0) cend = mid; else cbeg = mid;
+    }
     // Block sparsity: the sweeps visit only the key blocks that the caller's mask lists for this query tile, plus
     // the ones that are always attended -- the blocks of the first head_rows keys (so that every row keeps enough
     // keys for its system to be well posed and the directly-solved rows are untouched) and the tile's diagonal blocks.
@@ -216,7 +231,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // 16-bit format).  The values of the copies equal the bf16 inputs (the pre-pass checks the range).  Every role
     // counts the CG sweeps it has seen, so all of them know a sweep's format, and the next one's, without being
     // told.  (Tiles whose rows see fewer than 8 D keys converge more slowly and keep the pairs for longer.)
-    const int precise = off + r0 + TC_BR <= 8 * D ? prm.precise_iters_early : prm.precise_iters;
+    const int precise = off + r0p + TC_BR <= 8 * D ? prm.precise_iters_early : prm.precise_iters;
     const bool f16_on = prm.f16_ok && *prm.f16_ok && precise < (1 << 29);
     const long long wcap = prm.wait_clocks;
 
@@ -237,6 +252,8 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         mbar_init(bar(B_EXIT), 1);
         mbar_init(bar(B_EXIT + 1), 1);
         mbar_init(bar(B_MFULL), 1);
+        mbar_init(bar(B_XREADY), TC_COMPUTE / 32);
+        mbar_init(bar(B_XFULL), TC_COMPUTE / 32);
         misc[4] = SW_STATS;
         misc[5] = SW_STATS;
         misc[2] = 0;
@@ -249,6 +266,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     }
     tc_fence_before();
     __syncthreads();
+    if (NS > 1) cluster_sync();        // the other block's barriers exist
     tc_fence_after();
     const uint32_t tmem = (uint32_t)misc[0];
 
@@ -434,7 +452,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const int quad = warp & 3, half = warp >> 2;
         const int lrow = quad * 32 + lane;                 // row inside the tile == TMEM lane
         const int row = r0 + lrow;
-        const int L = prm.causal ? off + row + 1 : n;
+        const int L = prm.causal && row < nq ? off + row % prm.nq_pos + 1 : n;
         const int jlo = (prm.causal && prm.window > 0) ? max(0, L - prm.window) : 0;     // first visible key
         const bool row_ok = row < nq && L >= prm.head_rows;
         const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
@@ -676,6 +694,42 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
             tc_fence_before();
         };
+        // The two blocks of a pair: vec (this thread's NCOL accumulator values, or nothing) and a become the sums over
+        // both, b the larger.  Both blocks add the same two numbers, so from here on they compute the same.
+        uint32_t x_uses = 0;
+        float* xsc = reinterpret_cast<float*>(smem + Cfg::SM_BLIST);      // [2][256] (a block-sparse call has no pairs)
+        auto exchange = [&](float* vec, float& a, float& b) {
+            const uint32_t other = rank ^ 1u, ph = x_uses++ & 1;
+            // this warp's sweep is over and it has read what the last exchange brought: the other block may write
+            __syncwarp();
+            if (lane == 0) mbar_arrive_peer(peer_addr(bar(B_XREADY), other));
+            if (ok) ok = mbar_wait_cluster(bar(B_XREADY), ph, abort_flag, wcap);
+            if (ok) {
+                const uint32_t dst = peer_addr(sbase + SM_PHI, other) + 4u * (c0 * TC_BR + lrow);
+                if (vec) {
+#pragma unroll
+                    for (int e = 0; e < NCOL; ++e) st_peer(dst + 4u * e * TC_BR, vec[e]);
+                }
+                const uint32_t sc = peer_addr(sbase + Cfg::SM_BLIST, other) + 4u * tid;
+                st_peer(sc, a);
+                st_peer(sc + 1024u, b);
+                fence_cluster();
+            }
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) {
+                if (lane == 0) mbar_arrive_peer(peer_addr(bar(B_XFULL), other));
+                ok = mbar_wait_cluster(bar(B_XFULL), ph, abort_flag, wcap);
+            }
+            ok = all_ok(ok);
+            if (!ok) return;
+            if (vec) {
+                const float* src = reinterpret_cast<const float*>(smem + SM_PHI) + c0 * TC_BR + lrow;
+#pragma unroll
+                for (int e = 0; e < NCOL; ++e) vec[e] += src[e * TC_BR];
+            }
+            a += xsc[tid];
+            b = fmaxf(b, xsc[256 + tid]);
+        };
         uint32_t ctl_phase = 0;
         auto start_sweep = [&](int kind, bool f16 = false) {
             if (f16 && !q_is_f16) convert_q();
@@ -785,6 +839,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 if (ok) acc_wait();
                 ok = all_ok(ok);
                 if (!ok) break;
+                if (NS > 1) {
+                    exchange(nullptr, part, smax);
+                    if (!ok) break;
+                }
                 tmax = pair_max(smax) + mx2;
                 if (attempt == 1 || !group_any(row_ok && !(fabsf(tmax) <= 8.f))) break;
                 mx2 = fabsf(tmax) < 1e30f ? tmax : 0.f;     // (a row without a finite score keeps shift zero)
@@ -801,6 +859,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     }
                 } else {
                     acc_load(acc);
+                    if (NS > 1) {
+                        float u0 = 0.f, u1 = 0.f;
+                        exchange(acc, u0, u1);
+                    }
                     omega = pair_sum(part);
                 }
                 inv_omega = 1.f / omega;
@@ -873,6 +935,11 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (!ok) break;
             float ap[NCOL];
             acc_load(ap);
+            if (NS > 1) {
+                float u0 = 0.f, u1 = 0.f;
+                exchange(ap, u0, u1);
+                if (!ok) break;
+            }
             // (the loops below keep four independent partial sums and move the row-vector state in
             //  batches of eight so that the loads overlap: two warps per scheduler hide no latency)
             float pp[4] = {0.f, 0.f, 0.f, 0.f};
@@ -975,7 +1042,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // ---- output sweep ----
         float gfac = 1.f;
         if (ok && prm.sol) {
-            if (row_ok && LLA_IN_BOUNDS((size_t)bh * nq + row, (size_t)gridDim.x * nq, prm.status, 101)) {
+            if (rank == 0 && row_ok && LLA_IN_BOUNDS((size_t)bh * nq + row, (size_t)(gridDim.x / NS) * nq, prm.status, 101)) {
                 const size_t rowi = (size_t)bh * nq + row;
 #pragma unroll
                 for (int e = 0; e < NCOL; ++e) prm.sol[rowi * D + c0 + e] = xs[(c0 + e) * TC_BR + lrow];
@@ -1008,17 +1075,22 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (out16) write_operand16_pair(y);
             else write_operand(y);
             start_sweep(SW_OUT, out16);
-            const float part = sweep(SW_OUT);
+            float part = sweep(SW_OUT);
             if (ok) acc_wait();
             ok = all_ok(ok);
             if (ok) {
                 float o[NCOL];
                 acc_load(o);
+                if (NS > 1) {
+                    float u1 = 0.f;
+                    exchange(o, part, u1);
+                }
                 den = pair_sum(part);
-                if (row_ok && LLA_IN_BOUNDS((size_t)bh * nq + row, (size_t)gridDim.x * nq, prm.status, 102)) {
+                if (ok && rank == 0 && row_ok && LLA_IN_BOUNDS((size_t)bh * nq + row, (size_t)(gridDim.x / NS) * nq, prm.status, 102)) {
                     const float inv_den = 1.f / den;
                     const size_t rowi = (size_t)bh * nq + row;
-                    TOut* orow = out + prm.so.at(bh / prm.H, bh % prm.H, row) + c0;
+                    const int hin = row / prm.nq_pos;       // head inside the unit
+                    TOut* orow = out + prm.so.at(bh / prm.H, (bh % prm.H) * (nq / prm.nq_pos) + hin, row - hin * prm.nq_pos) + c0;
 #pragma unroll
                     for (int e = 0; e < NCOL; ++e) store_out(orow + e, o[e] * inv_den);
                     if (prm.rho) {
@@ -1048,6 +1120,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // (on an aborted run the TMA warp and the MMA warps have waited above for what they had issued)
     tc_fence_before();
     __syncthreads();
+    if (NS > 1) cluster_sync();        // neither block leaves while the other may still write to it
     if (warp == 8) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS) : "memory");
@@ -1151,20 +1224,28 @@ int launch_t(const ForwardArgs& a) {
     const int hr = head_rows_count(a);
     if (!a.causal && hr >= a.nq) return LLA_OK;
     const int first_tile = a.causal ? hr / TC_BR : 0;
-    const int tiles = (a.nq + TC_BR - 1) / TC_BR - first_tile;
+    int tiles = (a.nq + TC_BR - 1) / TC_BR - first_tile;
     if (tiles <= 0) return LLA_OK;
     CUtensorMap mq, mk, mv, mk16, mm;
-    const int BH = a.B * a.H;
     const int Hk = a.H / a.kv_group;
+    // A chunk of queries far into the sequence under grouped heads: the heads of a group read the same keys, so their rows
+    // can fill tiles together where a head's own rows leave its last tile partly empty (257 rows of four heads: nine
+    // tiles instead of twelve).  Their rows must lie one behind the other in q, and none may be solved directly.
+    const int group = a.kv_group;
+    const bool pack = group > 1 && hr == 0 && !a.block_mask && !a.minv && a.sq.h == (long long)a.nq * a.sq.r &&
+                      (group * a.nq + TC_BR - 1) / TC_BR < group * tiles;
+    const int units = pack ? a.B * Hk : a.B * a.H;          // unit: the rows that are cut into tiles together
+    const int unit_rows = pack ? group * a.nq : a.nq;
+    if (pack) tiles = (unit_rows + TC_BR - 1) / TC_BR;
     const auto BF = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, F16 = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    if (!make_map_16bit_4d(&mq, a.q, a.B, a.H, a.nq, D, a.sq.b, a.sq.h, a.sq.r, TC_BR, BF) ||
+    if (!make_map_16bit_4d(&mq, a.q, a.B, pack ? Hk : a.H, unit_rows, D, a.sq.b, pack ? group * a.sq.h : a.sq.h, a.sq.r, TC_BR, BF) ||
         !make_map_16bit_4d(&mk, a.k, a.B, Hk, a.n, D, a.sk.b, a.sk.h, a.sk.r, TC_BC, BF) ||
         !make_map_16bit_4d(&mv, a.v, a.B, Hk, a.n, D, a.sv.b, a.sv.h, a.sv.r, TC_BC, BF))
         return LLA_ERR_CUDA;
     mk16 = mk;
     mm = mk;
     TcParams prm;
-    prm.n = a.n; prm.nq = a.nq; prm.causal = a.causal; prm.head_rows = a.head_rows > 0 ? a.head_rows : 0;
+    prm.n = a.n; prm.nq = unit_rows; prm.nq_pos = a.nq; prm.causal = a.causal; prm.head_rows = a.head_rows > 0 ? a.head_rows : 0;
     prm.max_iters = a.max_iters; prm.first_tile = first_tile;
     prm.precise_iters = a.precise_iters;
     prm.precise_iters_early = a.precise_iters_early;
@@ -1174,7 +1255,7 @@ int launch_t(const ForwardArgs& a) {
     prm.lambda_rows = a.lambda_rows; prm.ridge_mode = a.ridge_mode;
     prm.block_mask = a.block_mask; prm.block_mask_stride = a.block_mask_stride;
     prm.rhs = a.rhs; prm.sol = a.sol; prm.kbar_in = a.kbar_in; prm.stats_in = a.stats_in;
-    prm.H = a.H; prm.kv_group = a.kv_group > 0 ? a.kv_group : 1;
+    prm.H = pack ? Hk : a.H; prm.kv_group = pack ? 1 : group;
     prm.so = a.so;
     prm.rho = a.rho; prm.stats = a.stats; prm.iters = a.iters; prm.status = a.status;
     prm.scratch = nullptr;
@@ -1184,7 +1265,8 @@ int launch_t(const ForwardArgs& a) {
     char* ws = static_cast<char*>(a.workspace);
     size_t ws_left = a.workspace ? a.workspace_bytes : 0;
     prm.window = a.causal ? a.window : 0;
-    tile_order(prm, tiles, first_tile, a.n, a.n - a.nq, D, a.causal, prm.window, a.minv != nullptr);
+    if (pack) prm.use_order = 0;
+    else tile_order(prm, tiles, first_tile, a.n, a.n - a.nq, D, a.causal, prm.window, a.minv != nullptr);
     if constexpr (!Cfg::STATE_IN_SMEM) {
         int dev = 0, sms = 0;
         LLA_CUDA_TRY(cudaGetDevice(&dev));
@@ -1216,13 +1298,39 @@ int launch_t(const ForwardArgs& a) {
         if (!make_map_16bit_4d(&mm, a.minv, a.B, Hk, (long long)precond_blocks(a.n) * D, D, cm.b, cm.h, cm.r, 64, F16)) return LLA_ERR_CUDA;
         precond = true;
     }
-    auto kern = precond ? forward_tc_kernel<D, TOut, true> : forward_tc_kernel<D, TOut, false>;
+    // Pairs of blocks per tile when the grid leaves SMs idle.  A sweep costs about 7 + (key blocks) in units of 0.9 K clocks
+    // (three more with the exchange of a pair), a launch as many rounds of its longest blocks as the SMs need.
+    int sms = 148;
+    {
+        int dev = 0;
+        LLA_CUDA_TRY(cudaGetDevice(&dev));
+        LLA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    }
+    const long long grid1 = (long long)units * tiles;
+    const int most = ((prm.window > 0 ? std::min(a.n, prm.window + TC_BR) : a.n) + TC_BC - 1) / TC_BC;
+    const int least = !a.causal ? most : std::min(most, (a.n - a.nq + first_tile * TC_BR + TC_BC) / TC_BC);
+    const double one = (double)((grid1 + sms - 1) / sms) * (7 + most), two = (double)((2 * grid1 + sms - 1) / sms) * (10 + 0.5 * most);
+    const bool pairs = !precond && !a.block_mask && least >= 4 && two < 0.95 * one;
+    auto kern = precond ? forward_tc_kernel<D, TOut, true> : pairs ? forward_tc_kernel<D, TOut, false, false, 2> : forward_tc_kernel<D, TOut, false>;
     if constexpr (std::is_same<TOut, float>::value) {
-        if (a.sol && a.kbar_in && a.stats_in) kern = precond ? forward_tc_kernel<D, TOut, true, true> : forward_tc_kernel<D, TOut, false, true>;
+        if (a.sol && a.kbar_in && a.stats_in)
+            kern = precond ? forward_tc_kernel<D, TOut, true, true>
+                           : pairs ? forward_tc_kernel<D, TOut, false, true, 2> : forward_tc_kernel<D, TOut, false, true>;
     }
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SM_ALLOC));
-    dim3 grid(BH, tiles);
-    kern<<<grid, D == 128 ? 384 : TC_THREADS, Cfg::SM_ALLOC, a.stream>>>(mq, mk, mv, mk16, mm, (TOut*)a.out, prm);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(units * (pairs ? 2 : 1), tiles);
+    cfg.blockDim = dim3(D == 128 ? 384 : TC_THREADS);
+    cfg.dynamicSmemBytes = Cfg::SM_ALLOC;
+    cfg.stream = a.stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pairs ? 1 : 0;
+    LLA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, mq, mk, mv, mk16, mm, (TOut*)a.out, prm));
     LLA_CUDA_TRY(cudaGetLastError());
     return LLA_OK;
 }

@@ -65,6 +65,42 @@ __device__ __forceinline__ bool mbar_wait_landed(uint32_t bar, uint32_t parity, 
         if (clock64() - t0 > cap) return false;
     return true;
 }
+// ---- pairs of blocks in a cluster (distributed shared memory) ----
+__device__ __forceinline__ uint32_t cluster_rank() { uint32_t r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+// the address in block `rank` of the cluster that corresponds to this block's shared-memory address
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, float v) { asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory"); }
+__device__ __forceinline__ void mbar_arrive_peer(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Bounded wait for arrivals of the other block, whose writes before them are visible afterwards.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long cap) {
+    const long long t0 = clock64();
+    while (true) {
+        for (int i = 0; i < 64; ++i) {
+            uint32_t ok;
+            asm volatile(
+                "{\n\t.reg .pred p;\n\t"
+                "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+                "selp.u32 %0, 1, 0, p;\n\t}"
+                : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+            if (ok) return true;
+        }
+        if (*abort_flag) return false;
+        if (clock64() - t0 > cap) {
+            *abort_flag = 1;
+            return false;
+        }
+    }
+}
 // OR of a predicate over the threads of named barrier `id` (every thread gets the result)
 __device__ __forceinline__ bool bar_or(int id, int threads, bool v) {
     uint32_t r;

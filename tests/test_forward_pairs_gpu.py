@@ -1,0 +1,88 @@
+"""The tensor-core forward on grids that leave SMs idle: pairs of blocks per query tile (each sweeps half of the keys), and
+the rows of grouped heads cut into tiles together.  Every sampled row is checked against the oracle's single-query routine
+over exactly its visible keys; tolerance as in the other bf16 parity tests on an fp32 output buffer."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2510_01450_b200 import binding as L, inputs
+from tests.gpu_util import dev, row_err, stream_ptr
+from tests.test_parity_gpu import TOL_BF16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("d,H,Hkv,n,nq,window,causal", [
+    (64, 4, 4, 900, 300, 0, True),         # pairs, a ragged last tile
+    (64, 8, 2, 700, 129, 0, True),         # packed rows of four heads: tiles that run over a head's end; pairs
+    (128, 8, 2, 1000, 200, 0, True),
+    (128, 4, 1, 1500, 257, 700, True),     # packed, window: a tile's first block comes from the next head's first row
+    (64, 2, 2, 1000, 1000, 0, False),      # non-causal pairs
+    (128, 6, 3, 600, 1, 0, True),          # one query per head: two rows in a tile
+    (64, 16, 4, 2000, 700, 0, True),       # packed tiles, more of them than half the SMs
+])
+def test_pairs_and_packed_rows(oracle, d, H, Hkv, n, nq, window, causal):
+    B = 2
+    w = inputs.CONFIGS[2].shrink(B=B, H=H, n=n, d=d, dv=d, seed=500 + d + n)
+    q, _, _ = inputs.make_prefill(w)
+    _, k, v = inputs.make_prefill(w.shrink(H=Hkv, seed=501 + n))
+    qc = np.ascontiguousarray(q[:, :, n - nq:]) * np.float32(2.0)          # (exact in bf16; weights further from uniform)
+    out = torch.full((B, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+    rho, stats = torch.empty_like(out), torch.empty((B, H, nq, 3), dtype=torch.float32, device="cuda")
+    iters = torch.full((B, H, nq), -7, dtype=torch.int32, device="cuda")
+    status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+    nbytes = L.lla_forward_workspace_bytes(B, H, n, d, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    for _ in range(2):
+        L.lla_forward_ex(dev(qc, "bf16"), dev(k, "bf16"), dev(v, "bf16"), out, B, H, n, d, d, w.scale, w.lam, causal=causal,
+                         out_dtype=L.LLA_F32, q_rows=nq, kv_heads=Hkv, window=window, rho=rho, stats=stats, iters=iters,
+                         device_status=status, workspace=ws, workspace_bytes=nbytes, stream=stream_ptr())
+    torch.cuda.synchronize()
+    assert status.cpu().numpy()[L.STATUS_TIMEOUT] == 0
+    assert (iters.cpu().numpy() >= -1).all()
+    got = out.cpu().numpy().astype(np.float64)
+    rows = np.unique(np.concatenate([np.arange(min(nq, 12)), np.random.default_rng(3).integers(0, nq, 40), [nq - 1]]))
+    lo = [max(0, n - nq + r + 1 - window) if causal and window else 0 for r in rows]
+    cnt = np.array([(n - nq + r + 1 if causal else n) - l for r, l in zip(rows, lo)], dtype=np.int32)
+    kk, vv = np.repeat(k, H // Hkv, axis=1), np.repeat(v, H // Hkv, axis=1)
+    for b in range(B):
+        kc = np.zeros((len(rows), H, cnt.max(), d), dtype=np.float32)
+        vc = np.zeros_like(kc)
+        for s, (l, c) in enumerate(zip(lo, cnt)):
+            kc[s, :, :c], vc[s, :, :c] = kk[b, :, l:l + c], vv[b, :, l:l + c]
+        ref = oracle.decode(np.ascontiguousarray(qc[b][:, rows].transpose(1, 0, 2)), kc, vc, cnt, w.scale, w.lam)
+        err = row_err(got[b][:, rows].transpose(1, 0, 2), ref)
+        assert np.isfinite(err).all() and err.max() <= TOL_BF16, (b, float(err.max()), int(err.argmax()))
+    # o = sum_j w_j (1 - z_j . rho) v_j / delta with the saved tensors, for one row of the last head
+    r = int(rows[len(rows) // 2])
+    l, c = lo[len(rows) // 2], int(cnt[len(rows) // 2])
+    qr, kr, vr = qc[1, -1, r].astype(np.float64), kk[1, -1, l:l + c].astype(np.float64), vv[1, -1, l:l + c].astype(np.float64)
+    m, om, dl = stats.cpu().numpy()[1, -1, r].astype(np.float64)
+    wt = np.exp(w.scale * kr @ qr - m)
+    assert abs(wt.sum() / om - 1) < 1e-4
+    o = (wt * (1 - (kr - qr) @ rho.cpu().numpy()[1, -1, r])) @ vr / dl
+    assert np.linalg.norm(o - got[1, -1, r]) <= 2e-3 * np.linalg.norm(o)
+
+
+def test_a_pair_whose_waits_run_out_leaves_cleanly():
+    """No copy is issued, so every wait expires; both blocks of every pair leave, are counted, and the next call is right."""
+    B, H, n, d, nq = 1, 2, 1200, 64, 256
+    w = inputs.CONFIGS[2].shrink(B=B, H=H, n=n, d=d, dv=d, seed=520)
+    q, k, v = inputs.make_prefill(w)
+    args = [dev(np.ascontiguousarray(q[:, :, n - nq:]), "bf16"), dev(k, "bf16"), dev(v, "bf16")]
+
+    def run(**kw):
+        out = torch.full((B, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+        status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+        L.lla_forward_ex(*args, out, B, H, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, q_rows=nq, device_status=status,
+                         stream=stream_ptr(), **kw)
+        torch.cuda.synchronize()
+        return out.cpu().numpy(), status.cpu().numpy()
+
+    good, st = run()
+    assert st[L.STATUS_TIMEOUT] == 0 and np.isfinite(good).all()
+    _, st = run(debug_wait_clocks=1 << 20, debug_flags=L.LLA_DEBUG_NO_LOADS)
+    assert st[L.STATUS_TIMEOUT] == 2 * B * H * (nq // 128)
+    again, st = run()
+    assert st[L.STATUS_TIMEOUT] == 0 and np.array_equal(good, again)
