@@ -172,7 +172,8 @@ __device__ __noinline__ bool sv_eliminate(const float* src, double inv, double r
 // largest of the parts' maxima; weight and maximum are still those of each part.  Called by threads 0 .. D - 1 of a block.
 template <int D, typename TOut>
 __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qrow, const float* __restrict__ src, int splits, float lambda_u,
-                                           int ridge_mode, TOut* __restrict__ orow, int* __restrict__ status, SolveSmem<D>& sm, double* prow) {
+                                           int ridge_mode, TOut* __restrict__ orow, int* __restrict__ status, SolveSmem<D>& sm, double* prow,
+                                           float* ms) {
     using C = SvCfg<D>;
     constexpr int PF = DtCfg<D>::REC, NW = C::NW;
     const int r = threadIdx.x, lane = r & 31, wp = r >> 5;
@@ -192,13 +193,18 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
     const double ar = (double)src[2 * D * D + r] * inv, cb = (double)src[2 * D * D + D + r] * inv;
     sm.a[r] = ar;
     sv_sync<D>();
-    // row r of the centred matrix (column r: M is symmetric up to fp32 rounding and the loads are coalesced)
+    // row r of the centred matrix (column r: M is symmetric up to fp32 rounding and the loads are coalesced).  ms: shared
+    // memory for the column as it is, which the residuals below read again (null: src is in shared memory itself)
+    const float* mcol = ms ? ms + r : src + r;
     uint64_t row[D / 2];
 #pragma unroll
     for (int j = 0; j < D; j += 8) {
         float v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = src[(j + e) * D + r];
+        for (int e = 0; e < 8; ++e) {
+            v[e] = src[(j + e) * D + r];
+            if (ms) ms[(j + e) * D + r] = v[e];
+        }
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
             double s0 = (double)v[e] * inv - sm.a[j + e] * ar, s1 = (double)v[e + 1] * inv - sm.a[j + e + 1] * ar;
@@ -267,10 +273,10 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
         sm.x[r] = x;
         sv_sync<D>();
         double s0 = 0.0, s1 = 0.0;
-#pragma unroll 4
+#pragma unroll 8
         for (int j = 0; j < D; j += 2) {
-            s0 += (double)src[j * D + r] * sm.x[j];
-            s1 += (double)src[(j + 1) * D + r] * sm.x[j + 1];
+            s0 += (double)mcol[j * D] * sm.x[j];
+            s1 += (double)mcol[(j + 1) * D] * sm.x[j + 1];
         }
         const double ax = sv_sum<D>(ar * x, sm);
         res = b - ((s0 + s1) * inv - ar * ax + ridge * x);
@@ -285,8 +291,8 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
     const double yv = done ? x : sm.x[r];
     const double ky = sv_sum<D>(ar * yv, sm);
     double o0 = 0.0, o1 = 0.0;
-#pragma unroll 8
-    for (int j = 0; j < D; j += 2) {
+#pragma unroll 32
+    for (int j = 0; j < D; j += 2) {      // (the matrix row's registers are free: 64 loads in flight)
         o0 += (double)src[D * D + j * D + r] * sm.x[j];
         o1 += (double)src[D * D + (j + 1) * D + r] * sm.x[j + 1];
     }
@@ -301,7 +307,7 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
 template <int D, typename TOut>
 __device__ __noinline__ void solve_here(const __nv_bfloat16* qrow, const float* rec, float lambda_u, int ridge_mode, TOut* orow,
                                         int* status, SolveSmem<D>& sm, double* prow) {
-    solve_unit<D>(qrow, rec, 1, lambda_u, ridge_mode, orow, status, sm, prow);
+    solve_unit<D>(qrow, rec, 1, lambda_u, ridge_mode, orow, status, sm, prow, nullptr);
 }
 
 struct DtParams {
@@ -870,6 +876,7 @@ __global__ void __launch_bounds__(D, D == 64 ? 8 : 2)
 decode_solve_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict__ parts, TOut* __restrict__ out,
                     const int* __restrict__ lens, int H, int Lmax, int head_rows, float lambda, int splits,
                     int* __restrict__ status, const float* __restrict__ lambda_units, int ridge_mode, int window) {
+    extern __shared__ __align__(16) float sv_mat[];      // D x D
     __shared__ SolveSmem<D> sm;
     __shared__ double prow[D + 1];
     const int bh = blockIdx.x;
@@ -877,7 +884,7 @@ decode_solve_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (visible_keys(lens[bh / H], Lmax, window) < head_rows) return;
     solve_unit<D>(q + (size_t)bh * D, parts + (size_t)bh * splits * DtCfg<D>::REC, splits, lambda_units ? lambda_units[bh] : lambda,
-                  ridge_mode, out + (size_t)bh * D, status, sm, prow);
+                  ridge_mode, out + (size_t)bh * D, status, sm, prow, sv_mat);
 }
 
 template <int D, typename TOut>
@@ -932,6 +939,9 @@ int launch_t(const DecodeArgs& a) {
         cudaLaunchConfig_t cs = {};
         cs.gridDim = dim3(BH);
         cs.blockDim = dim3(D);
+        cs.dynamicSmemBytes = sizeof(float) * D * D;
+        LLA_CUDA_TRY(cudaFuncSetAttribute(decode_solve_kernel<D, TOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cs.dynamicSmemBytes));
+        LLA_CUDA_TRY(cudaFuncSetAttribute(decode_solve_kernel<D, TOut>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
         cs.stream = a.stream;
         cs.attrs = attr;
         cs.numAttrs = 1;
