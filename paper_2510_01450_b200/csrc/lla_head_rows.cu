@@ -1,13 +1,14 @@
-// Direct fp64 solve for the rows that see only a few keys.
+// Direct fp64 solve of the decode units that see only a few keys.
 //
-// For a row with L visible keys and L < head_rows (default 2d) the system Sigma_i rho_i = mu_i of
-// Eq. "query_specific" has condition numbers of 1e4..1e5 at the paper's ridge sizes (Sigma_i is
-// low rank plus lambda*I while L < d).  fp32 conjugate gradients cannot resolve that, so these few
-// rows are computed exactly as Section 2.3 writes them: explicit moments, an LDL^T factorisation
-// of the d x d matrix in shared memory, and the intercept of Eq. "lla".  They are 2d/n of the
-// rows and about (2d/n)^2 of the pair work.
+// For a unit with L < head_rows = 2d visible keys the system Sigma rho = mu of Eq. "query_specific" has condition
+// numbers of 1e4..1e5 at the paper's ridge sizes (Sigma is low rank plus lambda*I while L < d), which fp32 arithmetic
+// cannot resolve, so the unit is computed exactly as Section 2.3 writes it: explicit moments, an LDL^T factorisation
+// of the d x d matrix in shared memory, and the intercept of Eq. "lla".  A unit is one row, so nothing is shared
+// between blocks (the forward's direct rows share Gram products between the rows of a head: lla_direct_rows.cu), and
+// what bounds the kernel is the chain of the factorisation; for longer caches it returns at once, and the streaming
+// kernel behind it starts without waiting for it.
 //
-// One thread block per (batch*head, row).  All arithmetic is double precision.
+// One thread block per (sequence, head).  All arithmetic is double precision.
 #include "lla_common.cuh"
 
 namespace lla {
@@ -92,17 +93,13 @@ __device__ __forceinline__ void load2(const float* p, float& a, float& b) {
     b = f.y;
 }
 
-template <int D, int DV, typename TIn, typename TOut>
+template <int D, typename TIn, typename TOut>
 __global__ void __launch_bounds__(HrCfg<D>::THREADS, HrCfg<D>::BLOCKS_PER_SM)
 head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn* __restrict__ v,
-                 TOut* __restrict__ out, int n, int rows_per_head, int causal, double scale,
-                 double lambda, int lcap, float* __restrict__ rho_out, float* __restrict__ stats,
-                 int* __restrict__ iters, int* __restrict__ status, const int* __restrict__ lens, int H,
-                 const float* __restrict__ lambda_rows, int ridge_mode, int nq, int kv_group,
-                 const PagedKv paged, int window, const Strides sq, const Strides sk, const Strides sv, const Strides so) {
-    // Prefill (lens == nullptr): block (i, bh) solves row i of head bh; n is the sequence length.
-    // Decode (lens != nullptr): block (0, bh) solves the single query of (sequence, head) bh over
-    // lens[bh / H] cached keys, but only when that is at most lcap; n is the cache stride Lmax.
+                 TOut* __restrict__ out, int Lmax, double scale, double lambda, int lcap, int* __restrict__ status,
+                 const int* __restrict__ lens, int H, const float* __restrict__ lambda_units, int ridge_mode, int kv_group,
+                 const PagedKv paged, int window) {
+    // Block bh solves the single query of (sequence, head) bh over its visible keys when they are at most lcap.
     using C = HrCfg<D>;
     constexpr int HR_THREADS = C::THREADS;
     extern __shared__ __align__(16) double smem[];
@@ -114,31 +111,20 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
     double* zc = S;                         // HR_CHUNK * D  centred keys of the current chunk (over S)
 
     const int tid = threadIdx.x;
-    // decode: the streaming kernel launched behind this one as its programmatic dependent need not wait for it
-    if (lens) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // blockIdx.x (fastest in launch order) is the head, blockIdx.y counts rows from the last one down:
-    // rows with the most keys are the longest blocks and start first, so the tail of the launch is short
-    const int bh = blockIdx.x;
-    const int i = rows_per_head - 1 - blockIdx.y;   // row index inside the head
-    if (i >= rows_per_head) return;
-    int L = causal ? (n - nq) + i + 1 : n;    // query row i sits at position n - nq + i
-    if (lens) {
-        L = visible_keys(lens[bh / H], n, window);
-        if (L > lcap) return;               // long caches go through the moment kernel
-    }
-    const size_t row = lens ? (size_t)bh : (size_t)bh * nq + i;      // row of the contiguous per-row outputs (rho, stats, ...)
-    // (debug build: the keys must fit the shared-memory arrays sized for lcap, the row the per-row outputs)
-    if (!LLA_IN_BOUNDS(L, lcap + 1, status, 201) || !LLA_IN_BOUNDS(row, (size_t)gridDim.x * (lens ? 1 : nq), status, 202)) return;
-    // prefill: q, k, v and out are addressed through their strides; decode keeps its contiguous / paged layout
-    const TIn* qrow = lens ? q + row * D : q + sq.at(bh / H, bh % H, i);
-    // (decode over a paged cache: the at most lcap <= page_size keys of a directly-solved unit sit in its first page)
-    const int kstart = lens ? first_visible_key(lens[bh / H], n, window) : 0;      // sliding-window decode
-    const size_t kvrow = kv_row(paged, bh / H, (bh % H) / max(kv_group, 1), H / max(kv_group, 1), n, kstart);
-    const int hk = (bh % H) / max(kv_group, 1);
-    const TIn* kb = lens ? k + kvrow * D : k + sk.at(bh / H, hk, 0);
-    const TIn* vb = lens ? v + kvrow * DV : v + sv.at(bh / H, hk, 0);
-    const size_t krs = lens ? (size_t)D : (size_t)sk.r, vrs = lens ? (size_t)DV : (size_t)sv.r;      // row strides of k and v
-    TOut* orow = lens ? out + row * DV : out + so.at(bh / H, bh % H, i);
+    // the streaming kernel launched behind this one as its programmatic dependent need not wait for it
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int bh = blockIdx.x, b = bh / H;
+    const int L = visible_keys(lens[b], Lmax, window);
+    if (L > lcap) return;                   // long caches go through the moment kernel
+    // (debug build: the keys must fit the shared-memory arrays sized for lcap)
+    if (!LLA_IN_BOUNDS(L, lcap + 1, status, 201)) return;
+    const TIn* qrow = q + (size_t)bh * D;
+    TOut* orow = out + (size_t)bh * D;
+    const int kstart = first_visible_key(lens[b], Lmax, window);       // sliding window
+    const int hk = (bh % H) / kv_group, hkv = H / kv_group;
+    // the unit's keys lie in one run of rows, except that those of a paged cache may take several pages
+    const size_t row0 = kv_row(paged, b, hk, hkv, Lmax, kstart);
+    auto key_row = [&](int j) { return (paged.table ? kv_row(paged, b, hk, hkv, Lmax, kstart + j) : row0 + j) * D; };
 
     for (int c = tid; c < D; c += HR_THREADS) qd[c] = (double)to_f32(qrow[c]);
     __syncthreads();
@@ -146,7 +132,7 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
     // scores, their maximum, weights exp(s - m), ridge lambda * exp(-m)
     double lmax = -INFINITY;
     for (int j = tid; j < L; j += HR_THREADS) {
-        const double s = dot_row<D>(qd, kb + (size_t)j * krs) * scale;
+        const double s = dot_row<D>(qd, k + key_row(j)) * scale;
         w[j] = s;
         lmax = fmax(lmax, s);
     }
@@ -158,8 +144,8 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
         lsum += e;
     }
     const double omega = block_reduce<HR_THREADS>(lsum, false, red);
-    // per-row ridge if given (prefill: [B,H,n]; decode: [B,H]); see lla_ridge_mode for the two frames
-    const double lam_i = lambda_rows ? (double)lambda_rows[row] : lambda;
+    // per-unit ridge if given ([B, H]); see lla_ridge_mode for the two frames
+    const double lam_i = lambda_units ? (double)lambda_units[bh] : lambda;
     const double lambda_m = ridge_mode == LLA_RIDGE_PRINTED ? lam_i : lam_i * exp(-m);
 
     // Rows with at most d keys (and a positive ridge) go through the dual (Gram) form: with Z the
@@ -167,7 +153,7 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
     // (Z Z^T + lambda' diag(1/w)) alpha = 1  --  an L x L system instead of d x d, free of the
     // cancellation in 1 - z . rho, and rho = Z^T alpha.  The system is padded to a multiple of 8 with
     // identity rows.
-    double csum = 0.0, rho_val = 0.0;
+    double csum = 0.0;
     bool bad = false;
     const bool dual = L <= D && lambda_m > 0.0;          // block-uniform
     const int Lp = (L + 7) & ~7;                         // dual: system size padded to the panel width
@@ -197,7 +183,7 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
         double* zt = S;                                   // zt[c * LZ + j] = k_j[c] - q[c]  (over S: D * LZ <= S_DOUBLES)
         for (int e = tid; e < Lp * D; e += HR_THREADS) {
             const int j = e / D, c = e - j * D;
-            zt[c * LZ + j] = j < L ? (double)to_f32(kb[(size_t)j * krs + c]) - qd[c] : 0.0;
+            zt[c * LZ + j] = j < L ? (double)to_f32(k[key_row(j) + c]) - qd[c] : 0.0;
         }
         __syncthreads();
         // Gram matrix
@@ -241,11 +227,6 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
             w[j] = cj;
             csum += cj;
         }
-        if (rho_out && tid < D) {                         // rho = Z^T alpha
-            double acc_r = 0.0;
-            for (int j = 0; j < L; ++j) acc_r += rhs[j] * ((double)to_f32(kb[(size_t)j * krs + tid]) - qd[tid]);
-            rho_val = acc_r;
-        }
     } else {
         // moments: Sigma and mu
         double mu_acc = 0.0;  // thread tid < D owns mu[tid]
@@ -255,17 +236,17 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
         float pre[PAIRS][2];
         auto fetch = [&](int j0) {
             const int np = min(HR_CHUNK, L - j0) * (D / 2);
-    #pragma unroll
+#pragma unroll
             for (int u = 0; u < PAIRS; ++u) {
                 const int pi = tid + HR_THREADS * u;
-                if (pi < np) load2(kb + (size_t)(j0 + (2 * pi) / D) * krs + (2 * pi) % D, pre[u][0], pre[u][1]);
+                if (pi < np) load2(k + key_row(j0 + (2 * pi) / D) + (2 * pi) % D, pre[u][0], pre[u][1]);
             }
         };
         fetch(0);
         for (int j0 = 0; j0 < L; j0 += HR_CHUNK) {
             const int jn = min(HR_CHUNK, L - j0);
             __syncthreads();
-    #pragma unroll
+#pragma unroll
             for (int u = 0; u < PAIRS; ++u) {
                 const int pi = tid + HR_THREADS * u;
                 if (pi < jn * (D / 2)) {
@@ -277,7 +258,7 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
             if (j0 + HR_CHUNK < L) fetch(j0 + HR_CHUNK);
             if (tid < D)
                 for (int jj = 0; jj < jn; ++jj) mu_acc += w[j0 + jj] * zc[jj * D + tid];
-    #pragma unroll
+#pragma unroll
             for (int t = 0; t < C::TILES_PER_THREAD; ++t) {
                 if (tr[t] < 0) continue;
                 // interleaved 4x4 tile: rows tr + T1*a, columns tc + T1*b, so that neighbouring threads
@@ -286,25 +267,25 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
                 for (int jj = 0; jj < jn; ++jj) {
                     const double wj = w[j0 + jj];
                     double zr[4], zcv[4];
-    #pragma unroll
+#pragma unroll
                     for (int a = 0; a < 4; ++a) {
                         zr[a] = wj * zc[jj * D + r0 + C::TILES_1D * a];
                         zcv[a] = zc[jj * D + c0 + C::TILES_1D * a];
                     }
-    #pragma unroll
+#pragma unroll
                     for (int a = 0; a < 4; ++a)
-    #pragma unroll
+#pragma unroll
                         for (int b = 0; b < 4; ++b) acc[t][a][b] += zr[a] * zcv[b];
                 }
             }
         }
         __syncthreads();   // the staged keys (lying over S) are no longer read
-    #pragma unroll
+#pragma unroll
         for (int t = 0; t < C::TILES_PER_THREAD; ++t) {
             if (tr[t] < 0) continue;
-    #pragma unroll
+#pragma unroll
             for (int a = 0; a < 4; ++a)
-    #pragma unroll
+#pragma unroll
                 for (int b = 0; b < 4; ++b) {
                     const int r = tr[t] + C::TILES_1D * a, c = tc[t] + C::TILES_1D * b;
                     if (c <= r) S[r * C::LDS + c] = acc[t][a][b] + (r == c ? lambda_m : 0.0);
@@ -321,43 +302,31 @@ head_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const TIn
         double qrho = 0.0;
         for (int c = 0; c < D; ++c) qrho += qd[c] * rhs[c];
         for (int j = tid; j < L; j += HR_THREADS) {
-            const double t = dot_row<D>(rhs, kb + (size_t)j * krs) - qrho;
+            const double t = dot_row<D>(rhs, k + key_row(j)) - qrho;
             const double cj = w[j] * (1.0 - t);
             w[j] = cj;
             csum += cj;
         }
-        if (tid < D) rho_val = rhs[tid];
     }
     const double denom = block_reduce<HR_THREADS>(csum, false, red);
-    for (int c = tid; c < DV; c += HR_THREADS) {
+    for (int c = tid; c < D; c += HR_THREADS) {
         double o = 0.0;
-        for (int j = 0; j < L; ++j) o += w[j] * (double)to_f32(vb[(size_t)j * vrs + c]);
+        for (int j = 0; j < L; ++j) o += w[j] * (double)to_f32(v[key_row(j) + c]);
         store_out(orow + c, (float)(o / denom));
     }
-    if (rho_out && tid < D) rho_out[row * D + tid] = (float)rho_val;
-    if (tid == 0) {
-        if (stats) {
-            stats[row * 3 + 0] = (float)m;
-            stats[row * 3 + 1] = (float)omega;
-            stats[row * 3 + 2] = (float)denom;
-        }
-        if (iters) iters[row] = -1;
-        if (bad && status) atomicAdd(status + LLA_STATUS_BAD_PIVOT, 1);
-    }
+    if (tid == 0 && bad && status) atomicAdd(status + LLA_STATUS_BAD_PIVOT, 1);
 }
 
 template <int D, typename TIn, typename TOut>
 int launch_decode_t(const DecodeArgs& a, int lcap) {
     using C = HrCfg<D>;
     const size_t smem = sizeof(double) * C::smem_doubles(lcap);
-    auto kern = head_rows_kernel<D, D, TIn, TOut>;
+    auto kern = head_rows_kernel<D, TIn, TOut>;
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-    dim3 grid(a.B * a.H, 1);
-    kern<<<grid, C::THREADS, smem, a.stream>>>(
-        (const TIn*)a.q, (const TIn*)a.kcache, (const TIn*)a.vcache, (TOut*)a.out, a.Lmax, 1, 0,
-        (double)a.scale, (double)a.lambda, lcap, nullptr, nullptr, nullptr, a.status, a.lens, a.H, a.lambda_units,
-        a.ridge_mode, 1, a.kv_group, a.paged, a.window, Strides{0, 0, 0}, Strides{0, 0, 0}, Strides{0, 0, 0}, Strides{0, 0, 0});
+    kern<<<a.B * a.H, C::THREADS, smem, a.stream>>>((const TIn*)a.q, (const TIn*)a.kcache, (const TIn*)a.vcache, (TOut*)a.out, a.Lmax,
+                                                    (double)a.scale, (double)a.lambda, lcap, a.status, a.lens, a.H, a.lambda_units,
+                                                    a.ridge_mode, a.kv_group > 0 ? a.kv_group : 1, a.paged, a.window);
     LLA_CUDA_TRY(cudaGetLastError());
     return LLA_OK;
 }

@@ -13,16 +13,17 @@ from tests.test_parity_gpu import TOL_BF16, _to_pages
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("d,mode,splits", [(64, "plain", 1), (64, "late_max", 1), (64, "late_max", 2), (64, "short", 1), (128, "plain", 1),
-                                           (128, "plain", 3), (128, "late_max", 1), (128, "late_max", 2), (128, "short", 1),
-                                           (128, "paged_gqa", 1), (128, "paged_gqa", 2), (128, "window", 1)])
+@pytest.mark.parametrize("d,mode,splits", [(64, "plain", 1), (64, "late_max", 1), (64, "late_max", 2), (64, "short", 1), (64, "plain", 12),
+                                           (128, "plain", 1), (128, "plain", 3), (128, "plain", 12), (128, "late_max", 1),
+                                           (128, "late_max", 2), (128, "short", 1), (128, "paged_gqa", 1), (128, "paged_gqa", 2),
+                                           (128, "paged_gqa_short", 1), (128, "window", 1)])
 def test_tile_edges_and_options(oracle, d, mode, splits):
-    H, Hkv = 4, 2 if mode == "paged_gqa" else 4
+    H, Hkv = 4, 2 if mode.startswith("paged_gqa") else 4
     w = inputs.CONFIGS[5].shrink(B=6, H=H, n=1100, d=d, dv=d, len_min=10, len_max=1100, seed=400 + d)
     q, _, _, _ = inputs.make_decode(w)
     _, kc, vc, _ = inputs.make_decode(w.shrink(H=Hkv))
     lens = np.array([2 * d, 2 * d + 1, 319, 384, 385, 1100], dtype=np.int32)
-    if mode == "short":
+    if mode.endswith("short"):
         lens[:3] = [1, 17, 2 * d - 1]           # solved directly
     kw = {}
     if mode == "late_max":
@@ -42,7 +43,7 @@ def test_tile_edges_and_options(oracle, d, mode, splits):
     for b in range(w.B):                      # slots past the end may hold anything
         kc[b, :, lens[b]:] = np.nan
         vc[b, :, lens[b]:] = np.nan
-    if mode == "paged_gqa":
+    if mode.startswith("paged_gqa"):         # pages of 128 keys: the directly solved 2 d - 1 keys take two of them at d = 128
         kc, table, max_pages, num_pages = _to_pages(kc, lens, 128, np.random.default_rng(401))
         vc, _, _, _ = _to_pages(vc, lens, 128, np.random.default_rng(401))
         kw.update(kv_heads=Hkv, block_table=torch.from_numpy(table).cuda(), page_size=128, max_pages=max_pages, num_pages=num_pages)
