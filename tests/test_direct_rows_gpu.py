@@ -1,0 +1,74 @@
+"""The fp64 direct rows at the edges of their chunks of keys, of the rows of a block and of the two forms of the system:
+every row of a problem with fp32 inputs or d = 16, and the short rows of the backward.  Each forward row is checked against
+the oracle's single-query routine over exactly its visible keys."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2510_01450_b200 import binding as L, inputs
+from tests.gpu_util import LLA_DT, dev, row_err, stream_ptr
+from tests.test_backward_gpu import TOL, grad_err, run_backward
+from tests.test_parity_gpu import TOL_BF16, TOL_F32
+
+pytestmark = pytest.mark.gpu
+
+
+# n around the chunk (64 keys at d = 16, 72 at 64, 136 / 64 at 128), one row, rows that do not fill a block's teams
+@pytest.mark.parametrize("dtype,d,n,nq,H,Hkv,window,causal,mode", [
+    ("f32", 16, 1, 1, 1, 1, 0, True, ""), ("f32", 16, 64, 64, 2, 2, 0, True, ""), ("f32", 16, 65, 65, 3, 1, 0, True, ""),
+    ("bf16", 16, 131, 70, 2, 1, 0, True, ""), ("f32", 16, 193, 193, 1, 1, 40, True, ""), ("f32", 16, 97, 30, 2, 2, 0, False, ""),
+    ("f32", 64, 72, 72, 2, 2, 0, True, ""), ("f32", 64, 73, 73, 1, 1, 0, True, ""), ("f32", 64, 217, 75, 4, 2, 0, True, ""),
+    ("f32", 64, 300, 300, 1, 1, 131, True, ""), ("f32", 64, 145, 9, 2, 1, 0, False, ""), ("f32", 64, 310, 40, 2, 2, 0, True, "late_max"),
+    ("f32", 64, 64, 33, 1, 1, 0, False, ""), ("f32", 128, 137, 137, 1, 1, 0, True, ""), ("f32", 128, 300, 70, 2, 1, 0, True, "late_max"),
+    ("f32", 128, 129, 3, 2, 2, 0, False, ""), ("f32", 128, 300, 45, 1, 1, 256, True, "")])
+def test_every_row_direct(oracle, dtype, d, n, nq, H, Hkv, window, causal, mode):
+    B = 2
+    w = inputs.CONFIGS[2].shrink(B=B, H=H, n=n, d=d, dv=d, dtype=dtype, seed=700 + d + n)
+    q, _, _ = inputs.make_prefill(w)
+    _, k, v = inputs.make_prefill(w.shrink(H=Hkv, seed=701 + n))
+    qc = np.ascontiguousarray(q[:, :, n - nq:])
+    if mode == "late_max":       # the first 100 keys score about e^-700 below the rest: the reference of the weights moves
+        u = np.ones(d, dtype=np.float32) / np.sqrt(d)
+        qc = qc - (qc @ u)[..., None] * u + 4 * u
+        k = k - (k @ u)[..., None] * u
+        k[:, :, :100] -= (175.0 / w.scale) * u
+    rnd = inputs.round_to_bf16 if dtype == "bf16" else (lambda x: x.astype(np.float32))
+    qc, k, v = rnd(qc), rnd(k), rnd(v)
+    out = torch.full((B, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+    status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+    iters = torch.full((B, H, nq), -7, dtype=torch.int32, device="cuda")
+    L.lla_forward_ex(dev(qc, dtype), dev(k, dtype), dev(v, dtype), out, B, H, n, d, d, w.scale, w.lam, causal=causal,
+                     in_dtype=LLA_DT[dtype], out_dtype=L.LLA_F32, q_rows=nq, kv_heads=Hkv, window=window, iters=iters,
+                     device_status=status, stream=stream_ptr())
+    torch.cuda.synchronize()
+    assert status.cpu().numpy()[L.STATUS_BAD_PIVOT] == 0
+    it = iters.cpu().numpy()
+    seen = np.array([n - nq + r + 1 if causal else n for r in range(nq)])
+    head_rows = 2 * d if dtype == "f32" else d + d // 2
+    assert (it == np.where(seen < head_rows, -1, 0)).all()
+    kk, vv = np.repeat(k, H // Hkv, axis=1), np.repeat(v, H // Hkv, axis=1)
+    lo = np.maximum(0, seen - window) if causal and window else np.zeros(nq, dtype=int)
+    cnt = (seen - lo).astype(np.int32)
+    for b in range(B):
+        kc = np.zeros((nq, H, cnt.max(), d), dtype=np.float32)
+        vc = np.zeros_like(kc)
+        for r in range(nq):
+            kc[r, :, :cnt[r]], vc[r, :, :cnt[r]] = kk[b, :, lo[r]:seen[r]], vv[b, :, lo[r]:seen[r]]
+        ref = oracle.decode(np.ascontiguousarray(qc[b].transpose(1, 0, 2)), kc, vc, cnt, w.scale, w.lam)
+        err = row_err(out.cpu().numpy()[b].transpose(1, 0, 2), ref)
+        assert np.isfinite(err).all() and err.max() <= (TOL_F32 if dtype == "f32" else TOL_BF16), (b, float(err.max()), int(err.argmax()))
+
+
+# lengths at which every row is direct (up to 1.5 d - 1 keys) or nearly, and which leave part of a block's rows empty
+@pytest.mark.parametrize("d,n,H", [(64, 2, 1), (64, 5, 3), (64, 64, 1), (64, 65, 2), (64, 95, 1), (64, 97, 2), (128, 3, 1),
+                                   (128, 128, 2), (128, 130, 1), (128, 191, 1), (128, 193, 1)])
+def test_backward_short_rows(backward_oracle, d, n, H):
+    w = inputs.CONFIGS[2].shrink(B=1, H=H, n=n, d=d, dv=d, seed=800 + d + n)
+    q, k, v = inputs.make_prefill(w)
+    g = inputs.make_upstream_grad(w)
+    ref = backward_oracle.backward(q, k, v, g, w.scale, w.lam)
+    for name, a, b in zip(("dq", "dk", "dv"), run_backward(w, q, k, v, g), ref):
+        assert np.isfinite(a).all(), name
+        err = grad_err(a, b)
+        assert err.max() <= TOL, (name, float(err.max()), int(err.argmax()))
