@@ -45,7 +45,7 @@ using namespace sm100;
 constexpr int TC_BR = 128;           // query rows per block (TMEM lanes)
 constexpr int TC_BC = 64;            // keys per block
 constexpr int TC_COMPUTE = 256;      // compute threads (warps 0..7)
-constexpr int TC_THREADS = 352;      // + TMA warp + two MMA warps (d = 128: 384, with an idle warp that completes the third warpgroup)
+constexpr int TC_THREADS = 384;      // + TMA warp + two MMA warps + an idle warp that completes the third warpgroup
 constexpr int TC_TMEM_COLS = 512;
 constexpr int TC_NBUF = 3;           // S/A/U buffers in TMEM (128 columns each)
 constexpr int TC_ACC_COL = TC_NBUF * 128;   // ACC columns [384, 384 + D)
@@ -61,9 +61,10 @@ enum SweepKind : int { SW_STATS = 1, SW_CG = 2, SW_OUT = 3, SW_DONE = 4, SW_CG16
 
 // Shared-memory carve-up (bytes, from a 1024-byte aligned base), per head size D (64 or 128).
 // Operand tiles are stored as D/64 sub-tiles of 64 columns (128-byte rows, 128B swizzle) one after
-// the other.  For D = 64 the row vectors x and kbar live in shared memory as fp32 [D][128]; for
-// D = 128 there is no room for them, so x, kbar and r live in an L2-resident global scratch slot
-// owned by the SM (one block per SM at a time) and the ring has three stages.
+// the other.  For D = 64 the row vectors x and r live in the compute threads' registers and kbar in shared memory as
+// fp32 [D][128] (x in shared memory as well: 96 shared-memory accesses a thread between two sweeps, when nothing else
+// runs on the SM, 2.8 K clocks there instead of 1.9 K); for D = 128 there is no room for any of them, so x, kbar and r
+// live in an L2-resident global scratch slot owned by the SM (one block per SM at a time) and the ring has three stages.
 template <int D>
 struct TcCfg {
     static constexpr int KSUB = D / 64;                         // 64-column sub-tiles per operand row
@@ -74,14 +75,13 @@ struct TcCfg {
     static constexpr int OPER_BYTES = KSUB * QSUB_BYTES;        // Q, P_hi, P_lo
     static constexpr int KBLK_BYTES = KSUB * KSUB_BYTES;        // K block (V block follows it)
     static constexpr int STAGE_BYTES = 2 * KBLK_BYTES;
-    static constexpr bool STATE_IN_SMEM = D == 64;
+    static constexpr bool STATE_IN_REGS = D == 64;
     static constexpr int SM_Q = 0;
     static constexpr int SM_PHI = SM_Q + OPER_BYTES;
     static constexpr int SM_PLO = SM_PHI + OPER_BYTES;
     static constexpr int SM_KV = SM_PLO + OPER_BYTES;
-    static constexpr int SM_X = SM_KV + NST * STAGE_BYTES;                        // fp32 [D][128] (D = 64 only)
-    static constexpr int SM_KBAR = SM_X + (STATE_IN_SMEM ? D * TC_BR * 4 : 0);
-    static constexpr int SM_RED = SM_KBAR + (STATE_IN_SMEM ? D * TC_BR * 4 : 0);  // pair reductions: 2 buffers x 4 values x 2 x 128 floats
+    static constexpr int SM_KBAR = SM_KV + NST * STAGE_BYTES;                     // fp32 [D][128] (D = 64 only)
+    static constexpr int SM_RED = SM_KBAR + (STATE_IN_REGS ? D * TC_BR * 4 : 0);  // pair reductions: 2 buffers x 4 values x 2 x 128 floats
     static constexpr int SM_FLAGS = SM_RED + 8192;                                // 2 x 8 ints
     static constexpr int SM_BAR = SM_FLAGS + 64;                                  // mbarriers
     static constexpr int SM_MISC = SM_BAR + 256;                                  // tmem base, ctl kind, abort
@@ -90,7 +90,7 @@ struct TcCfg {
     static constexpr int SM_ALLOC = SM_TOTAL + 1024;                              // slack for 1024-byte alignment
     static constexpr uint32_t IDESC_TS = sm100::make_idesc(TC_BR, D, 0, 1);   // ACC: A from TMEM, B MN-major, N = D
     static constexpr uint32_t IDESC_TS16 = sm100::make_idesc(TC_BR, D, 0, 1, /*f16=*/1);   // same, both operands fp16
-    static constexpr size_t SCRATCH_FLOATS_PER_SM = STATE_IN_SMEM ? 0 : 3 * (size_t)D * TC_BR;   // x, kbar, r
+    static constexpr size_t SCRATCH_FLOATS_PER_SM = STATE_IN_REGS ? 0 : 3 * (size_t)D * TC_BR;   // x, kbar, r
 };
 static_assert(TcCfg<64>::SM_ALLOC <= 227 * 1024 && TcCfg<128>::SM_ALLOC <= 227 * 1024, "shared memory budget");
 
@@ -147,7 +147,7 @@ struct TcParams {
 // which nothing reads between two sweeps) and carry on with the same numbers.  For grids that leave much of the chip
 // idle; see launch_t.
 template <int D, typename TOut, bool PC, bool GIVEN = false, int NS = 1>
-__global__ void __launch_bounds__(D == 128 ? 384 : TC_THREADS, 1)
+__global__ void __launch_bounds__(TC_THREADS, 1)
 forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK16,
                   const __grid_constant__ CUtensorMap tmM, TOut* __restrict__ out, const TcParams prm) {
@@ -164,12 +164,9 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     auto bar = [&](int i) { return bars + 8u * i; };
     volatile int* misc = reinterpret_cast<volatile int*>(smem + SM_MISC);   // [0] tmem base, [2] abort, [3] kv unit, [4..5] kind
     volatile int* abort_flag = misc + 2;
-    // row-vector state: shared memory (D = 64) or this SM's slot of the global scratch (D = 128)
-    float* xs;
-    float* kbs;
-    float* rs = nullptr;
-    if constexpr (Cfg::STATE_IN_SMEM) {
-        xs = reinterpret_cast<float*>(smem + Cfg::SM_X);
+    // row-vector state x, r and kbar: registers and shared memory (D = 64), or this SM's slot of the global scratch (D = 128)
+    float *xs = nullptr, *kbs, *rs = nullptr;
+    if constexpr (Cfg::STATE_IN_REGS) {
         kbs = reinterpret_cast<float*>(smem + Cfg::SM_KBAR);
     } else {
         uint32_t smid;
@@ -257,6 +254,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         misc[4] = SW_STATS;
         misc[5] = SW_STATS;
         misc[2] = 0;
+        misc[8] = misc[9] = 0;
         fence_barrier_init();
     }
     if (warp == 8) {   // TMEM allocation by one full warp; the base address lands in shared memory
@@ -272,8 +270,8 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 
     // Register hand-over between the warpgroups: the copy- and MMA-issuing warps need few registers and give theirs
     // up, the compute warps take them (168 a thread at launch, the most that twelve warps can have).
-    auto regs_give = [&]() { if constexpr (D == 128) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;" ::: "memory"); };
-    auto regs_take = [&]() { if constexpr (D == 128) asm volatile("setmaxnreg.inc.sync.aligned.u32 216;" ::: "memory"); };
+    auto regs_give = [&]() { asm volatile("setmaxnreg.dec.sync.aligned.u32 64;" ::: "memory"); };
+    auto regs_take = [&]() { asm volatile("setmaxnreg.inc.sync.aligned.u32 216;" ::: "memory"); };
 
     if (warp == 8) {
         regs_give();
@@ -740,14 +738,22 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (lane == 0) mbar_arrive(bar(B_CTL));
         };
 
-        // residual r: registers for D = 64, the scratch slot for D = 128 (no registers to spare)
-        float r[Cfg::STATE_IN_SMEM ? NCOL : 1] = {}, p[NCOL];
+        // x and the residual r: registers for D = 64, the scratch slot for D = 128 (no registers to spare)
+        float x[Cfg::STATE_IN_REGS ? NCOL : 1] = {}, r[Cfg::STATE_IN_REGS ? NCOL : 1] = {}, p[NCOL];
+        auto x_get = [&](int e) -> float {
+            if constexpr (Cfg::STATE_IN_REGS) return x[e];
+            else return xs[(c0 + e) * TC_BR + lrow];
+        };
+        auto x_set = [&](int e, float v) {
+            if constexpr (Cfg::STATE_IN_REGS) x[e] = v;
+            else xs[(c0 + e) * TC_BR + lrow] = v;
+        };
         auto r_get = [&](int e) -> float {
-            if constexpr (Cfg::STATE_IN_SMEM) return r[e];
+            if constexpr (Cfg::STATE_IN_REGS) return r[e];
             else return rs[(c0 + e) * TC_BR + lrow];
         };
         auto r_set = [&](int e, float v) {
-            if constexpr (Cfg::STATE_IN_SMEM) r[e] = v;
+            if constexpr (Cfg::STATE_IN_REGS) r[e] = v;
             else rs[(c0 + e) * TC_BR + lrow] = v;
         };
         float rr = 0.f, stop = 0.f;
@@ -881,7 +887,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         const int col = ch * 8 + e;
                         const float kb = acc[col] * inv_omega;
                         kbs[(c0 + col) * TC_BR + lrow] = kb;
-                        xs[(c0 + col) * TC_BR + lrow] = 0.f;
+                        x_set(col, 0.f);
                         const float bv = !row_ok ? 0.f : prm.rhs ? prm.rhs[((size_t)bh * nq + row) * D + c0 + col] : kb - qv;
                         r_set(col, bv);
                         p[col] = bv;
@@ -922,17 +928,29 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
         }
         if (ok) write_p(0);
+        // One barrier for two questions: does any row go on, and did every thread's waits succeed (a thread that gave
+        // up leaves a mark before the barrier; two marks in turn, so that none is set while the last is still read)
+        uint32_t votes = 0;
+        auto go_on = [&](bool act) {
+            const int slot = 8 + (votes++ & 1);
+            if (!ok) misc[slot] = 1;
+            const bool any = group_any(act);
+            if (misc[slot]) ok = false;
+            return any && ok;
+        };
         // ---- conjugate gradients (Algorithm 2) ----
         int t = 0;      // CG sweeps run
         for (; ok && t < prm.max_iters; ++t) {
             active = active && rr > stop;
-            if (!group_any(active)) break;
+            if (!go_on(active)) break;
             const bool cheap = f16_on && t >= precise;
             start_sweep(cheap ? SW_CG16 : SW_CG, cheap);
             sweep(cheap ? SW_CG16 : SW_CG);
             if (ok) acc_wait();
-            ok = all_ok(ok);
-            if (!ok) break;
+            if (PC) {
+                ok = all_ok(ok);
+                if (!ok) break;
+            }
             float ap[NCOL];
             acc_load(ap);
             if (NS > 1) {
@@ -958,7 +976,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 float xv[8], kv[8], rv[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    xv[i] = xs[(c0 + e0 + i) * TC_BR + lrow];
+                    xv[i] = x_get(e0 + i);
                     kv[i] = kbs[(c0 + e0 + i) * TC_BR + lrow];
                     rv[i] = r_get(e0 + i);
                 }
@@ -972,7 +990,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    xs[(c0 + e0 + i) * TC_BR + lrow] = xv[i];
+                    x_set(e0 + i, xv[i]);
                     r_set(e0 + i, rv[i]);
                 }
             }
@@ -1045,7 +1063,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (rank == 0 && row_ok && LLA_IN_BOUNDS((size_t)bh * nq + row, (size_t)(gridDim.x / NS) * nq, prm.status, 101)) {
                 const size_t rowi = (size_t)bh * nq + row;
 #pragma unroll
-                for (int e = 0; e < NCOL; ++e) prm.sol[rowi * D + c0 + e] = xs[(c0 + e) * TC_BR + lrow];
+                for (int e = 0; e < NCOL; ++e) prm.sol[rowi * D + c0 + e] = x_get(e);
                 if (half == 0 && prm.iters) prm.iters[rowi] = its;
                 if (half == 0 && prm.status) {
                     if (at_cap) atomicAdd(prm.status + LLA_STATUS_ROWS_AT_CAP, 1);
@@ -1064,7 +1082,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     const float qv = q_elem(qw, e);
                     const int col = ch * 8 + e;
                     const float kb = kbs[(c0 + col) * TC_BR + lrow];
-                    y[col] = xs[(c0 + col) * TC_BR + lrow];
+                    y[col] = x_get(col);
                     yb_p += kb * y[col];
                     g_p += (kb - qv) * y[col];
                 }
@@ -1267,7 +1285,7 @@ int launch_t(const ForwardArgs& a) {
     prm.window = a.causal ? a.window : 0;
     if (pack) prm.use_order = 0;
     else tile_order(prm, tiles, first_tile, a.n, a.n - a.nq, D, a.causal, prm.window, a.minv != nullptr);
-    if constexpr (!Cfg::STATE_IN_SMEM) {
+    if constexpr (!Cfg::STATE_IN_REGS) {
         int dev = 0, sms = 0;
         LLA_CUDA_TRY(cudaGetDevice(&dev));
         LLA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1320,7 +1338,7 @@ int launch_t(const ForwardArgs& a) {
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SM_ALLOC));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(units * (pairs ? 2 : 1), tiles);
-    cfg.blockDim = dim3(D == 128 ? 384 : TC_THREADS);
+    cfg.blockDim = dim3(TC_THREADS);
     cfg.dynamicSmemBytes = Cfg::SM_ALLOC;
     cfg.stream = a.stream;
     cudaLaunchAttribute attr[1];
