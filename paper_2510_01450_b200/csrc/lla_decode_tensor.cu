@@ -177,6 +177,14 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
     using C = SvCfg<D>;
     constexpr int PF = DtCfg<D>::REC, NW = C::NW;
     const int r = threadIdx.x, lane = r & 31, wp = r >> 5;
+    // ms: shared memory for the second moments, which are on their way while the weights of the parts are looked at, and
+    // which the residuals read again (null: src is in shared memory itself)
+    if (ms) {
+#pragma unroll
+        for (int c = 0; c < D / 4; ++c)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(ms + 4 * (c * D + r))), "l"(src + 4 * (c * D + r)) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
     // weights of the parts: every warp finds the maximum, one lane per part and pass
     float m = -INFINITY;
     for (int p = lane; p < splits; p += 32) m = fmaxf(m, src[(size_t)p * PF + 2 * D * D + 2 * D + 1]);
@@ -192,19 +200,16 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
     const double ridge = (ridge_mode == LLA_RIDGE_PRINTED ? lam_u : lam_u * exp(-(double)m)) * inv;
     const double ar = (double)src[2 * D * D + r] * inv, cb = (double)src[2 * D * D + D + r] * inv;
     sm.a[r] = ar;
+    if (ms) asm volatile("cp.async.wait_group 0;" ::: "memory");
     sv_sync<D>();
-    // row r of the centred matrix (column r: M is symmetric up to fp32 rounding and the loads are coalesced).  ms: shared
-    // memory for the column as it is, which the residuals below read again (null: src is in shared memory itself)
+    // row r of the centred matrix (column r of the moments: M is symmetric up to fp32 rounding)
     const float* mcol = ms ? ms + r : src + r;
     uint64_t row[D / 2];
 #pragma unroll
     for (int j = 0; j < D; j += 8) {
         float v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            v[e] = src[(j + e) * D + r];
-            if (ms) ms[(j + e) * D + r] = v[e];
-        }
+        for (int e = 0; e < 8; ++e) v[e] = mcol[(j + e) * D];
 #pragma unroll
         for (int e = 0; e < 8; e += 2) {
             double s0 = (double)v[e] * inv - sm.a[j + e] * ar, s1 = (double)v[e + 1] * inv - sm.a[j + e + 1] * ar;
