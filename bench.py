@@ -40,7 +40,7 @@ NCU_TRAFFIC = {
     3: (4 * 17.06e6, "profiles/forward_tc_kernel_cfg3.md (8 of 32 units captured, x 4)"),
     4: (8 * (33.67e6 + 2.58e6), "profiles/forward_tc_kernel_cfg4.md (2 of 16 heads captured, x 8)"),
 }
-NCU_DECODE_TRAFFIC = (1.188e9 + 24.2e6 + 34.3e6, "profiles/decode_tc_kernel_cfg5.md")   # streaming read + record write, solve read
+NCU_DECODE_TRAFFIC = (1.188e9 + 25.2e6 + 34.3e6, "profiles/decode_tc_kernel_cfg5.md")   # streaming read + record write, solve read
 
 
 def env_int(name, default):

@@ -120,6 +120,8 @@ int lla_decode_f32(const void *q, const void *kcache, const void *vcache, const 
  *   head_rows : rows that see fewer than this many keys are solved directly in fp64 from the
  *               explicit d x d system instead of by CG (0 = default: 1.5*d for bf16 inputs, 2*d for
  *               fp32 inputs; negative disables).  Those early systems are too ill-conditioned for fp32 CG.
+ *               With max_iters, tol, head_rows, impl and phases all at their defaults, every row of a problem
+ *               that the tensor-core kernel does not take (fp32 inputs, d = 16) is solved that way
  *   impl      : lla_impl
  *   phases    : which groups of rows to compute: 0 = all; LLA_PHASE_DIRECT = only the rows
  *               solved directly; LLA_PHASE_ITERATIVE = only the rows solved by CG (profiling aid:
@@ -132,7 +134,7 @@ int lla_decode_f32(const void *q, const void *kcache, const void *vcache, const 
  *               shift zero whenever every maximum of the row tile lies within 2^+-8 (Eq. "lla" does not depend on
  *               the shift; m_i + log omega_i and m_i + log delta_i are the shift-free quantities)
  *   iters     : optional [B, H, n] int32, CG iterations executed for the row (-1 for rows solved
- *               directly)
+ *               directly because they see fewer than head_rows keys, 0 for other rows solved directly)
  *   device_status : optional int[LLA_STATUS_WORDS] on the device
  *   q_rows    : 0 (or n) for the plain forward; 0 < q_rows < n for a chunk of queries at the last
  *               q_rows positions against all n keys (see the field's comment below)
@@ -264,7 +266,7 @@ typedef struct lla_decode_params {
     int page_size, max_pages, num_pages;
     int window;     /* sliding window: 0 = the query sees all lens[b] cached keys; W > 0 = only the last
                        min(W, lens[b]) of them (positions lens[b] - W .. lens[b] - 1).  Not with a paged cache */
-    long long debug_wait_clocks; /* as in lla_forward_params, for the tensor-core streaming kernel (bf16, d = 64) */
+    long long debug_wait_clocks; /* as in lla_forward_params, for the tensor-core streaming kernel (bf16) */
     int debug_flags;             /* LLA_DEBUG_NO_LOADS: its copy-issuing warp issues nothing, every bounded wait expires
                                     with nothing in flight, device_status[LLA_STATUS_TIMEOUT] counts the blocks and
                                     their units' outputs are NaN (the record of a block that gave up is poisoned) */
