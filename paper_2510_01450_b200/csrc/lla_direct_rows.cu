@@ -117,7 +117,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     for (int j0 = jbeg; j0 < jend; j0 += ch) {
         const int nk = min(ch, jend - j0);
         __syncthreads();
-        stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
+        stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch);
         __syncthreads();
         dots<D>(row_of(sm.s), row_of(sm.q), sm.kv, nk, warp, lane);
         __syncthreads();
@@ -185,6 +185,11 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     const int nba = dual ? (L + 7) / 8 : NB;
     sm.dual[tm] = dual ? L : 0;
     sm.lam[tm] = lam_m;
+    if (dual) {
+        // the diagonal of the dual form: ridge over weight for live keys (weights kept away from zero); the padding to a
+        // multiple of eight is an identity block
+        for (int j = tt; j < 8 * nba; j += 32 * NW) sm.s[tm][j] = j < L ? lam_m / fmax(sm.s[tm][j], 1e-290) : 1.0;
+    }
     if (dual && w == 0) {
         double qq = 0.0;
         for (int e = lane; e < D; e += 32) qq += sm.q[tm][e] * sm.q[tm][e];
@@ -245,9 +250,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 double v0 = idx < Lt && jdx < Lt ? gm[u][0] + (si - sm.t[t][jdx]) : 0.0;
                 double v1 = idx < Lt && jdx + 1 < Lt ? gm[u][1] + (si - sm.t[t][jdx + 1]) : 0.0;
                 if (bi == bj) {
-                    // ridge over weight for live keys (weights kept away from zero); the padding to a multiple of eight
-                    // is an identity block
-                    const double dg = idx < Lt ? sm.lam[t] / fmax(sm.s[t][idx], 1e-290) : 1.0;
+                    const double dg = sm.s[t][idx];
                     if (g == 2 * t4) v0 += dg;
                     if (g == 2 * t4 + 1) v1 += dg;
                 }
@@ -316,7 +319,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         const int nk = min(ch, jend - j0);
         __syncthreads();
         if (keys) {
-            stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
+            stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch);
             __syncthreads();
             if (dual) {
                 if (rho_out)                                       // rho = Z^T alpha
@@ -342,7 +345,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 sm.s[tm][j] = cj;
                 csum += cj;
             }
-        stage<D>(sm.kv, vb, sv.r, j0, jend, ch);
+        stage<D, true>(sm.kv, vb, sv.r, j0, jend, ch);
         __syncthreads();
         if (half < C::HALVES) {
             const int s1 = (nk + 3) / 4;

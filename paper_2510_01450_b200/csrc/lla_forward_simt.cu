@@ -2,7 +2,7 @@
 // tensor-core kernel does not take when the caller sets something of the solver (iteration cap, tolerance, head_rows,
 // phases), and with impl = LLA_IMPL_SIMT for everything, as an independent cross-check.  Under the default settings
 // those problems are solved directly (lla_direct_rows.cu), which is faster: 1000 rows of 8 fp32 heads, d = 64,
-// take 1.03 ms there and 2.56 ms here.
+// take 1.01 ms there and 2.56 ms here.
 //
 // Structure follows Algorithm 1 (three sweeps over the key blocks per query block) with the
 // solver of Algorithm 2 in between, in the weighted-mean-centred form of Eq. "lla_decomp":
