@@ -10,7 +10,7 @@
 // as products over the block's rows, so that a block adds to a gradient entry once instead of once per row.
 //
 // Measured on B200 against one block per row with a shared-memory LDL^T on the CUDA cores and one atomic per row and
-// entry: 32 heads, n = 1000, d = 64 (95 rows a head): 305 -> 135 us; 16 heads, d = 128 (191 rows): 3.5 -> 1.1 ms.
+// entry: 32 heads, n = 1000, d = 64 (95 rows a head): 305 -> 130 us; 16 heads, d = 128 (191 rows): 3.5 -> 1.1 ms.
 #include "lla_rows.cuh"
 
 namespace lla {

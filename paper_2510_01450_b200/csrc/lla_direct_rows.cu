@@ -117,7 +117,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     for (int j0 = jbeg; j0 < jend; j0 += ch) {
         const int nk = min(ch, jend - j0);
         __syncthreads();
-        stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch);
+        stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
         __syncthreads();
         dots<D>(row_of(sm.s), row_of(sm.q), sm.kv, nk, warp, lane);
         __syncthreads();
@@ -319,7 +319,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         const int nk = min(ch, jend - j0);
         __syncthreads();
         if (keys) {
-            stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch);
+            stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
             __syncthreads();
             if (dual) {
                 if (rho_out)                                       // rho = Z^T alpha
@@ -345,7 +345,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 sm.s[tm][j] = cj;
                 csum += cj;
             }
-        stage<D, true>(sm.kv, vb, sv.r, j0, jend, ch);
+        stage<D>(sm.kv, vb, sv.r, j0, jend, ch);
         __syncthreads();
         if (half < C::HALVES) {
             const int s1 = (nk + 3) / 4;

@@ -37,10 +37,11 @@ __device__ __forceinline__ void load_pair<float>(const float* p, double& a, doub
     b = (double)f.y;
 }
 
-// keys (or values) j0 .. j0 + ch - 1 -> shared memory; rows from jend on are zero.  With TRIM the rounds that hold no row
-// before jend are left out, four at a time: their rows keep what they held, and nothing may read them.
-// (Rows of 1 to 95 keys, 32 heads, d = 64: 92 -> 87 us together with the dual form's diagonal made once per row.)
-template <int D, bool TRIM = false, typename TIn>
+// keys (or values) j0 .. j0 + ch - 1 -> shared memory; rows from jend on are zero, but the rounds
+// that hold no row before jend are left out, four at a time: their rows keep what they held, and nothing reads them.
+// (Rows of 1 to 95 keys, 32 heads, d = 64: 92 -> 87 us together with the dual form's
+// diagonal made once per row; the backward's rows 135 -> 130 us.)
+template <int D, typename TIn>
 __device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch) {
     using C = DrCfg<D>;
     constexpr int PER = C::CH * D / 2 / C::THREADS, PER_STEP = C::STEP * D / 2 / C::THREADS;
@@ -49,7 +50,7 @@ __device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* _
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
         if (u >= PER_STEP && ch == C::STEP) break;
-        if (TRIM && u % 4 == 0 && j0 + ROUND * u >= jend) break;
+        if (u % 4 == 0 && j0 + ROUND * u >= jend) break;
         const int e = threadIdx.x + C::THREADS * u, j = e / (D / 2), c = 2 * (e % (D / 2));
         double a = 0.0, b = 0.0;
         if (j0 + j < jend) load_pair(src + (size_t)(j0 + j) * stride + c, a, b);
