@@ -120,8 +120,9 @@ int lla_decode_f32(const void *q, const void *kcache, const void *vcache, const 
  *   head_rows : rows that see fewer than this many keys are solved directly in fp64 from the
  *               explicit d x d system instead of by CG (0 = default: 1.5*d for bf16 inputs, 2*d for
  *               fp32 inputs; negative disables).  Those early systems are too ill-conditioned for fp32 CG.
- *               With max_iters, tol, head_rows, impl and phases all at their defaults, every row of a problem
- *               that the tensor-core kernel does not take (fp32 inputs, d = 16) is solved that way
+ *               With max_iters, tol, head_rows, impl and phases all at their defaults, further rows of a problem
+ *               that the tensor-core kernel does not take (fp32 inputs, d = 16) are solved that way where that is
+ *               faster than CG: all of them, unless they see very many keys and the call is large
  *   impl      : lla_impl
  *   phases    : which groups of rows to compute: 0 = all; LLA_PHASE_DIRECT = only the rows
  *               solved directly; LLA_PHASE_ITERATIVE = only the rows solved by CG (profiling aid:

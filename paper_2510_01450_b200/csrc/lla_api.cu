@@ -201,10 +201,12 @@ int lla_forward_ex(const lla_forward_params* p) {
     if (p->block_mask && (!use_tensor || !a.causal || a.window > 0 || a.n > 65536 || p->block_mask_stride < 0)) return LLA_ERR_UNSUPPORTED;
     // the forward workspace is optional (see lla_forward_workspace_bytes); a misaligned one is an error
     if (a.workspace && a.workspace_bytes > 0 && ((uintptr_t)a.workspace & 255u)) return LLA_ERR_WORKSPACE;
-    // A problem that the tensor-core kernel does not take is solved row by row from explicit moments, unless the caller
-    // asks for something of the conjugate-gradient solver.
-    a.all_direct = !use_tensor && p->impl == LLA_IMPL_AUTO && p->phases == LLA_PHASE_ALL && p->max_iters == 0 && p->tol == 0.f && p->head_rows == 0;
+    // A problem that the tensor-core kernel does not take is solved row by row from explicit moments where that is
+    // faster, unless the caller asks for something of the conjugate-gradient solver.
+    if (!use_tensor && p->impl == LLA_IMPL_AUTO && p->phases == LLA_PHASE_ALL && p->max_iters == 0 && p->tol == 0.f && p->head_rows == 0)
+        a.direct_below = lla::direct_rows_worthwhile(a);
     if (a.status) LLA_CUDA_TRY(cudaMemsetAsync(a.status, 0, sizeof(int) * LLA_STATUS_WORDS, a.stream));
+    if (p->phases == LLA_PHASE_ALL && lla::head_rows_count(a) >= a.nq) return lla::launch_head_rows(a);      // no other rows
     // The two row groups write disjoint rows of `out`; when both run, the direct rows go to a side
     // stream so they fill the SMs the iterative kernel's last wave leaves idle.
     // (the pre-pass of the tensor-core kernel goes first so that the fork below comes after it: the direct rows
@@ -213,7 +215,6 @@ int lla_forward_ex(const lla_forward_params* p) {
         const int rc_pre = lla::forward_tensor_prepass(a);
         if (rc_pre != LLA_OK) return rc_pre;
     }
-    if (a.all_direct) return lla::launch_head_rows(a);
     const bool both = p->phases == LLA_PHASE_ALL && lla::head_rows_count(a) > 0;
     SideStream* side = both ? side_stream() : nullptr;
     if (side) {

@@ -87,7 +87,7 @@ struct ForwardArgs {
     int max_iters;
     float tol;
     int head_rows;   // rows seeing fewer keys than this are solved directly (fp64)
-    bool all_direct = false;     // every row is (the problems the tensor-core kernel does not take, default solver settings)
+    int direct_below = 0;        // > 0: so are those seeing fewer than this (problems the tensor-core kernel does not take)
     float* rho;      // optional
     float* stats;    // optional
     int* iters;      // optional
@@ -222,6 +222,8 @@ int launch_backward(const BackwardArgs& a);
 int launch_backward_rows(const BackwardArgs& a, int nq, int rows, cudaStream_t stream);      // the directly-solved rows
 
 // Launchers implemented in the other translation units; each returns an lla_status.
+int direct_rows_below(const ForwardArgs& a);  // rows that see fewer keys than this are solved directly
+int direct_rows_worthwhile(const ForwardArgs& a);  // the same where conjugate gradients in fp32 are the alternative
 int head_rows_count(const ForwardArgs& a);   // leading query rows per head solved directly
 int launch_head_rows(const ForwardArgs& a);
 int launch_forward_simt(const ForwardArgs& a);

@@ -4,9 +4,9 @@
 //   * rows that see fewer than head_rows keys (default 1.5 d for bf16 inputs, 2 d for fp32).  Their systems have condition
 //     numbers of 1e4 .. 1e5 at the paper's ridge sizes (rank-deficient plus ridge while L < d), which the conjugate
 //     gradients of the other kernels cannot resolve;
-//   * every row of a problem that the tensor-core kernel does not take (fp32 inputs, d = 16) under the default solver
-//     settings.  Matrix-free conjugate gradients in fp32 need 20 .. 40 sweeps of 6 d operations per (query, key) pair
-//     there, explicit moments d^2 + 8 d once.
+//   * the rows of a problem that the tensor-core kernel does not take (fp32 inputs, d = 16) under the default solver
+//     settings, all of them or up to a number of keys (direct_rows_worthwhile below).  Matrix-free conjugate gradients
+//     in fp32 need 10 .. 40 sweeps of 6 d operations per (query, key) pair there, explicit moments d^2 + 8 d once.
 //
 // A row with more than d visible keys solves the centred system C y = kbar - q of Eq. "lla_decomp",
 //     C = sum_j p_j k_j k_j^T - kbar kbar^T + (lambda' / omega) I,     p_j = w_j / omega,   lambda' = lambda e^{-m},
@@ -23,6 +23,8 @@
 // What bounds it: the matrix pipe in the moments of long rows (36 of the about 47 instructions per 4 keys and row at
 // d = 64; measured at 89 % of its rate), the chain of reciprocals in the pivot blocks for short ones, which the eight
 // systems of two blocks on an SM hide in part.
+#include <algorithm>
+
 #include "lla_rows.cuh"
 
 namespace lla {
@@ -409,15 +411,50 @@ int launch_d(const ForwardArgs& a, int rows) {
 
 }  // namespace
 
+int direct_rows_below(const ForwardArgs& a) { return std::max(a.head_rows, a.direct_below); }
+
+// Direct or fp32 conjugate gradients (lla_forward_simt.cu), for problems that the tensor-core kernel does not take.  A row
+// with L keys costs here kd L + c0 microseconds of an SM whatever the data, there about ks L + s0 (keys and queries of the
+// usual recipe; the iterations fall with L, sharper weights take more).  Measured:
+//     d = 128: 0.137 L + 10    0.0575 L + 50    equal at 500 keys   (16 heads, n = 4000: 121 ms direct, 73 ms)
+//     d = 64:  0.031 L + 2.5   0.0194 L + 35    equal at 2800 keys  (8 heads, n = 8000: 54 ms direct, 50 ms)
+//     d = 16:  0.0067 L + 0.5  0.0056 L + 7.4   equal at 6300 keys  (16 heads, n = 8000: 23 ms direct, 26 ms)
+// But conjugate gradients are as slow as their longest block, which takes its rows through all sweeps alone (2 heads, n =
+// 2000, d = 128: 4.1 ms direct, 5.5 ms): the rows from that line on go there only if the whole call is shorter for it.
+int direct_rows_worthwhile(const ForwardArgs& a) {
+    const double kd = a.d == 128 ? 0.137 : a.d == 64 ? 0.031 : 0.0067, c0 = a.d == 128 ? 10.0 : a.d == 64 ? 2.5 : 0.5;
+    const double ks = a.d == 128 ? 0.0575 : a.d == 64 ? 0.0194 : 0.0056, s0 = a.d == 128 ? 50.0 : a.d == 64 ? 35.0 : 7.4;
+    const int block_rows = a.d == 128 ? 32 : 64, off = a.n - a.nq;
+    const int all = a.n + 1;
+    auto seen = [&](int pos) { return (double)(!a.causal ? a.n : a.window > 0 ? std::min(pos, a.window) : pos); };
+    auto direct = [&](double L) { return kd * L + c0; };
+    auto iterative = [&](double L) { return ks * L + s0; };
+    int line = std::max(a.head_rows, 1);
+    while (line <= a.n && direct(seen(line)) <= iterative(seen(line))) line += 64;
+    if (!a.causal) line = direct(a.n) <= iterative(a.n) ? all : 1;
+    if (line > a.n) return all;
+    double t_direct = 0.0, t_split = 0.0;                // microseconds of an SM, summed over a head's rows
+    for (int r = 0; r < a.nq; r += 32) {
+        const int rows = std::min(32, a.nq - r), pos = off + r + rows;
+        t_direct += rows * direct(seen(pos));
+        t_split += rows * (pos < line ? direct(seen(pos)) : iterative(seen(pos)));
+    }
+    int dev = 0, sms = 148;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const double heads = (double)a.B * a.H, longest = block_rows * iterative(seen(a.n));
+    const double split = std::max(longest, heads * t_split / sms + 0.3 * longest);
+    return split < heads * t_direct / sms ? line : all;
+}
+
 // Number of leading rows per head handled directly (causal), or nq / 0 (non-causal).
 int head_rows_count(const ForwardArgs& a) {
-    if (a.all_direct) return a.nq;
-    if (a.head_rows <= 0) return 0;
+    const int below = direct_rows_below(a);
+    if (below <= 0) return 0;
     if (a.causal) {     // query row i sees n - nq + i + 1 keys
-        const int rows = a.head_rows - 1 - (a.n - a.nq);
+        const int rows = below - 1 - (a.n - a.nq);
         return rows < 0 ? 0 : (rows > a.nq ? a.nq : rows);
     }
-    return a.n < a.head_rows ? a.nq : 0;
+    return a.n < below ? a.nq : 0;
 }
 
 int launch_head_rows(const ForwardArgs& a) {

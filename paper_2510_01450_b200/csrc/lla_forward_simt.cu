@@ -1,7 +1,7 @@
 // LLA forward on CUDA cores, fp32 arithmetic, by conjugate gradients: for fp32 tensors, d = 16 and whatever else the
 // tensor-core kernel does not take when the caller sets something of the solver (iteration cap, tolerance, head_rows,
 // phases), and with impl = LLA_IMPL_SIMT for everything, as an independent cross-check.  Under the default settings
-// those problems are solved directly (lla_direct_rows.cu), which is faster: 1000 rows of 8 fp32 heads, d = 64,
+// it has the rows with many keys of large calls; the others are solved directly (lla_direct_rows.cu), which is faster: 1000 rows of 8 fp32 heads, d = 64,
 // take 1.01 ms there and 2.56 ms here.
 //
 // Structure follows Algorithm 1 (three sweeps over the key blocks per query block) with the
@@ -25,6 +25,8 @@
 // Thread mapping: TPR consecutive lanes share one query row, each owning D/TPR columns of every
 // row vector (q, kbar, x, r, p, C p) in registers; dot products finish with TPR-wide xor shuffles.
 // Key (and value) tiles are staged in shared memory as fp32 and read as broadcast float4s.
+#include <algorithm>
+
 #include "lla_common.cuh"
 
 namespace lla {
@@ -319,7 +321,7 @@ int launch_t(const ForwardArgs& a) {
     dim3 grid(tiles, a.B * a.H);
     kern<<<grid, FS_THREADS, smem, a.stream>>>(
         (const TIn*)a.q, (const TIn*)a.k, (const TIn*)a.v, (TOut*)a.out, a.n, a.causal, a.scale,
-        a.lambda, a.head_rows > 0 ? a.head_rows : 0, a.max_iters, a.tol, first_tile, a.rho, a.stats,
+        a.lambda, std::max(direct_rows_below(a), 0), a.max_iters, a.tol, first_tile, a.rho, a.stats,
         a.iters, a.status, a.lambda_rows, a.ridge_mode, a.nq, a.H, a.kv_group, a.window, a.sq, a.sk, a.sv, a.so);
     LLA_CUDA_TRY(cudaGetLastError());
     return LLA_OK;

@@ -72,3 +72,31 @@ def test_backward_short_rows(backward_oracle, d, n, H):
         assert np.isfinite(a).all(), name
         err = grad_err(a, b)
         assert err.max() <= TOL, (name, float(err.max()), int(err.argmax()))
+
+
+# calls large enough that the rows with many keys go to the conjugate gradients instead: part of the rows of a causal call,
+# every row of a non-causal one
+@pytest.mark.parametrize("n,nq,B,H,causal", [(1500, 1500, 2, 8, True), (1100, 1100, 2, 8, False), (2000, 700, 2, 8, True)])
+def test_direct_and_iterative_rows_side_by_side(oracle, n, nq, B, H, causal):
+    d = 128
+    w = inputs.CONFIGS[2].shrink(B=B, H=H, n=n, d=d, dv=d, dtype="f32", seed=900 + n)
+    q, k, v = inputs.make_prefill(w)
+    qc = np.ascontiguousarray(q[:, :, n - nq:])
+    out = torch.full((B, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+    iters = torch.full((B, H, nq), -7, dtype=torch.int32, device="cuda")
+    L.lla_forward_ex(dev(qc, "f32"), dev(k, "f32"), dev(v, "f32"), out, B, H, n, d, d, w.scale, w.lam, causal=causal,
+                     in_dtype=L.LLA_F32, out_dtype=L.LLA_F32, q_rows=nq, iters=iters, stream=stream_ptr())
+    torch.cuda.synchronize()
+    assert torch.isfinite(out).all()
+    it = iters.cpu().numpy()
+    assert (it >= -1).all() and (it[:, :, -1] > 0).all()
+    cut = int(np.argmax(it[0, 0] > 0))                       # the first row of the iterative kernel
+    assert (it[:, :, cut:] > 0).all() and (it[:, :, :cut] <= 0).all()
+    rows = np.unique(np.clip([0, cut - 1, cut, cut + 1, nq // 2, nq - 1], 0, nq - 1))
+    cnt = np.array([n - nq + r + 1 if causal else n for r in rows], dtype=np.int32)
+    for b in range(B):
+        kc = np.repeat(k[b][None], len(rows), axis=0)
+        vc = np.repeat(v[b][None], len(rows), axis=0)
+        ref = oracle.decode(np.ascontiguousarray(qc[b][:, rows].transpose(1, 0, 2)), kc, vc, cnt, w.scale, w.lam)
+        err = row_err(out.cpu().numpy()[b][:, rows].transpose(1, 0, 2), ref)
+        assert err.max() <= TOL_F32, (b, float(err.max()), int(err.argmax()))
