@@ -1213,11 +1213,12 @@ float* scratch_for_device(size_t bytes) {
 }
 
 // Launch order of the query tiles: longest first, so that the blocks left for the end are short.
-// A tile's cost is (sweeps) x (per-sweep overhead + key blocks).  Sweeps = 3 + CG iterations, and the
-// iteration count falls with the number of visible keys per dimension (the first tiles need several
-// times more than the rest), so at short sequence lengths the first tiles are the longest blocks
-// even though their sweeps are the shortest.  The numbers are a fit to measured runs; they only
-// steer the order, never the result.
+// A tile's cost is (sweeps) x (per-sweep overhead + key blocks).  Sweeps = 2 + CG iterations, and the iteration count
+// falls with the number of visible keys per dimension (measured at d / keys = 1/2, 1/4, 1/8, 1/16, 1/64: 37 .. 42, 24,
+// 10.5, 7.5, 5; the same at both head sizes), so at short sequence lengths the first tiles are the longest blocks even
+// though their sweeps are the shortest.  A sweep's overhead is worth 8.5 key blocks (10 at d = 128).  The numbers only
+// steer the order, never the result.  (Against a fit with a third fewer iterations for the first tiles: n = 1500, 16 heads,
+// d = 64: 317 -> 294 us; n = 3000, 8 heads: 336 -> 321 us.)
 void tile_order(TcParams& prm, int tiles, int first_tile, int n, int off, int d, int causal, int window, bool precond) {
     prm.use_order = 0;
     if (!causal || tiles > TC_ORDER_MAX) return;
@@ -1226,10 +1227,10 @@ void tile_order(TcParams& prm, int tiles, int first_tile, int n, int off, int d,
         const int r_end = std::min(n, off + (first_tile + t + 1) * TC_BR);      // keys the tile's last row sees
         const int seen = window > 0 ? std::min(r_end, window) : r_end;
         const float x = (float)d / (float)seen;
-        const float its = precond ? std::min(16.f, 4.f + 190.f * x * x) : 6.f + 50.f * x;
+        const float its = precond ? std::min(16.f, 4.f + 190.f * x * x) : std::min(40.f, 4.5f + 40.f * x + 150.f * x * x);
         const int c_first = window > 0 ? std::max(0, off + (first_tile + t) * TC_BR + 1 - window) / TC_BC : 0;
         const float nblk = (float)((r_end + TC_BC - 1) / TC_BC - c_first);
-        cost[t] = (its + 2.f) * (6.f + nblk) + (precond ? 3.f * its : 0.f);
+        cost[t] = (its + 2.f) * ((d == 64 ? 8.5f : 10.f) + nblk) + (precond ? 3.f * its : 0.f);
         prm.order[t] = (unsigned short)t;
     }
     std::stable_sort(prm.order, prm.order + tiles, [&](unsigned short x, unsigned short y) { return cost[x] > cost[y]; });
