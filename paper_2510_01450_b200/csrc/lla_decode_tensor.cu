@@ -200,6 +200,7 @@ __device__ __forceinline__ void solve_unit(const __nv_bfloat16* __restrict__ qro
     const double ridge = (ridge_mode == LLA_RIDGE_PRINTED ? lam_u : lam_u * exp(-(double)m)) * inv;
     const double ar = (double)src[2 * D * D + r] * inv, cb = (double)src[2 * D * D + D + r] * inv;
     sm.a[r] = ar;
+    sm.x[r] = 0.0;      // the solution where the right-hand side is zero and no round runs
     if (ms) asm volatile("cp.async.wait_group 0;" ::: "memory");
     sv_sync<D>();
     // row r of the centred matrix (column r of the moments: M is symmetric up to fp32 rounding)

@@ -82,3 +82,32 @@ def test_solve_falls_back_to_elimination(oracle, d):
     torch.cuda.synchronize()
     # bf16 operand pairs of w k carry 2^-17 relative error per key, features at 1e-3 of the largest: 1e-2 covers it
     assert row_err(out.cpu().numpy(), ref).max() <= 1e-2
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("mode", ["zero", "constant", "paired"])
+def test_query_at_the_weighted_key_mean(oracle, d, mode):
+    """A right-hand side of the solve that is exactly zero: the slope term vanishes and the output is the weighted value
+    mean.  Runs behind an ordinary decode, so that shared memory holds another unit's solution."""
+    B, H, n = 2, 4, 512
+    w = inputs.CONFIGS[5].shrink(B=B, H=H, n=n, d=d, dv=d, len_min=n, len_max=n, seed=430 + d)
+    q, kc, vc, _ = inputs.make_decode(w)
+    lens = np.array([n, 256], dtype=np.int32)          # (powers of two: the mean of equal keys is exact)
+    q0, k0 = np.zeros_like(q), np.zeros_like(kc)
+    if mode == "constant":
+        q0 = q.copy()
+        k0 = np.ascontiguousarray(np.broadcast_to(q[:, :, None], kc.shape))
+    if mode == "paired":                              # keys in +/- pairs, a zero query
+        k0 = kc.copy()
+        k0[:, :, 1::2] = -k0[:, :, ::2]
+    ref = oracle.decode(q0, k0, vc, lens, w.scale, w.lam)
+    nbytes = 4 * B * H * (2 * d * d + 2 * d + 4)
+    dl, dv_ = torch.from_numpy(lens).cuda(), dev(vc, "bf16")
+    for ws in (torch.empty(nbytes, dtype=torch.uint8, device="cuda"), None):
+        for qq, kk in ((q, kc), (q0, k0)):
+            out = torch.full((B, H, d), float("nan"), dtype=torch.float32, device="cuda")
+            L.lla_decode_ex(dev(qq, "bf16"), dev(kk, "bf16"), dv_, dl, out, B, H, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32,
+                            splits=1, workspace=ws, workspace_bytes=nbytes if ws is not None else 0, stream=stream_ptr())
+        torch.cuda.synchronize()
+        err = row_err(out.cpu().numpy(), ref)
+        assert np.isfinite(err).all() and err.max() <= TOL_BF16, (float(err.max()), int(err.argmax()))
