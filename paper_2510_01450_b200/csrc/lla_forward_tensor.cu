@@ -36,6 +36,7 @@
 #include <mutex>
 
 #include "lla_sm100.cuh"
+#include "lla_voted_loop.cuh"
 
 namespace lla {
 namespace {
@@ -928,35 +929,23 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
         }
         if (ok) write_p(0);
-        // One barrier for two questions: does any row go on, and did every thread's waits succeed (a thread that gave
-        // up leaves a mark before the barrier; two marks in turn, so that none is set while the last is still read)
-        uint32_t votes = 0;
-        auto go_on = [&](bool act) {
-            const int slot = 8 + (votes++ & 1);
-            if (!ok) misc[slot] = 1;
-            const bool any = group_any(act);
-            if (misc[slot]) ok = false;
-            return any && ok;
-        };
         // ---- conjugate gradients (Algorithm 2) ----
-        int t = 0;      // CG sweeps run
-        for (; ok && t < prm.max_iters; ++t) {
-            active = active && rr > stop;
-            if (!go_on(active)) break;
+        auto still_active = [&]() { return active = active && rr > stop; };
+        auto cg_pass = [&](int t) -> bool {
             const bool cheap = f16_on && t >= precise;
             start_sweep(cheap ? SW_CG16 : SW_CG, cheap);
             sweep(cheap ? SW_CG16 : SW_CG);
             if (ok) acc_wait();
             if (PC) {
                 ok = all_ok(ok);
-                if (!ok) break;
+                if (!ok) return false;
             }
             float ap[NCOL];
             acc_load(ap);
             if (NS > 1) {
                 float u0 = 0.f, u1 = 0.f;
                 exchange(ap, u0, u1);
-                if (!ok) break;
+                if (!ok) return false;
             }
             // (the loops below keep four independent partial sums and move the row-vector state in
             //  batches of eight so that the loads overlap: two warps per scheduler hide no latency)
@@ -1014,7 +1003,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 rr2 = pair_sum(rr2);
                 precondition(ap, rr2);
                 ok = all_ok(ok);
-                if (!ok) break;
+                if (!ok) return false;
                 float rz_p = 0.f, kz_p = 0.f, zz_p = 0.f;
 #pragma unroll
                 for (int e0 = 0; e0 < NCOL; e0 += 8) {
@@ -1055,7 +1044,9 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
             }
             write_p(t + 1);
-        }
+            return true;
+        };
+        const int t = voted_loop(prm.max_iters, ok, misc + 8, still_active, cg_pass, group_any);      // CG sweeps run
         const bool at_cap = active && rr > stop;
         // ---- output sweep ----
         float gfac = 1.f;
