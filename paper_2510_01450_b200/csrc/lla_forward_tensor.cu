@@ -760,11 +760,11 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         float rr = 0.f, stop = 0.f;
         int its = 0;
         bool active = false;
-        // P operand for CG iteration t_next: bf16 hi + lo for the first precise_iters iterations, one fp16 after
+        // P operand of CG iteration t: bf16 hi + lo for the first precise_iters iterations, one fp16 after
         // (the products of an iteration enter x and r scaled by |p|, which has fallen by then: the coarser
         // operands of the later iterations cost no accuracy that the early ones have not already spent)
-        auto write_p = [&](int t_next) {
-            if (f16_on && t_next >= precise) {
+        auto write_p = [&](int t) {
+            if (f16_on && t >= precise) {
                 const int e2 = (int)((__float_as_uint(pn2) >> 23) & 0xffu) - 127;      // floor(log2 |p|^2)
                 const int k = max(-100, min(100, -(e2 >> 1)));
                 psc = __uint_as_float((uint32_t)(127 + k) << 23);
@@ -928,11 +928,13 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
             }
         }
-        if (ok) write_p(0);
         // ---- conjugate gradients (Algorithm 2) ----
         auto still_active = [&]() { return active = active && rr > stop; };
         auto cg_pass = [&](int t) -> bool {
             const bool cheap = f16_on && t >= precise;
+            // (behind the vote, which all compute threads take: in a pair of blocks the other block's sums, which lie
+            //  over the operand tiles in another layout, have been read by everyone then)
+            write_p(t);
             start_sweep(cheap ? SW_CG16 : SW_CG, cheap);
             sweep(cheap ? SW_CG16 : SW_CG);
             if (ok) acc_wait();
@@ -1043,7 +1045,6 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     ++its;
                 }
             }
-            write_p(t + 1);
             return true;
         };
         const int t = voted_loop(prm.max_iters, ok, misc + 8, still_active, cg_pass, group_any);      // CG sweeps run
@@ -1081,6 +1082,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             abar = pair_sum(yb_p);
             gfac = 1.f + pair_sum(g_p);
             const bool out16 = f16_on && t >= precise;      // the format every role derives from the CG sweeps it has seen
+            // (over the other block's last sums, like p: the vote that ended the loop lies in between)
             if (out16) write_operand16_pair(y);
             else write_operand(y);
             start_sweep(SW_OUT, out16);

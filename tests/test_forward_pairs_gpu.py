@@ -86,3 +86,23 @@ def test_a_pair_whose_waits_run_out_leaves_cleanly():
     assert st[L.STATUS_TIMEOUT] == 2 * B * H * (nq // 128)
     again, st = run()
     assert st[L.STATUS_TIMEOUT] == 0 and np.array_equal(good, again)
+
+
+@pytest.mark.parametrize("d,H,n,nq", [(64, 4, 3000, 500), (128, 4, 2500, 400)])
+def test_pairs_repeat_exactly(d, H, n, nq):
+    """The two blocks of a pair leave their sums in each other's operand tiles; who reads and who overwrites them when must
+    not show: every run gives the same bits (weights far from uniform, so that the rows take many iterations)."""
+    w = inputs.CONFIGS[2].shrink(B=1, H=H, n=n, d=d, dv=d, seed=540 + d)
+    q, k, v = inputs.make_prefill(w)
+    s = np.float32(d ** 0.5)
+    args = [dev(inputs.round_to_bf16(x), "bf16") for x in (np.ascontiguousarray(q[:, :, n - nq:]) * s, k * s, v)]
+    nbytes = L.lla_forward_workspace_bytes(1, H, n, d, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    first = None
+    for _ in range(25):
+        out = torch.full((1, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+        L.lla_forward_ex(*args, out, 1, H, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, q_rows=nq, workspace=ws,
+                         workspace_bytes=nbytes, stream=stream_ptr())
+        assert torch.isfinite(out).all()
+        first = out if first is None else first
+        assert torch.equal(out, first)
