@@ -86,6 +86,29 @@ __device__ __forceinline__ void sync(int bar_id) {
     else asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(32 * NW) : "memory");
 }
 
+// Inverse (j00 j01; j01 j11) of the symmetric block (a b; b c); false if it is not positive definite.
+// The entries span the doubles' whole range (a diagonal of the dual form is lambda e^-score), so their products may not
+// be representable where the inverse is.  A determinant with an exponent beyond 2^+-823 is formed again from the
+// entries scaled by powers of two that bring a and c to [1, 2).  (The same operands in every lane: the branch does not diverge.)
+__device__ __forceinline__ bool invert_pivot(double a, double b, double c, double& j00, double& j01, double& j11) {
+    double det = a * c - b * b;
+    const double inv = fast_rcp(det);
+    j00 = c * inv;
+    j01 = -b * inv;
+    j11 = a * inv;
+    if ((((unsigned)__double2hiint(det)) >> 20) - 200u >= 1646u) {      // (a sign, infinity and NaN come here too)
+        const double sa = __hiloint2double(0x7fe00000 - (__double2hiint(a) & 0x7ff00000), 0);
+        const double sc = __hiloint2double(0x7fe00000 - (__double2hiint(c) & 0x7ff00000), 0);
+        const double as = a * sa, cs = c * sc;
+        det = as * cs - (b * sa) * (b * sc);
+        const double is = fast_rcp(det);
+        j00 = (cs * is) * sa;
+        j01 = -((b * sa) * is) * sc;
+        j11 = (as * is) * sc;
+    }
+    return a > 0.0 && det > 0.0;
+}
+
 // Solve for the right-hand sides in sm.b.  c: the lower block triangle (destroyed); nba: block rows in use (the rest is
 // not touched); w, lane: warp inside the team and lane.  The solution is in sm.x[w].  Everything must be visible to
 // the team before the call.  Returns false if a pivot was not positive (the same in every warp).
@@ -108,9 +131,8 @@ __device__ __forceinline__ bool solve(double (*c)[64], Smem<D, NW, NRHS>& sm, in
             const double v0 = __shfl_sync(FULL, a0, 8 * k + 4 + t4), v1 = __shfl_sync(FULL, a1, 8 * k + 4 + t4);
             const double r0 = __shfl_sync(FULL, w0, 8 * k + t4), r1 = __shfl_sync(FULL, w1, 8 * k + t4);
             const double s0 = __shfl_sync(FULL, w0, 8 * k + 4 + t4), s1 = __shfl_sync(FULL, w1, 8 * k + 4 + t4);
-            const double det = pa * pc - pb * pb, inv = fast_rcp(det);
-            ok = ok && pa > 0.0 && det > 0.0;
-            const double j00 = pc * inv, j01 = -pb * inv, j11 = pa * inv;
+            double j00, j01, j11;
+            ok = invert_pivot(pa, pb, pc, j00, j01, j11) && ok;
             const double m0 = g > 2 * k + 1 ? x0 * j00 + x1 * j01 : 0.0, m1 = g > 2 * k + 1 ? x0 * j01 + x1 * j11 : 0.0;
             a0 -= m0 * u0 + m1 * v0;
             a1 -= m0 * u1 + m1 * v1;

@@ -100,3 +100,63 @@ def test_direct_and_iterative_rows_side_by_side(oracle, n, nq, B, H, causal):
         ref = oracle.decode(np.ascontiguousarray(qc[b][:, rows].transpose(1, 0, 2)), kc, vc, cnt, w.scale, w.lam)
         err = row_err(out.cpu().numpy()[b][:, rows].transpose(1, 0, 2), ref)
         assert err.max() <= TOL_F32, (b, float(err.max()), int(err.argmax()))
+
+
+def _scores_far_from_zero(dtype, d, n, mode):
+    """Raw scores far below zero, where the systems' diagonal lambda e^{-s_j} is beyond 1e154: of every key ("low") or
+    of every other key ("mixed"); or pairs of keys that equal the query, whose diagonal is lambda e^{-s} below 1e-154 ("high")."""
+    rng = np.random.default_rng(950 + d + n)
+    scale = np.float32(d ** -0.5)
+    u = np.ones(d, dtype=np.float32) / np.float32(np.sqrt(d))
+    a = np.float32(np.sqrt({"low": 520.0, "mixed": 520.0, "high": 600.0}[mode] / scale))
+    noise = lambda: rng.standard_normal((1, 2, n, d)).astype(np.float32) * scale
+    q, k, v = a * u + noise(), noise(), noise() * np.float32(np.sqrt(d))
+    if mode == "low":
+        k -= a * u
+    if mode == "mixed":
+        k[:, :, ::2] -= a * u
+    if mode == "high":
+        q[:] = a * u
+        k[:, :, :2] = a * u
+    rnd = inputs.round_to_bf16 if dtype == "bf16" else (lambda x: x.astype(np.float32))
+    return (*map(rnd, (q, k, v)), float(scale))
+
+
+FAR_SIZES = [("bf16", 64, 95), ("f32", 16, 130), ("f32", 64, 200), ("bf16", 128, 140), ("f32", 128, 150)]
+
+
+@pytest.mark.parametrize("dtype,d,n,mode", [(*size, mode) for size in FAR_SIZES for mode in ("low", "mixed")] +
+                         [("bf16", 64, 95, "high"), ("bf16", 128, 140, "high")])
+def test_scores_far_from_zero(oracle, dtype, d, n, mode):
+    q, k, v, scale = _scores_far_from_zero(dtype, d, n, mode)
+    if mode == "high":
+        # every row sees the two keys at its query: z = 0 for both, the others weigh e^-600 -- the mean of the two values
+        # (rows with more than d keys are left out: e^-600 of the identity is no ridge in the explicit form)
+        n = d
+        q, k, v = (np.ascontiguousarray(x[:, :, :n]) for x in (q, k, v))
+        ref = np.repeat(v[:, :, :2].astype(np.float64).mean(axis=2, keepdims=True), n, axis=2)
+        ref[:, :, 0] = v[:, :, 0]
+    else:
+        ref = oracle.forward(q, k, v, scale, 1e-3)
+    out = torch.full(q.shape, float("nan"), dtype=torch.float32, device="cuda")
+    status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+    L.lla_forward_ex(dev(q, dtype), dev(k, dtype), dev(v, dtype), out, 1, 2, n, d, d, scale, 1e-3, in_dtype=LLA_DT[dtype],
+                     out_dtype=L.LLA_F32, device_status=status, stream=stream_ptr())
+    torch.cuda.synchronize()
+    assert status.cpu().numpy()[L.STATUS_BAD_PIVOT] == 0
+    err = row_err(out.cpu().numpy(), ref)
+    assert np.isfinite(err).all() and err.max() <= (TOL_F32 if dtype == "f32" else TOL_BF16), (float(np.nanmax(err)), int(np.isnan(err).sum()))
+
+
+@pytest.mark.parametrize("mode", ["low", "mixed"])
+def test_backward_scores_far_from_zero(backward_oracle, mode):
+    d, n = 64, 95
+    q, k, v, scale = _scores_far_from_zero("bf16", d, n, mode)
+    w = inputs.CONFIGS[2].shrink(B=1, H=2, n=n, d=d, dv=d)
+    assert abs(w.scale - scale) < 1e-6
+    g = inputs.make_upstream_grad(w)
+    ref = backward_oracle.backward(q, k, v, g, w.scale, w.lam)
+    for name, a, b in zip(("dq", "dk", "dv"), run_backward(w, q, k, v, g), ref):
+        assert np.isfinite(a).all(), name
+        err = grad_err(a, b)
+        assert err.max() <= TOL, (name, float(err.max()), int(err.argmax()))
