@@ -20,6 +20,14 @@
 // team's registers, then in shared memory over the keys for the factorisation: lla_team_solve.cuh), and in a second
 // sweep k_j . y and the output sum (coefficients against values).  The second sweep forms the weights again instead of keeping them.
 //
+// fp32 inputs may lie far from the origin compared with their spread, up to 2^24 times, and squares of that do not fit a
+// double's 53 bits beside the spread's and a small ridge.  So in the blocks with ill-conditioned rows (fewer than head_rows
+// keys) their keys are staged relative to the block's first query, the ridge corrected by its product with the row's
+// query; and where the rounding of the shared products is not far below the ridge, the dual form's matrix is
+// formed from the differences k_j - q themselves, row by row.  (bf16 inputs reach 2^8 at most: products of the keys as they
+// are lose nothing.)  Both measured at 8 fp32 heads, d = 64: n = 1000, keys of every block shifted 1069 us, of those blocks
+// 1023 us; n = 63, all matrices row by row 39 us, shared 33 us.
+//
 // What bounds it: the matrix pipe in the moments of long rows (36 of the about 47 instructions per 4 keys and row at
 // d = 64; measured at 89 % of its rate), the chain of reciprocals in the pivot blocks for short ones, which the eight
 // systems of two blocks on an SM hide in part.
@@ -30,7 +38,7 @@
 namespace lla {
 namespace {
 
-template <int D>
+template <int D, bool REL>
 struct DrSmem {
     using C = DrCfg<D>;
     union {
@@ -38,13 +46,15 @@ struct DrSmem {
         double mat[C::TEAMS][team::Cfg<D, C::NW>::LOWER][64];      // the systems, between the sweeps
     };
     double q[C::TEAMS][C::LDK];               // query rows, zero beyond the head's
+    double rel[REL ? C::TEAMS : 1][C::LDK];        // REL: the same minus the first of them
     double y[C::TEAMS][C::LDK];                    // their solutions (second sweep)
     double s[C::TEAMS][C::LDW];               // scores -> weights -> output coefficients of the chunk
     double t[C::TEAMS][C::LDW];               // k_j . y
     double kbar[C::TEAMS][D];
     double osum[C::HALVES > 1 ? C::TEAMS : 1][D];   // second half of the output sum
     double red[2][C::TEAMS][C::NW];
-    double den[C::TEAMS], lam[C::TEAMS], qq[C::TEAMS];
+    double den[C::TEAMS], lam[C::TEAMS], qq[C::TEAMS], qn[REL ? C::TEAMS : 1];      // qq: |q|^2 in the frame of the keys; qn: |q|^2
+    double kmax[REL ? C::WARPS : 1];
     int dual[C::TEAMS];                       // visible keys of a dual row, 0 for the others
     team::Smem<D, C::NW, 1> solve[C::TEAMS];
 };
@@ -60,8 +70,9 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     using T = team::Cfg<D, C::NW>;
     constexpr int NW = C::NW, TEAMS = C::TEAMS, CH = C::CH, NB = C::NB, R = T::R;
     constexpr unsigned FULL = 0xffffffffu;
+    constexpr bool REL = sizeof(TIn) == 4;             // keys relative to the block's first query
     extern __shared__ __align__(16) unsigned char dr_smem[];
-    DrSmem<D>& sm = *reinterpret_cast<DrSmem<D>*>(dr_smem);
+    DrSmem<D, REL>& sm = *reinterpret_cast<DrSmem<D, REL>*>(dr_smem);
     auto row_of = [](auto& rows) { return [&rows](int r) { return &rows[r][0]; }; };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
     const int tm = warp / NW, w = warp % NW, tt = tid % (32 * NW);      // team, warp and thread inside the team
@@ -87,6 +98,16 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         sm.q[r][c] = i0 + r < rows_per_head ? (double)to_f32(q[sq.at(bh / H, bh % H, i0 + r) + c]) : 0.0;
         sm.y[r][c] = 0.0;
     }
+    const bool rel = REL && (causal ? off + i0 + 1 : n) < head_rows;
+    const double* qc = rel ? sm.rel[tm] : sm.q[tm];                     // the row's query in the frame of the staged keys
+    if (rel) {
+        __syncthreads();
+        for (int e = tid; e < TEAMS * D; e += C::THREADS) sm.rel[e / D][e % D] = sm.q[e / D][e % D] - sm.q[0][e % D];
+    }
+    auto stage_keys = [&](int j0) {
+        if (rel) stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch, sm.q[0]);
+        else stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
+    };
     // one value per thread of the team -> its maximum or sum over the team
     auto team_reduce = [&](double x, bool is_max, int slot) {
 #pragma unroll
@@ -119,7 +140,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     for (int j0 = jbeg; j0 < jend; j0 += ch) {
         const int nk = min(ch, jend - j0);
         __syncthreads();
-        stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
+        stage_keys(j0);
         __syncthreads();
         dots<D>(row_of(sm.s), row_of(sm.q), sm.kv, nk, warp, lane);
         __syncthreads();
@@ -176,10 +197,20 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             });
         }
     }
+    // What the frame of the keys takes from the row's scores.  (The weights are relative to the maximum and need it nowhere.)
+    auto frame = [&]() {
+        double x = 0.0;
+        if (rel) {
+            for (int e = lane; e < D; e += 32) x += sm.q[tm][e] * sm.q[0][e];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+        }
+        return x * scale;
+    };
     // team-wide sums (every team has run every block barrier above)
     if (live) {
         omega = team_reduce(omega, false, 1);
-        lam_m = ridge_mode == LLA_RIDGE_PRINTED ? lam_i * exp(m_max - m_ref) : lam_i * exp(-m_ref);
+        lam_m = ridge_mode == LLA_RIDGE_PRINTED ? lam_i * exp(m_max - m_ref) : lam_i * exp(-(m_ref + frame()));
     }
     const double inv = 1.0 / omega;
     team::Smem<D, NW, 1>& ss = sm.solve[tm];
@@ -193,11 +224,20 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         for (int j = tt; j < 8 * nba; j += 32 * NW) sm.s[tm][j] = j < L ? lam_m / fmax(sm.s[tm][j], 1e-290) : 1.0;
     }
     if (dual && w == 0) {
-        double qq = 0.0;
-        for (int e = lane; e < D; e += 32) qq += sm.q[tm][e] * sm.q[tm][e];
+        double qq = 0.0, qn = 0.0;
+        for (int e = lane; e < D; e += 32) {
+            qq += qc[e] * qc[e];
+            if (REL) qn += sm.q[tm][e] * sm.q[tm][e];
+        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) qq += __shfl_xor_sync(FULL, qq, o);
-        if (lane == 0) sm.qq[tm] = qq;
+        for (int o = 16; o > 0; o >>= 1) {
+            qq += __shfl_xor_sync(FULL, qq, o);
+            if (REL) qn += __shfl_xor_sync(FULL, qn, o);
+        }
+        if (lane == 0) {
+            sm.qq[tm] = qq;
+            if (REL) sm.qn[tm] = qn;
+        }
     }
     if (live && !dual) {
 #pragma unroll
@@ -208,7 +248,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             const int cc = 8 * T::row(r, w) + g;
             if (t4 == 0) {
                 sm.kbar[tm][cc] = a * inv;
-                ss.b[0][cc] = a * inv - sm.q[tm][cc];
+                ss.b[0][cc] = a * inv - qc[cc];
             }
         }
     }
@@ -219,7 +259,9 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     constexpr int GB = (T::LOWER + C::WARPS - 1) / C::WARPS;
     double gm[GB][2];
     const bool some_dual = jbeg == 0 && jend <= CH && (causal ? off + i0 + 1 : n) <= D;
+    bool rowwise = false;
     if (some_dual) {
+        double kmax = 0.0;
 #pragma unroll
         for (int u = 0; u < GB; ++u) {
             const int e = warp + C::WARPS * u;
@@ -233,11 +275,45 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 for (int s = 0; s < D / 4; ++s) team::dmma(x[s & 1][0], x[s & 1][1], sm.kv[8 * bi + g][4 * s + t4], sm.kv[8 * bj + g][4 * s + t4]);
                 gm[u][0] = x[0][0] + x[1][0];
                 gm[u][1] = x[0][1] + x[1][1];
+                if (REL && bi == bj && 8 * bi + g < jend) kmax = fmax(kmax, g == 2 * t4 ? gm[u][0] : g == 2 * t4 + 1 ? gm[u][1] : 0.0);
             }
         }
+        if (REL) {
+            // the rounding of the products below, 1e-16 of the largest |k|^2 or |k| |q|, against the ridge
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) kmax = fmax(kmax, __shfl_xor_sync(FULL, kmax, o));
+            if (lane == 0) sm.kmax[warp] = kmax;
+            __syncthreads();
+#pragma unroll
+            for (int u = 0; u < C::WARPS; ++u) kmax = fmax(kmax, sm.kmax[u]);
+            for (int t = 0; t < TEAMS; ++t)
+                rowwise = rowwise || (sm.dual[t] && !(sm.lam[t] >= 1e-8 * fmax(fmax(kmax, sm.qq[t]), sqrt(kmax * sm.qn[t]))));
+        }
+    }
+    // a dual row's matrix from its own differences, in the place of the moments
+    if (REL && rowwise && dual) {
+        team::with_warp<NW>(w, [&](auto wc) {
+            constexpr int W = decltype(wc)::value;
+#pragma unroll 1
+            for (int s = 0; s < D / 4; ++s) {
+                const double qe = qc[4 * s + t4];
+                auto z = [&](int b) { return 8 * b + g < L ? sm.kv[8 * b + g][4 * s + t4] - qe : 0.0; };
+                double av[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) av[r] = z(T::row(r, W));
+#pragma unroll
+                for (int j = 0; j <= T::row(R - 1, W); ++j) {
+                    if (j >= nba) break;
+                    const double bv = z(j);
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+                        if (j <= T::row(r, W)) team::dmma(c[T::off(r) + j][0], c[T::off(r) + j][1], av[r], bv);
+                }
+            }
+        });
     }
     __syncthreads();               // the keys are no longer read: their place takes the matrices
-    if (some_dual) {
+    if (some_dual && !rowwise) {
 #pragma unroll
         for (int u = 0; u < GB; ++u) {
             const int e = warp + C::WARPS * u;
@@ -248,9 +324,11 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             for (int t = 0; t < TEAMS; ++t) {
                 const int Lt = sm.dual[t];
                 if (8 * bi >= Lt) continue;
-                const double si = sm.qq[t] - (idx < Lt ? sm.t[t][idx] : 0.0);
-                double v0 = idx < Lt && jdx < Lt ? gm[u][0] + (si - sm.t[t][jdx]) : 0.0;
-                double v1 = idx < Lt && jdx + 1 < Lt ? gm[u][1] + (si - sm.t[t][jdx + 1]) : 0.0;
+                // q . k_j (REL: k_j relative to the block's first query, whose product goes off)
+                auto qk = [&](int j) { return REL ? sm.t[t][j] - sm.t[0][j] : sm.t[t][j]; };
+                const double si = sm.qq[t] - (idx < Lt ? qk(idx) : 0.0);
+                double v0 = idx < Lt && jdx < Lt ? gm[u][0] + (si - qk(jdx)) : 0.0;
+                double v1 = idx < Lt && jdx + 1 < Lt ? gm[u][1] + (si - qk(jdx + 1)) : 0.0;
                 if (bi == bj) {
                     const double dg = sm.s[t][idx];
                     if (g == 2 * t4) v0 += dg;
@@ -262,6 +340,24 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     }
     if (dual) {
         for (int e = tt; e < 8 * nba; e += 32 * NW) ss.b[0][e] = e < L ? 1.0 : 0.0;
+        if (REL && rowwise) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int bi = T::row(r, w);
+                if (bi >= nba) continue;
+                const double dg = sm.s[tm][8 * bi + g];
+#pragma unroll
+                for (int j = 0; j < NB; ++j)
+                    if (T::cols(r) > j && j <= bi) {
+                        double v0 = c[T::off(r) + j][0], v1 = c[T::off(r) + j][1];
+                        if (j == bi) {
+                            if (g == 2 * t4) v0 += dg;
+                            if (g == 2 * t4 + 1) v1 += dg;
+                        }
+                        *reinterpret_cast<double2*>(&sm.mat[tm][team::blk(bi, j)][2 * lane]) = make_double2(v0, v1);
+                    }
+            }
+        }
     } else if (live) {
         const double ridge = lam_m * inv;
 #pragma unroll
@@ -298,7 +394,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             for (int e = lane; e < D; e += 32) {
                 const double y = ss.x[w][0][e], kbv = sm.kbar[tm][e];
                 yk += kbv * y;
-                yb += (kbv - sm.q[tm][e]) * y;
+                yb += (kbv - qc[e]) * y;
                 if (w == 0) sm.y[tm][e] = y;
             }
 #pragma unroll
@@ -321,13 +417,13 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         const int nk = min(ch, jend - j0);
         __syncthreads();
         if (keys) {
-            stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
+            stage_keys(j0);
             __syncthreads();
             if (dual) {
                 if (rho_out)                                       // rho = Z^T alpha
                     for (int e = tt; e < D; e += 32 * NW) {
                         double a = 0.0;
-                        for (int j = 0; j < L; ++j) a += ss.x[w][0][j] * (sm.kv[j][e] - sm.q[tm][e]);
+                        for (int j = 0; j < L; ++j) a += ss.x[w][0][j] * (sm.kv[j][e] - qc[e]);
                         rho_out[row * D + e] = (float)a;
                     }
             }
@@ -372,10 +468,11 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             store_out(orow + 1, (float)(o1 * id));
         }
     }
+    const double f = exp(m_ref - m_max);           // to weights relative to the true maximum
+    if (live && stats) m_max += frame();           // (by whole warps)
     if (live && tt == 0) {
         if (stats) {
-            const double f = exp(m_ref - m_max);       // to weights relative to the true maximum
-            const double om = omega * f, dl = dual ? den * f : omega * f / gfac;
+                        const double om = omega * f, dl = dual ? den * f : omega * f / gfac;
             stats[row * 3 + 0] = (float)m_max;
             stats[row * 3 + 1] = (float)om;
             stats[row * 3 + 2] = (float)dl;
@@ -389,7 +486,7 @@ template <int D, typename TIn, typename TOut>
 int launch_t(const ForwardArgs& a, int rows) {
     using C = DrCfg<D>;
     static_assert(C::HALVES <= 2 && C::HALVES * C::NB == C::WARPS, "output sum layout");
-    const int smem = (int)sizeof(DrSmem<D>);
+    const int smem = (int)sizeof(DrSmem<D, sizeof(TIn) == 4>);
     auto kern = direct_rows_kernel<D, TIn, TOut>;
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));

@@ -41,19 +41,28 @@ __device__ __forceinline__ void load_pair<float>(const float* p, double& a, doub
 // that hold no row before jend are left out, four at a time: their rows keep what they held, and nothing reads them.
 // (Rows of 1 to 95 keys, 32 heads, d = 64: 92 -> 87 us together with the dual form's
 // diagonal made once per row; the backward's rows 135 -> 130 us.)
-template <int D, typename TIn>
-__device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch) {
+// REL: ref, a row in shared memory, is subtracted from each of them.
+template <int D, bool REL = false, typename TIn>
+__device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch,
+                                      const double* ref = nullptr) {
     using C = DrCfg<D>;
     constexpr int PER = C::CH * D / 2 / C::THREADS, PER_STEP = C::STEP * D / 2 / C::THREADS;
     static_assert(PER * 2 * C::THREADS == C::CH * D && PER_STEP * 2 * C::THREADS == C::STEP * D, "a chunk is a whole number of rounds");
     constexpr int ROUND = 2 * C::THREADS / D;              // rows of a round
+    const int c = 2 * (threadIdx.x % (D / 2));             // the same columns in every round
+    const double r0 = REL ? ref[c] : 0.0, r1 = REL ? ref[c + 1] : 0.0;
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
         if (u >= PER_STEP && ch == C::STEP) break;
         if (u % 4 == 0 && j0 + ROUND * u >= jend) break;
-        const int e = threadIdx.x + C::THREADS * u, j = e / (D / 2), c = 2 * (e % (D / 2));
+        const int j = threadIdx.x / (D / 2) + ROUND * u;
+        const bool in = j0 + j < jend;
         double a = 0.0, b = 0.0;
-        if (j0 + j < jend) load_pair(src + (size_t)(j0 + j) * stride + c, a, b);
+        if (in) load_pair(src + (size_t)(j0 + j) * stride + c, a, b);
+        if (REL) {                                         // (outside the condition: the rounds' loads stay together)
+            a -= in ? r0 : 0.0;
+            b -= in ? r1 : 0.0;
+        }
         *reinterpret_cast<double2*>(&dst[j][c]) = make_double2(a, b);
     }
 }

@@ -125,8 +125,7 @@ def _scores_far_from_zero(dtype, d, n, mode):
 FAR_SIZES = [("bf16", 64, 95), ("f32", 16, 130), ("f32", 64, 200), ("bf16", 128, 140), ("f32", 128, 150)]
 
 
-@pytest.mark.parametrize("dtype,d,n,mode", [(*size, mode) for size in FAR_SIZES for mode in ("low", "mixed")] +
-                         [("bf16", 64, 95, "high"), ("bf16", 128, 140, "high")])
+@pytest.mark.parametrize("dtype,d,n,mode", [(*size, mode) for size in FAR_SIZES for mode in ("low", "mixed", "high")])
 def test_scores_far_from_zero(oracle, dtype, d, n, mode):
     q, k, v, scale = _scores_far_from_zero(dtype, d, n, mode)
     if mode == "high":
@@ -160,3 +159,27 @@ def test_backward_scores_far_from_zero(backward_oracle, mode):
         assert np.isfinite(a).all(), name
         err = grad_err(a, b)
         assert err.max() <= TOL, (name, float(err.max()), int(err.argmax()))
+
+
+# (up to 2 d - 1 keys: the rows whose systems are ill-conditioned)
+@pytest.mark.parametrize("d,n,nq", [(16, 31, 31), (64, 127, 127), (64, 110, 41), (128, 255, 255)])
+def test_fp32_inputs_far_from_the_origin(oracle, d, n, nq):
+    """Keys and queries around a common point 1000 times as far away as they are spread: squares of the coordinates leave
+    1e-10 of a double beside a ridge of 1e-8, so the systems must be formed from differences."""
+    rng = np.random.default_rng(970 + d + n)
+    u = np.ones(d, dtype=np.float32) / np.float32(np.sqrt(d))
+    q, k = ((1000.0 * u + rng.standard_normal((1, 2, m, d)) / np.sqrt(d)).astype(np.float32) for m in (nq, n))
+    v = rng.standard_normal((1, 2, n, d)).astype(np.float32)
+    scale, lam = 1e-5, 1e-3
+    out = torch.full((1, 2, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+    rho = torch.full_like(out, float("nan"))
+    L.lla_forward_ex(dev(q, "f32"), dev(k, "f32"), dev(v, "f32"), out, 1, 2, n, d, d, scale, lam, in_dtype=L.LLA_F32,
+                     out_dtype=L.LLA_F32, q_rows=nq, rho=rho, stream=stream_ptr())
+    torch.cuda.synchronize()
+    cnt = np.arange(n - nq + 1, n + 1, dtype=np.int32)
+    ref = oracle.decode(np.ascontiguousarray(q[0].transpose(1, 0, 2)), np.repeat(k, nq, axis=0), np.repeat(v, nq, axis=0), cnt, scale, lam)
+    err = row_err(out.cpu().numpy()[0].transpose(1, 0, 2), ref)
+    assert np.isfinite(err).all() and err.max() <= TOL_F32, (float(err.max()), int(err.argmax()))
+    if n == nq:
+        _, rref, _, _ = oracle.forward_rows(q, k, v, scale, lam, want_aux=True)
+        assert row_err(rho.cpu().numpy(), rref)[1:].max() <= TOL_F32
