@@ -229,7 +229,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     // 16-bit format).  The values of the copies equal the bf16 inputs (the pre-pass checks the range).  Every role
     // counts the CG sweeps it has seen, so all of them know a sweep's format, and the next one's, without being
     // told.  (Tiles whose rows see fewer than 8 D keys converge more slowly and keep the pairs for longer.)
-    const int precise = off + r0p + TC_BR <= 8 * D ? prm.precise_iters_early : prm.precise_iters;
+    // (A tile of several heads' rows goes by the earliest position in it, at the tiles that a head's rows are cut into
+    //  when it is alone: packing heads never takes iterations with pairs from a row.)
+    const int first_pos = off + (wraps ? 0 : r0p / TC_BR * TC_BR);
+    const int precise = first_pos + TC_BR <= 8 * D ? prm.precise_iters_early : prm.precise_iters;
     const bool f16_on = prm.f16_ok && *prm.f16_ok && precise < (1 << 29);
     const long long wcap = prm.wait_clocks;
 
