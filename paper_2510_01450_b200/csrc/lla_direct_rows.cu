@@ -508,6 +508,8 @@ int launch_d(const ForwardArgs& a, int rows) {
 
 }  // namespace
 
+constexpr int kMaxRowBlocks = 65535;      // blocks of rows in the second dimension of the grid
+
 int direct_rows_below(const ForwardArgs& a) { return std::max(a.head_rows, a.direct_below); }
 
 // Direct or fp32 conjugate gradients (lla_forward_simt.cu), for problems that the tensor-core kernel does not take.  A row
@@ -518,11 +520,13 @@ int direct_rows_below(const ForwardArgs& a) { return std::max(a.head_rows, a.dir
 //     d = 16:  0.0067 L + 0.5  0.0056 L + 7.4   equal at 6300 keys  (16 heads, n = 8000: 23 ms direct, 26 ms)
 // But conjugate gradients are as slow as their longest block, which takes its rows through all sweeps alone (2 heads, n =
 // 2000, d = 128: 4.1 ms direct, 5.5 ms): the rows from that line on go there only if the whole call is shorter for it.
+// (And with a window, which keeps the keys few however long the sequence, those that a launch has no blocks left for.)
 int direct_rows_worthwhile(const ForwardArgs& a) {
     const double kd = a.d == 128 ? 0.137 : a.d == 64 ? 0.031 : 0.0067, c0 = a.d == 128 ? 10.0 : a.d == 64 ? 2.5 : 0.5;
     const double ks = a.d == 128 ? 0.0575 : a.d == 64 ? 0.0194 : 0.0056, s0 = a.d == 128 ? 50.0 : a.d == 64 ? 35.0 : 7.4;
     const int block_rows = a.d == 128 ? 32 : 64, off = a.n - a.nq;
-    const int all = a.n + 1;
+    const long long room = off + kMaxRowBlocks * (a.d == 128 ? DrCfg<128>::TEAMS : a.d == 64 ? DrCfg<64>::TEAMS : DrCfg<16>::TEAMS) + 1ll;
+    const int all = (int)std::min<long long>(a.n + 1, room);
     auto seen = [&](int pos) { return (double)(!a.causal ? a.n : a.window > 0 ? std::min(pos, a.window) : pos); };
     auto direct = [&](double L) { return kd * L + c0; };
     auto iterative = [&](double L) { return ks * L + s0; };

@@ -183,3 +183,28 @@ def test_fp32_inputs_far_from_the_origin(oracle, d, n, nq):
     if n == nq:
         _, rref, _, _ = oracle.forward_rows(q, k, v, scale, lam, want_aux=True)
         assert row_err(rho.cpu().numpy(), rref)[1:].max() <= TOL_F32
+
+
+# more blocks of rows than the second dimension of a grid holds (65535 blocks of four rows, two at d = 128)
+@pytest.mark.parametrize("d,n,window", [(16, 262200, 64), (128, 131100, 384)])
+def test_long_windowed_sequences(oracle, d, n, window):
+    rng = np.random.default_rng(980 + d)
+    q, k, v = (rng.standard_normal((1, 1, n, d), dtype=np.float32) / np.float32(s) for s in (d ** 0.5, d ** 0.5, 1.0))
+    out = torch.full((1, 1, n, d), float("nan"), dtype=torch.float32, device="cuda")
+    iters = torch.full((1, 1, n), -7, dtype=torch.int32, device="cuda")
+    scale, lam = d ** -0.5, 1e-3
+    L.lla_forward_ex(dev(q, "f32"), dev(k, "f32"), dev(v, "f32"), out, 1, 1, n, d, d, scale, lam, in_dtype=L.LLA_F32,
+                     out_dtype=L.LLA_F32, window=window, iters=iters, stream=stream_ptr())
+    torch.cuda.synchronize()
+    assert torch.isfinite(out).all()
+    last = 65535 * (2 if d == 128 else 4)
+    assert (iters[0, 0, 2 * d:last] == 0).all() and (iters[0, 0, last:] > 0).all()
+    rows = np.unique(np.concatenate([np.arange(4), [last - 1, last, last + 1], rng.integers(0, n, 30), [n - 2, n - 1]]))
+    lo = np.maximum(0, rows + 1 - window)
+    cnt = (rows + 1 - lo).astype(np.int32)
+    kc, vc = (np.zeros((len(rows), 1, window, d), dtype=np.float32) for _ in range(2))
+    for s, (r, l, c) in enumerate(zip(rows, lo, cnt)):
+        kc[s, 0, :c], vc[s, 0, :c] = k[0, 0, l:r + 1], v[0, 0, l:r + 1]
+    ref = oracle.decode(np.ascontiguousarray(q[0, :, rows].reshape(len(rows), 1, d)), kc, vc, cnt, scale, lam)
+    err = row_err(out.cpu().numpy()[0, 0, rows], ref)
+    assert err.max() <= TOL_F32, (float(err.max()), int(err.argmax()))
