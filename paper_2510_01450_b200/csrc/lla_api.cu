@@ -334,6 +334,8 @@ int lla_decode_ex(const lla_decode_params* p) {
             a.workspace = mem; a.workspace_bytes = need;
         }
     }
+    const int refused = lla::decode_refusal(a);
+    if (refused != LLA_OK) return refused;
     if (a.status) LLA_CUDA_TRY(cudaMemsetAsync(a.status, 0, sizeof(int) * LLA_STATUS_WORDS, a.stream));
     // The units with short caches go to the direct kernel, which writes rows of `out` nobody else writes and returns
     // at once for every other unit.  It goes first and the streaming kernel is its programmatic dependent, so the two

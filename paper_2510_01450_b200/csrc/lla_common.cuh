@@ -242,6 +242,8 @@ size_t precond_minv_bytes(int units, int n, int d);     // the fp16 matrices [un
 int launch_precond(const void* k, int B, int Hk, Strides sk, int n, int d, float lambda, int window, void* gram, void* minv,
                    cudaStream_t st);
 int launch_decode(const DecodeArgs& a);
+int decode_refusal(const DecodeArgs& a);       // the status with which launch_decode refuses the call (before the first launch)
+constexpr int kDecodeMaxSplits = 64;           // parts of a (sequence, head) that the tensor-core path merges
 int launch_head_rows_decode(const DecodeArgs& a);
 bool decode_records_fit(const DecodeArgs& a);
 bool decode_tensor_supported(const DecodeArgs& a);

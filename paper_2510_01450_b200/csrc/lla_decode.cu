@@ -265,6 +265,12 @@ decode_combine_kernel(const TIn* __restrict__ q, const float* __restrict__ parts
                     out + (size_t)bh * D, status);
 }
 
+// The tensor-core path keeps its moments relative to the first tile's maximum, not the true one,
+// which the printed ridge variant is defined against: that variant runs on the kernels above.
+bool on_tensor_cores(const DecodeArgs& a) {
+    return a.impl != LLA_IMPL_SIMT && a.ridge_mode == LLA_RIDGE_DEFINITION && decode_tensor_supported(a);
+}
+
 template <int D>
 constexpr size_t decode_smem_bytes() {
     const size_t stream = sizeof(float) * (2 * (size_t)DC_BK * D + DC_BK + D);
@@ -276,18 +282,10 @@ template <int D, typename TIn, typename TOut>
 int launch_t(const DecodeArgs& a) {
     const int splits = a.splits < 1 ? 1 : a.splits;
     const size_t smem = decode_smem_bytes<D>();
-    if (splits > 1) {
-        const size_t need = decode_workspace_bytes(a.B, a.H, a.d, a.dv, splits);
-        if (!a.workspace || a.workspace_bytes < need) return LLA_ERR_WORKSPACE;
-    }
-    // The tensor-core path keeps its moments relative to the first tile's maximum, not the true one,
-    // which the printed ridge variant is defined against: that variant runs on the kernels below.
-    if (a.impl == LLA_IMPL_TENSOR && a.ridge_mode == LLA_RIDGE_PRINTED) return LLA_ERR_UNSUPPORTED;
-    if (a.impl != LLA_IMPL_SIMT && a.ridge_mode == LLA_RIDGE_DEFINITION && decode_tensor_supported(a)) {
+    if (on_tensor_cores(a)) {
         // tensor-core path: streaming kernel plus its own solve kernel (or fused epilogue)
         return launch_decode_tensor_moments(a);
     } else {
-        if (a.impl == LLA_IMPL_TENSOR) return LLA_ERR_UNSUPPORTED;
         auto k1 = decode_moments_kernel<D, TIn, TOut>;
         LLA_CUDA_TRY(cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         dim3 grid(splits, a.B * a.H);
@@ -326,6 +324,14 @@ size_t decode_workspace_bytes(int B, int H, int d, int dv, int splits) {
     if (splits <= 1) return 0;
     (void)dv;
     return sizeof(float) * (size_t)B * H * splits * (2 * (size_t)d * d + 2 * d + 4);
+}
+
+int decode_refusal(const DecodeArgs& a) {
+    if (a.splits > 1 && (!a.workspace || a.workspace_bytes < decode_workspace_bytes(a.B, a.H, a.d, a.dv, a.splits))) return LLA_ERR_WORKSPACE;
+    const bool tensor = on_tensor_cores(a);
+    if (a.impl == LLA_IMPL_TENSOR && !tensor) return LLA_ERR_UNSUPPORTED;
+    if (tensor && a.d == 64 && a.splits > kDecodeMaxSplits) return LLA_ERR_INVALID_ARG;      // (at d = 128 the call runs with as many as that)
+    return LLA_OK;
 }
 
 int launch_decode(const DecodeArgs& a) {
@@ -405,7 +411,8 @@ extern "C" int lla_decode_noalloc(const void* q, const void* kcache, const void*
         a.workspace = scratch;
         a.workspace_bytes = LLA_NOALLOC_SCRATCH_BYTES;
     }
-    const int st = lla::launch_head_rows_decode(a);
+    int st = lla::decode_refusal(a);
+    if (st == LLA_OK) st = lla::launch_head_rows_decode(a);
     if (st != LLA_OK) return st;
     a.behind_direct = true;
     return lla::launch_decode(a);

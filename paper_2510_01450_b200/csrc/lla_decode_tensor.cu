@@ -110,7 +110,6 @@ struct SvCfg {
     // d = 128: where the error of the fp32 moments stands.
     static constexpr double TOL = D == 64 ? 1e-4 : 1e-6;
 };
-constexpr int DS_MAX_SPLITS = 64;
 template <int D>
 struct alignas(16) SolveSmem {
     float p[D];                              // vector of the current product, fp32
@@ -850,7 +849,7 @@ template <int D>
 __global__ void __launch_bounds__(DM_THREADS)
 decode_merge_kernel(float* __restrict__ parts, const int* __restrict__ lens, int H, int Lmax, int head_rows, int splits, int window) {
     constexpr int PF = DtCfg<D>::REC;
-    __shared__ float s_f[DS_MAX_SPLITS];
+    __shared__ float s_f[kDecodeMaxSplits];
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
     asm volatile("griddepcontrol.wait;" ::: "memory");      // a programmatic dependent of the streaming kernel
     if (visible_keys(lens[bh / H], Lmax, window) < head_rows) return;
@@ -896,10 +895,9 @@ decode_solve_kernel(const __nv_bfloat16* __restrict__ q, const float* __restrict
 template <int D, typename TOut>
 int launch_t(const DecodeArgs& a) {
     using C = DtCfg<D>;
-    const int splits = a.splits < 1 ? 1 : a.splits;
+    const int splits = a.splits < 1 ? 1 : a.splits > kDecodeMaxSplits ? kDecodeMaxSplits : a.splits;
     const bool have_ws = decode_records_fit(a);
     if ((splits > 1 || D == 128) && !have_ws) return LLA_ERR_WORKSPACE;
-    if (splits > DS_MAX_SPLITS) return LLA_ERR_INVALID_ARG;
     CUtensorMap mk, mv;
     const int BH = a.B * a.H;
     const int kvg = a.kv_group > 0 ? a.kv_group : 1;

@@ -111,3 +111,35 @@ def test_query_at_the_weighted_key_mean(oracle, d, mode):
         torch.cuda.synchronize()
         err = row_err(out.cpu().numpy(), ref)
         assert np.isfinite(err).all() and err.max() <= TOL_BF16, (float(err.max()), int(err.argmax()))
+
+
+def test_more_parts_than_the_merge_takes(oracle):
+    """More than 64 parts: at d = 128 the call runs (with a caller's buffer and with the library's), at d = 64 it is refused
+    before anything has been launched."""
+    B, H, n, splits = 1, 2, 6000, 80
+    for d in (128, 64):
+        w = inputs.CONFIGS[5].shrink(B=B, H=H, n=n, d=d, dv=d, len_min=n, len_max=n, seed=440 + d)
+        q, kc, vc, lens = inputs.make_decode(w)
+        lens = np.array([n if d == 128 else 2 * d - 1], dtype=np.int32)
+        args = [dev(q, "bf16"), dev(kc, "bf16"), dev(vc, "bf16"), torch.from_numpy(lens).cuda()]
+        nbytes = L.lla_decode_workspace_bytes(B, H, n, d, d, L.LLA_BF16, splits)
+        ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+
+        def run(call, **kw):
+            out = torch.full((B, H, d), float("nan"), dtype=torch.float32, device="cuda")
+            try:
+                call(*args, out, B, H, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, splits=splits, stream=stream_ptr(), **kw)
+                status = 0
+            except L.LlaError as e:
+                status = e.status
+            torch.cuda.synchronize()
+            return status, out.cpu().numpy()
+
+        for call, kw in ((L.lla_decode_ex, dict(workspace=ws, workspace_bytes=nbytes)), (L.lla_decode_noalloc, {})):
+            status, got = run(call, **kw)
+            if d == 128:
+                assert status == 0
+                err = row_err(got, oracle.decode(q, kc, vc, lens, w.scale, w.lam))
+                assert err.max() <= TOL_BF16, float(err.max())
+            else:
+                assert status == 1 and np.isnan(got).all()          # invalid argument, and no kernel has written
