@@ -240,8 +240,10 @@ int lla_forward_ex(const lla_forward_params *p);
  *               is optional: given one, the tensor-core path (bf16, d = dv = 64 or 128) writes each
  *               (sequence, head)'s moments there and solves in a second kernel, which is faster
  *               than solving at the end of the streaming kernel; the result is the same.  At
- *               d = 128 it needs 4 B H (2 d^2 + 2 d + 4) bytes for that; without them the call takes
- *               them from the stream-ordered pool (as lla_decode does; see the note on it below).
+ *               d = 128 it needs 4 B H (2 d^2 + 2 d + 4) bytes for that (lla_decode_workspace_bytes answers 0
+ *               there): given them, the call allocates nothing.  Without them it takes them from a stream-ordered
+ *               pool of the library's own, which keeps at most 128 MB between calls, or, while `stream` is
+ *               captured, solves at the end of the streaming kernel and allocates nothing either.
  */
 typedef struct lla_decode_params {
     const void *q, *kcache, *vcache;
@@ -286,8 +288,8 @@ int lla_decode_ex(const lla_decode_params *p);
  * buffers); `stream` is joined with them before the call returns.
  * lla_decode_host reads lens[] on the host and uploads only the first lens[b] rows of every
  * (sequence, head) cache.
- * Side effect on the process: the entry points that take scratch from the pool (these two, lla_forward,
- * lla_decode and lla_decode_ex at d = 128 without room for its records) set the release threshold of the current device's DEFAULT stream-ordered memory pool to
+ * Side effect on the process: the entry points that take scratch from the pool (these two, lla_forward and
+ * lla_decode) set the release threshold of the current device's DEFAULT stream-ordered memory pool to
  * "keep everything", once per device, so that repeated calls do not return their scratch to the driver.
  * A host program that trims that pool itself should use the _ex forms with its own workspace instead.
  */

@@ -22,8 +22,7 @@
 // m_ref is the maximum of the first tile.  The threads only note whether a later score exceeds it by more
 // than 2^90 (no check per tile across threads); if one did, the whole pass is repeated with the true maximum, which
 // is known by then (never triggered by bounded scores, covered by a test).  After the last tile the moments go to
-// the workspace as a record for the solve kernel, or, without a workspace (d = 64), to shared memory and are solved
-// on the spot.
+// the workspace as a record for the solve kernel, or, without one, to shared memory and are solved on the spot.
 #include "lla_sm100.cuh"
 
 namespace lla {
@@ -319,7 +318,7 @@ struct DtParams {
     int B, H, Lmax, splits, head_rows;
     float scale, lambda;
     const int* lens;
-    float* parts;        // moment records; null: solve in the epilogue (d = 64, one part)
+    float* parts;        // moment records; null: solve in the epilogue (one part)
     int* status;
     const float* lambda_units;   // optional per-(sequence, head) ridge
     int ridge_mode;
@@ -829,15 +828,13 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C::TMEM) : "memory");
     }
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    if constexpr (D == 64) {
-        if (prm.parts || tid >= D) return;
-        // no workspace, one part: solve here
-        static_assert(8192 + 4 * C::REC <= C::SM_BAR, "the record does not fit");
-        __shared__ SolveSmem<D> sm;
-        __shared__ double prow[D + 1];
-        solve_here<D>(q + (size_t)bh * D, s_rec, prm.lambda_units ? prm.lambda_units[bh] : prm.lambda, prm.ridge_mode,
-                      out + (size_t)bh * D, prm.status, sm, prow);
-    }
+    if (prm.parts || tid >= D) return;
+    // no workspace, one part: solve here
+    static_assert(8192 + 4 * C::REC <= C::SM_BAR, "the record does not fit");
+    __shared__ SolveSmem<D> sm;
+    __shared__ double prow[D + 1];
+    solve_here<D>(q + (size_t)bh * D, s_rec, prm.lambda_units ? prm.lambda_units[bh] : prm.lambda, prm.ridge_mode,
+                  out + (size_t)bh * D, prm.status, sm, prow);
 }
 
 // Sum of the parts' moments of one unit into the record of its first part, each scaled to the largest of their maxima
@@ -897,7 +894,7 @@ int launch_t(const DecodeArgs& a) {
     using C = DtCfg<D>;
     const int splits = a.splits < 1 ? 1 : a.splits > kDecodeMaxSplits ? kDecodeMaxSplits : a.splits;
     const bool have_ws = decode_records_fit(a);
-    if ((splits > 1 || D == 128) && !have_ws) return LLA_ERR_WORKSPACE;
+    if (splits > 1 && !have_ws) return LLA_ERR_WORKSPACE;
     CUtensorMap mk, mv;
     const int BH = a.B * a.H;
     const int kvg = a.kv_group > 0 ? a.kv_group : 1;
@@ -970,15 +967,12 @@ bool decode_records_fit(const DecodeArgs& a) {
     return a.workspace && ((uintptr_t)a.workspace & 15u) == 0 && a.workspace_bytes >= decode_record_bytes(a.B, a.H, a.d, a.dv, a.splits);
 }
 
-// d = 128 has no room to solve in the streaming kernel's epilogue: it needs the record buffer.
 bool decode_tensor_supported(const DecodeArgs& a) {
-    if (a.in_dtype != LLA_BF16 || a.d != a.dv || sm100::get_encode() == nullptr) return false;
-    return a.d == 64 || (a.d == 128 && decode_records_fit(a));
+    return a.in_dtype == LLA_BF16 && a.d == a.dv && (a.d == 64 || a.d == 128) && sm100::get_encode() != nullptr;
 }
 
-// Tensor-core decode.  With a record buffer (always for splits > 1 and for d = 128, optional for a single part at
-// d = 64) the streaming kernel writes moment records and a solve kernel follows; without one, single-part
-// blocks solve in their own epilogue.
+// Tensor-core decode.  With a record buffer (always for splits > 1, optional for a single part) the streaming kernel writes
+// moment records and a solve kernel follows; without one, single-part blocks solve in their own epilogue.
 int launch_decode_tensor_moments(const DecodeArgs& a) {
     if (!decode_tensor_supported(a)) return LLA_ERR_UNSUPPORTED;
     return a.d == 64 ? launch_d<64>(a) : launch_d<128>(a);

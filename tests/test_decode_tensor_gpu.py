@@ -1,12 +1,17 @@
 """The decode's tensor-core streaming kernel (bf16, d = 64 and 128) at the edges of its tiles of 64 keys, with the options
 that change which rows a tile reads, with short caches beside long ones, and with a first tile whose maximum is useless
 as the reference of the weights.  Tolerances are those of the other bf16 parity tests on an fp32 output buffer."""
+import ctypes
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
 
 from paper_2510_01450_b200 import binding as L, inputs
+from tests.conftest import ROOT
 from tests.gpu_util import dev, row_err, stream_ptr
 from tests.test_parity_gpu import TOL_BF16, _to_pages
 
@@ -143,3 +148,57 @@ def test_more_parts_than_the_merge_takes(oracle):
                 assert err.max() <= TOL_BF16, float(err.max())
             else:
                 assert status == 1 and np.isnan(got).all()          # invalid argument, and no kernel has written
+
+
+def _decode_d128(seed):
+    B, H, n, d = 4, 4, 1100, 128
+    w = inputs.CONFIGS[5].shrink(B=B, H=H, n=n, d=d, dv=d, len_min=10, len_max=n, seed=seed)
+    q, kc, vc, _ = inputs.make_decode(w)
+    lens = np.array([100, 2 * d, 385, n], dtype=np.int32)
+    return w, (q, kc, vc, lens), [dev(q, "bf16"), dev(kc, "bf16"), dev(vc, "bf16"), torch.from_numpy(lens).cuda()]
+
+
+def test_captured_calls_allocate_nothing(oracle):
+    """d = 128 without a buffer for the records, captured: the graph holds no allocation (a clone of it can be made) and its
+    replays are right."""
+    w, (q, kc, vc, lens), args = _decode_d128(450)
+    d = w.d
+    ref = oracle.decode(q, kc, vc, lens, w.scale, w.lam)
+    for splits in (0, 1):
+        out = torch.empty((w.B, w.H, d), dtype=torch.float32, device="cuda")
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph):
+            L.lla_decode_ex(*args, out, w.B, w.H, w.n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, splits=splits, stream=stream_ptr())
+        cuda, clone = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p()
+        assert cuda.cuGraphClone(ctypes.byref(clone), ctypes.c_void_p(graph.raw_cuda_graph())) == 0
+        assert cuda.cuGraphDestroy(clone) == 0
+        for _ in range(3):
+            out.fill_(float("nan"))
+            graph.replay()
+            torch.cuda.synchronize()
+            err = row_err(out.cpu().numpy(), ref)
+            assert np.isfinite(err).all() and err.max() <= TOL_BF16, float(err.max())
+
+
+def test_the_default_pool_is_left_alone():
+    """d = 128 without a buffer for the records: they come from a pool of the library's own (in a process of its own, for
+    other entry points do set the default pool's threshold)."""
+    code = """
+import ctypes, torch
+from tests.test_decode_tensor_gpu import L, _decode_d128, stream_ptr
+w, _, args = _decode_d128(451)
+cuda, pool, value = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), ctypes.c_uint64(77)
+def threshold():
+    assert cuda.cuDeviceGetDefaultMemPool(ctypes.byref(pool), 0) == 0
+    assert cuda.cuMemPoolGetAttribute(pool, 4, ctypes.byref(value)) == 0
+    return value.value
+before = threshold()
+out = torch.empty((w.B, w.H, w.d), dtype=torch.float32, device="cuda")
+L.lla_decode_ex(*args, out, w.B, w.H, w.n, w.d, w.d, w.scale, w.lam, out_dtype=L.LLA_F32, stream=stream_ptr())
+torch.cuda.synchronize()
+print("thresholds", before, threshold())
+"""
+    res = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
+    _, before, after = res.stdout.split()[-3:]
+    assert before == after
