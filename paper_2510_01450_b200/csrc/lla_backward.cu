@@ -448,7 +448,7 @@ int launch_t(const BackwardArgs& a) {
     const int kvg = a.kv_group > 0 ? a.kv_group : 1;
     const long long kvrows = (long long)a.B * a.H * a.n / kvg; // rows of k, v, dk, dv
     if (a.workspace_bytes < ws_own_bytes(rows, D, BH) || !a.workspace) return LLA_ERR_WORKSPACE;
-    if (first > 0 && off + first > 2 * D) return LLA_ERR_UNSUPPORTED;      // (head_rows beyond 2 d + 1)
+    if (first > 0 && off + first > backward_rows_most_keys(D)) return LLA_ERR_UNSUPPORTED;      // (a very large head_rows)
     float* kbar = static_cast<float*>(a.workspace);
     float* hvec = kbar + rows * D;
     float* tvec = hvec + rows * D;

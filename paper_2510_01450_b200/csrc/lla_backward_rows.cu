@@ -9,6 +9,10 @@
 //     dK += DS^T Q + U^T Y + W^T T,   dV += A^T G
 // as products over the block's rows, so that a block adds to a gradient entry once instead of once per row.
 //
+// A row's weights and per-key coefficients stay in shared memory for its up to 2 d keys.  Where the caller raises head_rows
+// beyond that (LONG) only the weights and gamma do, in rows as long as needed, and e_j and f_j are formed a chunk of
+// keys at a time, e_j once more before for g . o_i.
+//
 // Measured on B200 against one block per row with a shared-memory LDL^T on the CUDA cores and one atomic per row and
 // entry: 32 heads, n = 1000, d = 64 (95 rows a head): 305 -> 130 us; 16 heads, d = 128 (191 rows): 3.5 -> 1.1 ms.
 #include "lla_rows.cuh"
@@ -16,7 +20,7 @@
 namespace lla {
 namespace {
 
-template <int D>
+template <int D, bool LONG>
 struct BrSmem {
     using C = DrCfg<D>;
     static constexpr int LMAX = 2 * D, LDL = LMAX + 4;             // most keys of a row, and a row stride of 4 mod 16
@@ -25,26 +29,29 @@ struct BrSmem {
         double mat[C::TEAMS][team::Cfg<D, C::NW>::LOWER][64];
     };
     double q[C::TEAMS][C::LDK], g[C::TEAMS][C::LDK];               // query rows and upstream gradients
-    double p[C::TEAMS][LDL];                                       // scores -> weights -> a_j
-    double gam[C::TEAMS][LDL];                                     // gamma_j -> scale dL/ds_j
+    double p[LONG ? 1 : C::TEAMS][LDL];                            // scores -> weights -> a_j              (LONG: these two
+    double gam[LONG ? 1 : C::TEAMS][LDL];                          // gamma_j -> scale dL/ds_j               lie behind the struct)
     double kbar[C::TEAMS][D];
     team::Smem<D, C::NW, 2> solve[C::TEAMS];                       // afterwards e_j and f_j lie over its first part
     double red[2][C::TEAMS][C::NW];
     static_assert(64 + D / 8 * 24 + 4 * D >= 2 * LDL, "e and f lie over the solver's w, piv, b and z");
+    static_assert(LDL >= C::CH, "e and f of a chunk");
 };
+// LONG: row stride of the weights and of gamma for rows of up to lmax keys (in whole eights, 4 mod 16 doubles)
+__host__ __device__ constexpr int long_stride(int lmax) { return (lmax + 15) / 16 * 16 + 4; }
 
 __device__ __forceinline__ double ld_any(const void* p, int dtype, size_t i) {
     return dtype == LLA_F32 ? (double)static_cast<const float*>(p)[i] : (double)__bfloat162float(static_cast<const __nv_bfloat16*>(p)[i]);
 }
 
-template <int D>
-__global__ void __launch_bounds__(DrCfg<D>::THREADS, D == 64 ? 2 : 1)
+template <int D, bool LONG>
+__global__ void __launch_bounds__(DrCfg<D>::THREADS, D == 64 && !LONG ? 2 : 1)
 bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
                 const void* __restrict__ dout, int dout_dtype, float* __restrict__ dq, float* __restrict__ dk, float* __restrict__ dv,
                 int n, int nq, int rows_per_head, double scale, double lambda, int* __restrict__ status, float* __restrict__ dlambda,
-                int H, int kv_group) {
+                int H, int kv_group, int lmax) {
     using C = DrCfg<D>;
-    using S = BrSmem<D>;
+    using S = BrSmem<D, LONG>;
     using T = team::Cfg<D, C::NW>;
     constexpr int NW = C::NW, TEAMS = C::TEAMS, CH = C::CH, NB = C::NB, R = T::R;
     constexpr unsigned FULL = 0xffffffffu;
@@ -61,13 +68,17 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
     const int off = n - nq;
     const int L = live ? off + i + 1 : 0;                               // query row i sits at position off + i
     const int Lb = off + min(i0 + TEAMS, rows_per_head);                // keys of the block
-    if (!LLA_IN_BOUNDS(Lb, S::LMAX + 1, status, 602)) return;           // (debug build: the keys must fit the arrays)
+    if (!LLA_IN_BOUNDS(Lb, lmax + 1, status, 602)) return;              // (debug build: the keys must fit the arrays)
+    const int ldl = LONG ? long_stride(lmax) : S::LDL, lpad = LONG ? ldl - 4 : S::LMAX;
+    double* const ps = LONG ? reinterpret_cast<double*>(br_smem + sizeof(S)) : &sm.p[0][0];
+    double* const gams = LONG ? ps + TEAMS * ldl : &sm.gam[0][0];
+    auto p_of = [&](int r) { return ps + r * ldl; };
+    auto gam_of = [&](int r) { return gams + r * ldl; };
     const size_t base = (size_t)bh * nq;                                // rows of q, dout, dq, dlambda
     const size_t kvbase = (size_t)kv_unit(bh, H, kv_group) * n;         // grouped heads: the key/value head's rows
     const __nv_bfloat16* kb = k + kvbase * D;
     const __nv_bfloat16* vb = v + kvbase * D;
     auto row_of = [](auto& rows) { return [&rows](int r) { return &rows[r][0]; }; };
-    auto row_at = [](auto& rows, int j0) { return [&rows, j0](int r) { return &rows[r][j0]; }; };
     auto team_sum = [&](double x, int slot, bool is_max = false) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -93,24 +104,24 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
         __syncthreads();
         stage<D>(sm.kv, vb, D, j0, Lb, CH);
         __syncthreads();
-        dots<D>(row_at(sm.gam, j0), row_of(sm.g), sm.kv, nk, warp, lane);
+        dots<D>([&](int r) { return gam_of(r) + j0; }, row_of(sm.g), sm.kv, nk, warp, lane);
         __syncthreads();
         stage<D>(sm.kv, kb, D, j0, Lb, CH);
         __syncthreads();
-        dots<D>(row_at(sm.p, j0), row_of(sm.q), sm.kv, nk, warp, lane);
+        dots<D>([&](int r) { return p_of(r) + j0; }, row_of(sm.q), sm.kv, nk, warp, lane);
     }
     __syncthreads();
     // ---- weights (relative to the row maximum) ----
     double m = -1e300;
-    for (int j = tt; j < L; j += 32 * NW) m = fmax(m, sm.p[tm][j] * scale);
+    for (int j = tt; j < L; j += 32 * NW) m = fmax(m, p_of(tm)[j] * scale);
     m = team_sum(m, 0, true);
     double omega = 0.0, gsum = 0.0;
-    for (int j = tt; j < S::LMAX; j += 32 * NW) {
-        const double e = j < L ? exp(sm.p[tm][j] * scale - m) : 0.0;
+    for (int j = tt; j < lpad; j += 32 * NW) {
+        const double e = j < L ? exp(p_of(tm)[j] * scale - m) : 0.0;
         omega += e;
-        if (j < L) gsum += e * sm.gam[tm][j];
-        sm.p[tm][j] = e;
-        if (j >= L) sm.gam[tm][j] = 0.0;
+        if (j < L) gsum += e * gam_of(tm)[j];
+        p_of(tm)[j] = e;
+        if (j >= L) gam_of(tm)[j] = 0.0;
     }
     omega = team_sum(omega, 1);
     gsum = team_sum(gsum, 0);
@@ -132,7 +143,7 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
 #pragma unroll 1
             for (int s = 0; s < ns; ++s) {
                 const double* kr = sm.kv[4 * s + t4] + g;
-                const double wj = sm.p[tm][j0 + 4 * s + t4], gj = sm.gam[tm][j0 + 4 * s + t4];
+                const double wj = p_of(tm)[j0 + 4 * s + t4], gj = gam_of(tm)[j0 + 4 * s + t4];
                 double av[R];
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
@@ -223,33 +234,47 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
     auto t_of = [&](int r) { return &sm.solve[r].x[0][1][0]; };
     auto e_of = [&](int r) { return reinterpret_cast<double*>(&sm.solve[r]); };
     auto f_of = [&](int r) { return reinterpret_cast<double*>(&sm.solve[r]) + S::LDL; };
+    // (LONG: of the chunk from e0 on, which lies at the arrays' start)
+    auto kappa_of = [&](int from, int to, int e0) {
+        double x = 0.0;
+        for (int j = from + tt; j < to; j += 32 * NW) x += p_of(tm)[j] * (1.0 - (e_of(tm)[j - e0] - ky)) * gam_of(tm)[j];
+        return x;
+    };
+    double kappa = 0.0;
     for (int j0 = 0; j0 < Lb; j0 += CH) {
-        const int nk = min(CH, Lb - j0);
+        const int nk = min(CH, Lb - j0), at = LONG ? 0 : j0;
         __syncthreads();
         stage<D>(sm.kv, kb, D, j0, Lb, CH);
         __syncthreads();
-        dots<D>([&](int r) { return e_of(r) + j0; }, y_of, sm.kv, nk, warp, lane);
-        dots<D>([&](int r) { return f_of(r) + j0; }, t_of, sm.kv, nk, warp, lane);
+        dots<D>([&](int r) { return e_of(r) + at; }, y_of, sm.kv, nk, warp, lane);
+        if constexpr (!LONG) {
+            dots<D>([&](int r) { return f_of(r) + at; }, t_of, sm.kv, nk, warp, lane);
+        } else {
+            __syncthreads();
+            kappa += kappa_of(j0, min(L, j0 + nk), j0);
+        }
     }
     __syncthreads();
     // ---- per key: a_j -> p, scale dL/ds_j -> gam, p (f - gamma + gbar) -> f, p (e - 1) -> e ----
-    double kappa = 0.0;
-    for (int j = tt; j < L; j += 32 * NW) kappa += sm.p[tm][j] * (1.0 - (e_of(tm)[j] - ky)) * sm.gam[tm][j];
+    if constexpr (!LONG) kappa = kappa_of(0, L, 0);
     kappa = team_sum(kappa, 1) * inv + tmb;                              // g . o_i + t . (kbar - q)
-    for (int j = tt; j < S::LMAX; j += 32 * NW) {
-        double a = 0.0, ds = 0.0, fu = 0.0, ew = 0.0;
-        if (j < L) {
-            const double p = sm.p[tm][j] * inv, e = e_of(tm)[j] - ky, f = f_of(tm)[j] - kt, gj = sm.gam[tm][j];
-            a = p * (1.0 - e);
-            ds = scale * p * (gj * (1.0 - e) + (gbar + f) * e - f - kappa);
-            fu = p * (f - gj + gbar);
-            ew = p * (e - 1.0);
+    auto coefficients = [&](int from, int to, int e0) {
+        for (int j = from + tt; j < to; j += 32 * NW) {
+            double a = 0.0, ds = 0.0, fu = 0.0, ew = 0.0;
+            if (j < L) {
+                const double p = p_of(tm)[j] * inv, e = e_of(tm)[j - e0] - ky, f = f_of(tm)[j - e0] - kt, gj = gam_of(tm)[j];
+                a = p * (1.0 - e);
+                ds = scale * p * (gj * (1.0 - e) + (gbar + f) * e - f - kappa);
+                fu = p * (f - gj + gbar);
+                ew = p * (e - 1.0);
+            }
+            p_of(tm)[j] = a;
+            gam_of(tm)[j] = ds;
+            f_of(tm)[j - e0] = fu;
+            e_of(tm)[j - e0] = ew;
         }
-        sm.p[tm][j] = a;
-        sm.gam[tm][j] = ds;
-        f_of(tm)[j] = fu;
-        e_of(tm)[j] = ew;
-    }
+    };
+    if constexpr (!LONG) coefficients(0, S::LMAX, 0);
     // ---- dQ = t + DS K;  dK += DS^T Q + U^T Y + W^T T;  dV += A^T G ----
     double o0 = 0.0, o1 = 0.0;
     const int tr = t4 < TEAMS ? t4 : 0;                                  // A^T operands: row t4 of the block
@@ -261,19 +286,27 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
             stage<D>(sm.kv, kb, D, j0, Lb, CH);
             __syncthreads();
         }
+        const int at = LONG ? j0 : 0;                                    // e and f: their first key
+        if constexpr (LONG) {
+            dots<D>(e_of, y_of, sm.kv, nk, warp, lane);
+            dots<D>(f_of, t_of, sm.kv, nk, warp, lane);
+            __syncthreads();
+            coefficients(j0, j0 + (nk + 7) / 8 * 8, j0);
+            __syncthreads();
+        }
         // (warp: columns 8 warp .. + 7)
         for (int s = 0; 4 * s < nk; ++s)
-            team::dmma(o0, o1, g < TEAMS ? sm.gam[g][j0 + 4 * s + t4] : 0.0, sm.kv[4 * s + t4][8 * warp + g]);
+            team::dmma(o0, o1, g < TEAMS ? gam_of(g)[j0 + 4 * s + t4] : 0.0, sm.kv[4 * s + t4][8 * warp + g]);
         const double bq = tin ? sm.q[tr][8 * warp + g] : 0.0, bg = tin ? sm.g[tr][8 * warp + g] : 0.0;
         const double by = tin ? y_of(tr)[8 * warp + g] : 0.0, bt = tin ? t_of(tr)[8 * warp + g] : 0.0;
 #pragma unroll 2
         for (int kk = 0; 8 * kk < nk; ++kk) {
-            const int j = j0 + 8 * kk + g;                               // (j < LMAX; the arrays are zero from L on)
+            const int j = j0 + 8 * kk + g;                               // (the arrays are zero from L on)
             double x0 = 0.0, x1 = 0.0, z0 = 0.0, z1 = 0.0;
-            team::dmma(x0, x1, tin ? sm.gam[tr][j] : 0.0, bq);
-            team::dmma(z0, z1, tin ? sm.p[tr][j] : 0.0, bg);
-            team::dmma(x0, x1, tin ? f_of(tr)[j] : 0.0, by);
-            team::dmma(x0, x1, tin ? e_of(tr)[j] : 0.0, bt);
+            team::dmma(x0, x1, tin ? gam_of(tr)[j] : 0.0, bq);
+            team::dmma(z0, z1, tin ? p_of(tr)[j] : 0.0, bg);
+            team::dmma(x0, x1, tin ? f_of(tr)[j - at] : 0.0, by);
+            team::dmma(x0, x1, tin ? e_of(tr)[j - at] : 0.0, bt);
             if (j < Lb) {
                 const size_t at = (kvbase + j) * D + 8 * warp + 2 * t4;
                 atomicAdd(reinterpret_cast<float2*>(dk + at), make_float2((float)x0, (float)x1));
@@ -287,27 +320,31 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
     }
 }
 
-template <int D>
+template <int D, bool LONG>
 int launch_t(const BackwardArgs& a, int nq, int rows, cudaStream_t stream) {
     using C = DrCfg<D>;
-    const int smem = (int)sizeof(BrSmem<D>);
-    auto kern = bwd_rows_kernel<D>;
+    const int lmax = LONG ? a.n - nq + rows : BrSmem<D, LONG>::LMAX;
+    const int smem = (int)(sizeof(BrSmem<D, LONG>) + (LONG ? 2 * sizeof(double) * C::TEAMS * long_stride(lmax) : 0));
+    auto kern = bwd_rows_kernel<D, LONG>;
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
     dim3 grid(a.B * a.H, (rows + C::TEAMS - 1) / C::TEAMS);
     kern<<<grid, C::THREADS, smem, stream>>>((const __nv_bfloat16*)a.q, (const __nv_bfloat16*)a.k, (const __nv_bfloat16*)a.v, a.dout, a.dout_dtype,
                                              a.dq, a.dk, a.dv, a.n, nq, rows, (double)a.scale, (double)a.lambda, a.status, a.dlambda, a.H,
-                                             a.kv_group > 0 ? a.kv_group : 1);
+                                             a.kv_group > 0 ? a.kv_group : 1, lmax);
     LLA_CUDA_TRY(cudaGetLastError());
     return LLA_OK;
 }
 
 }  // namespace
 
-// The first `rows` query rows of every head (they see at most 2 d keys) on `stream`; dK and dV are added to.
+int backward_rows_most_keys(int d) { return d == 64 ? 1222 : 323; }
+
+// The first `rows` query rows of every head (they see at most backward_rows_most_keys keys) on `stream`; dK and dV are added to.
 int launch_backward_rows(const BackwardArgs& a, int nq, int rows, cudaStream_t stream) {
-    if (a.d == 64) return launch_t<64>(a, nq, rows, stream);
-    if (a.d == 128) return launch_t<128>(a, nq, rows, stream);
+    const bool many = a.n - nq + rows > 2 * a.d;
+    if (a.d == 64) return many ? launch_t<64, true>(a, nq, rows, stream) : launch_t<64, false>(a, nq, rows, stream);
+    if (a.d == 128) return many ? launch_t<128, true>(a, nq, rows, stream) : launch_t<128, false>(a, nq, rows, stream);
     return LLA_ERR_UNSUPPORTED;
 }
 

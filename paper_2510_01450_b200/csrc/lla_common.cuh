@@ -220,6 +220,7 @@ int launch_backward_tensor(const BwdTensorArgs& a, int which);   // which: 0 = k
 size_t backward_workspace_bytes(int B, int H, int n, int d);
 int launch_backward(const BackwardArgs& a);
 int launch_backward_rows(const BackwardArgs& a, int nq, int rows, cudaStream_t stream);      // the directly-solved rows
+int backward_rows_most_keys(int d);      // keys that such a row may see: what shared memory holds beside the systems
 
 // Launchers implemented in the other translation units; each returns an lla_status.
 int direct_rows_below(const ForwardArgs& a);  // rows that see fewer keys than this are solved directly

@@ -208,3 +208,34 @@ def test_long_windowed_sequences(oracle, d, n, window):
     ref = oracle.decode(np.ascontiguousarray(q[0, :, rows].reshape(len(rows), 1, d)), kc, vc, cnt, scale, lam)
     err = row_err(out.cpu().numpy()[0, 0, rows], ref)
     assert err.max() <= TOL_F32, (float(err.max()), int(err.argmax()))
+
+
+def _gradients(w, q, k, v, g, head_rows=0):
+    """dq, dk, dv of a forward and a backward pass, whatever the status words say."""
+    t = [dev(x, "bf16") for x in (q, k, v)]
+    out, rho, dq, dk, dv_ = (torch.full(q.shape, float("nan"), dtype=torch.float32, device="cuda") for _ in range(5))
+    stats = torch.empty((w.B, w.H, w.n, 3), dtype=torch.float32, device="cuda")
+    nbytes = L.lla_backward_workspace_bytes(w.B, w.H, w.n, w.d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    L.lla_forward_ex(*t, out, w.B, w.H, w.n, w.d, w.d, w.scale, w.lam, out_dtype=L.LLA_F32, head_rows=head_rows, rho=rho, stats=stats,
+                     stream=stream_ptr())
+    L.lla_backward_ex(*t, out, dev(g, "f32"), rho, stats, dq, dk, dv_, w.B, w.H, w.n, w.d, w.scale, w.lam, head_rows=head_rows,
+                      workspace=ws, workspace_bytes=nbytes, stream=stream_ptr())
+    torch.cuda.synchronize()
+    return [x.cpu().numpy().astype(np.float64) for x in (dq, dk, dv_)]
+
+
+# head_rows raised beyond the default: rows with more than 2 d keys solved directly in both passes, part of a sequence or all of
+# it, up to the most keys that the backward takes
+@pytest.mark.parametrize("d,n,head_rows", [(64, 129, 130), (64, 300, 200), (64, 300, 301), (128, 262, 270), (128, 400, 324), (64, 1222, 1223)])
+def test_backward_with_more_direct_rows(backward_oracle, d, n, head_rows):
+    H = 1 if n > 1000 else 2
+    w = inputs.CONFIGS[2].shrink(B=1, H=H, n=n, d=d, dv=d, seed=860 + d + n)
+    q, k, v = inputs.make_prefill(w)
+    g = inputs.make_upstream_grad(w)
+    ref = backward_oracle.backward(q, k, v, g, w.scale, w.lam)
+    # fp64 throughout where every row is direct: the gradients' own fp32 rounding and sums
+    tol = 1e-5 if head_rows > n else TOL
+    for name, a, b in zip(("dq", "dk", "dv"), _gradients(w, q, k, v, g, head_rows), ref):
+        err = grad_err(a, b)
+        assert np.isfinite(err).all() and err.max() <= tol, (name, float(err.max()), int(err.argmax()))
