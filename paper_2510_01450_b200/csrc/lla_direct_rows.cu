@@ -210,7 +210,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     // team-wide sums (every team has run every block barrier above)
     if (live) {
         omega = team_reduce(omega, false, 1);
-        lam_m = ridge_mode == LLA_RIDGE_PRINTED ? lam_i * exp(m_max - m_ref) : lam_i * exp(-(m_ref + frame()));
+        lam_m = ridge_mode == LLA_RIDGE_PRINTED ? lam_i : lam_i * exp(-(m_max + frame()));      // beside weights relative to m_max
     }
     const double inv = 1.0 / omega;
     team::Smem<D, NW, 1>& ss = sm.solve[tm];
@@ -359,7 +359,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             }
         }
     } else if (live) {
-        const double ridge = lam_m * inv;
+        const double ridge = lam_m * (inv * exp(m_max - m_ref));
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int bi = T::row(r, w);

@@ -239,3 +239,26 @@ def test_backward_with_more_direct_rows(backward_oracle, d, n, head_rows):
     for name, a, b in zip(("dq", "dk", "dv"), _gradients(w, q, k, v, g, head_rows), ref):
         err = grad_err(a, b)
         assert np.isfinite(err).all() and err.max() <= tol, (name, float(err.max()), int(err.argmax()))
+
+
+@pytest.mark.parametrize("dtype,d,n", [("bf16", 128, 180), ("f32", 128, 250)])
+def test_reference_far_below_the_maximum(oracle, dtype, d, n):
+    """The first 130 keys score near -740, the others near -160: the weights' reference is the former's maximum, where
+    lambda e^-m has no double, the row's ridge is the latter's."""
+    rng = np.random.default_rng(985 + n)
+    scale = np.float32(d ** -0.5)
+    u = np.ones(d, dtype=np.float32) / np.float32(np.sqrt(d))
+    a = np.float32(np.sqrt(740.0 / scale))
+    noise = lambda: rng.standard_normal((1, 2, n, d)).astype(np.float32) * scale
+    q, k, v = a * u + noise() * np.float32(0.01), noise() * np.float32(0.1), noise() * np.float32(np.sqrt(d))
+    k[:, :, :130] -= a * u
+    k[:, :, 130:] -= np.float32(160.0 / 740.0) * a * u
+    rnd = inputs.round_to_bf16 if dtype == "bf16" else (lambda x: x.astype(np.float32))
+    q, k, v = map(rnd, (q, k, v))
+    ref = oracle.forward(q, k, v, float(scale), 1e-3)[:, :, 140:]
+    out = torch.full(q.shape, float("nan"), dtype=torch.float32, device="cuda")
+    L.lla_forward_ex(dev(q, dtype), dev(k, dtype), dev(v, dtype), out, 1, 2, n, d, d, float(scale), 1e-3, in_dtype=LLA_DT[dtype],
+                     out_dtype=L.LLA_F32, stream=stream_ptr())
+    torch.cuda.synchronize()
+    err = row_err(out.cpu().numpy()[:, :, 140:], ref)
+    assert np.isfinite(err).all() and err.max() <= (TOL_F32 if dtype == "f32" else TOL_BF16), float(np.nanmax(err))
