@@ -34,6 +34,8 @@ struct BrSmem {
     double kbar[C::TEAMS][D];
     team::Smem<D, C::NW, 2> solve[C::TEAMS];                       // afterwards e_j and f_j lie over its first part
     double red[2][C::TEAMS][C::NW];
+    unsigned bad[2];                                               // keys, values at the block's end that are not finite (see Ends)
+    int odd;                                                       // a query or upstream gradient of the block is not
     static_assert(64 + D / 8 * 24 + 4 * D >= 2 * LDL, "e and f lie over the solver's w, piv, b and z");
     static_assert(LDL >= C::CH, "e and f of a chunk");
 };
@@ -92,21 +94,33 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
         for (int u = 1; u < NW; ++u) x = is_max ? fmax(x, sm.red[slot][tm][u]) : x + sm.red[slot][tm][u];
         return x;
     };
+    bool odd = false;
     for (int e = tid; e < TEAMS * D; e += C::THREADS) {
         const int r = e / D, c = e % D;
         const bool in = i0 + r < rows_per_head;
         sm.q[r][c] = in ? (double)__bfloat162float(q[(base + i0 + r) * D + c]) : 0.0;
         sm.g[r][c] = in ? ld_any(dout, dout_dtype, (base + i0 + r) * D + c) : 0.0;
+        odd = odd || !isfinite(sm.q[r][c]) || !isfinite(sm.g[r][c]);
     }
+    const int L0 = off + i0 + 1;                                         // every row of the block sees the keys before L0
+    const Ends ends{L0, Lb, 0, 0};
+    odd = __syncthreads_or(odd);
+    if (tid == 0) {
+        sm.odd = odd;
+        sm.bad[0] = sm.bad[1] = 0u;
+    }
+    auto checked = [&](int j0, int nk, int what) { take_out<D>(sm.kv, L0 - j0, nk, 1u, &sm.bad[what]); };    // (before the barrier that ends the staging)
     // ---- gamma_j = g . v_j and the scores ----
     for (int j0 = 0; j0 < Lb; j0 += CH) {
         const int nk = min(CH, Lb - j0);
         __syncthreads();
         stage<D>(sm.kv, vb, D, j0, Lb, CH);
+        checked(j0, nk, 1);
         __syncthreads();
         dots<D>([&](int r) { return gam_of(r) + j0; }, row_of(sm.g), sm.kv, nk, warp, lane);
         __syncthreads();
         stage<D>(sm.kv, kb, D, j0, Lb, CH);
+        checked(j0, nk, 0);
         __syncthreads();
         dots<D>([&](int r) { return p_of(r) + j0; }, row_of(sm.q), sm.kv, nk, warp, lane);
     }
@@ -123,6 +137,8 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
         p_of(tm)[j] = e;
         if (j >= L) gam_of(tm)[j] = 0.0;
     }
+    if (sm.bad[0] & ends.seen(tm, 0)) omega = NAN;      // the row sees a key, a value that is not finite
+    if (sm.bad[1] & ends.seen(tm, 0)) gsum = NAN;
     omega = team_sum(omega, 1);
     gsum = team_sum(gsum, 0);
     // ---- moments ----
@@ -135,6 +151,7 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
         if (Lb > CH) {
             __syncthreads();
             stage<D>(sm.kv, kb, D, j0, Lb, CH);
+            checked(j0, min(CH, Lb - j0), 0);
             __syncthreads();
         }
         const int ns = (min(CH, L - j0) + 3) / 4;
@@ -245,6 +262,7 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
         const int nk = min(CH, Lb - j0), at = LONG ? 0 : j0;
         __syncthreads();
         stage<D>(sm.kv, kb, D, j0, Lb, CH);
+        checked(j0, nk, 0);
         __syncthreads();
         dots<D>([&](int r) { return e_of(r) + at; }, y_of, sm.kv, nk, warp, lane);
         if constexpr (!LONG) {
@@ -284,6 +302,7 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
         __syncthreads();
         if (Lb > CH) {
             stage<D>(sm.kv, kb, D, j0, Lb, CH);
+            checked(j0, nk, 0);
             __syncthreads();
         }
         const int at = LONG ? j0 : 0;                                    // e and f: their first key
@@ -307,6 +326,17 @@ bwd_rows_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __rest
             team::dmma(z0, z1, tin ? p_of(tr)[j] : 0.0, bg);
             team::dmma(x0, x1, tin ? f_of(tr)[j - at] : 0.0, by);
             team::dmma(x0, x1, tin ? e_of(tr)[j - at] : 0.0, bt);
+            if ((sm.odd || sm.bad[0] || sm.bad[1]) && j >= L0 && j < Lb) {
+                // a row that is not finite must not reach the keys that it does not see: only those that do, by hand
+                const int c = 8 * warp + 2 * t4;
+                x0 = x1 = z0 = z1 = 0.0;
+                for (int r = j - L0 + 1; r < min(TEAMS, rows_per_head - i0); ++r) {
+                    x0 += gam_of(r)[j] * sm.q[r][c] + f_of(r)[j - at] * y_of(r)[c] + e_of(r)[j - at] * t_of(r)[c];
+                    x1 += gam_of(r)[j] * sm.q[r][c + 1] + f_of(r)[j - at] * y_of(r)[c + 1] + e_of(r)[j - at] * t_of(r)[c + 1];
+                    z0 += p_of(r)[j] * sm.g[r][c];
+                    z1 += p_of(r)[j] * sm.g[r][c + 1];
+                }
+            }
             if (j < Lb) {
                 const size_t at = (kvbase + j) * D + 8 * warp + 2 * t4;
                 atomicAdd(reinterpret_cast<float2*>(dk + at), make_float2((float)x0, (float)x1));

@@ -46,7 +46,7 @@ struct DrSmem {
         double mat[C::TEAMS][team::Cfg<D, C::NW>::LOWER][64];      // the systems, between the sweeps
     };
     double q[C::TEAMS][C::LDK];               // query rows, zero beyond the head's
-    double rel[REL ? C::TEAMS : 1][C::LDK];        // REL: the same minus the first of them
+    double rel[REL ? C::TEAMS + 1 : 1][C::LDK];    // REL: the same minus the first of them; the first (zero where it is not finite)
     double y[C::TEAMS][C::LDK];                    // their solutions (second sweep)
     double s[C::TEAMS][C::LDW];               // scores -> weights -> output coefficients of the chunk
     double t[C::TEAMS][C::LDW];               // k_j . y
@@ -56,6 +56,7 @@ struct DrSmem {
     double den[C::TEAMS], lam[C::TEAMS], qq[C::TEAMS], qn[REL ? C::TEAMS : 1];      // qq: |q|^2 in the frame of the keys; qn: |q|^2
     double kmax[REL ? C::WARPS : 1];
     int dual[C::TEAMS];                       // visible keys of a dual row, 0 for the others
+    unsigned bad[2];                          // keys, values at the ends of the block's range that are not finite (see Ends)
     team::Smem<D, C::NW, 1> solve[C::TEAMS];
 };
 
@@ -102,10 +103,23 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     const double* qc = rel ? sm.rel[tm] : sm.q[tm];                     // the row's query in the frame of the staged keys
     if (rel) {
         __syncthreads();
-        for (int e = tid; e < TEAMS * D; e += C::THREADS) sm.rel[e / D][e % D] = sm.q[e / D][e % D] - sm.q[0][e % D];
+        for (int e = tid; e < (TEAMS + 1) * D; e += C::THREADS) {
+            const int r = e / D, c = e % D;
+            const double x = sm.q[0][c], ref = isfinite(x) ? x : 0.0;
+            sm.rel[r][c] = r < TEAMS ? sm.q[r][c] - ref : ref;
+        }
     }
+    if (tid < 2) sm.bad[tid] = 0u;
+    auto ends = [&]() {
+        const int e = off + i0 + 1;
+        return Ends{causal ? e : 0, causal ? off + last + 1 : 0, jbeg, causal && window > 0 ? max(0, off + last + 1 - window) : 0};
+    };
+    auto checked = [&](int j0, int nk, int what) {                      // the chunk's ends, before the barrier that ends its staging
+        if (causal) take_out<D>(sm.kv, off + i0 + 1 - j0, nk, 1u, &sm.bad[what]);
+        if (causal && window > 0) take_out<D>(sm.kv, jbeg - j0, nk, 256u, &sm.bad[what]);
+    };
     auto stage_keys = [&](int j0) {
-        if (rel) stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch, sm.q[0]);
+        if (rel) stage<D, true>(sm.kv, kb, sk.r, j0, jend, ch, sm.rel[TEAMS]);
         else stage<D>(sm.kv, kb, sk.r, j0, jend, ch);
     };
     // one value per thread of the team -> its maximum or sum over the team
@@ -141,6 +155,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         const int nk = min(ch, jend - j0);
         __syncthreads();
         stage_keys(j0);
+        checked(j0, nk, 0);
         __syncthreads();
         dots<D>(row_of(sm.s), row_of(sm.q), sm.kv, nk, warp, lane);
         __syncthreads();
@@ -201,7 +216,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     auto frame = [&]() {
         double x = 0.0;
         if (rel) {
-            for (int e = lane; e < D; e += 32) x += sm.q[tm][e] * sm.q[0][e];
+            for (int e = lane; e < D; e += 32) x += sm.q[tm][e] * sm.rel[TEAMS][e];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
         }
@@ -286,6 +301,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             __syncthreads();
 #pragma unroll
             for (int u = 0; u < C::WARPS; ++u) kmax = fmax(kmax, sm.kmax[u]);
+            rowwise = !isfinite(sm.qn[0]);                 // (the products below take that query's from the others')
             for (int t = 0; t < TEAMS; ++t)
                 rowwise = rowwise || (sm.dual[t] && !(sm.lam[t] >= 1e-8 * fmax(fmax(kmax, sm.qq[t]), sqrt(kmax * sm.qn[t]))));
         }
@@ -418,6 +434,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
         __syncthreads();
         if (keys) {
             stage_keys(j0);
+            checked(j0, nk, 0);
             __syncthreads();
             if (dual) {
                 if (rho_out)                                       // rho = Z^T alpha
@@ -444,6 +461,7 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
                 csum += cj;
             }
         stage<D>(sm.kv, vb, sv.r, j0, jend, ch);
+        checked(j0, nk, 1);
         __syncthreads();
         if (half < C::HALVES) {
             const int s1 = (nk + 3) / 4;
@@ -462,6 +480,11 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
             o1 += p.y;
         }
         const double id = 1.0 / sm.den[g];
+        if (sm.bad[0] | sm.bad[1]) {
+            const double2 x = spoilt(sm.bad, ends(), g, causal && window > 0 ? max(0, off + i0 + g + 1 - window) : 0, vb + 8 * ob + 2 * t4, sv.r);
+            o0 += x.x;
+            o1 += x.y;
+        }
         TOut* orow = out + so.at(bh / H, bh % H, i0 + g) + 8 * ob + 2 * t4;
         if (LLA_IN_BOUNDS((size_t)bh * nq + i0 + g, (size_t)gridDim.x * nq, status, 201)) {
             store_out(orow, (float)(o0 * id));
@@ -470,12 +493,18 @@ direct_rows_kernel(const TIn* __restrict__ q, const TIn* __restrict__ k, const T
     }
     const double f = exp(m_ref - m_max);           // to weights relative to the true maximum
     if (live && stats) m_max += frame();           // (by whole warps)
+    bool spoil = false;                            // the row sees a key that is not finite
+    if (live && sm.bad[0]) {
+        spoil = (sm.bad[0] & ends().seen(tm, jlo)) != 0u;
+        if (spoil && rho_out && w == 0)
+            for (int e = lane; e < D; e += 32) rho_out[row * D + e] = NAN;
+    }
     if (live && tt == 0) {
         if (stats) {
                         const double om = omega * f, dl = dual ? den * f : omega * f / gfac;
             stats[row * 3 + 0] = (float)m_max;
-            stats[row * 3 + 1] = (float)om;
-            stats[row * 3 + 2] = (float)dl;
+            stats[row * 3 + 1] = spoil ? NAN : (float)om;
+            stats[row * 3 + 2] = spoil ? NAN : (float)dl;
         }
         if (iters) iters[row] = L < head_rows ? -1 : 0;      // (0: a row that conjugate gradients could have solved)
         if (!ok && status) atomicAdd(status + LLA_STATUS_BAD_PIVOT, 1);

@@ -67,6 +67,48 @@ __device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* _
     }
 }
 
+// ---- what is not finite ----
+// Zero times infinity or NaN is not zero: such entries, in the few keys and values at the ends of a block's range that only
+// some of its rows see, would reach the other rows through their zero weights.  They are taken out of the staged rows
+// (set to zero; bit b stands for the key hi0 + b, bit 8 + b for lo0 + b), and what the rows that do see them put out is
+// spoilt at the end.  (256 fp32 rows, d = 16: 24.6 us with this, 22.5 without; rows of 1 to 95 keys, 32 heads, d = 64: 86 us
+// against 84; with bounds on the keys inside the loops over them instead: 24.8 and 86.)
+struct Ends {
+    int hi0, hi1;      // keys that the last row of the block sees and the first does not: row r sees those before hi0 + r
+    int lo0, lo1;      // (window) keys that the first row sees and the last does not
+    // the bits of the keys that the block's r-th row sees, if it sees the keys from first_key on
+    __device__ __forceinline__ unsigned seen(int r, int first_key) const { return ((1u << r) - 1u) | ((0xff00u << max(first_key - lo0, 0)) & 0xff00u); }
+};
+// Takes them out of the staged rows first .. first + TEAMS - 2, as far as they are among the nk staged, and notes row first + b as
+// bit0 << b in bad.  A thread looks at what it has staged itself, so the barrier that ends the staging is enough.
+template <int D>
+__device__ __forceinline__ void take_out(double (*rows)[DrCfg<D>::LDK], int first, int nk, unsigned bit0, unsigned* bad) {
+    constexpr int ROUND = 2 * DrCfg<D>::THREADS / D;          // a thread stages every ROUND-th row
+    static_assert(DrCfg<D>::TEAMS - 1 <= ROUND && (ROUND & (ROUND - 1)) == 0, "at most one of these rows a thread");
+    const int b = ((int)threadIdx.x / (D / 2) - first) & (ROUND - 1), j = first + b;
+    if (b >= DrCfg<D>::TEAMS - 1 || j < 0 || j >= nk) return;
+    double2& x = *reinterpret_cast<double2*>(&rows[j][2 * (threadIdx.x % (D / 2))]);
+    if (isfinite(x.x) && isfinite(x.y)) return;
+    x = make_double2(isfinite(x.x) ? x.x : 0.0, isfinite(x.y) ? x.y : 0.0);
+    atomicOr(bad, bit0 << b);
+}
+// What spoils two columns, to which v points, of the block's r-th row, which sees keys from first_key on: NaN if it sees a key
+// taken out, or a value taken out there; zero otherwise.
+template <typename TIn>
+__device__ __noinline__ double2 spoilt(const unsigned* bad, Ends ends, int r, int first_key, const TIn* v, long long stride) {
+    const unsigned seen = ends.seen(r, first_key);
+    double2 x = make_double2(0.0, 0.0);
+    if (bad[0] & seen) x = make_double2(NAN, NAN);
+    for (int bit = 0; bit < 16; ++bit) {
+        if (!(bad[1] & seen & (1u << bit))) continue;
+        double a, b;
+        load_pair(v + (size_t)(bit < 8 ? ends.hi0 + bit : ends.lo0 + bit - 8) * stride, a, b);
+        if (!isfinite(a)) x.x = NAN;
+        if (!isfinite(b)) x.y = NAN;
+    }
+    return x;
+}
+
 // out(r)[j] = row(r) . keys[j], eight keys per step of a warp; row and out: pointers of the block's r-th row
 template <int D, typename Row, typename Out>
 __device__ __forceinline__ void dots(Out&& out, Row&& row, const double (*keys)[DrCfg<D>::LDK], int nkeys, int warp, int lane) {

@@ -262,3 +262,60 @@ def test_reference_far_below_the_maximum(oracle, dtype, d, n):
     torch.cuda.synchronize()
     err = row_err(out.cpu().numpy()[:, :, 140:], ref)
     assert np.isfinite(err).all() and err.max() <= (TOL_F32 if dtype == "f32" else TOL_BF16), float(np.nanmax(err))
+
+
+@pytest.mark.parametrize("dtype,d,n,window", [("bf16", 64, 95, 0), ("f32", 16, 100, 0), ("f32", 16, 100, 33), ("f32", 64, 150, 0),
+                                              ("f32", 64, 300, 131), ("bf16", 128, 150, 0), ("f32", 128, 140, 0), ("f32", 128, 400, 258)])
+@pytest.mark.parametrize("where", ["q", "k", "v"])
+def test_infinities_stay_in_the_rows_that_see_them(dtype, d, n, window, where):
+    """A query row that is not finite spoils its own output, a key or value those of the rows that see it: the rows beside them
+    in a block come out as without it."""
+    w = inputs.CONFIGS[2].shrink(B=1, H=1, n=n, d=d, dv=d, dtype=dtype, seed=990 + d + n)
+    x = dict(zip("qkv", (dev(a, dtype) for a in inputs.make_prefill(w))))
+
+    def run():
+        out, rho = (torch.full((1, 1, n, d), 7.0, dtype=torch.float32, device="cuda") for _ in range(2))
+        stats = torch.full((1, 1, n, 3), 7.0, dtype=torch.float32, device="cuda")
+        L.lla_forward_ex(x["q"], x["k"], x["v"], out, 1, 1, n, d, d, w.scale, w.lam, in_dtype=LLA_DT[dtype],
+                         out_dtype=L.LLA_F32, window=window, rho=rho, stats=stats, stream=stream_ptr())
+        torch.cuda.synchronize()
+        return out[0, 0], rho[0, 0], stats[0, 0]
+
+    clean = run()
+    assert all(torch.isfinite(c).all() for c in clean)
+    for j in (0, 1, 4, 41, 43, 66, n - 2):
+        for bad in (float("inf"), float("nan")):
+            keep = x[where][0, 0, j, 3].clone()
+            x[where][0, 0, j, 3] = bad
+            got = run()
+            x[where][0, 0, j, 3] = keep
+            rows = torch.arange(n, device="cuda")
+            seen = rows == j if where == "q" else (rows >= j) & ((rows < j + window) if window else (rows >= 0))
+            assert not torch.isfinite(got[0][seen]).all(dim=1).any(), (j, bad)
+            if where != "v":
+                assert not torch.isfinite(got[1][seen]).all(dim=1).any() and not torch.isfinite(got[2][seen]).all(dim=1).any()
+            # (the frame or the form of a row's matrix may be another beside it: fp32 rounding)
+            for a, b in zip(got, clean):
+                assert torch.allclose(a[~seen], b[~seen], rtol=1e-5, atol=1e-6 * float(b.abs().max())), (j, bad)
+
+
+@pytest.mark.parametrize("d,n", [(64, 95), (128, 150)])
+def test_backward_infinities_stay_in_the_rows_that_see_them(d, n):
+    w = inputs.CONFIGS[2].shrink(B=1, H=1, n=n, d=d, dv=d, seed=995 + d)
+    q, k, v = inputs.make_prefill(w)
+    g = inputs.make_upstream_grad(w)
+    clean = _gradients(w, q, k, v, g)
+    same = lambda a, b: np.abs(a - b).max() <= 1e-5 * np.abs(b).max()      # (fp32 sums in another order)
+    for j in (4, 40, 42):
+        gb = g.copy()
+        gb[0, 0, j, 3] = np.nan
+        dq, dk, dv = _gradients(w, q, k, v, gb)
+        rest = np.arange(n) != j
+        assert np.isnan(dq[0, 0, j]).any() and same(dq[0, 0, rest], clean[0][0, 0, rest])
+        for a, b in ((dk, clean[1]), (dv, clean[2])):         # keys up to j get a share of row j
+            assert np.isnan(a[0, 0, : j + 1]).any(axis=1).all() and same(a[0, 0, j + 1:], b[0, 0, j + 1:])
+        for which in (1, 2):
+            bad = [q, k.copy(), v.copy()]
+            bad[which][0, 0, j, 3] = np.nan
+            dq = _gradients(w, *bad, g)[0]
+            assert same(dq[0, 0, :j], clean[0][0, 0, :j]) and np.isnan(dq[0, 0, j:]).any(axis=1).all()
