@@ -122,7 +122,11 @@ int lla_decode_f32(const void *q, const void *kcache, const void *vcache, const 
  *               fp32 inputs; negative disables).  Those early systems are too ill-conditioned for fp32 CG.
  *               With max_iters, tol, head_rows, impl and phases all at their defaults, further rows of a problem
  *               that the tensor-core kernel does not take (fp32 inputs, d = 16) are solved that way where that is
- *               faster than CG: all of them, unless they see very many keys and the call is large
+ *               faster than CG: all of them, except that a call with enough (batch, head) pairs to fill the GPU
+ *               leaves the rows that see more than about 500 (d = 128), 2800 (d = 64) or 6300 (d = 16) keys to CG.
+ *               So the last bits of a sequence's output depend on how many others are in the call; so they do on
+ *               the tensor-core kernel, where small calls split a row's sums over two thread blocks.  Both stay within
+ *               the tolerance of the solver settings, and equal calls give equal bits
  *   impl      : lla_impl
  *   phases    : which groups of rows to compute: 0 = all; LLA_PHASE_DIRECT = only the rows
  *               solved directly; LLA_PHASE_ITERATIVE = only the rows solved by CG (profiling aid:
@@ -367,7 +371,8 @@ int lla_decode_default_splits(int B, int H, int Lmax);
  *               scale, lambda, head_rows and window (a causal forward with q_rows = n and the ridge of the
  *               definition; the call cannot tell and would return the gradient of that forward)
  *   dq, dk, dv: [B, H, n, d] fp32 on the device, overwritten
- *   max_iters, tol, head_rows : as in lla_forward_params (0 = defaults)
+ *   max_iters, tol, head_rows : as in lla_forward_params (0 = defaults); the directly-solved rows may see at most
+ *               1222 keys at d = 64, 323 at d = 128 (a larger head_rows: LLA_ERR_UNSUPPORTED)
  *   device_status : optional int[LLA_STATUS_WORDS], zeroed by the call
  *   workspace / workspace_bytes : device scratch of at least lla_backward_workspace_bytes(B, H, n, d)
  *               bytes, 256-byte aligned (required; LLA_ERR_WORKSPACE otherwise)

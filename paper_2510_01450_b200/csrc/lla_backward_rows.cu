@@ -13,8 +13,8 @@
 // beyond that (LONG) only the weights and gamma do, in rows as long as needed, and e_j and f_j are formed a chunk of
 // keys at a time, e_j once more before for g . o_i.
 //
-// Measured on B200 against one block per row with a shared-memory LDL^T on the CUDA cores and one atomic per row and
-// entry: 32 heads, n = 1000, d = 64 (95 rows a head): 305 -> 130 us; 16 heads, d = 128 (191 rows): 3.5 -> 1.1 ms.
+// Measured on B200: 32 heads, n = 1000, d = 64 (95 rows a head) 130 us; 16 heads, d = 128 (191 rows) 1.1 ms.  (One block per
+// row with a shared-memory LDL^T on the CUDA cores and one atomic per row and entry: 305 us and 3.5 ms.)
 #include "lla_rows.cuh"
 
 namespace lla {

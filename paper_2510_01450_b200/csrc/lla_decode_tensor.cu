@@ -1,8 +1,9 @@
 // LLA decode on tensor cores (bf16 caches, d = dv = 64 or 128): one pass over the KV cache.
 //
 // The cache is streamed a single time and folded into the weighted moments about the origin that the
-// centred form of Eq. "lla_decomp" needs, fp32 in TMEM:
-//     M = sum_j w_j k_j k_j^T,  N = sum_j w_j v_j k_j^T,  and on the CUDA cores omega = sum w, a = sum w k, c = sum w v.
+// centred form of Eq. "lla_decomp" needs:
+//     M = sum_j w_j k_j k_j^T,  N = sum_j w_j v_j k_j^T  (fp32 in TMEM),  omega = sum w (CUDA cores),
+//     a = sum w k,  c = sum w v  (d = 64: a column of the MMA; d = 128: CUDA cores).
 //
 // Per tile of 64 keys, each role at its own pace, coupled by mbarriers only:
 //   TMA         K and V tiles -> 128B-swizzled shared memory, where they are the MN-major B operand as they arrive:
@@ -15,9 +16,13 @@
 //   MMA (TS)    d = 64 : A = [wK ; wV]^T (128 rows), B = [K | 1] (N = 80):  D = [M a ; N c]
 //               d = 128: A = [wK]^T,                 B = [K | V] (N = 256): D = [M | N^T]; a, c on the CUDA cores
 //
-// Why this form: the earlier kernel had [K^T ; V^T] as A and the weighted keys as B, written to shared memory by the
-// threads: 80 KB of shared-memory traffic per 16 KB of cache, and one chain of dependent phases per tile.  Here it is
-// 56 KB (d = 64) and the phases of different tiles overlap.
+// Why this form: [K^T ; V^T] as A and the weighted keys as B, written to shared memory by the threads, take 80 KB of
+// shared-memory traffic per 16 KB of cache and one chain of dependent phases per tile (265 us at 64 sequences x 16
+// heads, d = 64).  Here it is 56 KB and the phases of different tiles overlap (230 us).
+//
+// Precision: the accumulators are fp32, added to once per 16 keys and operand half.  Against float64 the output at
+// d = 128 differs by 4e-6 (500 keys a part) to 3e-5 (8000), which grows with the number of these additions, not with the
+// operands' 17 bits; at d = 64 by the solve's tolerance, 5e-5.  The CUDA-core kernels (impl = LLA_IMPL_SIMT) give 1e-6.
 //
 // m_ref is the maximum of the first tile.  The threads only note whether a later score exceeds it by more
 // than 2^90 (no check per tile across threads); if one did, the whole pass is repeated with the true maximum, which
@@ -839,8 +844,8 @@ decode_tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant_
 
 // Sum of the parts' moments of one unit into the record of its first part, each scaled to the largest of their maxima
 // (the parts' weights and maxima stay as they are).  Split calls are small ones, which leave most of the chip idle:
-// merging in the solve kernel, whose few blocks would read every part through 64 threads, made that kernel 42 us long
-// at one sequence x 16 heads, d = 64, 8 parts; now 4 us here and 10 us there.
+// in the solve kernel, whose few blocks would read every part through 64 threads, merging and solving take 42 us at one
+// sequence x 16 heads, d = 64, 8 parts; 4 us here and 9 us there.
 constexpr int DM_THREADS = 256;
 template <int D>
 __global__ void __launch_bounds__(DM_THREADS)

@@ -1213,8 +1213,8 @@ float* scratch_for_device(size_t bytes) {
 // falls with the number of visible keys per dimension (measured at d / keys = 1/2, 1/4, 1/8, 1/16, 1/64: 37 .. 42, 24,
 // 10.5, 7.5, 5; the same at both head sizes), so at short sequence lengths the first tiles are the longest blocks even
 // though their sweeps are the shortest.  A sweep's overhead is worth 8.5 key blocks (10 at d = 128).  The numbers only
-// steer the order, never the result.  (Against a fit with a third fewer iterations for the first tiles: n = 1500, 16 heads,
-// d = 64: 317 -> 294 us; n = 3000, 8 heads: 336 -> 321 us.)
+// steer the order, never the result.  (With a third fewer iterations for the first tiles they start too late: n = 1500, 16
+// heads, d = 64: 317 us against 294; n = 3000, 8 heads: 336 against 321.)
 void tile_order(TcParams& prm, int tiles, int first_tile, int n, int off, int d, int causal, int window, bool precond) {
     prm.use_order = 0;
     if (!causal || tiles > TC_ORDER_MAX) return;

@@ -39,8 +39,7 @@ __device__ __forceinline__ void load_pair<float>(const float* p, double& a, doub
 
 // keys (or values) j0 .. j0 + ch - 1 -> shared memory; rows from jend on are zero, but the rounds
 // that hold no row before jend are left out, four at a time: their rows keep what they held, and nothing reads them.
-// (Rows of 1 to 95 keys, 32 heads, d = 64: 92 -> 87 us together with the dual form's
-// diagonal made once per row; the backward's rows 135 -> 130 us.)
+// (Of rows of 1 to 95 keys, 32 heads, d = 64, all rounds would take 4 % more, forward and backward.)
 // REL: ref, a row in shared memory, is subtracted from each of them.
 template <int D, bool REL = false, typename TIn>
 __device__ __forceinline__ void stage(double (*dst)[DrCfg<D>::LDK], const TIn* __restrict__ src, long long stride, int j0, int jend, int ch,

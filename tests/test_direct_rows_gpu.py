@@ -14,10 +14,13 @@ from tests.test_parity_gpu import TOL_BF16, TOL_F32
 pytestmark = pytest.mark.gpu
 
 
-# n around the chunk (64 keys at d = 16, 72 at 64, 136 / 64 at 128), one row, rows that do not fill a block's teams
+# n around the chunk (64 keys at d = 16; 128, in longer blocks 64, at d = 64; 136, in longer blocks 128, at d = 128), one row,
+# rows that do not fill a block's teams
 @pytest.mark.parametrize("dtype,d,n,nq,H,Hkv,window,causal,mode", [
     ("f32", 16, 1, 1, 1, 1, 0, True, ""), ("f32", 16, 64, 64, 2, 2, 0, True, ""), ("f32", 16, 65, 65, 3, 1, 0, True, ""),
     ("bf16", 16, 131, 70, 2, 1, 0, True, ""), ("f32", 16, 193, 193, 1, 1, 40, True, ""), ("f32", 16, 97, 30, 2, 2, 0, False, ""),
+    ("f32", 64, 127, 127, 1, 1, 0, True, ""), ("f32", 64, 128, 128, 2, 1, 0, True, ""), ("f32", 64, 129, 129, 1, 1, 0, True, ""),
+    ("f32", 64, 132, 132, 1, 1, 0, True, ""), ("f32", 64, 193, 193, 1, 1, 0, True, ""), ("f32", 128, 136, 136, 1, 1, 0, True, ""),
     ("f32", 64, 72, 72, 2, 2, 0, True, ""), ("f32", 64, 73, 73, 1, 1, 0, True, ""), ("f32", 64, 217, 75, 4, 2, 0, True, ""),
     ("f32", 64, 300, 300, 1, 1, 131, True, ""), ("f32", 64, 145, 9, 2, 1, 0, False, ""), ("f32", 64, 310, 40, 2, 2, 0, True, "late_max"),
     ("f32", 64, 64, 33, 1, 1, 0, False, ""), ("f32", 128, 137, 137, 1, 1, 0, True, ""), ("f32", 128, 300, 70, 2, 1, 0, True, "late_max"),
