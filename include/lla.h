@@ -182,17 +182,17 @@ typedef struct lla_forward_params {
     int window;     /* causal sliding window: 0 = a row sees every earlier position; W > 0 = only its last W
                        positions (itself included).  Needs causal != 0 and W >= the direct-row threshold
                        (head_rows; 1.5 d for bf16, 2 d for fp32 by default), else LLA_ERR_UNSUPPORTED */
-    int cg_precise_iters; /* tensor-core kernel only.  The operands formed on the fly in a CG iteration (the search
-                       direction P and the weighted products W .* (P K^T) of Algorithm 2) enter the tensor cores
-                       as bf16 hi + lo pairs (16 mantissa bits, two products each) during the first
+    int cg_precise_iters; /* tensor-core kernel only.  The weighted products W .* (P K^T) of Algorithm 2, formed on the fly in a
+                       CG iteration, enter the tensor cores as fp16 hi + lo pairs (two products each) during the first
                        cg_precise_iters iterations of a row tile and as single fp16 values (11 bits, one product)
                        afterwards: an iteration's products are scaled by the size of its search direction,
                        which has fallen by then, so the coarser operands of the later iterations add less
-                       error than the tolerance leaves.  The fp16 sweeps read an fp16 copy of k made by a
-                       pre-pass into `workspace` (without room for it there, or with an entry of q or k beyond
-                       6e4 in magnitude, every iteration uses pairs).  0 = default (1 iteration; 4 for the row
+                       error than the tolerance leaves.  The search direction P is rounded to fp16 before it is used at all, so
+                       its products are exact.  The sweeps read an fp16 copy of k made by a pre-pass into `workspace`
+                       (without room for it there, or with an entry of q or k beyond 6e4 in magnitude, they read the bf16
+                       inputs, and every iteration uses bf16 pairs for both operands).  0 = default (1 iteration; 4 for the row
                        tiles within the first 8 d positions, which converge more slowly); n > 0 = n
-                       iterations for every tile; LLA_CG_PRECISE_ALL = every iteration with pairs;
+                       iterations for every tile; LLA_CG_PRECISE_ALL = every iteration with bf16 pairs;
                        LLA_CG_PRECISE_NONE = fp16 from the first iteration on */
     long long q_strides[3], k_strides[3], v_strides[3], out_strides[3];
                           /* element strides (batch, head, row) of q [B, H, rows, d], k and v [B, kv heads, n, d] and

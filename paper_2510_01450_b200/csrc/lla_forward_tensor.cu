@@ -16,15 +16,16 @@
 //   MMA 2 (TS)     ACC += U_hi B + U_lo B, A operand straight from TMEM, B = the same K block read
 //                  MN-major (or the V block in the output sweep)
 //
-// S/A/U cycle through three TMEM buffers (3 x 128 columns) and ACC takes D more (all 512 columns for
-// D = 128); K/V blocks go through a 4-stage ring (3 stages for D = 128).  Operands wider than 64 columns
+// S/A/U cycle through three TMEM buffers (3 x 128 columns; for D = 128 three for S and U, two for A, and one holds Q) and ACC
+// takes D more (all 512 columns for D = 128); K and V blocks go through a ring of 8 slots (7 for D = 128).  Operands wider than 64 columns
 // are held as 64-column sub-tiles so every tile keeps the 128-byte swizzled row.  For D = 128 the fp32
 // row vectors x, kbar and r do not fit in shared memory or registers next to the operand tiles; each
 // thread keeps its own entries in a global scratch slot owned by the SM (L2-resident, thread-private).  Roles: warps 0-7 compute (warp w owns TMEM lanes 32*(w%4).. and key half w/4 of each
 // block; two threads share a row and exchange partial sums through shared memory), warp 8 issues TMA,
-// warps 9 and 10 issue the two MMA streams.  Every on-the-fly MMA operand (P, y, U) is carried as a bf16 pair hi + lo so
-// the products keep ~16 mantissa bits: a single bf16 rounding of those operands would leave a
-// 2e-3..5e-3 error in the output, above the 2e-3 gate.  Q, K, V are exact bf16 inputs.
+// warps 9 and 10 issue the two MMA streams.  The weights w and c and the solution y are carried as pairs hi + lo of 16-bit
+// values: a single bf16 rounding of those operands would leave a 2e-3..5e-3 error in the output, above the 2e-3 gate.  A search
+// direction P is rounded to one fp16 value per entry before it is used anywhere, so its products carry no rounding at all;
+// U is a pair in the first CG iterations and one fp16 value later.  Q, K, V are exact bf16 inputs.
 //
 // The mathematics is the centred form described in lla_forward_simt.cu (same CG, same freeze rule).
 // All waits on mbarriers are bounded; a wait that expires sets LLA_STATUS_TIMEOUT and the block
@@ -50,42 +51,55 @@ constexpr int TC_THREADS = 384;      // + TMA warp + two MMA warps + an idle war
 constexpr int TC_TMEM_COLS = 512;
 constexpr int TC_NBUF = 3;           // S/A/U buffers in TMEM (128 columns each)
 constexpr int TC_ACC_COL = TC_NBUF * 128;   // ACC columns [384, 384 + D)
-constexpr int TC_R_COL = 0;                 // preconditioner product, between sweeps: R (fp16) in buffer 0's columns,
-constexpr int TC_Z_COL = 128;               // Z = R M (fp32, D columns) from buffer 1's columns on
-constexpr int TC_NST_MAX = 4;
+constexpr int TC_A_COL = 192, TC_Q_COL = 320;   // D = 128: S / U slots at 0, 64, 128, two A slots, then Q as 16-bit pairs
+constexpr int TC_R_COL = 0;                 // preconditioner product, between sweeps: R (fp16, D / 2 columns),
+constexpr int TC_Z_COL = 64;                // Z = R M (fp32, D columns)
+constexpr int TC_SLOT_MAX = 8;
+constexpr int TC_PRE = 4;            // key blocks fetched ahead of a sweep
 constexpr int TC_ORDER_MAX = 256;    // launch-order table size (query tiles)
 constexpr int TC_BLIST_MAX = 1024;   // key blocks a block-sparse tile can list (n <= 65536)
 constexpr int TC_SPLIT_MAX = 4;      // sweeps of at most this many key blocks run in split mode (see the compute role)
 
-// SW_CG16: a CG sweep whose on-the-fly operands (P, U) are single fp16 values instead of bf16 hi + lo pairs
-enum SweepKind : int { SW_STATS = 1, SW_CG = 2, SW_OUT = 3, SW_DONE = 4, SW_CG16 = 5 };
+// SW_CG: a CG sweep on the bf16 inputs, P and U as bf16 hi + lo pairs.  SW_CG16, SW_CG16P: a CG sweep on the fp16 copies,
+// the search direction one fp16 value per entry (exactly: it is rounded before it is used anywhere), U = w (a - abar)
+// single fp16 values or fp16 hi + lo pairs.
+enum SweepKind : int { SW_STATS = 1, SW_CG = 2, SW_OUT = 3, SW_DONE = 4, SW_CG16 = 5, SW_CG16P = 6 };
 
 // Shared-memory carve-up (bytes, from a 1024-byte aligned base), per head size D (64 or 128).
 // Operand tiles are stored as D/64 sub-tiles of 64 columns (128-byte rows, 128B swizzle) one after
 // the other.  For D = 64 the row vectors x and r live in the compute threads' registers and kbar in shared memory as
 // fp32 [D][128] (x in shared memory as well: 96 shared-memory accesses a thread between two sweeps, when nothing else
 // runs on the SM, 2.8 K clocks there instead of 1.9 K); for D = 128 there is no room for any of them, so x, kbar and r
-// live in an L2-resident global scratch slot owned by the SM (one block per SM at a time) and the ring has three stages.
+// live in an L2-resident global scratch slot owned by the SM (one block per SM at a time).
 template <int D>
 struct TcCfg {
     static constexpr int KSUB = D / 64;                         // 64-column sub-tiles per operand row
     static constexpr int NCOL = D / 2;                          // row-vector columns per thread
-    static constexpr int NST = D == 64 ? 4 : 3;                 // K/V ring stages
     static constexpr int QSUB_BYTES = TC_BR * 128;              // one sub-tile of a 128-row operand
     static constexpr int KSUB_BYTES = TC_BC * 128;              // one sub-tile of a 64-key block
     static constexpr int OPER_BYTES = KSUB * QSUB_BYTES;        // Q, P_hi, P_lo
-    static constexpr int KBLK_BYTES = KSUB * KSUB_BYTES;        // K block (V block follows it)
-    static constexpr int STAGE_BYTES = 2 * KBLK_BYTES;
+    static constexpr int KBLK_BYTES = KSUB * KSUB_BYTES;        // a K or V block
+    // Ring slots, each for one K or V block.  A K block stays until its U K^T product is done, and a load takes longer than
+    // a block's products: with three slots for K (and three that only the output sweep used, for V) the D = 128 kernel
+    // waited for keys during 30 % of its time (16 heads, n = 16384: 13.5 -> 12.9 ms).
+    static constexpr int NSLOT = D == 64 ? 8 : 7;
     static constexpr bool STATE_IN_REGS = D == 64;
+    // D = 128: Q is copied to TMEM and S = Q K^T takes it from there: with both operands in shared memory an MMA of N = 64 is
+    // bound by reading them (48 clocks instead of 32).  Its 64 columns come from A having two slots instead of three;
+    // a slot is free as soon as it has been read.  (At D = 64, where the tensor pipe is not what a block waits for,
+    // the same was 2.5 % slower.)
+    static constexpr bool Q_IN_TMEM = D == 128;
+    static __device__ __forceinline__ uint32_t s_col(uint32_t b) { return b * (Q_IN_TMEM ? 64u : 128u); }
+    static __device__ __forceinline__ uint32_t a_col(uint32_t b, uint32_t a) { return Q_IN_TMEM ? TC_A_COL + 64u * (a & 1u) : b * 128u + 64u; }
     static constexpr int SM_Q = 0;
     static constexpr int SM_PHI = SM_Q + OPER_BYTES;
     static constexpr int SM_PLO = SM_PHI + OPER_BYTES;
     static constexpr int SM_KV = SM_PLO + OPER_BYTES;
-    static constexpr int SM_KBAR = SM_KV + NST * STAGE_BYTES;                     // fp32 [D][128] (D = 64 only)
+    static constexpr int SM_KBAR = SM_KV + NSLOT * KBLK_BYTES;                    // fp32 [D][128] (D = 64 only)
     static constexpr int SM_RED = SM_KBAR + (STATE_IN_REGS ? D * TC_BR * 4 : 0);  // pair reductions: 2 buffers x 4 values x 2 x 128 floats
     static constexpr int SM_FLAGS = SM_RED + 8192;                                // 2 x 8 ints
     static constexpr int SM_BAR = SM_FLAGS + 64;                                  // mbarriers
-    static constexpr int SM_MISC = SM_BAR + 256;                                  // tmem base, ctl kind, abort
+    static constexpr int SM_MISC = SM_BAR + 512;                                  // tmem base, ctl kind, abort
     static constexpr int SM_BLIST = SM_MISC + 64;                                 // block-sparse: the tile's key blocks (uint16)
     static constexpr int SM_TOTAL = SM_BLIST + 2 * TC_BLIST_MAX;
     static constexpr int SM_ALLOC = SM_TOTAL + 1024;                              // slack for 1024-byte alignment
@@ -96,14 +110,14 @@ struct TcCfg {
 static_assert(TcCfg<64>::SM_ALLOC <= 227 * 1024 && TcCfg<128>::SM_ALLOC <= 227 * 1024, "shared memory budget");
 
 // mbarrier indices
-enum { B_QFULL = 0, B_KVFULL = 1, B_KVEMPTY = B_KVFULL + TC_NST_MAX, B_VFULL = B_KVEMPTY + TC_NST_MAX,
-       B_SAFULL = B_VFULL + TC_NST_MAX,
+enum { B_QFULL = 0, B_KVFULL = 1, B_KVEMPTY = B_KVFULL + TC_SLOT_MAX, B_SAFULL = B_KVEMPTY + TC_SLOT_MAX,
        B_UFULL = B_SAFULL + TC_NBUF, B_BUFFREE = B_UFULL + TC_NBUF, B_ACCFULL = B_BUFFREE + TC_NBUF, B_CTL = B_ACCFULL + 1,
        B_EXIT = B_CTL + 1,   // two: the MMA warps' last commits on an aborted run
        B_MFULL = B_EXIT + 2, // the preconditioner matrix has landed
        B_XREADY = B_MFULL + 1, B_XFULL = B_XREADY + 1,   // exchange of a pair of blocks: the other's sweep is done, its sums are here
-       B_COUNT = B_XFULL + 1 };
-static_assert(B_COUNT * 8 <= 256, "barrier area too small");
+       B_AFREE = B_XFULL + 1,    // D = 128: an A slot has been read (two slots)
+       B_COUNT = B_AFREE + 2 };
+static_assert(B_COUNT * 8 <= 512, "barrier area too small");
 
 constexpr uint32_t IDESC_SS = make_idesc(TC_BR, TC_BC, 0, 0);   // S/A: A, B K-major; ACC uses make_idesc(128, D, 0, 1)
 constexpr uint32_t IDESC_SS16 = make_idesc(TC_BR, TC_BC, 0, 0, /*f16=*/1);   // the same products with both operands fp16
@@ -155,10 +169,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     using Cfg = TcCfg<D>;
-    constexpr int TC_NST = Cfg::NST, NCOL = Cfg::NCOL, KSUB = Cfg::KSUB;
+    constexpr int NSLOT = Cfg::NSLOT, NCOL = Cfg::NCOL, KSUB = Cfg::KSUB;
     constexpr int SM_Q = Cfg::SM_Q, SM_PHI = Cfg::SM_PHI, SM_PLO = Cfg::SM_PLO, SM_KV = Cfg::SM_KV;
     constexpr int SM_RED = Cfg::SM_RED, SM_FLAGS = Cfg::SM_FLAGS, SM_BAR = Cfg::SM_BAR, SM_MISC = Cfg::SM_MISC;
-    constexpr int STAGE = Cfg::STAGE_BYTES, KBLK = Cfg::KBLK_BYTES;
+    constexpr int KBLK = Cfg::KBLK_BYTES;
     constexpr uint32_t IDESC_TS = Cfg::IDESC_TS, IDESC_TS16 = Cfg::IDESC_TS16;
     const uint32_t sbase = smem_u32(smem);
     const uint32_t bars = sbase + SM_BAR;
@@ -223,12 +237,15 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     const int nblk = prm.block_mask ? misc[6] : cend - cbeg;      // key blocks per sweep
     auto kblock = [&](int c) { return prm.block_mask ? (int)blist[c] : cbeg + c; };     // c-th key block of a sweep
     const bool split = nblk <= TC_SPLIT_MAX;
-    // Operand format of a sweep over the keys.  The statistics sweep(s) and the first `precise` CG sweeps run on
-    // the bf16 inputs; every later sweep (the remaining CG sweeps and, if CG got that far, the output sweep) runs
-    // its Q K^T and P K^T products on fp16 copies of Q and K (one kind::f16 MMA takes both operands in the same
-    // 16-bit format).  The values of the copies equal the bf16 inputs (the pre-pass checks the range).  Every role
-    // counts the CG sweeps it has seen, so all of them know a sweep's format, and the next one's, without being
-    // told.  (Tiles whose rows see fewer than 8 D keys converge more slowly and keep the pairs for longer.)
+    // Ring positions (slot = position % NSLOT) of the blocks of a sweep that starts at position g0: K blocks one after the
+    // other; in the output sweep V blocks too, those of the fetched-ahead K blocks behind them, then K and V in turn.
+    const uint32_t pre = (uint32_t)min(TC_PRE, nblk);
+    auto kpos = [&](uint32_t g0, uint32_t c, bool out) { return out && c >= pre ? g0 + 2 * c : g0 + c; };
+    auto vpos = [&](uint32_t g0, uint32_t c) { return c < pre ? g0 + pre + c : g0 + 2 * c + 1; };
+    // Operand format: with fp16 copies of the inputs (the pre-pass checks that their values are those of the bf16 inputs) every
+    // sweep runs on them, else every sweep runs on the bf16 inputs: one kind::f16 MMA takes both operands in the same
+    // 16-bit format.  The first `precise` CG sweeps carry U as hi + lo pairs.  (Tiles whose rows see fewer than 8 D keys
+    // converge more slowly and keep the pairs for longer.)
     // (A tile of several heads' rows goes by the earliest position in it, at the tiles that a head's rows are cut into
     //  when it is alone: packing heads never takes iterations with pairs from a row.)
     const int first_pos = off + (wraps ? 0 : r0p / TC_BR * TC_BR);
@@ -238,10 +255,9 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 
     if (tid == 0) {
         mbar_init(bar(B_QFULL), 1);
-        for (int s = 0; s < TC_NST; ++s) {
+        for (int s = 0; s < NSLOT; ++s) {
             mbar_init(bar(B_KVFULL + s), 1);
             mbar_init(bar(B_KVEMPTY + s), 1);
-            mbar_init(bar(B_VFULL + s), 1);
         }
         for (int b = 0; b < TC_NBUF; ++b) {
             mbar_init(bar(B_SAFULL + b), 1);
@@ -255,6 +271,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         mbar_init(bar(B_MFULL), 1);
         mbar_init(bar(B_XREADY), TC_COMPUTE / 32);
         mbar_init(bar(B_XFULL), TC_COMPUTE / 32);
+        for (int a = 0; a < 2; ++a) mbar_init(bar(B_AFREE + a), (split ? TC_COMPUTE : TC_COMPUTE / 2) / 32);
         misc[4] = SW_STATS;
         misc[5] = SW_STATS;
         misc[2] = 0;
@@ -290,76 +307,59 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const int bb = bh / prm.H, hq = bh % prm.H, hk = hq / prm.kv_group;
             for (int sub = 0; sub < KSUB; ++sub)
                 tma_load_4d(sbase + SM_Q + sub * Cfg::QSUB_BYTES, &tmQ, bar(B_QFULL), 64 * sub, r0, hq, bb);
-            if (PC) {
-                // the preconditioner of this tile's key range: D x D fp16, laid out like D / 64 key blocks, into the
-                // V halves of the first ring stages (idle until the output sweep, when it is no longer needed)
+            if (PC && f16_on) {
+                // the preconditioner of this tile's key range: D x D fp16, laid out like D / 64 key blocks, in the P_lo tile
+                // (the fp16 CG sweeps do not use it; the output sweep does, when the matrix is no longer needed)
                 const int gm = precond_block_used((prm.causal ? min(n - 1, off + r0 + TC_BR - 1) : n - 1) / 128);
                 mbar_expect_tx(bar(B_MFULL), D * D * 2);
                 for (int rb = 0; rb < D / 64; ++rb)
                     for (int sub = 0; sub < KSUB; ++sub)
-                        tma_load_4d(sbase + SM_KV + rb * STAGE + KBLK + sub * Cfg::KSUB_BYTES, &tmM, bar(B_MFULL), 64 * sub,
+                        tma_load_4d(sbase + SM_PLO + rb * KBLK + sub * Cfg::KSUB_BYTES, &tmM, bar(B_MFULL), 64 * sub,
                                     gm * D + 64 * rb, hk, bb);
             }
-            uint32_t kit = 0;      // K blocks issued so far
-            int pre = 0;           // blocks of the coming sweep already issued
+            uint32_t kit = 0;      // blocks issued so far (the next ring position)
             bool ok = true;
-            auto issue_k = [&](int c, bool f16) {
-                const uint32_t s = kit % TC_NST;
-                if (!mbar_wait(bar(B_KVEMPTY + s), ((kit / TC_NST) & 1) ^ 1, abort_flag, wcap)) { ok = false; return; }
+            const CUtensorMap* tk = f16_on ? &tmK16 : &tmK;
+            auto issue = [&](const CUtensorMap* map, int c) {
+                const uint32_t s = kit % NSLOT;
+                if (!mbar_wait(bar(B_KVEMPTY + s), ((kit / NSLOT) & 1) ^ 1, abort_flag, wcap)) { ok = false; return; }
                 mbar_expect_tx(bar(B_KVFULL + s), KBLK);
                 for (int sub = 0; sub < KSUB; ++sub)
-                    tma_load_4d(sbase + SM_KV + s * STAGE + sub * Cfg::KSUB_BYTES, f16 ? &tmK16 : &tmK, bar(B_KVFULL + s), 64 * sub,
+                    tma_load_4d(sbase + SM_KV + s * KBLK + sub * Cfg::KSUB_BYTES, map, bar(B_KVFULL + s), 64 * sub,
                                 kblock(c) * TC_BC, hk, bb);
                 ++kit;
             };
-            uint32_t v_g0 = 0;
-            int v_issued = 0;      // V blocks issued (output sweep only), the first at ring position v_g0
-            auto issue_v = [&](int c, uint32_t g) {
-                if (v_issued == 0) v_g0 = g - c;
-                v_issued = c + 1;
-                const uint32_t s = g % TC_NST;
-                mbar_expect_tx(bar(B_VFULL + s), KBLK);
-                for (int sub = 0; sub < KSUB; ++sub)
-                    tma_load_4d(sbase + SM_KV + s * STAGE + KBLK + sub * Cfg::KSUB_BYTES, &tmV, bar(B_VFULL + s), 64 * sub, kblock(c) * TC_BC, hk, bb);
+            // first blocks of the next sweep, whatever kind it turns out to be
+            auto prefetch = [&]() {
+                for (int c = 0; c < (int)pre && ok; ++c) issue(tk, c);
             };
-            int cg_seen = 0;       // CG sweeps issued so far
+            prefetch();
+            uint32_t pre_out = pre;      // blocks fetched ahead and not announced yet
             for (uint32_t ctl = 0; ok; ++ctl) {
                 if (!mbar_wait(bar(B_CTL), ctl & 1, abort_flag, wcap)) break;
                 const int kind = misc[4 + (ctl & 1)];
                 if (kind == SW_DONE) {
-                    // prefetched blocks nobody will consume: wait until they have landed
-                    for (int i = 0; i < pre; ++i) {
-                        const uint32_t g = kit - pre + i;
-                        if (!mbar_wait(bar(B_KVFULL + g % TC_NST), (g / TC_NST) & 1, abort_flag, wcap)) break;
-                    }
+                    // fetched-ahead blocks nobody will consume: wait until they have landed
+                    for (uint32_t g = kit - pre_out; g < kit; ++g)
+                        if (!mbar_wait(bar(B_KVFULL + g % NSLOT), (g / NSLOT) & 1, abort_flag, wcap)) break;
                     break;
                 }
-                const uint32_t g0 = kit - pre;
                 if (kind == SW_OUT)
-                    for (int c = 0; c < pre; ++c) issue_v(c, g0 + c);
-                const bool f16_cur = kind == SW_CG16 || (kind == SW_OUT && f16_on && cg_seen >= precise);
-                for (int c = pre; c < nblk && ok; ++c) {
-                    issue_k(c, f16_cur);
-                    if (ok && kind == SW_OUT) issue_v(c, g0 + c);
+                    for (int c = 0; c < (int)pre && ok; ++c) issue(&tmV, c);
+                for (int c = (int)pre; c < nblk && ok; ++c) {
+                    issue(tk, c);
+                    if (ok && kind == SW_OUT) issue(&tmV, c);
                 }
-                pre = 0;
-                if (kind == SW_CG || kind == SW_CG16) ++cg_seen;
-                // first blocks of the next sweep, in the format it will have.  After a statistics sweep the next one
-                // is another statistics sweep, the first CG sweep or the output sweep: all on the bf16 inputs unless
-                // precise == 0, where nothing is fetched ahead
-                const bool f16_next = f16_on && cg_seen >= precise;
-                if (kind != SW_OUT && !(kind == SW_STATS && f16_next))
-                    for (int c = 0; c < min(TC_NST, nblk) && ok; ++c) { issue_k(c, f16_next); ++pre; }
+                pre_out = 0;
+                if (kind != SW_OUT) { prefetch(); pre_out = pre; }
             }
             if (*abort_flag) {
-                if (PC) (void)mbar_wait_landed(bar(B_MFULL), 0, wcap);
+                if (PC && f16_on) (void)mbar_wait_landed(bar(B_MFULL), 0, wcap);
                 // an aborted block: the copies issued above write into this block's shared memory, so they must
                 // have landed before the block exits (on a completed run their consumers have waited for them)
                 (void)mbar_wait_landed(bar(B_QFULL), 0, wcap);
-                for (uint32_t g = kit > (uint32_t)TC_NST ? kit - TC_NST : 0; g < kit; ++g)
-                    (void)mbar_wait_landed(bar(B_KVFULL + g % TC_NST), (g / TC_NST) & 1, wcap);
-                for (int c = max(0, v_issued - TC_NST); c < v_issued; ++c)
-                    (void)mbar_wait_landed(bar(B_VFULL + (v_g0 + c) % TC_NST), (c / TC_NST) & 1, wcap);
+                for (uint32_t g = kit > (uint32_t)NSLOT ? kit - NSLOT : 0; g < kit; ++g)
+                    (void)mbar_wait_landed(bar(B_KVFULL + g % NSLOT), (g / NSLOT) & 1, wcap);
             }
         }
     } else if (warp == 9) {
@@ -378,39 +378,48 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const uint64_t qdesc = make_desc(sb_u + SM_Q);
         const uint64_t phdesc = make_desc(sb_u + SM_PHI);
         const uint64_t pldesc = make_desc(sb_u + SM_PLO);
-        uint32_t it = 0;   // global block counter (stage = it % NST, buffer = it % NBUF)
-        int cg_seen = 0;   // CG sweeps issued so far
+        const uint32_t idesc = f16_on ? IDESC_SS16 : IDESC_SS;
+        uint32_t it = 0;   // global block counter (buffer = it % NBUF)
+        uint32_t g0 = 0;   // ring position of the sweep's first block
+        uint32_t at = 0;   // the same for the blocks with a product A (D = 128: slot = at % 2)
         for (uint32_t ctl = 0; ok; ++ctl) {
             if (!mbar_wait(bar(B_CTL), ctl & 1, abort_flag, wcap)) break;
             const int kind = misc[4 + (ctl & 1)];
             if (kind == SW_DONE) break;
             tc_fence_after();
-            const uint32_t idesc = (kind == SW_CG16 || (kind == SW_OUT && f16_on && cg_seen >= precise)) ? IDESC_SS16 : IDESC_SS;
-            if (kind == SW_CG || kind == SW_CG16) ++cg_seen;
             for (int c = 0; c < nblk && ok; ++c, ++it) {
-                const uint32_t s = it % TC_NST, b = it % TC_NBUF, bu = it / TC_NBUF;
-                if (!mbar_wait(bar(B_KVFULL + s), (it / TC_NST) & 1, abort_flag, wcap)) { ok = false; break; }
+                const uint32_t g = kpos(g0, c, kind == SW_OUT), s = g % NSLOT, b = it % TC_NBUF, bu = it / TC_NBUF;
+                if (!mbar_wait(bar(B_KVFULL + s), (g / NSLOT) & 1, abort_flag, wcap)) { ok = false; break; }
                 if (!mbar_wait(bar(B_BUFFREE + b), (bu & 1) ^ 1, abort_flag, wcap)) { ok = false; break; }
                 tc_fence_after();
-                const uint64_t kdesc = make_desc(sb_u + SM_KV + s * STAGE);
-                const uint32_t s_tm = tm_u + b * 128, a_tm = s_tm + 64;
+                const uint64_t kdesc = make_desc(sb_u + SM_KV + s * KBLK);
+                const uint32_t s_tm = tm_u + Cfg::s_col(b), a_tm = tm_u + Cfg::a_col(b, at);
                 // contraction over D: one group of four 16-wide steps per 64-column sub-tile
                 // (sub-tiles are QSUB_BYTES / KSUB_BYTES apart: 1024 / 512 descriptor units)
 #pragma unroll
-                for (int sub = 0; sub < KSUB; ++sub)
-                    mma_ss_k64(el, s_tm, qdesc + sub * (Cfg::QSUB_BYTES >> 4), kdesc + sub * (Cfg::KSUB_BYTES >> 4), idesc, sub > 0);
-                if (kind == SW_CG || kind == SW_OUT || kind == SW_CG16) {
+                for (int sub = 0; sub < KSUB; ++sub) {
+                    if constexpr (Cfg::Q_IN_TMEM) mma_ts_kmajor_k64(el, s_tm, tm_u + TC_Q_COL + 32 * sub, kdesc + sub * (Cfg::KSUB_BYTES >> 4), idesc, sub > 0);
+                    else mma_ss_k64(el, s_tm, qdesc + sub * (Cfg::QSUB_BYTES >> 4), kdesc + sub * (Cfg::KSUB_BYTES >> 4), idesc, sub > 0);
+                }
+                if (kind != SW_STATS) {
+                    if (Cfg::Q_IN_TMEM) {
+                        if (!mbar_wait(bar(B_AFREE + (at & 1)), ((at >> 1) & 1) ^ 1, abort_flag, wcap)) { ok = false; break; }
+                        tc_fence_after();
+                        ++at;
+                    }
 #pragma unroll
                     for (int sub = 0; sub < KSUB; ++sub)
                         mma_ss_k64(el, a_tm, phdesc + sub * (Cfg::QSUB_BYTES >> 4), kdesc + sub * (Cfg::KSUB_BYTES >> 4), idesc, sub > 0);
-                    if (kind != SW_CG16) {     // second half of the operand pair
+                    if (kind == SW_CG || kind == SW_OUT) {     // second half of the operand pair
 #pragma unroll
                         for (int sub = 0; sub < KSUB; ++sub)
                             mma_ss_k64(el, a_tm, pldesc + sub * (Cfg::QSUB_BYTES >> 4), kdesc + sub * (Cfg::KSUB_BYTES >> 4), idesc, 1);
                     }
                 }
                 tc_commit_el(el, bar(B_SAFULL + b));
+                if (kind == SW_OUT) tc_commit_el(el, bar(B_KVEMPTY + s));      // (else the key block is needed once more)
             }
+            g0 += kind == SW_OUT ? 2 * nblk : nblk;
         }
         if (*abort_flag) {      // an aborted block: the MMAs this warp issued must be done before TMEM and shared memory go
             tc_commit_el(el, bar(B_EXIT + 0));
@@ -423,24 +432,26 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         const uint32_t sb_u = __shfl_sync(0xffffffffu, sbase, 0);
         const uint32_t tm_u = __shfl_sync(0xffffffffu, tmem, 0);
         bool ok = true;
-        uint32_t it = 0;
+        uint32_t it = 0, g0 = 0;
         for (uint32_t ctl = 0; ok; ++ctl) {
             if (!mbar_wait(bar(B_CTL), ctl & 1, abort_flag, wcap)) break;
             const int kind = misc[4 + (ctl & 1)];
             if (kind == SW_DONE) break;
             for (int c = 0; c < nblk && ok; ++c, ++it) {
-                const uint32_t s = it % TC_NST, b = it % TC_NBUF, bu = it / TC_NBUF;
+                const uint32_t g = kind == SW_OUT ? vpos(g0, c) : kpos(g0, c, false), s = g % NSLOT, b = it % TC_NBUF, bu = it / TC_NBUF;
                 if (!mbar_wait(bar(B_UFULL + b), bu & 1, abort_flag, wcap)) { ok = false; break; }
-                if (kind == SW_OUT && !mbar_wait(bar(B_VFULL + s), (c / TC_NST) & 1, abort_flag, wcap)) { ok = false; break; }
+                if (kind == SW_OUT && !mbar_wait(bar(B_KVFULL + s), (g / NSLOT) & 1, abort_flag, wcap)) { ok = false; break; }
                 tc_fence_after();
-                const uint32_t bsm = sb_u + SM_KV + s * STAGE + (kind == SW_OUT ? KBLK : 0);
+                const uint32_t bsm = sb_u + SM_KV + s * KBLK;
                 // B = the K (or V) block read MN-major, N = D: 64-wide column groups are one sub-tile apart
-                if (kind == SW_CG16) mma_ts_k64(el, tm_u + TC_ACC_COL, tm_u + b * 128, make_desc(bsm, Cfg::KSUB_BYTES), IDESC_TS16, c > 0);
-                else mma_ts_hilo_k64(el, tm_u + TC_ACC_COL, tm_u + b * 128, make_desc(bsm, Cfg::KSUB_BYTES), IDESC_TS, c > 0);
+                if (kind == SW_CG16) mma_ts_k64(el, tm_u + TC_ACC_COL, tm_u + Cfg::s_col(b), make_desc(bsm, Cfg::KSUB_BYTES), IDESC_TS16, c > 0);
+                else mma_ts_hilo_k64(el, tm_u + TC_ACC_COL, tm_u + Cfg::s_col(b), make_desc(bsm, Cfg::KSUB_BYTES),
+                                     f16_on && kind != SW_OUT ? IDESC_TS16 : IDESC_TS, c > 0);
                 tc_commit_el(el, bar(B_KVEMPTY + s));
                 tc_commit_el(el, bar(B_BUFFREE + b));
                 if (c == nblk - 1) tc_commit_el(el, bar(B_ACCFULL));
             }
+            g0 += kind == SW_OUT ? 2 * nblk : nblk;
         }
         if (*abort_flag) {      // an aborted block: the MMAs this warp issued must be done before TMEM and shared memory go
             tc_commit_el(el, bar(B_EXIT + 1));
@@ -484,20 +495,6 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             pair_sync();
             a = buf[lrow] + buf[128 + lrow];
             b = buf[256 + lrow] + buf[384 + lrow];
-        };
-        // four sums for one barrier
-        auto pair_sum4 = [&](float& a, float& b, float& c, float& d4) {
-            float* buf = red + red_sel * 1024;
-            red_sel ^= 1;
-            buf[half * 128 + lrow] = a;
-            buf[256 + half * 128 + lrow] = b;
-            buf[512 + half * 128 + lrow] = c;
-            buf[768 + half * 128 + lrow] = d4;
-            pair_sync();
-            a = buf[lrow] + buf[128 + lrow];
-            b = buf[256 + lrow] + buf[384 + lrow];
-            c = buf[512 + lrow] + buf[640 + lrow];
-            d4 = buf[768 + lrow] + buf[896 + lrow];
         };
         auto pair_max = [&](float v) {
             float* buf = red + red_sel * 1024;
@@ -546,37 +543,51 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 *reinterpret_cast<uint4*>(smem + SM_PLO + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
         };
-        // Q tile: bf16 as loaded, or fp16 once the sweeps have switched format (converted in place by
-        // convert_q, each thread its own chunks, between two sweeps when no MMA reads the tile)
-        bool q_is_f16 = false;
+        // Q tile: bf16 as loaded, or fp16 (converted in place by prepare_q, each thread its own chunks)
         auto q_elem = [&](const uint32_t* qw, int e) -> float {
-            if (q_is_f16) {
+            if (f16_on) {
                 const __half2 h2 = *reinterpret_cast<const __half2*>(&qw[e >> 1]);
                 return (e & 1) ? __high2float(h2) : __low2float(h2);
             }
             return (e & 1) ? __uint_as_float(qw[e >> 1] & 0xFFFF0000u) : __uint_as_float(qw[e >> 1] << 16);
         };
-        auto convert_q = [&]() {
+        // before the first sweep: Q in the format of the sweeps, and at D = 128 to TMEM
+        auto prepare_q = [&]() {
+            uint32_t qt[Cfg::Q_IN_TMEM ? NCOL / 2 : 1];
 #pragma unroll
             for (int ch = 0; ch < NCOL / 8; ++ch) {
                 uint4* qp = reinterpret_cast<uint4*>(smem + SM_Q + oper_off(ch));
                 const uint4 qraw = *qp;
-                const uint32_t qw[4] = {qraw.x, qraw.y, qraw.z, qraw.w};
-                uint32_t h[4];
+                uint32_t qw[4] = {qraw.x, qraw.y, qraw.z, qraw.w};
+                if (f16_on) {
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    h[e] = pack_f16(__uint_as_float(qw[e] << 16), __uint_as_float(qw[e] & 0xFFFF0000u));
-                *qp = make_uint4(h[0], h[1], h[2], h[3]);
+                    for (int e = 0; e < 4; ++e)
+                        qw[e] = pack_f16(__uint_as_float(qw[e] << 16), __uint_as_float(qw[e] & 0xFFFF0000u));
+                    *qp = make_uint4(qw[0], qw[1], qw[2], qw[3]);
+                }
+                if constexpr (Cfg::Q_IN_TMEM) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) qt[4 * ch + e] = qw[e];
+                }
             }
-            q_is_f16 = true;
+            if constexpr (Cfg::Q_IN_TMEM) {
+                tmem_st32(tmem + lane_addr + TC_Q_COL + 32 * half, qt);
+                tc_wait_st();
+                tc_fence_before();
+            }
         };
-        // the same vector as one fp16 value per entry, scaled by the power of two sc (see write_p)
-        auto write_operand16 = [&](const float* vec, float sc) {
+        // vec rounded to fp16 after scaling by the power of two sc (isc = 1 / sc; see write_p), in the operand tile and in vec itself
+        auto write_operand16 = [&](float* vec, float sc, float isc) {
 #pragma unroll
             for (int ch = 0; ch < NCOL / 8; ++ch) {
                 uint32_t h[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) h[e] = pack_f16(vec[ch * 8 + 2 * e] * sc, vec[ch * 8 + 2 * e + 1] * sc);
+                for (int e = 0; e < 4; ++e) {
+                    h[e] = pack_f16(vec[ch * 8 + 2 * e] * sc, vec[ch * 8 + 2 * e + 1] * sc);
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[e]));
+                    vec[ch * 8 + 2 * e] = f.x * isc;
+                    vec[ch * 8 + 2 * e + 1] = f.y * isc;
+                }
                 *reinterpret_cast<uint4*>(smem + SM_PHI + oper_off(ch)) = make_uint4(h[0], h[1], h[2], h[3]);
             }
         };
@@ -585,26 +596,34 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         float mx2 = -INFINITY, omega = 0.f, inv_omega = 0.f, ridge = 0.f, den = 0.f;
         float abar = 0.f;                                     // kbar.p (CG) or kbar.y (output)
         // fp16 sweeps: the search direction is stored as p * psc with psc a power of two that brings |p| to
-        // [1, 2.83), so that its entries and u = w (a - abar) sit in the middle of the fp16 range whatever the
-        // scale of the right-hand side; pn2 tracks |p|^2 through the recurrence |p'|^2 = |r'|^2 + beta^2 |p|^2
+        // [1, 2.83) over the row's largest weight (where that is above one), so that its entries and u = w (a - abar) sit in
+        // the middle of the fp16 range whatever the scale of the right-hand side; pn2 tracks |p|^2 through the recurrence
+        // |p'|^2 = |r'|^2 + beta^2 |p|^2
         float pn2 = 0.f, psc = 1.f, ipsc = 1.f;
+        int wexp = 0;                                         // largest weight of the row is at most 2^wexp
+        uint32_t ablk = 0;                                    // blocks with a product A so far (D = 128: slot = ablk % 2)
         float smax = -INFINITY;                               // statistics sweep: largest score of the row, relative to the shift
         uint32_t blk = 0;                                     // global block counter (buffer = blk & 1)
         bool ok = true;
 
-        // One sweep over the key blocks.  kind is uniform over the block.
+        // One sweep over the key blocks: an instance of the loop per kind (and, for the statistics, format), so that it
+        // carries no branches on them.
         // Long sweeps: warps 0-3 (group 0) take the even blocks, warps 4-7 (group 1) the odd ones,
         // each thread all 64 keys of its row in two passes of 32: the two warps that share a
         // scheduler are then in different phases of the load -> math -> store chain and hide each
         // other's latency.  Short sweeps (split mode, the first query tiles) are latency-bound
         // instead: there both groups work on every block, each thread on its half of the keys, which
         // halves the time from a block's scores to its contribution.
-        auto sweep = [&](int kind) {
+        auto sweep_of = [&](auto kind_c, auto f16_c) {
+            constexpr int kind = decltype(kind_c)::value;
+            constexpr bool f16 = decltype(f16_c)::value;
             float part = 0.f;                                 // omega / den partial
             const uint64_t c1c1 = pk2(c1, c1), nmx = pk2(-mx2, -mx2);
-            const float ab_s = kind == SW_CG16 ? abar * psc : abar;
+            const float ab_s = kind == SW_CG16 || kind == SW_CG16P ? abar * psc : abar;
             const uint64_t nab = pk2(-ab_s, -ab_s), oab = pk2(1.f + abar, 1.f + abar), neg1 = pk2(-1.f, -1.f);
             uint64_t part2 = pk2(0.f, 0.f);
+            const uint32_t a0 = ablk;
+            if (kind != SW_STATS) ablk += nblk;
             for (int c = 0; c < nblk; ++c, ++blk) {
                 if (!split && (int)(blk & 1) != half) continue;
                 const uint32_t b = blk % TC_NBUF;
@@ -612,11 +631,16 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 tc_fence_after();
 #pragma unroll 1
                 for (int h = split ? half : 0; h < (split ? half + 1 : 2); ++h) {
-                    const uint32_t s_addr = tmem + lane_addr + b * 128 + 32 * h;
+                    const uint32_t s_addr = tmem + lane_addr + Cfg::s_col(b) + 32 * h;
                     uint32_t sv[32], av[32];
                     tmem_ld32(s_addr, sv);
-                    if (kind == SW_CG || kind == SW_OUT || kind == SW_CG16) tmem_ld32(s_addr + 64, av);
+                    if (kind != SW_STATS) tmem_ld32(tmem + lane_addr + Cfg::a_col(b, a0 + c) + 32 * h, av);
                     tc_wait_ld();
+                    if (Cfg::Q_IN_TMEM && kind != SW_STATS && (split || h == 1)) {      // the A slot has been read
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(B_AFREE + ((a0 + c) & 1)));
+                    }
                     // keys jfirst <= e < jlim of this half block are visible.  Only the diagonal blocks and a
                     // window's first blocks hide any: there the hidden scores are overwritten with a large negative
                     // number, whose weight is exactly zero, so the loops below carry no mask
@@ -651,16 +675,17 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                             upk2(t2, t0, t1);
                             if (kind == SW_STATS) smax = fmaxf(smax, fmaxf(t0, t1));     // largest score, relative to the shift
                             uint64_t u2 = pk2(ex2f(t0), ex2f(t1));
-                            if (kind == SW_CG)
+                            if (kind == SW_CG || kind == SW_CG16P)
                                 u2 = mul2(u2, add2(pk2(__uint_as_float(av[2 * e2]), __uint_as_float(av[2 * e2 + 1])), nab));
                             if (kind == SW_OUT)
                                 u2 = mul2(u2, fma2(pk2(__uint_as_float(av[2 * e2]), __uint_as_float(av[2 * e2 + 1])), neg1, oab));
                             float u0, u1;
                             upk2(u2, u0, u1);
-                            if (kind != SW_CG) part2 = add2(part2, u2);
+                            if (kind == SW_STATS || kind == SW_OUT) part2 = add2(part2, u2);
                             // 16 keys per k-step: 8 columns of hi, then 8 columns of lo
                             const int ks = e2 >> 3, e = e2 & 7;
-                            pk[ks * 16 + e] = split_bf16x2(u0, u1, pk[ks * 16 + 8 + e]);
+                            if (f16) pk[ks * 16 + e] = split_f16x2(u0, u1, pk[ks * 16 + 8 + e]);
+                            else pk[ks * 16 + e] = split_bf16x2(u0, u1, pk[ks * 16 + 8 + e]);
                         }
                         tmem_st32(s_addr, pk);
                     }
@@ -675,6 +700,15 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             upk2(part2, p0, p1);
             part = p0 + p1;
             return part;
+        };
+        auto sweep_stats = [&]() {
+            return f16_on ? sweep_of(std::integral_constant<int, SW_STATS>{}, std::true_type{})
+                          : sweep_of(std::integral_constant<int, SW_STATS>{}, std::false_type{});
+        };
+        auto sweep_cg = [&](int kind) {
+            if (kind == SW_CG16) (void)sweep_of(std::integral_constant<int, SW_CG16>{}, std::true_type{});
+            else if (kind == SW_CG16P) (void)sweep_of(std::integral_constant<int, SW_CG16P>{}, std::true_type{});
+            else (void)sweep_of(std::integral_constant<int, SW_CG>{}, std::false_type{});
         };
         // read this thread's NCOL ACC columns after the sweep's last MMA
         uint32_t acc_uses = 0;
@@ -733,8 +767,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             b = fmaxf(b, xsc[256 + tid]);
         };
         uint32_t ctl_phase = 0;
-        auto start_sweep = [&](int kind, bool f16 = false) {
-            if (f16 && !q_is_f16) convert_q();
+        auto start_sweep = [&](int kind) {
             if (tid == 0) misc[4 + (ctl_phase & 1)] = kind;
             ++ctl_phase;
             fence_proxy_async();       // operand tiles written with ordinary stores -> visible to the MMA
@@ -763,19 +796,52 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         float rr = 0.f, stop = 0.f;
         int its = 0;
         bool active = false;
-        // P operand of CG iteration t: bf16 hi + lo for the first precise_iters iterations, one fp16 after
-        // (the products of an iteration enter x and r scaled by |p|, which has fallen by then: the coarser
-        // operands of the later iterations cost no accuracy that the early ones have not already spent)
-        auto write_p = [&](int t) {
-            if (f16_on && t >= precise) {
+        // P operand of a CG iteration.  On fp16 copies of the inputs the direction itself is rounded to fp16 first, and the rounded
+        // vector is the one that enters x, r and the products: A = P K^T then carries no rounding of P at all, for half
+        // the products of a hi + lo pair (32 heads, n = 4096, d = 64: 1394 -> 1350 us, and the error against float64 falls from
+        // 1.5e-4 to 0.9e-4).  (Directions that are off by 2^-12 cost conjugacy, not consistency: x and r still
+        // belong together.)  What is left is the rounding of U, whose errors average over the keys.
+        auto write_p = [&]() {
+            if (f16_on) {
                 const int e2 = (int)((__float_as_uint(pn2) >> 23) & 0xffu) - 127;      // floor(log2 |p|^2)
-                const int k = max(-100, min(100, -(e2 >> 1)));
+                const int k = max(-100, min(100, -(e2 >> 1) - wexp));
                 psc = __uint_as_float((uint32_t)(127 + k) << 23);
                 ipsc = __uint_as_float((uint32_t)(127 - k) << 23);
-                write_operand16(p, psc);
+                write_operand16(p, psc, ipsc);
             } else {
                 write_operand(p);
             }
+        };
+        // D = 128: the search direction is not kept in registers over a sweep but read back from its operand tiles
+        auto reload_p = [&]() {
+#pragma unroll
+            for (int ch = 0; ch < NCOL / 8; ++ch) {
+                const uint4 h4 = *reinterpret_cast<const uint4*>(smem + SM_PHI + oper_off(ch));
+                const uint32_t h[4] = {h4.x, h4.y, h4.z, h4.w};
+                if (f16_on) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h[e]));
+                        p[ch * 8 + 2 * e] = f.x * ipsc;
+                        p[ch * 8 + 2 * e + 1] = f.y * ipsc;
+                    }
+                } else {
+                    const uint4 l4 = *reinterpret_cast<const uint4*>(smem + SM_PLO + oper_off(ch));
+                    const uint32_t l[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        p[ch * 8 + 2 * e] = __uint_as_float(h[e] << 16) + __uint_as_float(l[e] << 16);
+                        p[ch * 8 + 2 * e + 1] = __uint_as_float(h[e] & 0xFFFF0000u) + __uint_as_float(l[e] & 0xFFFF0000u);
+                    }
+                }
+            }
+        };
+        // kbar . p, once the sweep that needs it has been announced: the first products are on their way meanwhile
+        auto kbar_dot = [&](const float* vec) {
+            float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int e = 0; e < NCOL; ++e) s4[e & 3] = fmaf(kbs[(c0 + e) * TC_BR + lrow], vec[e], s4[e & 3]);
+            return pair_sum((s4[0] + s4[1]) + (s4[2] + s4[3]));
         };
 
         // z = M r with the tile's preconditioner: vec holds this thread's NCOL entries of r on entry (|r|^2 is about
@@ -806,7 +872,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
                     for (int rb = 0; rb < D / 64; ++rb)
                         mma_ts_k64c(el0, tm_c + TC_Z_COL, tm_c + TC_R_COL + 32 * rb,
-                                    make_desc(sb_c + SM_KV + rb * STAGE + KBLK, Cfg::KSUB_BYTES), IDESC_TS16, rb > 0);
+                                    make_desc(sb_c + SM_PLO + rb * KBLK, Cfg::KSUB_BYTES), IDESC_TS16, rb > 0);
                     tc_commit_el(el0, bar(B_ACCFULL));
                 }
             }
@@ -836,6 +902,8 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         {
             float part = 0.f;
             mx2 = 0.f;
+            ok = all_ok(mbar_wait(bar(B_QFULL), 0, abort_flag, wcap));
+            if (ok) prepare_q();
             // (solve mode with the row statistics given: nothing to sweep for)
             constexpr bool given = GIVEN;
             if (given && row_ok) {
@@ -845,7 +913,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             for (int attempt = 0; attempt < 2 && ok && !given; ++attempt) {
                 smax = -INFINITY;
                 start_sweep(SW_STATS);
-                part = sweep(SW_STATS);
+                part = sweep_stats();
                 if (ok) acc_wait();
                 ok = all_ok(ok);
                 if (!ok) break;
@@ -875,12 +943,13 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     }
                     omega = pair_sum(part);
                 }
+                wexp = given ? 0 : (int)fminf(fmaxf(ceilf(tmax - mx2), 0.f), 8.f);
                 inv_omega = 1.f / omega;
                 const float lam_i = (prm.lambda_rows && row < nq) ? prm.lambda_rows[(size_t)bh * nq + row] : prm.lambda;
                 // ridge in the frame of the shift: lambda e^{-shift} by the definition; the printed algorithm adds
                 // lambda in the frame of the row maximum, i.e. lambda e^{max - shift} here
                 ridge = lam_i * ex2f((prm.ridge_mode == LLA_RIDGE_PRINTED ? tmax : 0.f) - mx2) * inv_omega;
-                float rr_p = 0.f, ab_p = 0.f;
+                float rr_p = 0.f;
 #pragma unroll
                 for (int ch = 0; ch < NCOL / 8; ++ch) {
                     const uint4 qraw = *reinterpret_cast<const uint4*>(smem + SM_Q + oper_off(ch));
@@ -896,35 +965,34 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         r_set(col, bv);
                         p[col] = bv;
                         rr_p += bv * bv;
-                        ab_p += kb * bv;
                     }
                 }
                 rr = pair_sum(rr_p);
-                abar = pair_sum(ab_p);
                 stop = prm.tol * prm.tol * rr;
                 active = row_ok && rr > 0.f;
                 pn2 = rr;
                 rz = rr;
             }
         }
-        if (ok && PC) {
-            // preconditioned start: p = z = M r, with r . z, kbar . z and |z|^2 for the recurrences
+        const bool pc_on = PC && f16_on;      // (an input outside the fp16 range: plain CG on operand pairs, which need the P_lo tile)
+        if (PC && !pc_on) prec_row = false;
+        if (ok && pc_on) {
+            // preconditioned start: p = z = M r, with r . z and |z|^2 for the recurrences
             precondition(p, rr);
             ok = all_ok(ok);
             if (ok) {
-                float rz_p = 0.f, kz_p = 0.f, zz_p = 0.f, unused = 0.f;
+                float rz_p = 0.f, zz_p = 0.f;
 #pragma unroll
                 for (int e = 0; e < NCOL; ++e) {
                     rz_p = fmaf(r_get(e), p[e], rz_p);
-                    kz_p = fmaf(kbs[(c0 + e) * TC_BR + lrow], p[e], kz_p);
                     zz_p = fmaf(p[e], p[e], zz_p);
                 }
-                pair_sum4(rz_p, kz_p, zz_p, unused);
+                pair_sum2(rz_p, zz_p);
                 if (rz_p > 0.f) {
-                    rz = rz_p; abar = kz_p; pn2 = zz_p;
+                    rz = rz_p; pn2 = zz_p;
                 } else {
                     // the rounded matrix is not positive on this residual: the row runs unpreconditioned
-                    // (abar, pn2 and rz already hold the values for p = r)
+                    // (pn2 and rz already hold the values for p = r)
                     prec_row = false;
 #pragma unroll
                     for (int e = 0; e < NCOL; ++e) p[e] = r_get(e);
@@ -934,12 +1002,14 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // ---- conjugate gradients (Algorithm 2) ----
         auto still_active = [&]() { return active = active && rr > stop; };
         auto cg_pass = [&](int t) -> bool {
-            const bool cheap = f16_on && t >= precise;
+            const int kind = !f16_on ? SW_CG : t < precise ? SW_CG16P : SW_CG16;
             // (behind the vote, which all compute threads take: in a pair of blocks the other block's sums, which lie
             //  over the operand tiles in another layout, have been read by everyone then)
-            write_p(t);
-            start_sweep(cheap ? SW_CG16 : SW_CG, cheap);
-            sweep(cheap ? SW_CG16 : SW_CG);
+            write_p();
+            start_sweep(kind);
+            abar = kbar_dot(p);
+            sweep_cg(kind);
+            if constexpr (!Cfg::STATE_IN_REGS) reload_p();
             if (ok) acc_wait();
             if (PC) {
                 ok = all_ok(ok);
@@ -955,7 +1025,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             // (the loops below keep four independent partial sums and move the row-vector state in
             //  batches of eight so that the loads overlap: two warps per scheduler hide no latency)
             float pp[4] = {0.f, 0.f, 0.f, 0.f};
-            const float acc_scale = cheap ? inv_omega * ipsc : inv_omega;
+            const float acc_scale = f16_on ? inv_omega * ipsc : inv_omega;
 #pragma unroll
             for (int e = 0; e < NCOL; ++e) {
                 ap[e] = fmaf(ap[e], acc_scale, ridge * p[e]);
@@ -964,14 +1034,13 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const float pap = pair_sum((pp[0] + pp[1]) + (pp[2] + pp[3]));
             if (active && !(pap > 0.f)) active = false;
             const float alpha = active ? rz / pap : 0.f;       // rz = |r|^2 without a preconditioner
-            float r2[4] = {0.f, 0.f, 0.f, 0.f}, kr[4] = {0.f, 0.f, 0.f, 0.f};
+            float r2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int e0 = 0; e0 < NCOL; e0 += 8) {
-                float xv[8], kv[8], rv[8];
+                float xv[8], rv[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     xv[i] = x_get(e0 + i);
-                    kv[i] = kbs[(c0 + e0 + i) * TC_BR + lrow];
                     rv[i] = r_get(e0 + i);
                 }
 #pragma unroll
@@ -980,7 +1049,6 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     rv[i] = fmaf(-alpha, ap[e0 + i], rv[i]);
                     ap[e0 + i] = rv[i];                       // ap now holds the new residual
                     r2[i & 3] = fmaf(rv[i], rv[i], r2[i & 3]);
-                    kr[i & 3] = fmaf(kv[i], rv[i], kr[i & 3]);
                 }
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
@@ -988,15 +1056,12 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     r_set(e0 + i, rv[i]);
                 }
             }
-            float rr2 = (r2[0] + r2[1]) + (r2[2] + r2[3]), kbr = (kr[0] + kr[1]) + (kr[2] + kr[3]);
+            float rr2 = pair_sum((r2[0] + r2[1]) + (r2[2] + r2[3]));
             if constexpr (!PC) {
-                // ||r_new||^2 and kbar . r_new in one exchange; kbar . p_new follows from the recurrence
-                pair_sum2(rr2, kbr);
                 if (active) {
                     const float beta = rr2 / rr;
 #pragma unroll
                     for (int e = 0; e < NCOL; ++e) p[e] = fmaf(beta, p[e], ap[e]);
-                    abar = fmaf(beta, abar, kbr);
                     pn2 = fmaf(beta * beta, pn2, rr2);
                     rr = rr2;
                     rz = rr2;
@@ -1004,29 +1069,26 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
             } else {
                 // preconditioned: z = M r_new (ap <- z), then beta = (r_new . z_new) / (r . z), p = z + beta p;
-                // kbar . p and a bound on |p| follow from kbar . z and |z|
-                rr2 = pair_sum(rr2);
-                precondition(ap, rr2);
-                ok = all_ok(ok);
-                if (!ok) return false;
-                float rz_p = 0.f, kz_p = 0.f, zz_p = 0.f;
+                // a bound on |p| follows from |z|
+                if (pc_on) {
+                    precondition(ap, rr2);
+                    ok = all_ok(ok);
+                    if (!ok) return false;
+                }
+                float rz_p = 0.f, zz_p = 0.f;
 #pragma unroll
                 for (int e0 = 0; e0 < NCOL; e0 += 8) {
-                    float kv[8], rv[8];
+                    float rv[8];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        kv[i] = kbs[(c0 + e0 + i) * TC_BR + lrow];
-                        rv[i] = r_get(e0 + i);
-                    }
+                    for (int i = 0; i < 8; ++i) rv[i] = r_get(e0 + i);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         if (!prec_row) ap[e0 + i] = rv[i];           // a row whose preconditioner failed: z = r
                         rz_p = fmaf(rv[i], ap[e0 + i], rz_p);
-                        kz_p = fmaf(kv[i], ap[e0 + i], kz_p);
                         zz_p = fmaf(ap[e0 + i], ap[e0 + i], zz_p);
                     }
                 }
-                pair_sum4(rz_p, kz_p, zz_p, kbr);
+                pair_sum2(rz_p, zz_p);
                 if (active) {
                     float beta = rz_p / rz;
                     if (!(rz_p > 0.f)) {
@@ -1034,13 +1096,12 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         // row from its current x as plain CG, p = r
                         prec_row = false;
                         beta = 0.f;
-                        rz_p = rr2; kz_p = kbr; zz_p = rr2;
+                        rz_p = rr2; zz_p = rr2;
 #pragma unroll
                         for (int e = 0; e < NCOL; ++e) ap[e] = r_get(e);
                     }
 #pragma unroll
                     for (int e = 0; e < NCOL; ++e) p[e] = fmaf(beta, p[e], ap[e]);
-                    abar = fmaf(beta, abar, kz_p);
                     const float pn = sqrtf(zz_p) + fabsf(beta) * sqrtf(pn2);      // |p_new| <= |z| + |beta| |p|
                     pn2 = pn * pn;
                     rr = rr2;
@@ -1050,7 +1111,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
             return true;
         };
-        const int t = voted_loop(prm.max_iters, ok, misc + 8, still_active, cg_pass, group_any);      // CG sweeps run
+        voted_loop(prm.max_iters, ok, misc + 8, still_active, cg_pass, group_any);
         const bool at_cap = active && rr > stop;
         // ---- output sweep ----
         float gfac = 1.f;
@@ -1084,12 +1145,11 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
             abar = pair_sum(yb_p);
             gfac = 1.f + pair_sum(g_p);
-            const bool out16 = f16_on && t >= precise;      // the format every role derives from the CG sweeps it has seen
             // (over the other block's last sums, like p: the vote that ended the loop lies in between)
-            if (out16) write_operand16_pair(y);
+            if (f16_on) write_operand16_pair(y);
             else write_operand(y);
-            start_sweep(SW_OUT, out16);
-            float part = sweep(SW_OUT);
+            start_sweep(SW_OUT);
+            float part = sweep_of(std::integral_constant<int, SW_OUT>{}, std::false_type{});      // (V stays bf16)
             if (ok) acc_wait();
             ok = all_ok(ok);
             if (ok) {

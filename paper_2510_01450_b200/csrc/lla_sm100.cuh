@@ -211,6 +211,13 @@ __device__ __forceinline__ uint32_t pack_f16(float a, float b) {
     asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
     return r;
 }
+// Split two fp32 values into fp16 hi + lo pairs: hi is the value cut to 11 significant bits, lo the rounded remainder, so
+// hi + lo keeps 22 bits down to an absolute error of 2^-25 (half the spacing of the fp16 subnormals).
+__device__ __forceinline__ uint32_t split_f16x2(float a, float b, uint32_t& lo) {
+    const float ha = __uint_as_float(__float_as_uint(a) & 0xFFFFE000u), hb = __uint_as_float(__float_as_uint(b) & 0xFFFFE000u);
+    lo = pack_f16(a - ha, b - hb);
+    return pack_f16(ha, hb);
+}
 // {hi16: bf16(a), lo16: bf16(b)}
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     uint32_t r;
