@@ -235,13 +235,15 @@ size_t forward_tensor_scratch_bytes();         // d = 128 row-state scratch (0 i
 size_t forward_tensor_workspace_bytes(int B, int H, int n, int d);   // that scratch + the fp16 copy of k (upper bound: kv heads = H)
 // CG preconditioner of the tensor-core forward (lla_precond.cu): one d x d fp16 matrix per block of 128 keys
 int precond_blocks(int n);
-// Beyond the first 16 blocks (2048 keys) the covariance changes little from one block of 128 keys to the next: only
-// every fourth block gets a matrix of its own there, and a tile takes the last one at or before its key block.
-__host__ __device__ __forceinline__ int precond_block_used(int g) { return g < 16 ? g : ((g + 1) / 4) * 4 - 1; }
+// Beyond the first 16 blocks (2048 keys) the covariance changes little from one block of 128 keys to the next: two blocks share
+// a matrix there.  The last block of the group that holds block g of nb, whose matrix the tiles of the group take ...
+__host__ __device__ __forceinline__ int precond_block_used(int g, int nb) { return g < 16 ? g : (g | 1) < nb ? (g | 1) : nb - 1; }
+// ... and the first block of the group that ends with block g
+__host__ __device__ __forceinline__ int precond_group_start(int g) { return g < 16 ? g : g & ~1; }
 size_t precond_gram_bytes(int units, int n, int d);     // fp32 running Gram sums (scratch of the pre-pass)
 size_t precond_minv_bytes(int units, int n, int d);     // the fp16 matrices [units][blocks][d][d]
-int launch_precond(const void* k, int B, int Hk, Strides sk, int n, int d, float lambda, int window, void* gram, void* minv,
-                   cudaStream_t st);
+// the pre-pass with the matrices: the fp16 copy of k and the range check of q and k (into f16_ok, nonzero before) as well
+int launch_precond(const ForwardArgs& a, void* k16, int* f16_ok, void* gram, void* minv);
 int launch_decode(const DecodeArgs& a);
 int decode_refusal(const DecodeArgs& a);       // the status with which launch_decode refuses the call (before the first launch)
 constexpr int kDecodeMaxSplits = 64;           // parts of a (sequence, head) that the tensor-core path merges

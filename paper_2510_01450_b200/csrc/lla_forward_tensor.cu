@@ -96,7 +96,9 @@ struct TcCfg {
     static constexpr int SM_PLO = SM_PHI + OPER_BYTES;
     static constexpr int SM_KV = SM_PLO + OPER_BYTES;
     static constexpr int SM_KBAR = SM_KV + NSLOT * KBLK_BYTES;                    // fp32 [D][128] (D = 64 only)
-    static constexpr int SM_RED = SM_KBAR + (STATE_IN_REGS ? D * TC_BR * 4 : 0);  // pair reductions: 2 buffers x 4 values x 2 x 128 floats
+    // the preconditioner's matrix: at D = 128 where Q was, once that is in TMEM
+    static constexpr int SM_M = Q_IN_TMEM ? SM_Q : SM_KBAR + (STATE_IN_REGS ? D * TC_BR * 4 : 0);
+    static constexpr int SM_RED = Q_IN_TMEM ? SM_KBAR : SM_M + D * D * 2;         // pair reductions: 2 buffers x 4 values x 2 x 128 floats
     static constexpr int SM_FLAGS = SM_RED + 8192;                                // 2 x 8 ints
     static constexpr int SM_BAR = SM_FLAGS + 64;                                  // mbarriers
     static constexpr int SM_MISC = SM_BAR + 512;                                  // tmem base, ctl kind, abort
@@ -116,7 +118,8 @@ enum { B_QFULL = 0, B_KVFULL = 1, B_KVEMPTY = B_KVFULL + TC_SLOT_MAX, B_SAFULL =
        B_MFULL = B_EXIT + 2, // the preconditioner matrix has landed
        B_XREADY = B_MFULL + 1, B_XFULL = B_XREADY + 1,   // exchange of a pair of blocks: the other's sweep is done, its sums are here
        B_AFREE = B_XFULL + 1,    // D = 128: an A slot has been read (two slots)
-       B_COUNT = B_AFREE + 2 };
+       B_QREAD = B_AFREE + 2,    // D = 128: Q has been copied to TMEM
+       B_COUNT = B_QREAD + 1 };
 static_assert(B_COUNT * 8 <= 512, "barrier area too small");
 
 constexpr uint32_t IDESC_SS = make_idesc(TC_BR, TC_BC, 0, 0);   // S/A: A, B K-major; ACC uses make_idesc(128, D, 0, 1)
@@ -271,6 +274,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         mbar_init(bar(B_MFULL), 1);
         mbar_init(bar(B_XREADY), TC_COMPUTE / 32);
         mbar_init(bar(B_XFULL), TC_COMPUTE / 32);
+        mbar_init(bar(B_QREAD), TC_COMPUTE / 32);
         for (int a = 0; a < 2; ++a) mbar_init(bar(B_AFREE + a), (split ? TC_COMPUTE : TC_COMPUTE / 2) / 32);
         misc[4] = SW_STATS;
         misc[5] = SW_STATS;
@@ -307,16 +311,19 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const int bb = bh / prm.H, hq = bh % prm.H, hk = hq / prm.kv_group;
             for (int sub = 0; sub < KSUB; ++sub)
                 tma_load_4d(sbase + SM_Q + sub * Cfg::QSUB_BYTES, &tmQ, bar(B_QFULL), 64 * sub, r0, hq, bb);
-            if (PC && f16_on) {
-                // the preconditioner of this tile's key range: D x D fp16, laid out like D / 64 key blocks, in the P_lo tile
-                // (the fp16 CG sweeps do not use it; the output sweep does, when the matrix is no longer needed)
-                const int gm = precond_block_used((prm.causal ? min(n - 1, off + r0 + TC_BR - 1) : n - 1) / 128);
+            bool m_issued = false;
+            // the preconditioner of this tile's key range: D x D fp16, laid out like D / 64 key blocks
+            auto load_m = [&]() {
+                if (Cfg::Q_IN_TMEM && !mbar_wait(bar(B_QREAD), 0, abort_flag, wcap)) return;
+                const int last = !prm.causal ? n - 1 : min(n - 1, off + (wraps ? prm.nq_pos : r0p + TC_BR) - 1);
+                const int gm = precond_block_used(last / 128, (n + 127) / 128);
+                m_issued = true;
                 mbar_expect_tx(bar(B_MFULL), D * D * 2);
                 for (int rb = 0; rb < D / 64; ++rb)
                     for (int sub = 0; sub < KSUB; ++sub)
-                        tma_load_4d(sbase + SM_PLO + rb * KBLK + sub * Cfg::KSUB_BYTES, &tmM, bar(B_MFULL), 64 * sub,
+                        tma_load_4d(sbase + Cfg::SM_M + rb * KBLK + sub * Cfg::KSUB_BYTES, &tmM, bar(B_MFULL), 64 * sub,
                                     gm * D + 64 * rb, hk, bb);
-            }
+            };
             uint32_t kit = 0;      // blocks issued so far (the next ring position)
             bool ok = true;
             const CUtensorMap* tk = f16_on ? &tmK16 : &tmK;
@@ -334,6 +341,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 for (int c = 0; c < (int)pre && ok; ++c) issue(tk, c);
             };
             prefetch();
+            if (PC && f16_on && ok) load_m();
             uint32_t pre_out = pre;      // blocks fetched ahead and not announced yet
             for (uint32_t ctl = 0; ok; ++ctl) {
                 if (!mbar_wait(bar(B_CTL), ctl & 1, abort_flag, wcap)) break;
@@ -354,7 +362,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 if (kind != SW_OUT) { prefetch(); pre_out = pre; }
             }
             if (*abort_flag) {
-                if (PC && f16_on) (void)mbar_wait_landed(bar(B_MFULL), 0, wcap);
+                if (m_issued) (void)mbar_wait_landed(bar(B_MFULL), 0, wcap);
                 // an aborted block: the copies issued above write into this block's shared memory, so they must
                 // have landed before the block exits (on a completed run their consumers have waited for them)
                 (void)mbar_wait_landed(bar(B_QFULL), 0, wcap);
@@ -496,6 +504,18 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             a = buf[lrow] + buf[128 + lrow];
             b = buf[256 + lrow] + buf[384 + lrow];
         };
+        // three
+        auto pair_sum3 = [&](float& a, float& b, float& c) {
+            float* buf = red + red_sel * 1024;
+            red_sel ^= 1;
+            buf[half * 128 + lrow] = a;
+            buf[256 + half * 128 + lrow] = b;
+            buf[512 + half * 128 + lrow] = c;
+            pair_sync();
+            a = buf[lrow] + buf[128 + lrow];
+            b = buf[256 + lrow] + buf[384 + lrow];
+            c = buf[512 + lrow] + buf[640 + lrow];
+        };
         auto pair_max = [&](float v) {
             float* buf = red + red_sel * 1024;
             red_sel ^= 1;
@@ -543,7 +563,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 *reinterpret_cast<uint4*>(smem + SM_PLO + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             }
         };
-        // Q tile: bf16 as loaded, or fp16 (converted in place by prepare_q, each thread its own chunks)
+        // Q tile: bf16 as loaded, or fp16 (converted by prepare_q, each thread its own chunks)
         auto q_elem = [&](const uint32_t* qw, int e) -> float {
             if (f16_on) {
                 const __half2 h2 = *reinterpret_cast<const __half2*>(&qw[e >> 1]);
@@ -563,7 +583,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
                         qw[e] = pack_f16(__uint_as_float(qw[e] << 16), __uint_as_float(qw[e] & 0xFFFF0000u));
-                    *qp = make_uint4(qw[0], qw[1], qw[2], qw[3]);
+                    if constexpr (!Cfg::Q_IN_TMEM) *qp = make_uint4(qw[0], qw[1], qw[2], qw[3]);
                 }
                 if constexpr (Cfg::Q_IN_TMEM) {
 #pragma unroll
@@ -574,6 +594,24 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 tmem_st32(tmem + lane_addr + TC_Q_COL + 32 * half, qt);
                 tc_wait_st();
                 tc_fence_before();
+                if (PC) {      // the preconditioner's matrix may come
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_QREAD));
+                }
+            }
+        };
+        // this thread's entries of q, two to a word
+        auto load_q = [&](uint32_t* qt) {
+            if constexpr (Cfg::Q_IN_TMEM) {
+                tmem_ld32(tmem + lane_addr + TC_Q_COL + 32 * half, qt);
+                tc_wait_ld();
+            } else {
+#pragma unroll
+                for (int ch = 0; ch < NCOL / 8; ++ch) {
+                    const uint4 x = *reinterpret_cast<const uint4*>(smem + SM_Q + oper_off(ch));
+                    qt[4 * ch] = x.x; qt[4 * ch + 1] = x.y; qt[4 * ch + 2] = x.z; qt[4 * ch + 3] = x.w;
+                }
             }
         };
         // vec rounded to fp16 after scaling by the power of two sc (isc = 1 / sc; see write_p), in the operand tile and in vec itself
@@ -844,18 +882,20 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             return pair_sum((s4[0] + s4[1]) + (s4[2] + s4[3]));
         };
 
-        // z = M r with the tile's preconditioner: vec holds this thread's NCOL entries of r on entry (|r|^2 is about
-        // nrm2 over the whole row) and of z on return.  r goes to TMEM as fp16, scaled by a power of two into the
+        // Z = R M with the tile's preconditioner, left in TMEM: vec holds this thread's NCOL entries of r (|r|^2 is about
+        // nrm2 over the whole row).  r goes to TMEM as fp16, scaled by a power of two into the
         // middle of the fp16 range (M is stored with a largest entry of one); once every compute thread has stored
-        // its part, warp 0 issues the product Z = R M itself (no hand-over to the MMA warps, which are idle between
+        // its part, warp 0 issues the product itself (no hand-over to the MMA warps, which are idle between
         // sweeps, as are the TMEM columns of the S/A/U buffers that R and Z use).
         const uint32_t el0 = PC ? elect_one() : 0u;
         const uint32_t sb_c = PC ? __shfl_sync(0xffffffffu, sbase, 0) : 0u, tm_c = PC ? __shfl_sync(0xffffffffu, tmem, 0) : 0u;
         bool m_ready = false;
-        auto precondition = [&](float* vec, float nrm2) {
+        float zsc = 1.f;        // z = zsc Z
+        auto precondition = [&](const float* vec, float nrm2) {
             const int e2 = (int)((__float_as_uint(nrm2) >> 23) & 0xffu) - 127;
             const int k = max(-100, min(100, -(e2 >> 1)));
-            const float sc = __uint_as_float((uint32_t)(127 + k) << 23), isc = __uint_as_float((uint32_t)(127 - k) << 23);
+            const float sc = __uint_as_float((uint32_t)(127 + k) << 23);
+            zsc = __uint_as_float((uint32_t)(127 - k) << 23);
             uint32_t pk[NCOL / 2];
 #pragma unroll
             for (int e = 0; e < NCOL / 2; ++e) pk[e] = pack_f16(vec[2 * e] * sc, vec[2 * e + 1] * sc);
@@ -868,29 +908,45 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (warp == 0) {
                 if (!m_ready) m_ready = mbar_wait(bar(B_MFULL), 0, abort_flag, wcap);     // the matrix has landed (first use)
                 tc_fence_after();
-                if (m_ready) {
+                if (m_ready && !*abort_flag) {
 #pragma unroll
                     for (int rb = 0; rb < D / 64; ++rb)
                         mma_ts_k64c(el0, tm_c + TC_Z_COL, tm_c + TC_R_COL + 32 * rb,
-                                    make_desc(sb_c + SM_PLO + rb * KBLK, Cfg::KSUB_BYTES), IDESC_TS16, rb > 0);
+                                    make_desc(sb_c + Cfg::SM_M + rb * KBLK, Cfg::KSUB_BYTES), IDESC_TS16, rb > 0);
                     tc_commit_el(el0, bar(B_ACCFULL));
                 }
             }
-            if (!mbar_wait(bar(B_ACCFULL), acc_uses & 1, abort_flag, wcap)) { ok = false; return; }
-            ++acc_uses;
-            tc_fence_after();
+            acc_wait();
+        };
+        // f(e, z_e) for this thread's entries
+        auto each_z = [&](auto&& fn) {
 #pragma unroll
             for (int cb = 0; cb < NCOL; cb += 32) {
                 uint32_t v[32];
                 tmem_ld32(tmem + lane_addr + TC_Z_COL + c0 + cb, v);
                 tc_wait_ld();
 #pragma unroll
-                for (int e = 0; e < 32; ++e) vec[cb + e] = __uint_as_float(v[e]) * isc;
+                for (int e = 0; e < 32; ++e) fn(cb + e, __uint_as_float(v[e]) * zsc);
             }
             tc_fence_before();
         };
-        float rz = 0.f;      // r . z of the preconditioned recurrence
         bool prec_row = true;   // false once the preconditioner has failed this row (z = r from then on)
+        // From the residual in rv: r . z, |z|^2 and z . p ...
+        auto z_sums = [&](const float* rv, float& rz_p, float& zz_p, float& zp_p) {
+            rz_p = zz_p = zp_p = 0.f;
+            each_z([&](int e, float z) {
+                z = prec_row ? z : rv[e];
+                rz_p = fmaf(rv[e], z, rz_p);
+                zz_p = fmaf(z, z, zz_p);
+                zp_p = fmaf(z, p[e], zp_p);
+            });
+            pair_sum3(rz_p, zz_p, zp_p);
+        };
+        // ... and the direction dir = z + beta dir
+        auto z_step = [&](float* dir, const float* rv, float beta) {
+            each_z([&](int e, float z) { dir[e] = fmaf(beta, dir[e], prec_row ? z : rv[e]); });
+        };
+        float rz = 0.f;      // r . z of the preconditioned recurrence
 
         // ---- statistics sweep: omega and kbar ----
         // No sweep of its own finds the row maxima: Eq. "lla" is unchanged under a joint scaling of the weights and
@@ -950,13 +1006,13 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 // lambda in the frame of the row maximum, i.e. lambda e^{max - shift} here
                 ridge = lam_i * ex2f((prm.ridge_mode == LLA_RIDGE_PRINTED ? tmax : 0.f) - mx2) * inv_omega;
                 float rr_p = 0.f;
+                uint32_t qt[NCOL / 2];
+                load_q(qt);
 #pragma unroll
                 for (int ch = 0; ch < NCOL / 8; ++ch) {
-                    const uint4 qraw = *reinterpret_cast<const uint4*>(smem + SM_Q + oper_off(ch));
-                    const uint32_t qw[4] = {qraw.x, qraw.y, qraw.z, qraw.w};
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const float qv = q_elem(qw, e);
+                        const float qv = q_elem(qt + 4 * ch, e);
                         const int col = ch * 8 + e;
                         const float kb = acc[col] * inv_omega;
                         kbs[(c0 + col) * TC_BR + lrow] = kb;
@@ -981,22 +1037,16 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             precondition(p, rr);
             ok = all_ok(ok);
             if (ok) {
-                float rz_p = 0.f, zz_p = 0.f;
-#pragma unroll
-                for (int e = 0; e < NCOL; ++e) {
-                    rz_p = fmaf(r_get(e), p[e], rz_p);
-                    zz_p = fmaf(p[e], p[e], zz_p);
-                }
-                pair_sum2(rz_p, zz_p);
+                float rz_p, zz_p, unused;
+                z_sums(p, rz_p, zz_p, unused);
                 if (rz_p > 0.f) {
                     rz = rz_p; pn2 = zz_p;
                 } else {
-                    // the rounded matrix is not positive on this residual: the row runs unpreconditioned
-                    // (pn2 and rz already hold the values for p = r)
+                    // the rounded matrix is not positive on this residual: the row runs unpreconditioned, p = r
+                    // (pn2 and rz already hold the values for that)
                     prec_row = false;
-#pragma unroll
-                    for (int e = 0; e < NCOL; ++e) p[e] = r_get(e);
                 }
+                each_z([&](int e, float z) { p[e] = prec_row ? z : p[e]; });
             }
         }
         // ---- conjugate gradients (Algorithm 2) ----
@@ -1011,10 +1061,6 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             sweep_cg(kind);
             if constexpr (!Cfg::STATE_IN_REGS) reload_p();
             if (ok) acc_wait();
-            if (PC) {
-                ok = all_ok(ok);
-                if (!ok) return false;
-            }
             float ap[NCOL];
             acc_load(ap);
             if (NS > 1) {
@@ -1023,7 +1069,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 if (!ok) return false;
             }
             // (the loops below keep four independent partial sums and move the row-vector state in
-            //  batches of eight so that the loads overlap: two warps per scheduler hide no latency)
+            //  batches of sixteen so that the loads overlap: two warps per scheduler hide no latency)
             float pp[4] = {0.f, 0.f, 0.f, 0.f};
             const float acc_scale = f16_on ? inv_omega * ipsc : inv_omega;
 #pragma unroll
@@ -1036,22 +1082,22 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const float alpha = active ? rz / pap : 0.f;       // rz = |r|^2 without a preconditioner
             float r2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-            for (int e0 = 0; e0 < NCOL; e0 += 8) {
-                float xv[8], rv[8];
+            for (int e0 = 0; e0 < NCOL; e0 += 16) {
+                float xv[16], rv[16];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
+                for (int i = 0; i < 16; ++i) {
                     xv[i] = x_get(e0 + i);
                     rv[i] = r_get(e0 + i);
                 }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
+                for (int i = 0; i < 16; ++i) {
                     xv[i] = fmaf(alpha, p[e0 + i], xv[i]);
                     rv[i] = fmaf(-alpha, ap[e0 + i], rv[i]);
                     ap[e0 + i] = rv[i];                       // ap now holds the new residual
                     r2[i & 3] = fmaf(rv[i], rv[i], r2[i & 3]);
                 }
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
+                for (int i = 0; i < 16; ++i) {
                     x_set(e0 + i, xv[i]);
                     r_set(e0 + i, rv[i]);
                 }
@@ -1068,42 +1114,29 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     ++its;
                 }
             } else {
-                // preconditioned: z = M r_new (ap <- z), then beta = (r_new . z_new) / (r . z), p = z + beta p;
-                // a bound on |p| follows from |z|
+                // preconditioned: z = M r_new (the new residual is in ap), then beta = (r_new . z_new) / (r . z), p = z + beta p;
+                // |p|^2 follows from |z|^2 and z . p (a bound from |z| alone grows away from it where beta is near one, and a direction
+                // scaled by it would lose its bits to the fp16 subnormals)
+                if (pc_on) precondition(ap, rr2);
+                float rz_p = rr2, zz_p = rr2, zp_p = 0.f;
+                if (pc_on) z_sums(ap, rz_p, zz_p, zp_p);
+                float beta = rz_p / rz;
+                if (active && !(rz_p > 0.f)) {
+                    // r . M r is not positive (the rounded matrix is not definite on this residual): restart the
+                    // row from its current x as plain CG, p = r
+                    prec_row = false;
+                    beta = 0.f;
+                    rz_p = rr2; zz_p = rr2;
+                }
+                if (!active) beta = 0.f;
                 if (pc_on) {
-                    precondition(ap, rr2);
-                    ok = all_ok(ok);
-                    if (!ok) return false;
-                }
-                float rz_p = 0.f, zz_p = 0.f;
-#pragma unroll
-                for (int e0 = 0; e0 < NCOL; e0 += 8) {
-                    float rv[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) rv[i] = r_get(e0 + i);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        if (!prec_row) ap[e0 + i] = rv[i];           // a row whose preconditioner failed: z = r
-                        rz_p = fmaf(rv[i], ap[e0 + i], rz_p);
-                        zz_p = fmaf(ap[e0 + i], ap[e0 + i], zz_p);
-                    }
-                }
-                pair_sum2(rz_p, zz_p);
-                if (active) {
-                    float beta = rz_p / rz;
-                    if (!(rz_p > 0.f)) {
-                        // r . M r is not positive (the rounded matrix is not definite on this residual): restart the
-                        // row from its current x as plain CG, p = r
-                        prec_row = false;
-                        beta = 0.f;
-                        rz_p = rr2; zz_p = rr2;
-#pragma unroll
-                        for (int e = 0; e < NCOL; ++e) ap[e] = r_get(e);
-                    }
+                    z_step(p, ap, beta);
+                } else {
 #pragma unroll
                     for (int e = 0; e < NCOL; ++e) p[e] = fmaf(beta, p[e], ap[e]);
-                    const float pn = sqrtf(zz_p) + fabsf(beta) * sqrtf(pn2);      // |p_new| <= |z| + |beta| |p|
-                    pn2 = pn * pn;
+                }
+                if (active) {
+                    pn2 = fmaxf(fmaf(beta, fmaf(beta, pn2, 2.f * zp_p), zz_p), 1e-3f * zz_p);
                     rr = rr2;
                     rz = rz_p;
                     ++its;
@@ -1129,13 +1162,13 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         } else if (ok) {
             float y[NCOL];
             float yb_p = 0.f, g_p = 0.f;
+            uint32_t qt[NCOL / 2];
+            load_q(qt);
 #pragma unroll
             for (int ch = 0; ch < NCOL / 8; ++ch) {
-                const uint4 qraw = *reinterpret_cast<const uint4*>(smem + SM_Q + oper_off(ch));
-                const uint32_t qw[4] = {qraw.x, qraw.y, qraw.z, qraw.w};
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
-                    const float qv = q_elem(qw, e);
+                    const float qv = q_elem(qt + 4 * ch, e);
                     const int col = ch * 8 + e;
                     const float kb = kbs[(c0 + col) * TC_BR + lrow];
                     y[col] = x_get(col);
@@ -1283,7 +1316,7 @@ void tile_order(TcParams& prm, int tiles, int first_tile, int n, int off, int d,
         const int r_end = std::min(n, off + (first_tile + t + 1) * TC_BR);      // keys the tile's last row sees
         const int seen = window > 0 ? std::min(r_end, window) : r_end;
         const float x = (float)d / (float)seen;
-        const float its = precond ? std::min(16.f, 4.f + 190.f * x * x) : std::min(40.f, 4.5f + 40.f * x + 150.f * x * x);
+        const float its = precond ? std::min(16.f, 2.7f + 14.f * x + 90.f * x * x) : std::min(40.f, 4.5f + 40.f * x + 150.f * x * x);
         const int c_first = window > 0 ? std::max(0, off + (first_tile + t) * TC_BR + 1 - window) / TC_BC : 0;
         const float nblk = (float)((r_end + TC_BC - 1) / TC_BC - c_first);
         cost[t] = (its + 2.f) * ((d == 64 ? 8.5f : 10.f) + nblk) + (precond ? 3.f * its : 0.f);
@@ -1307,7 +1340,7 @@ int launch_t(const ForwardArgs& a) {
     // can fill tiles together where a head's own rows leave its last tile partly empty (257 rows of four heads: nine
     // tiles instead of twelve).  Their rows must lie one behind the other in q, and none may be solved directly.
     const int group = a.kv_group;
-    const bool pack = group > 1 && hr == 0 && !a.block_mask && !a.minv && a.sq.h == (long long)a.nq * a.sq.r &&
+    const bool pack = group > 1 && hr == 0 && !a.block_mask && a.sq.h == (long long)a.nq * a.sq.r &&
                       (group * a.nq + TC_BR - 1) / TC_BR < group * tiles;
     const int units = pack ? a.B * Hk : a.B * a.H;          // unit: the rows that are cut into tiles together
     const int unit_rows = pack ? group * a.nq : a.nq;
@@ -1385,12 +1418,13 @@ int launch_t(const ForwardArgs& a) {
     const int most = ((prm.window > 0 ? std::min(a.n, prm.window + TC_BR) : a.n) + TC_BC - 1) / TC_BC;
     const int least = !a.causal ? most : std::min(most, (a.n - a.nq + first_tile * TC_BR + TC_BC) / TC_BC);
     const double one = (double)((grid1 + sms - 1) / sms) * (7 + most), two = (double)((2 * grid1 + sms - 1) / sms) * (10 + 0.5 * most);
-    const bool pairs = !precond && !a.block_mask && least >= 4 && two < 0.95 * one;
-    auto kern = precond ? forward_tc_kernel<D, TOut, true> : pairs ? forward_tc_kernel<D, TOut, false, false, 2> : forward_tc_kernel<D, TOut, false>;
+    const bool pairs = !a.block_mask && least >= 4 && two < 0.95 * one;
+    auto kern = precond ? (pairs ? forward_tc_kernel<D, TOut, true, false, 2> : forward_tc_kernel<D, TOut, true>)
+                        : (pairs ? forward_tc_kernel<D, TOut, false, false, 2> : forward_tc_kernel<D, TOut, false>);
     if constexpr (std::is_same<TOut, float>::value) {
         if (a.sol && a.kbar_in && a.stats_in)
-            kern = precond ? forward_tc_kernel<D, TOut, true, true>
-                           : pairs ? forward_tc_kernel<D, TOut, false, true, 2> : forward_tc_kernel<D, TOut, false, true>;
+            kern = precond ? (pairs ? forward_tc_kernel<D, TOut, true, true, 2> : forward_tc_kernel<D, TOut, true, true>)
+                           : (pairs ? forward_tc_kernel<D, TOut, false, true, 2> : forward_tc_kernel<D, TOut, false, true>);
     }
     LLA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SM_ALLOC));
     cudaLaunchConfig_t cfg = {};
@@ -1439,24 +1473,25 @@ int forward_tensor_prepass(ForwardArgs& a) {
     uint4* k16 = reinterpret_cast<uint4*>(ws);
     int* okw = reinterpret_cast<int*>(ws + round256(k_elems * 2));
     LLA_CUDA_TRY(cudaMemsetAsync(okw, 1, sizeof(int), a.stream));
+    // with the preconditioner's matrices behind the copy (Gram scratch first), if enabled and there is room: one pass
+    // over k makes all of it
+    const int units = a.B * a.H / a.kv_group;
+    const size_t used = head + f16_copy_bytes(k_elems);
+    const size_t gram_b = precond_gram_bytes(units, a.n, a.d), minv_b = precond_minv_bytes(units, a.n, a.d);
+    a.k16 = k16;
+    a.f16_ok = okw;
+    if (a.precondition && a.workspace_bytes >= used + gram_b + minv_b) {
+        char* gram = static_cast<char*>(a.workspace) + used;
+        const int rc = launch_precond(a, k16, okw, gram, gram + gram_b);
+        if (rc != LLA_OK) return rc;
+        a.minv = gram + gram_b;
+        return LLA_OK;
+    }
     const size_t k_vec = k_elems / 8;
     const unsigned blocks = (unsigned)std::min<size_t>((k_vec + 255) / 256, 148 * 8);
     f16_copy_kernel<<<blocks, 256, 0, a.stream>>>(static_cast<const __nv_bfloat16*>(a.k), k16, a.H / a.kv_group, a.n, a.d, a.sk,
                                                    static_cast<const __nv_bfloat16*>(a.q), a.H, a.nq, a.sq, a.B, okw);
     LLA_CUDA_TRY(cudaGetLastError());
-    a.k16 = k16;
-    a.f16_ok = okw;
-    // the preconditioner behind it, if enabled and there is room (Gram scratch, then the matrices)
-    const int units = a.B * a.H / a.kv_group;
-    const size_t used = head + f16_copy_bytes(k_elems);
-    const size_t gram_b = precond_gram_bytes(units, a.n, a.d), minv_b = precond_minv_bytes(units, a.n, a.d);
-    if (a.precondition && a.workspace_bytes >= used + gram_b + minv_b) {
-        char* gram = static_cast<char*>(a.workspace) + used;
-        char* minv = gram + gram_b;
-        const int rc = launch_precond(a.k, a.B, a.H / a.kv_group, a.sk, a.n, a.d, a.lambda, a.causal ? a.window : 0, gram, minv, a.stream);
-        if (rc != LLA_OK) return rc;
-        a.minv = minv;
-    }
     return LLA_OK;
 }
 

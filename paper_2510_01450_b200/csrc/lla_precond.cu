@@ -4,224 +4,384 @@
 // The system of query row i is C_i = sum_j p_ij (k_j - kbar_i)(k_j - kbar_i)^T + ridge_i I with weights
 // p_ij = w_ij / omega_i over the visible keys.  With all weights equal it is the covariance of those keys,
 // which is the same matrix for every row that sees the same keys and changes slowly from row to row.  Its
-// inverse, formed once per block of 128 keys for the keys up to the end of that block, is a good
-// preconditioner wherever the weights are not far from uniform: on the synthetic workloads it halves the
-// iteration count.  It never changes the solution, only the path to it, so it is built in fp32 and stored
-// in fp16; a block whose inversion breaks down gets the identity.
+// inverse, formed once per group of key blocks, is a good preconditioner wherever the weights are not far from uniform: on
+// the synthetic workloads it takes away more than half of the iterations.  It never changes the solution, only the path to
+// it, so it is built in fp32 and stored in fp16; a block whose inversion breaks down gets the identity.
+//
+// The rows of a tile see between none and all of the tile's own keys, so those enter with the mean of that, half their
+// weight: a row's own covariance is then off by half a block's worth of keys at most, whichever row of the tile it is.
+// (With full weight the first row is off by a whole block: 15.8 instead of 12.1 iterations in the second tile at d = 64, 6.0
+// instead of 5.0 in the sixth, three instead of two past 14 K keys at d = 128.)
 //
 // Three kernels, all on the caller's stream ahead of the forward kernel:
-//   gram_blocks_kernel   G_b = sum_j k_j k_j^T and s_b = sum_j k_j over the keys of block b
-//   gram_scan_kernel     running sums over b (in place)
-//   precond_invert_kernel   M_g = (G / L - s s^T / L^2 + (lambda / L) I)^{-1} by Gauss-Jordan elimination in
-//                        shared memory, scaled to a largest entry of one (conjugate gradients do not see the
-//                        scale of a preconditioner), rounded to fp16
+//   precond_gram_kernel     a chunk of key blocks each: running sums of k_j k_j^T and k_j inside the chunk, one record per
+//                           block that is asked for.  It reads every key once, so it also makes the fp16 copy of k and
+//                           checks that k and q fit the fp16 range.  Bound by its loads; the products run on mma.sync,
+//                           whose operands come straight from the tiles (ldmatrix.trans).  16 heads, n = 16384, d = 128:
+//                           85 us, where Gram sums on the CUDA cores, their scan over every block and a copy kernel took 430
+//   precond_scan_kernel     the sums of whole chunks (the records of their last blocks) become running sums over the sequence
+//   precond_invert_kernel   M_g = (G / L - s s^T / L^2 + (lambda / L) I)^{-1}, G and s from the records of the block and of
+//                           the chunk before it, by Gauss-Jordan elimination in registers, scaled to a largest entry of one
+//                           (conjugate gradients do not see the scale of a preconditioner), rounded to fp16.
 #include <cuda_fp16.h>
 
-#include "lla_common.cuh"
+#include <algorithm>
+
+#include "lla_sm100.cuh"
 
 namespace lla {
 namespace {
 
+using sm100::pack_f16;
+using sm100::smem_u32;
+
 constexpr int PC_THREADS = 256;
 constexpr int PC_BLOCK = 128;      // keys per Gram block
+constexpr int PC_CHUNKS = 8;       // at most
+
+struct PcParams {
+    const __nv_bfloat16* k;
+    const __nv_bfloat16* q;
+    float* gram;       // [units][blocks][D * D + D]
+    uint4* k16;        // [units][n][D] fp16
+    int* f16_ok;       // cleared if an entry of k or q lies outside the fp16 range
+    __half* minv;      // [units][blocks][D][D]
+    int n, nb, cb;     // keys; blocks; blocks per chunk
+    int g0;            // first block that a query sees last
+    int B, Hk, H, nq;
+    int causal, window, head_rows;
+    float lambda;
+    Strides sk, sq;
+};
+
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// a pair of bf16 values as a pair of fp16 values; bad: one of them is beyond 60000 (or not a number)
+__device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w, bool& bad) {
+    const float a = __uint_as_float(w << 16), b = __uint_as_float(w & 0xFFFF0000u);
+    bad |= !(fabsf(a) <= 60000.f) || !(fabsf(b) <= 60000.f);
+    return pack_f16(a, b);
+}
 
 template <int D>
 __global__ void __launch_bounds__(PC_THREADS)
-gram_blocks_kernel(const __nv_bfloat16* __restrict__ k, float* __restrict__ gram, int n, int nb, int Hk, Strides sk) {
-    constexpr int LD = D + 1, TR = D / 16;
-    extern __shared__ float pc_smem[];
-    float* ks = pc_smem;                                   // [PC_BLOCK][LD]
-    const int b = blockIdx.x, u = blockIdx.y, tid = threadIdx.x;
-    const int j0 = b * PC_BLOCK, rows = min(PC_BLOCK, n - j0);
-    const __nv_bfloat16* src = k + sk.at(u / Hk, u % Hk, j0);
-    for (int idx = tid; idx < PC_BLOCK * (D / 8); idx += PC_THREADS) {
-        const int r = idx / (D / 8), c = (idx % (D / 8)) * 8;
-        float x[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (r < rows) load8(src + (size_t)r * sk.r + c, x);
+precond_gram_kernel(const PcParams p) {
+    constexpr int LD = D + 8;                       // rows 16 bytes apart modulo 128: ldmatrix without bank conflicts
+    constexpr int CPR = D / 8, RPI = PC_THREADS / CPR, NLD = PC_BLOCK / RPI;      // 16-byte pieces per row, rows per step, steps
+    constexpr int MT = D / 64, NT = D / 16;         // a warp's tiles of 16 x 8: 4 x 2 warps
+    extern __shared__ __align__(16) uint8_t pc_raw[];
+    __nv_bfloat16* ks = reinterpret_cast<__nv_bfloat16*>(pc_raw);                     // [2][PC_BLOCK][LD]
+    float* sums = reinterpret_cast<float*>(pc_raw + 2 * PC_BLOCK * LD * 2);           // [PC_THREADS][9]
+    const int u = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int b0 = blockIdx.x * p.cb, b1 = min(p.nb, b0 + p.cb);
+    const int col = tid % CPR, row0 = tid / CPR;
+    const __nv_bfloat16* src = p.k + p.sk.at(u / p.Hk, u % p.Hk, 0) + 8 * col;
+    uint4* dst16 = p.k16 + (size_t)u * p.n * CPR + col;
+    uint4 raw[NLD];
+    auto fetch = [&](int b) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) ks[r * LD + c + e] = x[e];
+        for (int i = 0; i < NLD; ++i) {
+            const int j = b * PC_BLOCK + row0 + i * RPI;
+            raw[i] = j < p.n ? *reinterpret_cast<const uint4*>(src + (long long)j * p.sk.r) : make_uint4(0, 0, 0, 0);
+        }
+    };
+    bool bad = false;
+    float s8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float acc[MT][NT][4] = {};
+    const int m0 = (warp & 3) * 16 * MT, n0 = (warp >> 2) * 8 * NT;
+    const int mat = lane >> 3, l8 = lane & 7;
+    if (b0 < b1) fetch(b0);
+    for (int b = b0; b < b1; ++b) {
+        __nv_bfloat16* t = ks + (b & 1) * PC_BLOCK * LD;
+#pragma unroll
+        for (int i = 0; i < NLD; ++i) {
+            const int r = row0 + i * RPI, j = b * PC_BLOCK + r;
+            *reinterpret_cast<uint4*>(t + r * LD + 8 * col) = raw[i];
+            const uint32_t w[4] = {raw[i].x, raw[i].y, raw[i].z, raw[i].w};
+            uint32_t h[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                h[e] = bf16x2_to_f16x2(w[e], bad);
+                s8[2 * e] += __uint_as_float(w[e] << 16);
+                s8[2 * e + 1] += __uint_as_float(w[e] & 0xFFFF0000u);
+            }
+            if (j < p.n) dst16[(size_t)j * CPR] = make_uint4(h[0], h[1], h[2], h[3]);
+        }
+        if (b + 1 < b1) fetch(b + 1);
+        __syncthreads();
+        const uint32_t tb = smem_u32(t);
+#pragma unroll 2
+        for (int k0 = 0; k0 < PC_BLOCK; k0 += 16) {
+            uint32_t a[MT][4], bb[NT / 2][4];      // bb: two tiles of 8 columns each
+#pragma unroll
+            for (int i = 0; i < MT; ++i)
+                ldmatrix_x4_trans(a[i], tb + 2u * ((k0 + (mat >> 1) * 8 + l8) * LD + m0 + 16 * i + (mat & 1) * 8));
+#pragma unroll
+            for (int i = 0; i < NT / 2; ++i)
+                ldmatrix_x4_trans(bb[i], tb + 2u * ((k0 + (mat & 1) * 8 + l8) * LD + n0 + 16 * i + (mat >> 1) * 8));
+#pragma unroll
+            for (int i = 0; i < MT; ++i)
+#pragma unroll
+                for (int jn = 0; jn < NT; ++jn) mma_bf16(acc[i][jn], a[i], bb[jn >> 1][2 * (jn & 1)], bb[jn >> 1][2 * (jn & 1) + 1]);
+        }
+        if (p.window > 0 || b == b1 - 1 || precond_block_used(b, p.nb) == b) {
+            float* rec = p.gram + ((size_t)u * p.nb + b) * (D * D + D);
+#pragma unroll
+            for (int i = 0; i < MT; ++i)
+#pragma unroll
+                for (int jn = 0; jn < NT; ++jn) {
+                    float* o = rec + (m0 + 16 * i + (lane >> 2)) * D + n0 + 8 * jn + 2 * (lane & 3);
+                    *reinterpret_cast<float2*>(o) = make_float2(acc[i][jn][0], acc[i][jn][1]);
+                    *reinterpret_cast<float2*>(o + 8 * D) = make_float2(acc[i][jn][2], acc[i][jn][3]);
+                }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) sums[tid * 9 + e] = s8[e];
+            __syncthreads();
+            if (tid < D) {
+                float s = 0.f;
+                for (int r = 0; r < RPI; ++r) s += sums[(r * CPR + tid / 8) * 9 + tid % 8];
+                rec[D * D + tid] = s;
+            }
+            __syncthreads();
+        }
+        // (the next tile goes to the other buffer; the one after it is written behind the next barrier)
     }
-    __syncthreads();
-    const int ti = tid >> 4, tj = tid & 15;
-    float acc[TR][TR] = {};
-    for (int r = 0; r < PC_BLOCK; ++r) {
-        float a[TR], c[TR];
+    // the range of q, shared out over the grid: eight loads in flight a thread where q is one piece
+    const size_t nthr = (size_t)gridDim.x * gridDim.y * PC_THREADS, q_vec = (size_t)p.B * p.H * p.nq * CPR;
+    const bool flat = p.sq.r == D && p.sq.h == (long long)p.nq * D && p.sq.b == (long long)p.H * p.nq * D;
+    auto check = [&](const uint4& x) {
+        (void)bf16x2_to_f16x2(x.x, bad); (void)bf16x2_to_f16x2(x.y, bad); (void)bf16x2_to_f16x2(x.z, bad); (void)bf16x2_to_f16x2(x.w, bad);
+    };
+    size_t i = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * PC_THREADS + tid;
+    if (flat) {
+        const uint4* qv = reinterpret_cast<const uint4*>(p.q);
+        for (; i + 7 * nthr < q_vec; i += 8 * nthr) {
+            uint4 x[8];
 #pragma unroll
-        for (int e = 0; e < TR; ++e) { a[e] = ks[r * LD + ti + 16 * e]; c[e] = ks[r * LD + tj + 16 * e]; }
+            for (int e = 0; e < 8; ++e) x[e] = qv[i + e * nthr];
 #pragma unroll
-        for (int x = 0; x < TR; ++x)
-#pragma unroll
-            for (int y = 0; y < TR; ++y) acc[x][y] = fmaf(a[x], c[y], acc[x][y]);
+            for (int e = 0; e < 8; ++e) check(x[e]);
+        }
+        for (; i < q_vec; i += nthr) check(qv[i]);
+    } else {
+        for (; i < q_vec; i += nthr) {
+            const size_t rowi = i / CPR;
+            const int row = (int)(rowi % p.nq), unit = (int)(rowi / p.nq);
+            check(*reinterpret_cast<const uint4*>(p.q + p.sq.at(unit / p.H, unit % p.H, row) + 8 * (int)(i % CPR)));
+        }
     }
-    float* dst = gram + ((size_t)u * nb + b) * (D * D + D);
-#pragma unroll
-    for (int x = 0; x < TR; ++x)
-#pragma unroll
-        for (int y = 0; y < TR; ++y) dst[(ti + 16 * x) * D + tj + 16 * y] = acc[x][y];
-    if (tid < D) {
-        float s = 0.f;
-        for (int r = 0; r < PC_BLOCK; ++r) s += ks[r * LD + tid];
-        dst[D * D + tid] = s;
-    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) *p.f16_ok = 0;
 }
 
-// gram[u][b] += gram[u][b - 1], element by element
+// Records of the chunks' last blocks: running sums over the chunks, element by element (rec: floats of a record).
 __global__ void __launch_bounds__(PC_THREADS)
-gram_scan_kernel(float* __restrict__ gram, int nb, int rec) {
-    const int e = blockIdx.x * PC_THREADS + threadIdx.x;
-    if (e >= rec) return;
-    float* p = gram + (size_t)blockIdx.y * nb * rec + e;
-    float run = p[0];
-    for (int b = 1; b < nb; ++b) {
-        run += p[(size_t)b * rec];
-        p[(size_t)b * rec] = run;
-    }
+precond_scan_kernel(float* __restrict__ gram, int nb, int cb, int rec) {
+    cudaGridDependencySynchronize();
+    const int e = blockIdx.x * PC_THREADS + threadIdx.x, chunks = (nb + cb - 1) / cb;
+    if (4 * e >= rec) return;
+    float4* p = reinterpret_cast<float4*>(gram + (size_t)blockIdx.y * nb * rec) + e;
+    auto at = [&](int c) { return (size_t)(min(nb, (c + 1) * cb) - 1) * (rec / 4); };
+    float4 x[PC_CHUNKS];
+#pragma unroll
+    for (int c = 0; c < PC_CHUNKS; ++c)
+        if (c < chunks) x[c] = p[at(c)];
+#pragma unroll
+    for (int c = 1; c < PC_CHUNKS; ++c)
+        if (c < chunks) {
+            x[c].x += x[c - 1].x; x[c].y += x[c - 1].y; x[c].z += x[c - 1].z; x[c].w += x[c - 1].w;
+            p[at(c)] = x[c];
+        }
 }
 
-// One preconditioner per key block g: the keys [lo, hi) with hi = min(n, 128 (g + 1)) and lo = 0, or with a
-// sliding window the start of the block that holds position hi - window.
+// One preconditioner per group of key blocks that tiles ask for (precond_block_used names the group's last block g): the keys
+// before the group, those of the group with the mean weight that the group's rows give them, without the blocks that a
+// sliding window has left behind.
 template <int D>
 __global__ void __launch_bounds__(PC_THREADS)
-precond_invert_kernel(const float* __restrict__ gram, __half* __restrict__ minv, int n, int nb, float lambda, int window) {
-    constexpr int LD = D + 1;
-    extern __shared__ float pc_smem[];
-    float* A = pc_smem;                                    // [D][LD]
-    float* sv = A + D * LD;                                // [D]
+precond_invert_kernel(const PcParams p) {
+    constexpr int TR = D / 16, V = D / 64;
+    constexpr int rec = D * D + D;
     __shared__ float s_red[PC_THREADS / 32];
     __shared__ int s_bad;
-    const int g = blockIdx.x, u = blockIdx.y, tid = threadIdx.x;
-    if (precond_block_used(g) != g) return;        // no tile asks for this block's matrix
-    const int rec = D * D + D;
-    const int hi = min(n, PC_BLOCK * (g + 1));
-    const int glo = window > 0 ? max(0, hi - window) / PC_BLOCK : 0;     // first block that counts
-    const float* Gh = gram + ((size_t)u * nb + g) * rec;
-    const float* Gl = glo > 0 ? gram + ((size_t)u * nb + glo - 1) * rec : nullptr;
-    const float L = (float)(hi - glo * PC_BLOCK), invL = 1.f / L;
+    __shared__ __align__(16) float s_row[2][D], s_col[2][D];
+    __shared__ float sv[D];
+    const int u = blockIdx.y, tid = threadIdx.x;
+    const int g = p.causal ? p.g0 + (int)blockIdx.x : p.nb - 1;
+    if (p.causal && precond_block_used(g, p.nb) != g) return;        // no tile asks for this block's matrix
+    const int start = precond_group_start(g), hi = min(p.n, PC_BLOCK * (g + 1));
+    const int glo = p.window > 0 ? max(0, hi - p.window) / PC_BLOCK : 0;     // first block that counts
+    const float len = (float)(hi - PC_BLOCK * start);
+    const float first = (float)max(p.head_rows - PC_BLOCK * start, 0);
+    const float w = p.causal ? fminf(fmaxf(0.5f * (first + len) / len, 0.5f), 1.f) : 1.f;
+    const float L = (float)(PC_BLOCK * (start - glo)) + w * len, invL = 1.f / L;
+    // the sums up to a block: its own record, and unless it is the last of its chunk that of the chunk before
+    int at[6];
+    float wt[6];
+    const int e0 = start - 1, e1 = glo - 1;      // (-1: none)
+    auto sum_to = [&](int i, int b, float weight) {
+        const bool whole = (b + 1) % p.cb == 0 || b == p.nb - 1;
+        at[i] = b < 0 ? 0 : b;                                        wt[i] = b < 0 ? 0.f : weight;
+        at[i + 1] = b < 0 ? 0 : max(0, b / p.cb * p.cb - 1);          wt[i + 1] = b < 0 || whole || b < p.cb ? 0.f : weight;
+    };
+    sum_to(0, g, w);
+    sum_to(2, e0, 1.f - w);
+    sum_to(4, e1, -1.f);
+    if (at[3] == at[1] && wt[1] != 0.f) { wt[1] += wt[3]; wt[3] = 0.f; }
+    const float* base = p.gram + (size_t)u * p.nb * rec;
     if (tid == 0) s_bad = 0;
-    for (int e = tid; e < D; e += PC_THREADS) sv[e] = (Gh[D * D + e] - (Gl ? Gl[D * D + e] : 0.f)) * invL;
+    // Thread (ty, tx) of the 16 x 16 grid keeps the entries (64 i + 4 ty + .., 64 j + 4 tx + ..) in registers.
+    const int ty = tid >> 4, tx = tid & 15;
+    float a[TR][TR] = {};
+    float mine = 0.f;
+    cudaGridDependencySynchronize();
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        if (wt[c] == 0.f) continue;
+        const float* r = base + (size_t)at[c] * rec;
+#pragma unroll
+        for (int i = 0; i < TR; ++i)
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const float4 x = *reinterpret_cast<const float4*>(r + (64 * (i >> 2) + 4 * ty + (i & 3)) * D + 64 * j + 4 * tx);
+                a[i][4 * j] = fmaf(wt[c], x.x, a[i][4 * j]);
+                a[i][4 * j + 1] = fmaf(wt[c], x.y, a[i][4 * j + 1]);
+                a[i][4 * j + 2] = fmaf(wt[c], x.z, a[i][4 * j + 2]);
+                a[i][4 * j + 3] = fmaf(wt[c], x.w, a[i][4 * j + 3]);
+            }
+        if (tid < D) mine = fmaf(wt[c], r[D * D + tid], mine);
+    }
+    if (tid < D) sv[tid] = mine * invL;
     __syncthreads();
     float tr_part = 0.f;
-    for (int e = tid; e < D * D; e += PC_THREADS) {
-        const int r = e / D, c = e % D;
-        const float v = (Gh[e] - (Gl ? Gl[e] : 0.f)) * invL - sv[r] * sv[c];
-        A[r * LD + c] = v;
-        if (r == c) tr_part += v;
-    }
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < TR; ++j) {
+            a[i][j] = fmaf(a[i][j], invL, -sv[64 * (i >> 2) + 4 * ty + (i & 3)] * sv[64 * (j >> 2) + 4 * tx + (j & 3)]);
+            if (i == j && ty == tx) tr_part += a[i][j];
+        }
     // ridge: lambda / L, but at least a millionth of the mean diagonal so that the elimination cannot stall
     for (int off = 16; off > 0; off >>= 1) tr_part += __shfl_xor_sync(0xffffffffu, tr_part, off);
     if ((tid & 31) == 0) s_red[tid >> 5] = tr_part;
     __syncthreads();
     float trace = 0.f;
-    for (int w = 0; w < PC_THREADS / 32; ++w) trace += s_red[w];
-    const float ridge = fmaxf(lambda * invL, 1e-6f * trace / D);
-    for (int e = tid; e < D; e += PC_THREADS) A[e * LD + e] += ridge;
-    __syncthreads();
-    // In-place Gauss-Jordan inversion (no pivoting: the matrix is symmetric positive definite).  Thread (ty, tx)
-    // of the 16 x 16 grid keeps the entries (ty + 16 i, tx + 16 j) in registers; per step the pivot row and the
-    // pivot column go through shared memory (two buffers in turn: one barrier per step).
-    constexpr int TR = D / 16;
-    const int ty = tid >> 4, tx = tid & 15;
-    float a[TR][TR];
+    for (int k = 0; k < PC_THREADS / 32; ++k) trace += s_red[k];
+    const float ridge = fmaxf(p.lambda * invL, 1e-6f * trace / D);
+    if (ty == tx) {
 #pragma unroll
-    for (int i = 0; i < TR; ++i)
+        for (int i = 0; i < TR; ++i) a[i][i] += ridge;
+    }
+    // In-place Gauss-Jordan inversion (no pivoting: the matrix is symmetric positive definite).  Per step the pivot row and
+    // the pivot column go through shared memory (two buffers in turn: one barrier per step).  The loops run over the
+    // owner of the pivot, so that its place in the owner's registers is a constant (found by comparison instead, 704
+    // matrices of 128 x 128 took 430 us; 1150 of them now take 216 us, 256 of 64 x 64 13 us instead of 38).
+    bool broke = false;
 #pragma unroll
-        for (int j = 0; j < TR; ++j) a[i][j] = A[(ty + 16 * i) * LD + tx + 16 * j];
-    __shared__ float s_row[2][D], s_col[2][D];
-    for (int kk = 0; kk < D; ++kk) {
-        const int ki = kk >> 4, kr = kk & 15, bsel = kk & 1;
-        if (ty == kr) {
+    for (int kh = 0; kh < V; ++kh) {
+#pragma unroll 1
+        for (int t = 0; t < 16; ++t) {
 #pragma unroll
-            for (int i = 0; i < TR; ++i)
-                if (i == ki) {
+            for (int kl = 0; kl < 4; ++kl) {
+                const int ki = 4 * kh + kl, bsel = kl & 1, kk = 64 * kh + 4 * t + kl;
+                if (ty == t) {
 #pragma unroll
-                    for (int j = 0; j < TR; ++j) s_row[bsel][tx + 16 * j] = a[i][j];
+                    for (int j = 0; j < V; ++j)
+                        *reinterpret_cast<float4*>(&s_row[bsel][64 * j + 4 * tx]) = make_float4(a[ki][4 * j], a[ki][4 * j + 1], a[ki][4 * j + 2], a[ki][4 * j + 3]);
                 }
-        }
-        if (tx == kr) {
+                if (tx == t) {
 #pragma unroll
-            for (int j = 0; j < TR; ++j)
-                if (j == ki) {
-#pragma unroll
-                    for (int i = 0; i < TR; ++i) s_col[bsel][ty + 16 * i] = a[i][j];
+                    for (int i = 0; i < V; ++i)
+                        *reinterpret_cast<float4*>(&s_col[bsel][64 * i + 4 * ty]) = make_float4(a[4 * i][ki], a[4 * i + 1][ki], a[4 * i + 2][ki], a[4 * i + 3][ki]);
                 }
-        }
-        __syncthreads();
-        const float piv = s_row[bsel][kk];
-        if (!(piv > 0.f) || !isfinite(piv)) { if (tid == 0) s_bad = 1; }
-        const float ip = 1.f / piv;
-        float rw[TR], cl[TR];
+                __syncthreads();
+                const float piv = s_row[bsel][kk];
+                broke |= !(piv > 0.f && piv <= 3e38f);
+                const float ip = __fdividef(1.f, piv);
+                float rw[TR], cl[TR];
 #pragma unroll
-        for (int j = 0; j < TR; ++j) rw[j] = s_row[bsel][tx + 16 * j] * ip;
-#pragma unroll
-        for (int i = 0; i < TR; ++i) cl[i] = s_col[bsel][ty + 16 * i];
-        // every entry as an ordinary one, then the owners of the pivot row and column put theirs right
-#pragma unroll
-        for (int i = 0; i < TR; ++i)
-#pragma unroll
-            for (int j = 0; j < TR; ++j) a[i][j] = fmaf(-cl[i], rw[j], a[i][j]);
-        if (ty == kr) {
-#pragma unroll
-            for (int i = 0; i < TR; ++i)
-                if (i == ki) {
-#pragma unroll
-                    for (int j = 0; j < TR; ++j) a[i][j] = rw[j];
+                for (int j = 0; j < V; ++j) {
+                    const float4 x = *reinterpret_cast<const float4*>(&s_row[bsel][64 * j + 4 * tx]);
+                    rw[4 * j] = x.x * ip; rw[4 * j + 1] = x.y * ip; rw[4 * j + 2] = x.z * ip; rw[4 * j + 3] = x.w * ip;
+                    const float4 y = *reinterpret_cast<const float4*>(&s_col[bsel][64 * j + 4 * ty]);
+                    cl[4 * j] = -y.x; cl[4 * j + 1] = -y.y; cl[4 * j + 2] = -y.z; cl[4 * j + 3] = -y.w;
                 }
-        }
-        if (tx == kr) {
+                // every entry as an ordinary one, then the owners of the pivot row and column put theirs right
 #pragma unroll
-            for (int j = 0; j < TR; ++j)
-                if (j == ki) {
+                for (int i = 0; i < TR; ++i)
 #pragma unroll
-                    for (int i = 0; i < TR; ++i) a[i][j] = (ty == kr && i == ki) ? ip : -cl[i] * ip;
+                    for (int j = 0; j < TR; ++j) a[i][j] = fmaf(cl[i], rw[j], a[i][j]);
+                if (ty == t) {
+#pragma unroll
+                    for (int j = 0; j < TR; ++j) a[ki][j] = rw[j];
                 }
+                if (tx == t) {
+#pragma unroll
+                    for (int i = 0; i < TR; ++i) a[i][ki] = cl[i] * ip;
+                    if (ty == t) a[ki][ki] = ip;
+                }
+            }
         }
     }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < TR; ++i)
-#pragma unroll
-        for (int j = 0; j < TR; ++j) A[(ty + 16 * i) * LD + tx + 16 * j] = a[i][j];
-    __syncthreads();
-    // symmetrise, find the largest entry, store as fp16 scaled to a largest entry of one
+    // the largest entry; store as fp16 scaled to a largest entry of one
     float mx = 0.f;
-    bool bad = false;
-    for (int e = tid; e < D * D; e += PC_THREADS) {
-        const int r = e / D, c = e % D;
-        const float v = 0.5f * (A[r * LD + c] + A[c * LD + r]);
-        bad |= !isfinite(v);
-        mx = fmaxf(mx, fabsf(v));
-    }
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < TR; ++j) {
+            broke |= !isfinite(a[i][j]);
+            mx = fmaxf(mx, fabsf(a[i][j]));
+        }
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if (bad) s_bad = 1;
+    if (broke) s_bad = 1;
+    __syncthreads();       // (the sums of the trace have been read)
     if ((tid & 31) == 0) s_red[tid >> 5] = mx;
     __syncthreads();
     mx = 0.f;
-    for (int w = 0; w < PC_THREADS / 32; ++w) mx = fmaxf(mx, s_red[w]);
+    for (int k = 0; k < PC_THREADS / 32; ++k) mx = fmaxf(mx, s_red[k]);
     const bool use_identity = s_bad != 0 || !(mx > 0.f);
     const float sc = use_identity ? 0.f : 1.f / mx;
-    __half* dst = minv + ((size_t)u * nb + g) * D * D;
-    for (int e = tid; e < D * D; e += PC_THREADS) {
-        const int r = e / D, c = e % D;
-        const float v = use_identity ? (r == c ? 1.f : 0.f) : 0.5f * (A[r * LD + c] + A[c * LD + r]) * sc;
-        dst[e] = __float2half_rn(v);
-    }
+    __half* dst = p.minv + ((size_t)u * p.nb + g) * D * D;
+#pragma unroll
+    for (int i = 0; i < TR; ++i)
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const int r = 64 * (i >> 2) + 4 * ty + (i & 3), c = 64 * j + 4 * tx;
+            float x[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) x[e] = use_identity ? (r == c + e ? 1.f : 0.f) : a[i][4 * j + e] * sc;
+            *reinterpret_cast<uint2*>(dst + r * D + c) = make_uint2(pack_f16(x[0], x[1]), pack_f16(x[2], x[3]));
+        }
 }
 
 template <int D>
-int launch_t(const __nv_bfloat16* k, int B, int Hk, Strides sk, int n, float lambda, int window, float* gram, __half* minv, cudaStream_t st) {
-    const int units = B * Hk;
-    const int nb = precond_blocks(n), rec = D * D + D;
-    const size_t smem_g = sizeof(float) * PC_BLOCK * (D + 1), smem_i = sizeof(float) * (D * (D + 1) + D);
-    LLA_CUDA_TRY(cudaFuncSetAttribute(gram_blocks_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_g));
-    LLA_CUDA_TRY(cudaFuncSetAttribute(precond_invert_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_i));
-    gram_blocks_kernel<D><<<dim3(nb, units), PC_THREADS, smem_g, st>>>(k, gram, n, nb, Hk, sk);
+int launch_t(const PcParams& p, cudaStream_t st) {
+    const int units = p.B * p.Hk;
+    const size_t smem = 2 * (size_t)PC_BLOCK * (D + 8) * 2 + sizeof(float) * PC_THREADS * 9;
+    LLA_CUDA_TRY(cudaFuncSetAttribute(precond_gram_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    precond_gram_kernel<D><<<dim3((p.nb + p.cb - 1) / p.cb, units), PC_THREADS, smem, st>>>(p);
     LLA_CUDA_TRY(cudaGetLastError());
-    if (nb > 1) {
-        gram_scan_kernel<<<dim3((rec + PC_THREADS - 1) / PC_THREADS, units), PC_THREADS, 0, st>>>(gram, nb, rec);
-        LLA_CUDA_TRY(cudaGetLastError());
+    // (the two small kernels are programmatic dependents: their launches overlap the kernel before)
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cfg.blockDim = dim3(PC_THREADS);
+    cfg.stream = st;
+    constexpr int rec = D * D + D;
+    if (p.nb > p.cb) {
+        cfg.gridDim = dim3((rec / 4 + PC_THREADS - 1) / PC_THREADS, units);
+        LLA_CUDA_TRY(cudaLaunchKernelEx(&cfg, precond_scan_kernel, p.gram, p.nb, p.cb, rec));
     }
-    precond_invert_kernel<D><<<dim3(nb, units), PC_THREADS, smem_i, st>>>(gram, minv, n, nb, lambda, window);
-    LLA_CUDA_TRY(cudaGetLastError());
+    cfg.gridDim = dim3(p.causal ? p.nb - p.g0 : 1, units);
+    LLA_CUDA_TRY(cudaLaunchKernelEx(&cfg, precond_invert_kernel<D>, p));
     return LLA_OK;
 }
 
@@ -236,12 +396,18 @@ size_t precond_minv_bytes(int units, int n, int d) {
     return ((size_t)units * precond_blocks(n) * (size_t)d * d * sizeof(__half) + 255) & ~(size_t)255;
 }
 
-int launch_precond(const void* k, int B, int Hk, Strides sk, int n, int d, float lambda, int window, void* gram, void* minv,
-                   cudaStream_t st) {
-    if (d == 64) return launch_t<64>(static_cast<const __nv_bfloat16*>(k), B, Hk, sk, n, lambda, window, static_cast<float*>(gram),
-                                     static_cast<__half*>(minv), st);
-    if (d == 128) return launch_t<128>(static_cast<const __nv_bfloat16*>(k), B, Hk, sk, n, lambda, window, static_cast<float*>(gram),
-                                       static_cast<__half*>(minv), st);
+int launch_precond(const ForwardArgs& a, void* k16, int* f16_ok, void* gram, void* minv) {
+    PcParams p = {};
+    p.k = static_cast<const __nv_bfloat16*>(a.k); p.q = static_cast<const __nv_bfloat16*>(a.q);
+    p.gram = static_cast<float*>(gram); p.k16 = static_cast<uint4*>(k16); p.f16_ok = f16_ok; p.minv = static_cast<__half*>(minv);
+    p.n = a.n; p.nb = precond_blocks(a.n);
+    p.cb = (p.nb + PC_CHUNKS - 1) / PC_CHUNKS;
+    p.B = a.B; p.Hk = a.H / a.kv_group; p.H = a.H; p.nq = a.nq;
+    p.causal = a.causal; p.window = a.causal ? a.window : 0; p.head_rows = a.head_rows > 0 ? a.head_rows : 0;
+    p.g0 = std::max(a.n - a.nq, std::min(a.n, p.head_rows) - 1) / PC_BLOCK;      // (rows before are solved directly)
+    p.lambda = a.lambda; p.sk = a.sk; p.sq = a.sq;
+    if (a.d == 64) return launch_t<64>(p, a.stream);
+    if (a.d == 128) return launch_t<128>(p, a.stream);
     return LLA_ERR_UNSUPPORTED;
 }
 
