@@ -213,17 +213,18 @@ class Prefill:
         nws = L.lla_forward_workspace_bytes(w.B, w.H, w.n, w.d, w.dv)
         self.ws = torch.empty(max(nws, 256), dtype=torch.uint8, device="cuda") if nws else None
         self.ws_bytes = nws
-        self.precondition = 0
+        self.solver_kw = {}        # default solver settings: conjugate gradients preconditioned by the library's own choice
 
     def step(self, i, phases=0):
         w, L = self.w, self.L
         q, k, v = self.sets[i % self.rot]
         L.lla_forward_ex(q, k, v, self.outs[i % self.rot], w.B, w.H, w.n, w.d, w.dv, w.scale, w.lam, causal=1,
                          phases=phases, workspace=self.ws, workspace_bytes=self.ws_bytes, stream=self.sp,
-                         cg_precondition=self.precondition)
+                         **self.solver_kw)
 
     def probe(self):
-        """Iterations actually executed (for the algorithmic flop count) and an fp32 copy of set 0's
+        """Iterations actually executed (for the algorithmic flop count; cg_precondition = 1 is what the timed calls run, which
+        a call that asks for iteration counts has to name) and an fp32 copy of set 0's
         output for the parity figures; outside every timed region."""
         w, L, torch = self.w, self.L, self.torch
         iters = torch.zeros((w.B, w.H, w.n), dtype=torch.int32, device="cuda")
@@ -231,7 +232,7 @@ class Prefill:
         out32 = torch.empty((w.B, w.H, w.n, w.dv), dtype=torch.float32, device="cuda")
         L.lla_forward_ex(*self.sets[0], out32, w.B, w.H, w.n, w.d, w.dv, w.scale, w.lam, causal=1, iters=iters,
                          out_dtype=L.LLA_F32, device_status=status, workspace=self.ws, workspace_bytes=self.ws_bytes,
-                         stream=self.sp)
+                         stream=self.sp, cg_precondition=1)
         torch.cuda.synchronize()
         self.iters = iters.cpu().numpy()
         self.status = status.cpu().numpy()
@@ -268,26 +269,25 @@ class Prefill:
                 "direct_rows_ms_per_launch": ms_direct, "sm_mhz": c["sm_mhz"],
                 "ms_x_mhz": ms_kernel * c["sm_mhz"] if c["sm_mhz"] else None}
 
-    def preconditioned(self, peaks, steps, warmup):
-        """The same step with cg_precondition = 1 (inverse key covariance per block of 128 keys as CG preconditioner,
-        built by a pre-pass inside the timed call): fewer iterations, so fewer algorithmic flops and less time."""
+    def plain_cg(self, peaks, steps, warmup):
+        """The same step by Algorithm 2 as it stands (its iteration cap given, which takes the choice from the library)."""
         w, L, torch = self.w, self.L, self.torch
-        self.precondition = 1
+        self.solver_kw = {"max_iters": 64}
         iters = torch.zeros((w.B, w.H, w.n), dtype=torch.int32, device="cuda")
         L.lla_forward_ex(*self.sets[0], self.outs[0], w.B, w.H, w.n, w.d, w.dv, w.scale, w.lam, causal=1, iters=iters,
-                         workspace=self.ws, workspace_bytes=self.ws_bytes, stream=self.sp, cg_precondition=1)
+                         workspace=self.ws, workspace_bytes=self.ws_bytes, stream=self.sp, **self.solver_kw)
         torch.cuda.synchronize()
         it = iters.cpu().numpy()
         ms, clk = self.timed(steps, warmup)
-        self.precondition = 0
+        self.solver_kw = {}
         ms /= steps
         fl = algorithmic_flops(w, it)
         cg = it[it >= 0]
         c = clk.summary()
         return {"ms_per_step": ms, "tokens_per_s": w.B * w.n / (ms * 1e-3), "cg_mean_iters": float(cg.mean()) if cg.size else 0.0,
                 "tflops": fl / (ms * 1e-3) / 1e12, "frac_of_bf16_peak_whole_step": fl / (ms * 1e-3) / 1e12 / peaks["bf16_tflops"],
-                "sm_mhz": c["sm_mhz"], "note": "optional mode (lla_forward_params.cg_precondition = 1); pre-pass kernels "
-                "inside the timed step; flops count the iterations executed, which this mode roughly halves"}, clk
+                "sm_mhz": c["sm_mhz"], "note": "without the preconditioner (max_iters given); flops count the iterations executed, "
+                "about twice as many"}, clk
 
     def solver(self):
         L = self.L
@@ -307,8 +307,8 @@ def measure_leg(L, torch, peaks, w, local, steps, warmup):
     ms_d, _ = p.timed(steps, 3, L.LLA_PHASE_DIRECT)
     ms_step = ms_all / steps
     c = clk_all.summary()
-    pre, clk_p = p.preconditioned(peaks, max(10, steps // 2), 3)
-    leg = {"config": workload_config(w), "steps": steps, "ms_per_step": ms_step, "preconditioned": pre,
+    pre, clk_p = p.plain_cg(peaks, max(10, steps // 2), 3)
+    leg = {"config": workload_config(w), "steps": steps, "ms_per_step": ms_step, "plain_cg": pre,
            "tokens_per_s": w.B * w.n / (ms_step * 1e-3),
            "tflops": algorithmic_flops(w, p.iters) / (ms_step * 1e-3) / 1e12,
            "frac_of_bf16_peak_whole_step": algorithmic_flops(w, p.iters) / (ms_step * 1e-3) / 1e12 / peaks["bf16_tflops"],
@@ -365,7 +365,7 @@ def run_ours(args):
     ms_kernel /= args.steps
     ms_direct /= args.steps
 
-    pre_leg, clk_p = head.preconditioned(peaks, max(5, args.steps // 2), 3)
+    pre_leg, clk_p = head.plain_cg(peaks, max(5, args.steps // 2), 3)
     samplers.append(clk_p)
 
     # ---- end to end through the host-buffer entry point (pinned memory) ----
@@ -434,14 +434,14 @@ def run_ours(args):
         "tflops": flops_step / (ms_step * 1e-3) / 1e12,
         "frac_of_bf16_peak_whole_step": flops_step / (ms_step * 1e-3) / 1e12 / peaks["bf16_tflops"],
         "sm_mhz": c_head["sm_mhz"], "ms_x_mhz": ms_step * c_head["sm_mhz"] if c_head["sm_mhz"] else None,
-        "roofline": roof, "preconditioned": pre_leg,
+        "roofline": roof, "plain_cg": pre_leg,
         "e2e": {"value": world * tokens_step * e2e_steps / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": int(pout.numel() * 2), "steps": e2e_steps,
                 "ms_per_step": 1e3 * e2e_s / e2e_steps,
                 "note": "lla_forward_host on pinned buffers; the host link carries "
                         f"{(h2d + pout.numel() * 2) / 1e6:.0f} MB per step"},
         # per step: the fp16 copy of k, the iterative-rows kernel, the direct-rows kernel
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": 5 * args.steps,
     }
     line.update(legs)
     if decode is not None:
@@ -524,7 +524,7 @@ def bench_backward(L, torch, peaks, pre, local, steps=20, warmup=3, nsets=4):
         L.lla_backward_ex(*saved[i % nsets], *grads, w.B, w.H, w.n, w.d, w.scale, w.lam, workspace=ws,
                           workspace_bytes=nbytes, stream=sp, **kw)
 
-    step(0, iters=iters)
+    step(0, iters=iters, cg_precondition=1)      # what the timed steps run
     torch.cuda.synchronize()
     it = iters.cpu().numpy().reshape(-1, w.n).astype(np.float64)
     pairs = np.arange(1, w.n + 1, dtype=np.float64)
@@ -542,13 +542,13 @@ def bench_backward(L, torch, peaks, pre, local, steps=20, warmup=3, nsets=4):
         e1.record(stream)
         torch.cuda.synchronize()
     ms = e0.elapsed_time(e1) / steps
-    # the same steps with the extra solve preconditioned (optional mode, as in the forward)
-    step(0, iters=iters, cg_precondition=1)
+    # the same steps with plain conjugate gradients in the extra solve (the iteration cap given, as in the forward)
+    step(0, iters=iters, max_iters=64)
     torch.cuda.synchronize()
     it_pc = iters.cpu().numpy().reshape(-1, w.n).astype(np.float64)
     e0.record(stream)
     for i in range(steps):
-        step(warmup + i, cg_precondition=1)
+        step(warmup + i, max_iters=64)
     e1.record(stream)
     torch.cuda.synchronize()
     ms_pc = e0.elapsed_time(e1) / steps
@@ -559,12 +559,12 @@ def bench_backward(L, torch, peaks, pre, local, steps=20, warmup=3, nsets=4):
             "frac_of_bf16_peak": flops / (ms * 1e-3) / 1e12 / peaks["bf16_tflops"],
             "roofline": {"bound": "tensor", "achieved": flops / (ms * 1e-3) / 1e12, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                          "frac": flops / (ms * 1e-3) / 1e12 / peaks["bf16_tflops"], "traffic": None,
-                         "kernel": "the whole pass (eight launches: solve, dK/dV, dQ, moments, direct rows, ...; profiles/backward_cfg3.md)",
+                         "kernel": "the whole pass (ten launches: solve, dK/dV, dQ, moments, direct rows, ...; profiles/backward_cfg3.md)",
                          "peak_source": f"{peaks['source']} burst bf16 (MEASURED_PEAKS.json)"},
             "cg_mean_iters": float(it[it >= 0].mean()) if (it >= 0).any() else 0.0,
-            "preconditioned": {"ms_per_step": ms_pc, "cg_mean_iters": float(it_pc[it_pc >= 0].mean()) if (it_pc >= 0).any() else 0.0,
-                               "note": "optional mode (lla_backward_params.cg_precondition = 1)"},
-            "algorithmic_flops_per_step": flops, "gpu_launches_per_step": 8,
+            "plain_cg": {"ms_per_step": ms_pc, "cg_mean_iters": float(it_pc[it_pc >= 0].mean()) if (it_pc >= 0).any() else 0.0,
+                               "note": "extra solve without the preconditioner (max_iters given)"},
+            "algorithmic_flops_per_step": flops, "gpu_launches_per_step": 10,
             "sm_mhz": c["sm_mhz"], "ms_x_mhz": ms * c["sm_mhz"] if c["sm_mhz"] else None,
             "l2": f"inputs and saved tensors rotate over {nsets} sets ({nsets * set_bytes / 1e6:.0f} MB > 126 MB L2)",
             "inputs": "bf16 q, k, v; fp32 upstream gradient, forward output, rho, stats; fp32 gradients"}, clk

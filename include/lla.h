@@ -209,14 +209,16 @@ typedef struct lla_forward_params {
                        and the directly-solved rows are untouched) and the blocks on the tile's diagonal.  NULL =
                        dense.  n <= 65536.  Shapes the tensor-core kernel does not cover: LLA_ERR_UNSUPPORTED */
     long long block_mask_stride;     /* bytes from one (batch, head) unit's mask to the next; 0 = one mask for all */
-    int cg_precondition;  /* tensor-core kernel only.  0 = plain conjugate gradients as in Algorithm 2 (default).
-                       1 = preconditioned with the inverse covariance of the visible keys: one d x d matrix per
-                       block of 128 keys, built by a pre-pass into `workspace` (plain CG without room for it
-                       there).  The system of a row is that covariance under the row's attention weights, so the
-                       closer the weights are to uniform the fewer iterations remain -- about half on the
-                       synthetic workloads; with sharply peaked weights it may not pay for its pre-pass.  The
+    int cg_precondition;  /* tensor-core kernel only.  1 = conjugate gradients preconditioned with the inverse covariance of the
+                       visible keys: a d x d matrix per block of 128 keys, built by a pre-pass into `workspace` (plain CG
+                       without room for it there).  The system of a row is that covariance under the row's attention
+                       weights, so the closer the weights are to uniform the fewer iterations remain -- half and less
+                       on the synthetic workloads, four fifths with scores of unit variance.  The
                        solution is the same within the tolerance; a row on which the rounded matrix turns out
-                       not to be positive definite carries on with plain CG */
+                       not to be positive definite carries on with plain CG.
+                       0 = default: with the other solver settings (max_iters, tol, cg_precise_iters, impl) at their
+                       defaults, no `iters`, no lambda_rows and the ridge of the definition, the library chooses, which at
+                       present means as with 1 unless there are fewer than n / 4 query rows; otherwise plain conjugate gradients as in Algorithm 2 */
     long long debug_wait_clocks; /* tensor-core kernel only: cap, in SM clocks, of every bounded wait on a barrier
                        inside the kernel (0 = default, about 2^31).  A wait that runs out makes its thread block
                        stop: the block waits for the copies and MMAs it has issued itself, releases its tensor
@@ -410,7 +412,8 @@ typedef struct lla_backward_params {
     int window;   /* as in lla_forward_params: the forward being differentiated ran with this causal sliding window
                      (0: none).  At least head_rows, and not with impl = LLA_IMPL_SIMT: LLA_ERR_UNSUPPORTED otherwise */
     int cg_precondition; /* as in lla_forward_params: 1 = the extra solve runs the preconditioned conjugate gradients
-                     (about half the iterations; same result within the tolerance) */
+                     (about half the iterations; same result within the tolerance), 0 = the library's choice unless
+                     max_iters, tol, impl or iters is given */
     const unsigned char *block_mask; /* as in lla_forward_params: the forward being differentiated ran with this block
                      mask (same layout, same always-attended blocks; NULL = dense).  Not with a window, n > 65536 or
                      impl = LLA_IMPL_SIMT: LLA_ERR_UNSUPPORTED */

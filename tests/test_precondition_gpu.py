@@ -1,0 +1,87 @@
+"""The solver that a call with default settings gets: conjugate gradients preconditioned per group of key blocks."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2510_01450_b200 import binding as L, inputs
+from tests.gpu_util import dev, row_err, stream_ptr
+from tests.test_parity_gpu import TOL_BF16
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(d, n, nq, H, Hkv, spread, seed):
+    w = inputs.CONFIGS[2].shrink(B=1, H=H, n=n, d=d, dv=d, seed=seed)
+    q, _, _ = inputs.make_prefill(w)
+    _, k, v = inputs.make_prefill(w.shrink(H=Hkv, seed=seed + 1))
+    return w, inputs.round_to_bf16(q[:, :, n - nq:] * np.float32(spread)), k, v
+
+
+@pytest.mark.parametrize("d,n,nq,H,Hkv,window,causal,spread", [
+    (64, 97, 97, 2, 2, 0, True, 1.0),          # two rows beyond the directly solved ones
+    (64, 129, 129, 2, 2, 0, True, 1.0),        # a second block of one key
+    (128, 193, 193, 2, 2, 0, True, 1.0),
+    (64, 2305, 2305, 1, 1, 0, True, 1.0),      # pairs of blocks share a matrix, the last group has one block of one key
+    (128, 1177, 300, 4, 2, 0, True, 1.0),      # a chunk of queries: heads packed, pairs of thread blocks
+    (64, 1000, 257, 4, 1, 0, True, 12.0),      # the same with sharply peaked weights
+    (64, 1400, 1400, 2, 2, 333, True, 1.0),    # window
+    (64, 700, 700, 2, 2, 0, False, 1.0),       # every row sees every key
+])
+def test_default_solver_against_explicit_solves(d, n, nq, H, Hkv, window, causal, spread):
+    """Both solvers stop at a residual of 1e-4; the default one may not be further from the float64 solution than the plain
+    one is, beyond the half that two stopping points below the same bound can differ by."""
+    w, q, k, v = _case(d, n, nq, H, Hkv, spread, 700 + n)
+    nbytes = L.lla_forward_workspace_bytes(1, H, n, d, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    args = [dev(x, "bf16") for x in (q, k, v)]
+    outs = []
+    for kw in ({}, {"max_iters": 64}):
+        out = torch.full((1, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+        status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+        L.lla_forward_ex(*args, out, 1, H, n, d, d, w.scale, w.lam, causal=causal, out_dtype=L.LLA_F32, q_rows=nq, kv_heads=Hkv,
+                         window=window, device_status=status, workspace=ws, workspace_bytes=nbytes, stream=stream_ptr(), **kw)
+        torch.cuda.synchronize()
+        st = status.cpu().tolist()
+        assert st[L.STATUS_TIMEOUT] == 0 and st[L.STATUS_ROWS_AT_CAP] == 0
+        outs.append((out.cpu().numpy()[0].astype(np.float64), st[L.STATUS_ITER_SUM]))
+    assert np.isfinite(outs[0][0]).all()
+    rows = np.unique(np.concatenate([np.arange(0, nq, max(1, nq // 40)), [nq - 1]]))
+    errs = [[], []]
+    for h in range(H):
+        K, V = k[0, h * Hkv // H].astype(np.float64), v[0, h * Hkv // H].astype(np.float64)
+        for r in rows:
+            c = n - nq + r + 1 if causal else n
+            lo = max(0, c - window) if window else 0
+            s = w.scale * K[lo:c] @ q[0, h, r].astype(np.float64)
+            wt, z = np.exp(s - s.max()), K[lo:c] - q[0, h, r]
+            rho = np.linalg.solve((wt[:, None] * z).T @ z + w.lam * np.exp(-s.max()) * np.eye(d), wt @ z)
+            a = wt * (1 - z @ rho)
+            ref = a @ V[lo:c] / a.sum()
+            for e, (o, _) in zip(errs, outs):
+                e.append(row_err(o[h, r], ref[None])[0])
+    default, plain = (np.asarray(e) for e in errs)
+    assert default.max() <= TOL_BF16
+    assert np.sqrt(np.mean(default ** 2)) <= 1.5 * np.sqrt(np.mean(plain ** 2)) + 1e-6
+    if spread == 1.0:
+        assert outs[0][1] < outs[1][1]            # fewer iterations: it is the preconditioned solver that ran
+
+
+def test_an_input_outside_the_fp16_range_turns_the_matrices_off():
+    # an entry of k beyond 6e4, in a key that no row sees: the copies, and with them the preconditioner, are off on the
+    # device, and what runs is the plain solver on operand pairs
+    n, nq = 300, 100
+    w, q, k, v = _case(64, n, nq, 1, 1, 1.0, 31)
+    nbytes = L.lla_forward_workspace_bytes(1, 1, n, 64, 64)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    sums = []
+    for entry in (1.0, 70000.0):
+        k[0, 0, 7, 5] = entry
+        out = torch.full((1, 1, nq, 64), float("nan"), dtype=torch.float32, device="cuda")
+        status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+        L.lla_forward_ex(dev(q, "bf16"), dev(k, "bf16"), dev(v, "bf16"), out, 1, 1, n, 64, 64, w.scale, w.lam, out_dtype=L.LLA_F32,
+                         q_rows=nq, window=150, device_status=status, workspace=ws, workspace_bytes=nbytes, stream=stream_ptr())
+        torch.cuda.synchronize()
+        sums.append((out.cpu().numpy(), status.cpu().tolist()[L.STATUS_ITER_SUM]))
+    assert sums[0][1] < sums[1][1]
+    assert row_err(sums[0][0], sums[1][0].astype(np.float64)).max() <= 4e-4      # two stopping points below 1e-4 each
