@@ -494,17 +494,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             pair_sync();
             return buf[lrow] + buf[128 + lrow];
         };
-        // two sums for one barrier
-        auto pair_sum2 = [&](float& a, float& b) {
-            float* buf = red + red_sel * 1024;
-            red_sel ^= 1;
-            buf[half * 128 + lrow] = a;
-            buf[256 + half * 128 + lrow] = b;
-            pair_sync();
-            a = buf[lrow] + buf[128 + lrow];
-            b = buf[256 + lrow] + buf[384 + lrow];
-        };
-        // three
+        // three sums for one barrier
         auto pair_sum3 = [&](float& a, float& b, float& c) {
             float* buf = red + red_sel * 1024;
             red_sel ^= 1;
