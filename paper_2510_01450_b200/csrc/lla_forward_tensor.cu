@@ -316,7 +316,8 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             auto load_m = [&]() {
                 if (Cfg::Q_IN_TMEM && !mbar_wait(bar(B_QREAD), 0, abort_flag, wcap)) return;
                 const int last = !prm.causal ? n - 1 : min(n - 1, off + (wraps ? prm.nq_pos : r0p + TC_BR) - 1);
-                const int gm = precond_block_used(last / 128, (n + 127) / 128);
+                // (with a window one per query tile of a head; for the tiles that grouped heads share, the one of the middle row)
+                const int gm = prm.window > 0 && prm.causal ? min(r0p + TC_BR / 2, prm.nq_pos - 1) / TC_BR : precond_block_used(last / 128, (n + 127) / 128);
                 m_issued = true;
                 mbar_expect_tx(bar(B_MFULL), D * D * 2);
                 for (int rb = 0; rb < D / 64; ++rb)
@@ -1335,7 +1336,10 @@ int launch_t(const ForwardArgs& a) {
     // can fill tiles together where a head's own rows leave its last tile partly empty (257 rows of four heads: nine
     // tiles instead of twelve).  Their rows must lie one behind the other in q, and none may be solved directly.
     const int group = a.kv_group;
+    // Nor with a narrow window and the preconditioner, whose matrix then is that of one head's tile: a row elsewhere in
+    // the sequence sees other keys, too few of them (fewer than 8 d) for their covariance to be much the same.
     const bool pack = group > 1 && hr == 0 && !a.block_mask && a.sq.h == (long long)a.nq * a.sq.r &&
+                      !(a.minv && a.causal && a.window > 0 && a.window < 8 * D) &&
                       (group * a.nq + TC_BR - 1) / TC_BR < group * tiles;
     const int units = pack ? a.B * Hk : a.B * a.H;          // unit: the rows that are cut into tiles together
     const int unit_rows = pack ? group * a.nq : a.nq;

@@ -13,6 +13,11 @@
 // (With full weight the first row is off by a whole block: 15.8 instead of 12.1 iterations in the second tile at d = 64, 6.0
 // instead of 5.0 in the sixth, three instead of two past 14 K keys at d = 128.)
 //
+// A sliding window moves with the row, so there every query tile has a matrix of its own, in which each block of keys has the
+// weight of its mean share in the windows of the tile's rows: the block that the first rows see none of, and the one that
+// the last rows have left behind, count by the keys that a row of the tile sees of them on average.  The weights lie between
+// zero and one and add up to the mean number of visible keys, which is at least one: nothing here divides by zero.
+//
 // Three kernels, all on the caller's stream ahead of the forward kernel:
 //   precond_gram_kernel     a chunk of key blocks each: running sums of k_j k_j^T and k_j inside the chunk, one record per
 //                           block that is asked for.  It reads every key once, so it also makes the fp16 copy of k and
@@ -45,9 +50,10 @@ struct PcParams {
     float* gram;       // [units][blocks][D * D + D]
     uint4* k16;        // [units][n][D] fp16
     int* f16_ok;       // cleared if an entry of k or q lies outside the fp16 range
-    __half* minv;      // [units][blocks][D][D]
+    __half* minv;      // [units][blocks][D][D]; with a window the first [tiles] of a unit's are in use
     int n, nb, cb;     // keys; blocks; blocks per chunk
-    int g0;            // first block that a query sees last
+    int g0;            // first block that a query sees last; with a window the first query tile that is not solved directly
+    int tiles;         // query tiles of 128 rows per head
     int B, Hk, H, nq;
     int causal, window, head_rows;
     float lambda;
@@ -199,62 +205,102 @@ precond_scan_kernel(float* __restrict__ gram, int nb, int cb, int rec) {
         }
 }
 
+// The integers t <= y of min(max(t, 0), len) added up.
+__device__ __forceinline__ long long sum_clamped(long long y, long long len) {
+    return y <= 0 ? 0 : y <= len ? y * (y + 1) / 2 : len * (len + 1) / 2 + (y - len) * len;
+}
+
+// The matrix of query tile t under a sliding window: the mean share of key block b in the windows of the tile's rows, which sit
+// at the positions first .. last.  (A row at i sees the keys i + 1 - window .. i from zero on.)
+__device__ __forceinline__ float window_share(int first, int last, int window, int b, int n) {
+    if (b < 0 || PC_BLOCK * b > last) return 0.f;
+    const long long len = min(n - PC_BLOCK * b, PC_BLOCK), e = last + 1ll - PC_BLOCK * b, f = first - (long long)PC_BLOCK * b;
+    const long long seen = sum_clamped(e, len) - sum_clamped(f, len);
+    const long long left = sum_clamped(e - window, len) - sum_clamped(f - window, len);
+    return (float)(seen - left) / (float)(len * (last - first + 1));
+}
+
 // One preconditioner per group of key blocks that tiles ask for (precond_block_used names the group's last block g): the keys
-// before the group, those of the group with the mean weight that the group's rows give them, without the blocks that a
-// sliding window has left behind.
+// before the group, those of the group with the mean weight that the group's rows give them.  With a sliding window one per
+// query tile: every block of keys with its mean share in the windows of the tile's rows.
+constexpr int PC_TERMS = 12;
 template <int D>
 __global__ void __launch_bounds__(PC_THREADS)
 precond_invert_kernel(const PcParams p) {
     constexpr int TR = D / 16, V = D / 64;
     constexpr int rec = D * D + D;
     __shared__ float s_red[PC_THREADS / 32];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_at[PC_TERMS], s_terms;
     __shared__ __align__(16) float s_row[2][D], s_col[2][D];
-    __shared__ float sv[D];
+    __shared__ float sv[D], s_wt[PC_TERMS];
     const int u = blockIdx.y, tid = threadIdx.x;
-    const int g = p.causal ? p.g0 + (int)blockIdx.x : p.nb - 1;
-    if (p.causal && precond_block_used(g, p.nb) != g) return;        // no tile asks for this block's matrix
-    const int start = precond_group_start(g), hi = min(p.n, PC_BLOCK * (g + 1));
-    const int glo = p.window > 0 ? max(0, hi - p.window) / PC_BLOCK : 0;     // first block that counts
-    const float len = (float)(hi - PC_BLOCK * start);
-    const float first = (float)max(p.head_rows - PC_BLOCK * start, 0);
-    const float w = p.causal ? fminf(fmaxf(0.5f * (first + len) / len, 0.5f), 1.f) : 1.f;
-    const float L = (float)(PC_BLOCK * (start - glo)) + w * len, invL = 1.f / L;
-    // the sums up to a block: its own record, and unless it is the last of its chunk that of the chunk before
-    int at[6];
-    float wt[6];
-    const int e0 = start - 1, e1 = glo - 1;      // (-1: none)
-    auto sum_to = [&](int i, int b, float weight) {
-        const bool whole = (b + 1) % p.cb == 0 || b == p.nb - 1;
-        at[i] = b < 0 ? 0 : b;                                        wt[i] = b < 0 ? 0.f : weight;
-        at[i + 1] = b < 0 ? 0 : max(0, b / p.cb * p.cb - 1);          wt[i + 1] = b < 0 || whole || b < p.cb ? 0.f : weight;
+    const int g = p.causal ? p.g0 + (int)blockIdx.x : p.nb - 1;      // the matrix's place; a query tile with a window
+    float L;
+    int terms = 0;
+    // the sums up to block b: its own record, and unless it is the last of its chunk that of the chunk before
+    auto add = [&](int at, float weight) {
+        for (int i = 0; i < terms; ++i)
+            if (s_at[i] == at) { s_wt[i] += weight; return; }
+        s_at[terms] = at;
+        s_wt[terms++] = weight;
     };
-    sum_to(0, g, w);
-    sum_to(2, e0, 1.f - w);
-    sum_to(4, e1, -1.f);
-    if (at[3] == at[1] && wt[1] != 0.f) { wt[1] += wt[3]; wt[3] = 0.f; }
+    auto sum_to = [&](int b, float weight) {
+        if (b < 0 || weight == 0.f) return;
+        add(b, weight);
+        if ((b + 1) % p.cb != 0 && b != p.nb - 1 && b >= p.cb) add(b / p.cb * p.cb - 1, weight);
+    };
+    if (p.window > 0) {
+        if (g >= p.tiles) return;
+        const int off = p.n - p.nq;
+        const int last = min(p.n - 1, off + PC_BLOCK * g + PC_BLOCK - 1);
+        const int first = min(max(off + PC_BLOCK * g, p.head_rows - 1), last);
+        auto share = [&](int b) { return window_share(first, last, p.window, b, p.n); };
+        // the mean number of visible keys
+        L = (float)(sum_clamped(last + 1, p.window) - sum_clamped(first, p.window)) / (float)(last - first + 1);
+        if (tid == 0) {
+            // sum_b share(b) block(b) in the running sums: the shares change at the two blocks that hold the first rows' and the
+            // last rows' first keys and at the two that hold the rows themselves
+            const int lo = max(0, first + 1 - p.window) / PC_BLOCK, hi = last / PC_BLOCK;
+            for (int b = lo - 1; b <= min(lo + 1, hi); ++b) sum_to(b, share(b) - share(b + 1));
+            for (int b = max(lo + 2, hi - 2); b <= hi; ++b) sum_to(b, share(b) - share(b + 1));
+            s_terms = terms;
+        }
+    } else {
+        if (p.causal && precond_block_used(g, p.nb) != g) return;        // no tile asks for this block's matrix
+        const int start = precond_group_start(g), hi = min(p.n, PC_BLOCK * (g + 1));
+        const float len = (float)(hi - PC_BLOCK * start);
+        const float first = (float)max(p.head_rows - PC_BLOCK * start, 0);
+        const float w = p.causal ? fminf(fmaxf(0.5f * (first + len) / len, 0.5f), 1.f) : 1.f;
+        L = (float)(PC_BLOCK * start) + w * len;
+        if (tid == 0) {
+            sum_to(g, w);
+            sum_to(start - 1, 1.f - w);
+            s_terms = terms;
+        }
+    }
+    const float invL = 1.f / L;
     const float* base = p.gram + (size_t)u * p.nb * rec;
     if (tid == 0) s_bad = 0;
     // Thread (ty, tx) of the 16 x 16 grid keeps the entries (64 i + 4 ty + .., 64 j + 4 tx + ..) in registers.
     const int ty = tid >> 4, tx = tid & 15;
     float a[TR][TR] = {};
     float mine = 0.f;
+    __syncthreads();
     cudaGridDependencySynchronize();
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-        if (wt[c] == 0.f) continue;
-        const float* r = base + (size_t)at[c] * rec;
+    for (int c = 0; c < s_terms; ++c) {
+        const float wt = s_wt[c];
+        const float* r = base + (size_t)s_at[c] * rec;
 #pragma unroll
         for (int i = 0; i < TR; ++i)
 #pragma unroll
             for (int j = 0; j < V; ++j) {
                 const float4 x = *reinterpret_cast<const float4*>(r + (64 * (i >> 2) + 4 * ty + (i & 3)) * D + 64 * j + 4 * tx);
-                a[i][4 * j] = fmaf(wt[c], x.x, a[i][4 * j]);
-                a[i][4 * j + 1] = fmaf(wt[c], x.y, a[i][4 * j + 1]);
-                a[i][4 * j + 2] = fmaf(wt[c], x.z, a[i][4 * j + 2]);
-                a[i][4 * j + 3] = fmaf(wt[c], x.w, a[i][4 * j + 3]);
+                a[i][4 * j] = fmaf(wt, x.x, a[i][4 * j]);
+                a[i][4 * j + 1] = fmaf(wt, x.y, a[i][4 * j + 1]);
+                a[i][4 * j + 2] = fmaf(wt, x.z, a[i][4 * j + 2]);
+                a[i][4 * j + 3] = fmaf(wt, x.w, a[i][4 * j + 3]);
             }
-        if (tid < D) mine = fmaf(wt[c], r[D * D + tid], mine);
+        if (tid < D) mine = fmaf(wt, r[D * D + tid], mine);
     }
     if (tid < D) sv[tid] = mine * invL;
     __syncthreads();
@@ -380,7 +426,7 @@ int launch_t(const PcParams& p, cudaStream_t st) {
         cfg.gridDim = dim3((rec / 4 + PC_THREADS - 1) / PC_THREADS, units);
         LLA_CUDA_TRY(cudaLaunchKernelEx(&cfg, precond_scan_kernel, p.gram, p.nb, p.cb, rec));
     }
-    cfg.gridDim = dim3(p.causal ? p.nb - p.g0 : 1, units);
+    cfg.gridDim = dim3(p.window > 0 ? std::max(p.tiles - p.g0, 1) : p.causal ? p.nb - p.g0 : 1, units);
     LLA_CUDA_TRY(cudaLaunchKernelEx(&cfg, precond_invert_kernel<D>, p));
     return LLA_OK;
 }
@@ -404,7 +450,9 @@ int launch_precond(const ForwardArgs& a, void* k16, int* f16_ok, void* gram, voi
     p.cb = (p.nb + PC_CHUNKS - 1) / PC_CHUNKS;
     p.B = a.B; p.Hk = a.H / a.kv_group; p.H = a.H; p.nq = a.nq;
     p.causal = a.causal; p.window = a.causal ? a.window : 0; p.head_rows = a.head_rows > 0 ? a.head_rows : 0;
-    p.g0 = std::max(a.n - a.nq, std::min(a.n, p.head_rows) - 1) / PC_BLOCK;      // (rows before are solved directly)
+    p.tiles = (a.nq + PC_BLOCK - 1) / PC_BLOCK;
+    p.g0 = p.window > 0 ? head_rows_count(a) / PC_BLOCK          // (rows before are solved directly)
+                        : std::max(a.n - a.nq, std::min(a.n, p.head_rows) - 1) / PC_BLOCK;
     p.lambda = a.lambda; p.sk = a.sk; p.sq = a.sq;
     if (a.d == 64) return launch_t<64>(p, a.stream);
     if (a.d == 128) return launch_t<128>(p, a.stream);

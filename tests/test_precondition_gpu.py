@@ -85,3 +85,60 @@ def test_an_input_outside_the_fp16_range_turns_the_matrices_off():
         sums.append((out.cpu().numpy(), status.cpu().tolist()[L.STATUS_ITER_SUM]))
     assert sums[0][1] < sums[1][1]
     assert row_err(sums[0][0], sums[1][0].astype(np.float64)).max() <= 4e-4      # two stopping points below 1e-4 each
+
+
+def _solve(w, q, k, v, nq, Hkv, **kw):
+    """Output (float64 numpy), iterations per row, rows at the cap; the cap as in a default call."""
+    nbytes = L.lla_forward_workspace_bytes(1, w.H, w.n, w.d, w.d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    out = torch.full((1, w.H, nq, w.d), float("nan"), dtype=torch.float32, device="cuda")
+    status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+    iters = torch.full((1, w.H, nq), -1, dtype=torch.int32, device="cuda")
+    L.lla_forward_ex(dev(q, "bf16"), dev(k, "bf16"), dev(v, "bf16"), out, 1, w.H, w.n, w.d, w.d, w.scale, w.lam, out_dtype=L.LLA_F32,
+                     q_rows=nq, kv_heads=Hkv, device_status=status, iters=iters, workspace=ws, workspace_bytes=nbytes, stream=stream_ptr(),
+                     **{"max_iters": 64, **kw})
+    torch.cuda.synchronize()
+    st = status.cpu().tolist()
+    assert st[L.STATUS_TIMEOUT] == 0
+    return out.cpu().numpy()[0].astype(np.float64), iters.cpu().numpy()[0], st[L.STATUS_ROWS_AT_CAP]
+
+
+def _exact(w, q, k, v, h, hk, rows, nq, window=0):
+    ref = []
+    K, V = k[0, hk].astype(np.float64), v[0, hk].astype(np.float64)
+    for r in rows:
+        c = w.n - nq + r + 1
+        lo = max(0, c - window) if window else 0
+        s = w.scale * K[lo:c] @ q[0, h, r].astype(np.float64)
+        wt, z = np.exp(s - s.max()), K[lo:c] - q[0, h, r]
+        rho = np.linalg.solve((wt[:, None] * z).T @ z + w.lam * np.exp(-s.max()) * np.eye(w.d), wt @ z)
+        a = wt * (1 - z @ rho)
+        ref.append(a @ V[lo:c] / a.sum())
+    return np.asarray(ref)
+
+
+@pytest.mark.parametrize("d,n,nq,H,Hkv,window,spread", [
+    (64, 2637, 2637, 2, 2, 96, 1.0),       # the narrowest window: a tile's windows lie in two blocks of keys
+    (64, 2500, 2500, 2, 2, 128, 1.0),
+    (64, 2637, 1111, 4, 2, 160, 1.0),      # a chunk whose tiles do not start at a block of keys, grouped heads
+    (128, 2500, 2500, 2, 2, 192, 1.0),
+    (128, 2637, 2637, 2, 2, 256, 1.0),
+    (128, 2637, 2637, 2, 2, 224, 8 * 2 ** 0.5),      # scores of unit variance
+    (64, 2500, 2500, 2, 2, 333, 8.0),
+])
+def test_the_matrices_of_a_window_are_made_of_the_keys_that_its_rows_see(d, n, nq, H, Hkv, window, spread):
+    """Past 2048 keys and below it: fewer iterations than plain conjugate gradients in the first and in the second tile of every
+    256 rows, no more rows that run into the cap, and no larger error (two stopping points below one bound: half)."""
+    w, q, k, v = _case(d, n, nq, H, Hkv, 1.0, 900 + n + window)
+    s = np.float32(d ** 0.5 if spread > 1 else 1.0)      # (q and k ~ N(0, 1): q . k / sqrt(d) of unit variance)
+    q, k = inputs.round_to_bf16(q * s), inputs.round_to_bf16(k * s)
+    rows = np.unique(np.concatenate([np.linspace(max(0, d + d // 2 - (n - nq)), nq - 1, 30).astype(int), [nq - 129, nq - 1]]))
+    got = [_solve(w, q, k, v, nq, Hkv, window=window, **kw) for kw in ({"cg_precondition": 1}, {})]
+    ref = _exact(w, q, k, v, H - 1, Hkv - 1, rows, nq, window)
+    rms = [np.sqrt(np.mean(row_err(o[H - 1, rows], ref) ** 2)) for o, _, _ in got]
+    assert rms[0] <= 1.5 * rms[1] + 1e-6
+    assert got[0][2] <= got[1][2]
+    for part in (0, 1):
+        its = [i[:, (np.arange(nq) // 128 % 2) == part] for _, i, _ in got]
+        its = [i[i >= 0].mean() for i in its]
+        assert its[0] < 0.9 * its[1], (part, its)
