@@ -304,21 +304,26 @@ precond_invert_kernel(const PcParams p) {
     }
     if (tid < D) sv[tid] = mine * invL;
     __syncthreads();
-    float tr_part = 0.f;
+    float sq_part = 0.f;
 #pragma unroll
     for (int i = 0; i < TR; ++i)
 #pragma unroll
         for (int j = 0; j < TR; ++j) {
             a[i][j] = fmaf(a[i][j], invL, -sv[64 * (i >> 2) + 4 * ty + (i & 3)] * sv[64 * (j >> 2) + 4 * tx + (j & 3)]);
-            if (i == j && ty == tx) tr_part += a[i][j];
+            sq_part = fmaf(a[i][j], a[i][j], sq_part);
         }
-    // ridge: lambda / L, but at least a millionth of the mean diagonal so that the elimination cannot stall
-    for (int off = 16; off > 0; off >>= 1) tr_part += __shfl_xor_sync(0xffffffffu, tr_part, off);
-    if ((tid & 31) == 0) s_red[tid >> 5] = tr_part;
+    // Ridge: lambda / L, but at least a 4000th of the covariance's Frobenius norm, which bounds its largest eigenvalue.  The fp16
+    // entries of the inverse, the largest of which is one, are off by 2^-12, the matrix as a whole by about 1e-4; without the
+    // bound the inverse of keys in a subspace is all ridge, and what it says of the subspace lies below that: r . M r has any sign, and
+    // rows with such a matrix needed more iterations than without (keys of rank 60, d = 64, n = 2500: 20.6 instead of
+    // 14.6 with 1269 rows at the cap).  Where the spectrum spans more than the bound the iterations grow with the square root of what
+    // is beyond (standard deviations from 1 to 0.01: 5 -> 10 iterations, plain conjugate gradients: 64 and more).
+    for (int off = 16; off > 0; off >>= 1) sq_part += __shfl_xor_sync(0xffffffffu, sq_part, off);
+    if ((tid & 31) == 0) s_red[tid >> 5] = sq_part;
     __syncthreads();
-    float trace = 0.f;
-    for (int k = 0; k < PC_THREADS / 32; ++k) trace += s_red[k];
-    const float ridge = fmaxf(p.lambda * invL, 1e-6f * trace / D);
+    float sq = 0.f;
+    for (int k = 0; k < PC_THREADS / 32; ++k) sq += s_red[k];
+    const float ridge = fmaxf(p.lambda * invL, sqrtf(sq) * (1.f / 4000.f));
     if (ty == tx) {
 #pragma unroll
         for (int i = 0; i < TR; ++i) a[i][i] += ridge;
@@ -385,7 +390,7 @@ precond_invert_kernel(const PcParams p) {
         }
     for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
     if (broke) s_bad = 1;
-    __syncthreads();       // (the sums of the trace have been read)
+    __syncthreads();       // (the sums of the squares have been read)
     if ((tid & 31) == 0) s_red[tid >> 5] = mx;
     __syncthreads();
     mx = 0.f;

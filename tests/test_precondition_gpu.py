@@ -142,3 +142,26 @@ def test_the_matrices_of_a_window_are_made_of_the_keys_that_its_rows_see(d, n, n
         its = [i[:, (np.arange(nq) // 128 % 2) == part] for _, i, _ in got]
         its = [i[i >= 0].mean() for i in its]
         assert its[0] < 0.9 * its[1], (part, its)
+
+
+@pytest.mark.parametrize("d,n,rank,distinct", [(64, 1700, 32, 0), (64, 2500, 60, 0), (128, 2500, 124, 0), (128, 1300, 64, 0)])
+def test_keys_that_do_not_span_the_space(d, n, rank, distinct):
+    """Keys (and queries) in a subspace, up to their rounding to bf16, or few different keys: an inverse covariance that is all
+    ridge outside the subspace must not drown what it says inside.  Not more iterations than plain conjugate gradients,
+    nor rows at the cap, nor a larger error."""
+    H = 2
+    w, q, k, v = _case(d, n, n, H, H, 1.0, 1200 + n + rank)
+    rng = np.random.default_rng(7)
+    basis = np.linalg.qr(rng.standard_normal((d, d)))[0][:, :rank]
+    proj = (basis @ basis.T * (d / rank) ** 0.5).astype(np.float32)
+    if distinct:
+        k = k[:, :, rng.integers(0, distinct, n)]
+    else:
+        q, k = inputs.round_to_bf16(q @ proj), inputs.round_to_bf16(k @ proj)
+    rows = np.linspace(d + d // 2, n - 1, 40).astype(int)
+    got = [_solve(w, q, k, v, n, H, **kw) for kw in ({"cg_precondition": 1}, {})]
+    ref = _exact(w, q, k, v, H - 1, H - 1, rows, n)
+    rms = [np.sqrt(np.mean(row_err(o[H - 1, rows], ref) ** 2)) for o, _, _ in got]
+    its = [i[i >= 0].mean() for _, i, _ in got]
+    assert its[0] < its[1] and got[0][2] <= got[1][2], (its, got[0][2], got[1][2])
+    assert rms[0] <= 1.5 * rms[1] + 1e-6, rms
