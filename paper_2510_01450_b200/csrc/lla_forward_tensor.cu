@@ -535,14 +535,14 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
         };
 
-        // the same vector as an fp16 hi + lo pair (the output sweep's y once the sweeps run on fp16 operands)
-        auto write_operand16_pair = [&](const float* vec) {
+        // the same vector times sc as an fp16 hi + lo pair (the output sweep's y where the sweeps run on fp16 operands)
+        auto write_operand16_pair = [&](const float* vec, float sc) {
 #pragma unroll
             for (int ch = 0; ch < NCOL / 8; ++ch) {
                 uint32_t hi[4], lo[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float a = vec[ch * 8 + 2 * e], b = vec[ch * 8 + 2 * e + 1];
+                    const float a = vec[ch * 8 + 2 * e] * sc, b = vec[ch * 8 + 2 * e + 1] * sc;
                     const __half2 h2 = __floats2half2_rn(a, b);
                     const float2 f = __half22float2(h2);
                     const __half2 l2 = __floats2half2_rn(a - f.x, b - f.y);
@@ -628,7 +628,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // [1, 2.83) over the row's largest weight (where that is above one), so that its entries and u = w (a - abar) sit in
         // the middle of the fp16 range whatever the scale of the right-hand side; pn2 tracks |p|^2 through the recurrence
         // |p'|^2 = |r'|^2 + beta^2 |p|^2
-        float pn2 = 0.f, psc = 1.f, ipsc = 1.f;
+        float pn2 = 0.f, psc = 1.f, ipsc = 1.f;               // (in the output sweep ipsc undoes the scale of y)
         int wexp = 0;                                         // largest weight of the row is at most 2^wexp
         uint32_t ablk = 0;                                    // blocks with a product A so far (D = 128: slot = ablk % 2)
         float smax = -INFINITY;                               // statistics sweep: largest score of the row, relative to the shift
@@ -649,7 +649,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             float part = 0.f;                                 // omega / den partial
             const uint64_t c1c1 = pk2(c1, c1), nmx = pk2(-mx2, -mx2);
             const float ab_s = kind == SW_CG16 || kind == SW_CG16P ? abar * psc : abar;
-            const uint64_t nab = pk2(-ab_s, -ab_s), oab = pk2(1.f + abar, 1.f + abar), neg1 = pk2(-1.f, -1.f);
+            const uint64_t nab = pk2(-ab_s, -ab_s), oab = pk2(1.f + abar, 1.f + abar), neg1 = pk2(-ipsc, -ipsc);
             uint64_t part2 = pk2(0.f, 0.f);
             const uint32_t a0 = ablk;
             if (kind != SW_STATS) ablk += nblk;
@@ -830,12 +830,15 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // the products of a hi + lo pair (32 heads, n = 4096, d = 64: 1394 -> 1350 us, and the error against float64 falls from
         // 1.5e-4 to 0.9e-4).  (Directions that are off by 2^-12 cost conjugacy, not consistency: x and r still
         // belong together.)  What is left is the rounding of U, whose errors average over the keys.
+        auto scale_of = [&](float nrm2, int below) {
+            const int e2 = (int)((__float_as_uint(nrm2) >> 23) & 0xffu) - 127;      // floor(log2 |p|^2)
+            const int k = max(-100, min(100, -(e2 >> 1) - below));
+            psc = __uint_as_float((uint32_t)(127 + k) << 23);
+            ipsc = __uint_as_float((uint32_t)(127 - k) << 23);
+        };
         auto write_p = [&]() {
             if (f16_on) {
-                const int e2 = (int)((__float_as_uint(pn2) >> 23) & 0xffu) - 127;      // floor(log2 |p|^2)
-                const int k = max(-100, min(100, -(e2 >> 1) - wexp));
-                psc = __uint_as_float((uint32_t)(127 + k) << 23);
-                ipsc = __uint_as_float((uint32_t)(127 - k) << 23);
+                scale_of(pn2, wexp);
                 write_operand16(p, psc, ipsc);
             } else {
                 write_operand(p);
@@ -1157,7 +1160,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
         } else if (ok) {
             float y[NCOL];
-            float yb_p = 0.f, g_p = 0.f;
+            float yb_p = 0.f, g_p = 0.f, yy_p = 0.f;
             uint32_t qt[NCOL / 2];
             load_q(qt);
 #pragma unroll
@@ -1170,13 +1173,21 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                     y[col] = x_get(col);
                     yb_p += kb * y[col];
                     g_p += (kb - qv) * y[col];
+                    yy_p += y[col] * y[col];
                 }
             }
-            abar = pair_sum(yb_p);
-            gfac = 1.f + pair_sum(g_p);
-            // (over the other block's last sums, like p: the vote that ended the loop lies in between)
-            if (f16_on) write_operand16_pair(y);
-            else write_operand(y);
+            pair_sum3(yb_p, g_p, yy_p);
+            abar = yb_p;
+            gfac = 1.f + g_p;
+            // (over the other block's last sums, like p: the vote that ended the loop lies in between.)  In fp16 scaled by a power of
+            // two that brings |y| to [1, 2.83): y grows with the inverse of the ridge where the keys are small or few, beyond the range
+            ipsc = 1.f;
+            if (f16_on) {
+                scale_of(yy_p, 0);
+                write_operand16_pair(y, psc);
+            } else {
+                write_operand(y);
+            }
             start_sweep(SW_OUT);
             float part = sweep_of(std::integral_constant<int, SW_OUT>{}, std::false_type{});      // (V stays bf16)
             if (ok) acc_wait();

@@ -144,7 +144,7 @@ def test_the_matrices_of_a_window_are_made_of_the_keys_that_its_rows_see(d, n, n
         assert its[0] < 0.9 * its[1], (part, its)
 
 
-@pytest.mark.parametrize("d,n,rank,distinct", [(64, 1700, 32, 0), (64, 2500, 60, 0), (128, 2500, 124, 0), (128, 1300, 64, 0)])
+@pytest.mark.parametrize("d,n,rank,distinct", [(64, 1700, 32, 0), (64, 2500, 60, 0), (128, 2500, 124, 0), (128, 1300, 64, 0), (64, 1300, 64, 40)])
 def test_keys_that_do_not_span_the_space(d, n, rank, distinct):
     """Keys (and queries) in a subspace, up to their rounding to bf16, or few different keys: an inverse covariance that is all
     ridge outside the subspace must not drown what it says inside.  Not more iterations than plain conjugate gradients,
@@ -165,3 +165,16 @@ def test_keys_that_do_not_span_the_space(d, n, rank, distinct):
     its = [i[i >= 0].mean() for _, i, _ in got]
     assert its[0] < its[1] and got[0][2] <= got[1][2], (its, got[0][2], got[1][2])
     assert rms[0] <= 1.5 * rms[1] + 1e-6, rms
+
+
+@pytest.mark.parametrize("d,scale_k,n", [(64, 1e-3, 700), (64, 1e-2, 1500), (128, 1e-2, 1300)])
+def test_solutions_beyond_the_fp16_range(d, scale_k, n):
+    """Small keys under ordinary queries: the solution grows with the inverse of the ridge, beyond 65504, and the coefficients
+    formed from it must not."""
+    w, q, k, v = _case(d, n, n, 1, 1, 1.0, 1300 + n)
+    k = inputs.round_to_bf16(k * np.float32(scale_k))
+    rows = np.linspace(d + d // 2, n - 1, 30).astype(int)
+    ref = _exact(w, q, k, v, 0, 0, rows, n)
+    for kw in ({"max_iters": 0}, {}, {"cg_precondition": 1}):
+        out, _, _ = _solve(w, q, k, v, n, 1, **kw)
+        assert row_err(out[0, rows], ref).max() <= TOL_BF16, kw
