@@ -924,7 +924,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             }
             tc_fence_before();
         };
-        bool prec_row = true;   // false once the preconditioner has failed this row (z = r from then on)
+        // false: z = r.  From the start for rows that see fewer than 1.5 D keys (head_rows below its default), whose covariance
+        // has too little in common with that of the tile's mean row (head_rows = 0, n = 500, 4 heads: twice the rows at the cap
+        // with z = M r), and once the preconditioner has failed a row
+        bool prec_row = !prm.causal || L - jlo >= D + D / 2;
         // From the residual in rv: r . z, |z|^2 and z . p ...
         auto z_sums = [&](const float* rv, float& rz_p, float& zz_p, float& zp_p) {
             rz_p = zz_p = zp_p = 0.f;
@@ -1038,7 +1041,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             if (ok) {
                 float rz_p, zz_p, unused;
                 z_sums(p, rz_p, zz_p, unused);
-                if (rz_p > 0.f) {
+                if (prec_row && rz_p > 0.f) {
                     rz = rz_p; pn2 = zz_p;
                 } else {
                     // the rounded matrix is not positive on this residual: the row runs unpreconditioned, p = r

@@ -178,3 +178,16 @@ def test_solutions_beyond_the_fp16_range(d, scale_k, n):
     for kw in ({"max_iters": 0}, {}, {"cg_precondition": 1}):
         out, _, _ = _solve(w, q, k, v, n, 1, **kw)
         assert row_err(out[0, rows], ref).max() <= TOL_BF16, kw
+
+
+@pytest.mark.parametrize("d,n,kw", [(64, 500, dict(head_rows=-1)), (128, 500, dict(head_rows=40)), (64, 2600, dict(head_rows=16, window=48)),
+                                    (128, 700, dict(head_rows=-1, window=20))])
+def test_rows_of_few_keys_run_plain_conjugate_gradients(d, n, kw):
+    """With head_rows below 1.5 d the solver gets rows whose covariance is not the tile's: by default the call is plain, and where the
+    preconditioner is asked for it leaves those rows alone."""
+    w, q, k, v = _case(d, n, n, 2, 2, 1.0, 1400 + n)
+    plain, default, asked = (_solve(w, q, k, v, n, 2, **s, **kw) for s in ({}, {"max_iters": 0}, {"cg_precondition": 1}))
+    assert np.array_equal(plain[0], default[0], equal_nan=True)
+    few = np.arange(n) + 1 < d + d // 2 if "window" not in kw else np.ones(n, dtype=bool)
+    at_cap = [(r[1][:, few] >= 64).sum() for r in (plain, asked)]
+    assert at_cap[1] <= 1.1 * at_cap[0] + 2, at_cap
