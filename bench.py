@@ -223,8 +223,7 @@ class Prefill:
                          **self.solver_kw)
 
     def probe(self):
-        """Iterations actually executed (for the algorithmic flop count; cg_precondition = 1 is what the timed calls run, which
-        a call that asks for iteration counts has to name) and an fp32 copy of set 0's
+        """Iterations actually executed (for the algorithmic flop count) and an fp32 copy of set 0's
         output for the parity figures; outside every timed region."""
         w, L, torch = self.w, self.L, self.torch
         iters = torch.zeros((w.B, w.H, w.n), dtype=torch.int32, device="cuda")
@@ -232,7 +231,7 @@ class Prefill:
         out32 = torch.empty((w.B, w.H, w.n, w.dv), dtype=torch.float32, device="cuda")
         L.lla_forward_ex(*self.sets[0], out32, w.B, w.H, w.n, w.d, w.dv, w.scale, w.lam, causal=1, iters=iters,
                          out_dtype=L.LLA_F32, device_status=status, workspace=self.ws, workspace_bytes=self.ws_bytes,
-                         stream=self.sp, cg_precondition=1)
+                         stream=self.sp)
         torch.cuda.synchronize()
         self.iters = iters.cpu().numpy()
         self.status = status.cpu().numpy()
@@ -524,7 +523,7 @@ def bench_backward(L, torch, peaks, pre, local, steps=20, warmup=3, nsets=4):
         L.lla_backward_ex(*saved[i % nsets], *grads, w.B, w.H, w.n, w.d, w.scale, w.lam, workspace=ws,
                           workspace_bytes=nbytes, stream=sp, **kw)
 
-    step(0, iters=iters, cg_precondition=1)      # what the timed steps run
+    step(0, iters=iters)
     torch.cuda.synchronize()
     it = iters.cpu().numpy().reshape(-1, w.n).astype(np.float64)
     pairs = np.arange(1, w.n + 1, dtype=np.float64)

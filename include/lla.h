@@ -217,7 +217,7 @@ typedef struct lla_forward_params {
                        solution is the same within the tolerance; a row on which the rounded matrix turns out
                        not to be positive definite carries on with plain CG.
                        0 = default: with the other solver settings (max_iters, tol, cg_precise_iters, impl) at their
-                       defaults, head_rows at its default or above 1.5 d, no `iters`, no lambda_rows and the ridge of the definition, the library chooses, which at
+                       defaults, head_rows at its default or above 1.5 d, no lambda_rows and the ridge of the definition, the library chooses, which at
                        present means as with 1 unless there are fewer than n / 4 query rows; otherwise plain conjugate gradients as in Algorithm 2 */
     long long debug_wait_clocks; /* tensor-core kernel only: cap, in SM clocks, of every bounded wait on a barrier
                        inside the kernel (0 = default, about 2^31).  A wait that runs out makes its thread block
@@ -413,7 +413,7 @@ typedef struct lla_backward_params {
                      (0: none).  At least head_rows, and not with impl = LLA_IMPL_SIMT: LLA_ERR_UNSUPPORTED otherwise */
     int cg_precondition; /* as in lla_forward_params: 1 = the extra solve runs the preconditioned conjugate gradients
                      (about half the iterations; same result within the tolerance), 0 = the library's choice unless
-                     max_iters, tol, impl, iters or a head_rows below 1.5 d is given */
+                     max_iters, tol, impl or a head_rows below 1.5 d is given */
     const unsigned char *block_mask; /* as in lla_forward_params: the forward being differentiated ran with this block
                      mask (same layout, same always-attended blocks; NULL = dense).  Not with a window, n > 65536 or
                      impl = LLA_IMPL_SIMT: LLA_ERR_UNSUPPORTED */

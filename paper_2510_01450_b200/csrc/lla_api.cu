@@ -130,10 +130,10 @@ ForwardArgs to_args(const lla_forward_params* p) {
         if (src[0] || src[1] || src[2]) dst = lla::Strides{src[0], src[1], src[2]};
     };
     take(a.sq, p->q_strides); take(a.sk, p->k_strides); take(a.sv, p->v_strides); take(a.so, p->out_strides);
-    // Under the default solver settings the solver is the library's choice (a call that asks for iteration counts or sets
-    // anything of the solver gets Algorithm 2 as it stands); the matrices know the scalar ridge of the definition only, and
+    // Under the default solver settings the solver is the library's choice (a call that sets anything of the solver gets
+    // Algorithm 2 as it stands; `iters` only reports, so it has no say); the matrices know the scalar ridge of the definition only, and
     // rows of fewer than 1.5 d keys, which a smaller head_rows leaves to the solver, are better off without.
-    const bool free_choice = p->max_iters == 0 && p->tol == 0.f && p->cg_precise_iters == 0 && p->impl == LLA_IMPL_AUTO && !p->iters &&
+    const bool free_choice = p->max_iters == 0 && p->tol == 0.f && p->cg_precise_iters == 0 && p->impl == LLA_IMPL_AUTO &&
                              !p->lambda_rows && p->ridge_mode == LLA_RIDGE_DEFINITION && a.head_rows >= p->d + p->d / 2;
     a.precondition = p->cg_precondition > 0 || (free_choice && precondition_pays(a.n, a.nq)) ? 1 : 0;
     a.no_loads = (p->debug_flags & LLA_DEBUG_NO_LOADS) ? 1 : 0;
@@ -463,7 +463,7 @@ int lla_backward_ex(const lla_backward_params* p) {
     a.window = p->window;
     if (p->cg_precondition != 0 && p->cg_precondition != 1) return LLA_ERR_INVALID_ARG;
     // (as in the forward: the solver is the library's choice unless the call says something of it)
-    a.precondition = p->cg_precondition || (p->max_iters == 0 && p->tol == 0.f && p->impl == LLA_IMPL_AUTO && !p->iters &&
+    a.precondition = p->cg_precondition || (p->max_iters == 0 && p->tol == 0.f && p->impl == LLA_IMPL_AUTO &&
                                             a.head_rows >= p->d + p->d / 2 && precondition_pays(p->n, p->q_rows > 0 ? p->q_rows : p->n));
     // block sparsity: under the forward's conditions, and in the tensor-core kernels only
     if (p->block_mask && (a.cuda_core_pairs || a.window > 0 || p->n > 65536 || p->block_mask_stride < 0)) return LLA_ERR_UNSUPPORTED;

@@ -343,7 +343,7 @@ def test_backward_with_preconditioned_solve(backward_oracle):
     g = inputs.make_upstream_grad(w)
     ref = backward_oracle.backward(q, k, v, g, w.scale, w.lam)
     its = [torch.full((w.B, w.H, w.n), -1, dtype=torch.int32, device="cuda") for _ in range(2)]
-    plain = run_backward(w, q, k, v, g, iters=its[0])
+    plain = run_backward(w, q, k, v, g, iters=its[0], max_iters=64)      # (a cap that is given: conjugate gradients as they stand)
     got = run_backward(w, q, k, v, g, iters=its[1], cg_precondition=1)
     for name, a, b in zip(("dq", "dk", "dv"), got, ref):
         assert grad_err(a, b).max() <= TOL, name

@@ -13,6 +13,7 @@ from tests.test_parity_gpu import TOL_BF16
 pytestmark = pytest.mark.gpu
 
 
+@pytest.mark.parametrize("solver", [{}, {"max_iters": 64}, {"cg_precondition": 1}], ids=["default", "plain", "preconditioned"])
 @pytest.mark.parametrize("d,H,Hkv,n,nq,window,causal", [
     (64, 4, 4, 900, 300, 0, True),         # pairs, a ragged last tile
     (64, 8, 2, 700, 129, 0, True),         # packed rows of four heads: tiles that run over a head's end; pairs
@@ -22,7 +23,7 @@ pytestmark = pytest.mark.gpu
     (128, 6, 3, 600, 1, 0, True),          # one query per head: two rows in a tile
     (64, 16, 4, 2000, 700, 0, True),       # packed tiles, more of them than half the SMs
 ])
-def test_pairs_and_packed_rows(oracle, d, H, Hkv, n, nq, window, causal):
+def test_pairs_and_packed_rows(oracle, d, H, Hkv, n, nq, window, causal, solver):
     B = 2
     w = inputs.CONFIGS[2].shrink(B=B, H=H, n=n, d=d, dv=d, seed=500 + d + n)
     q, _, _ = inputs.make_prefill(w)
@@ -37,7 +38,7 @@ def test_pairs_and_packed_rows(oracle, d, H, Hkv, n, nq, window, causal):
     for _ in range(2):
         L.lla_forward_ex(dev(qc, "bf16"), dev(k, "bf16"), dev(v, "bf16"), out, B, H, n, d, d, w.scale, w.lam, causal=causal,
                          out_dtype=L.LLA_F32, q_rows=nq, kv_heads=Hkv, window=window, rho=rho, stats=stats, iters=iters,
-                         device_status=status, workspace=ws, workspace_bytes=nbytes, stream=stream_ptr())
+                         device_status=status, workspace=ws, workspace_bytes=nbytes, stream=stream_ptr(), **solver)
     torch.cuda.synchronize()
     assert status.cpu().numpy()[L.STATUS_TIMEOUT] == 0
     assert (iters.cpu().numpy() >= -1).all()

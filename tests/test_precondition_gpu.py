@@ -191,3 +191,24 @@ def test_rows_of_few_keys_run_plain_conjugate_gradients(d, n, kw):
     few = np.arange(n) + 1 < d + d // 2 if "window" not in kw else np.ones(n, dtype=bool)
     at_cap = [(r[1][:, few] >= 64).sum() for r in (plain, asked)]
     assert at_cap[1] <= 1.1 * at_cap[0] + 2, at_cap
+
+
+@pytest.mark.parametrize("d,n,nq", [(64, 700, 700), (128, 900, 400)])
+def test_asking_for_iteration_counts_changes_nothing(d, n, nq):
+    """The same bits with and without `iters`, and counts that are those of the solver that ran."""
+    w, q, k, v = _case(d, n, nq, 2, 2, 1.0, 1500 + n)
+    args = [dev(x, "bf16") for x in (q, k, v)]
+    nbytes = L.lla_forward_workspace_bytes(1, 2, n, d, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    outs = []
+    iters = torch.full((1, 2, nq), -1, dtype=torch.int32, device="cuda")
+    for it in (None, iters):
+        out = torch.full((1, 2, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+        status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+        L.lla_forward_ex(*args, out, 1, 2, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, q_rows=nq, device_status=status, iters=it,
+                         workspace=ws, workspace_bytes=nbytes, stream=stream_ptr())
+        torch.cuda.synchronize()
+        outs.append((out, status.cpu().tolist()[L.STATUS_ITER_SUM]))
+    assert torch.equal(outs[0][0], outs[1][0]) and outs[0][1] == outs[1][1]
+    it = iters.cpu().numpy()
+    assert it[it > 0].sum() == outs[1][1]
