@@ -218,7 +218,7 @@ typedef struct lla_forward_params {
                        not to be positive definite carries on with plain CG.
                        0 = default: with the other solver settings (max_iters, tol, cg_precise_iters, impl) at their
                        defaults, head_rows at its default or above 1.5 d, no lambda_rows and the ridge of the definition, the library chooses, which at
-                       present means as with 1 unless there are fewer than n / 4 query rows; otherwise plain conjugate gradients as in Algorithm 2 */
+                       present means as with 1 unless there are fewer than n / 4 query rows or a block mask; otherwise plain conjugate gradients as in Algorithm 2 */
     long long debug_wait_clocks; /* tensor-core kernel only: cap, in SM clocks, of every bounded wait on a barrier
                        inside the kernel (0 = default, about 2^31).  A wait that runs out makes its thread block
                        stop: the block waits for the copies and MMAs it has issued itself, releases its tensor

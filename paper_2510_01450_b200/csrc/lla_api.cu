@@ -72,7 +72,9 @@ bool head_size_ok(int d, int dv) { return d == dv && (d == 16 || d == 64 || d ==
 // The preconditioner's pre-pass reads every key, its gain is in the sweeps of the query tiles: whole sequences gain 15 % (32
 // heads, n = 1024, d = 64: 309 -> 266 us) to 30 % (16 heads, n = 16384, d = 128: 12.9 -> 9.0 ms), a chunk of 257 queries on 5003
 // keys with scores of unit variance loses (16 heads over 4, d = 128: 577 -> 633 us).
-bool precondition_pays(int n, int nq) { return 4ll * nq >= n; }
+// Nor under a block mask: the matrices are those of all keys, and a row that attends some needs as many iterations with them as
+// without (8 heads, n = 8192, d = 64, 5 % of the blocks: 474 -> 546 us; d = 128, n = 4096, scores of unit variance: 1377 -> 1767 us).
+bool precondition_pays(int n, int nq, bool masked) { return 4ll * nq >= n && !masked; }
 
 int check_forward(const lla_forward_params* p) {
     if (!p) return LLA_ERR_INVALID_ARG;
@@ -135,7 +137,7 @@ ForwardArgs to_args(const lla_forward_params* p) {
     // rows of fewer than 1.5 d keys, which a smaller head_rows leaves to the solver, are better off without.
     const bool free_choice = p->max_iters == 0 && p->tol == 0.f && p->cg_precise_iters == 0 && p->impl == LLA_IMPL_AUTO &&
                              !p->lambda_rows && p->ridge_mode == LLA_RIDGE_DEFINITION && a.head_rows >= p->d + p->d / 2;
-    a.precondition = p->cg_precondition > 0 || (free_choice && precondition_pays(a.n, a.nq)) ? 1 : 0;
+    a.precondition = p->cg_precondition > 0 || (free_choice && precondition_pays(a.n, a.nq, p->block_mask != nullptr)) ? 1 : 0;
     a.no_loads = (p->debug_flags & LLA_DEBUG_NO_LOADS) ? 1 : 0;
     if (p->cg_precise_iters != 0) {
         a.precise_iters = p->cg_precise_iters == LLA_CG_PRECISE_NONE ? 0 : p->cg_precise_iters < 0 ? (1 << 30) : p->cg_precise_iters;
@@ -464,7 +466,7 @@ int lla_backward_ex(const lla_backward_params* p) {
     if (p->cg_precondition != 0 && p->cg_precondition != 1) return LLA_ERR_INVALID_ARG;
     // (as in the forward: the solver is the library's choice unless the call says something of it)
     a.precondition = p->cg_precondition || (p->max_iters == 0 && p->tol == 0.f && p->impl == LLA_IMPL_AUTO &&
-                                            a.head_rows >= p->d + p->d / 2 && precondition_pays(p->n, p->q_rows > 0 ? p->q_rows : p->n));
+                                            a.head_rows >= p->d + p->d / 2 && precondition_pays(p->n, p->q_rows > 0 ? p->q_rows : p->n, p->block_mask != nullptr));
     // block sparsity: under the forward's conditions, and in the tensor-core kernels only
     if (p->block_mask && (a.cuda_core_pairs || a.window > 0 || p->n > 65536 || p->block_mask_stride < 0)) return LLA_ERR_UNSUPPORTED;
     a.block_mask = p->block_mask; a.block_mask_stride = p->block_mask_stride;

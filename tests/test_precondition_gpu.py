@@ -212,3 +212,13 @@ def test_asking_for_iteration_counts_changes_nothing(d, n, nq):
     assert torch.equal(outs[0][0], outs[1][0]) and outs[0][1] == outs[1][1]
     it = iters.cpu().numpy()
     assert it[it > 0].sum() == outs[1][1]
+
+
+def test_a_block_mask_runs_plain_conjugate_gradients():
+    """The matrices are those of all keys, a masked row sees some: by default the call is the plain one, bit for bit."""
+    n, d = 1500, 64
+    w, q, k, v = _case(d, n, n, 2, 2, 1.0, 1600)
+    mask = (np.random.default_rng(3).random(((n + 127) // 128, (n + 63) // 64)) < 0.2).astype(np.uint8)
+    m = torch.from_numpy(mask).cuda()
+    plain, default = (_solve(w, q, k, v, n, 2, block_mask=m, **s) for s in ({}, {"max_iters": 0}))
+    assert np.array_equal(plain[0], default[0]) and np.array_equal(plain[1], default[1])
