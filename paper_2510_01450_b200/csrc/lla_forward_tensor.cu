@@ -1022,11 +1022,12 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                 }
                 rr = pair_sum(rr_p);
                 stop = prm.tol * prm.tol * rr;
-                // The preconditioned solver goes on to half the residual in the tile next to the directly solved rows, whose
-                // systems turn a residual into a many times larger error: the largest element error of a gradient is found
-                // there (n = 16384, d = 128: 6.5e-3 -> 5.1e-3 of the gradient's mean square root from one call to another),
-                // for one iteration in that tile.
-                if (PC && first_pos + TC_BR <= 2 * D) stop *= 0.25f;
+                // The preconditioned solver goes on to half the residual in rows of at most 2 D keys, whose systems turn a
+                // residual into a many times larger error: the largest element error of a gradient is found in those next to
+                // the directly solved ones (n = 16384, d = 128: 6.5e-3 -> 5.1e-3 of the gradient's mean square root from
+                // one call to another), for one or two iterations.  (By the row's keys and not by its tile: a
+                // chunk's tiles start anywhere, and under a narrow window every row is such a row.)
+                if (PC && L - jlo <= 2 * D) stop *= 0.25f;
                 active = row_ok && rr > 0.f;
                 pn2 = rr;
                 rz = rr;

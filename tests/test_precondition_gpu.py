@@ -222,3 +222,35 @@ def test_a_block_mask_runs_plain_conjugate_gradients():
     m = torch.from_numpy(mask).cuda()
     plain, default = (_solve(w, q, k, v, n, 2, block_mask=m, **s) for s in ({}, {"max_iters": 0}))
     assert np.array_equal(plain[0], default[0]) and np.array_equal(plain[1], default[1])
+
+
+@pytest.mark.parametrize("d,n,nq,window", [(64, 500, 460, 0), (64, 500, 439, 0), (128, 700, 580, 0), (64, 1500, 1500, 120), (128, 1500, 1500, 250)])
+def test_rows_of_few_keys_go_on_to_half_the_residual(d, n, nq, window):
+    """Whatever tile a row of at most 2 d keys falls into: in a chunk whose tiles start elsewhere, and under a window.  The residual
+    is that of the saved solution, in float64: y = rho / (1 - b . rho) solves C y = b to half of 1e-4; nine rows in ten
+    within another quarter of the tolerance for what rounding adds to the solver's own residual (operand pairs in every iteration:
+    of the order of 1e-5)."""
+    H = 4
+    w, q, k, v = _case(d, n, nq, H, H, 1.0, 1700 + nq)
+    seen = np.arange(n - nq, n) + 1
+    seen = np.minimum(seen, window) if window else seen
+    rows = np.flatnonzero((seen >= d + d // 2) & (seen <= 2 * d))
+    rows = rows[:: max(1, len(rows) // 40)]
+    rho = torch.zeros((1, H, nq, d), dtype=torch.float32, device="cuda")
+    _solve(w, q, k, v, nq, H, window=window, cg_precondition=1, cg_precise_iters=64, rho=rho)
+    rho = rho.cpu().numpy()[0].astype(np.float64)
+    res = []
+    for h in range(H):
+        K = k[0, h].astype(np.float64)
+        for r in rows:
+            c = n - nq + r + 1
+            kk = K[max(0, c - window) if window else 0:c]
+            sc = w.scale * kk @ q[0, h, r].astype(np.float64)
+            wt = np.exp(sc - sc.max())
+            kb = wt @ kk / wt.sum()
+            b = kb - q[0, h, r]
+            y = rho[h, r] / (1 - b @ rho[h, r])
+            cy = (wt * ((kk - kb) @ y)) @ (kk - kb) / wt.sum() + w.lam * np.exp(-sc.max()) / wt.sum() * y
+            res.append(np.linalg.norm(b - cy) / np.linalg.norm(b))
+    res = np.asarray(res)
+    assert np.quantile(res, 0.5) <= 0.5e-4 and np.quantile(res, 0.9) <= 0.75e-4, np.sort(res)[::8]
