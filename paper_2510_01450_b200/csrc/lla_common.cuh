@@ -118,8 +118,8 @@ struct ForwardArgs {
     int no_loads = 0;           // aid: issue no copy at all (lla_forward_params.debug_*)
     const void* minv = nullptr; // CG preconditioner matrices (fp16), set by forward_tensor_prepass when enabled
     int precondition = 0;       // 1: preconditioned CG when the workspace has room for the matrices
-    const void* k16 = nullptr;  // fp16 copy of k and its validity word, set by forward_tensor_prepass
-    const int* f16_ok = nullptr;
+    const void* k16 = nullptr;  // fp16 copy of k, and the largest magnitudes of k and q (bf16 bit patterns): set by
+    const uint32_t* f16_range = nullptr;   // forward_tensor_prepass
     int precise_iters = 1;      // tensor-core kernel: CG iterations run with bf16 hi + lo operand pairs before the
     int precise_iters_early = 4;   // switch to single fp16 operands (see lla_forward_params.cg_precise_iters); the
                                 // second value is for row tiles that end within the first 8 d positions
@@ -242,8 +242,8 @@ __host__ __device__ __forceinline__ int precond_block_used(int g, int nb) { retu
 __host__ __device__ __forceinline__ int precond_group_start(int g) { return g < 16 ? g : g & ~1; }
 size_t precond_gram_bytes(int units, int n, int d);     // fp32 running Gram sums (scratch of the pre-pass)
 size_t precond_minv_bytes(int units, int n, int d);     // the fp16 matrices [units][blocks][d][d]
-// the pre-pass with the matrices: the fp16 copy of k and the range check of q and k (into f16_ok, nonzero before) as well
-int launch_precond(const ForwardArgs& a, void* k16, int* f16_ok, void* gram, void* minv);
+// the pre-pass with the matrices: the fp16 copy of k and the largest magnitudes of k and q (range[2], zero before) as well
+int launch_precond(const ForwardArgs& a, void* k16, uint32_t* range, void* gram, void* minv);
 int launch_decode(const DecodeArgs& a);
 int decode_refusal(const DecodeArgs& a);       // the status with which launch_decode refuses the call (before the first launch)
 constexpr int kDecodeMaxSplits = 64;           // parts of a (sequence, head) that the tensor-core path merges

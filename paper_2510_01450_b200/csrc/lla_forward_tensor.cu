@@ -133,8 +133,8 @@ struct TcParams {
     int precise_iters_early;   // the same for the row tiles that end within the first 8 D positions
     long long wait_clocks;   // cap of every bounded wait, in SM clocks
     int no_loads;        // test aid: the TMA warp issues no copy at all, so that every wait expires with nothing in flight
-    const int* f16_ok;   // device word written by the conversion pre-pass: nonzero = q and k fit the fp16 range and
-                         // the fp16 copy of k (tmK16) is valid; NULL or zero = every sweep in bf16
+    const uint32_t* f16_range;   // the largest magnitudes of k and q as the conversion pre-pass found them (bf16 bit patterns): where
+                         // they fit (fits_f16) the sweeps run on the fp16 copy of k (tmK16); NULL: every sweep in bf16
     float scale, lambda, tol;
     float* rho;
     float* stats;
@@ -253,7 +253,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     //  when it is alone: packing heads never takes iterations with pairs from a row.)
     const int first_pos = off + (wraps ? 0 : r0p / TC_BR * TC_BR);
     const int precise = first_pos + TC_BR <= 8 * D ? prm.precise_iters_early : prm.precise_iters;
-    const bool f16_on = prm.f16_ok && *prm.f16_ok && precise < (1 << 29);
+    const bool f16_on = prm.f16_range && fits_f16(prm.f16_range[0], prm.f16_range[1]) && precise < (1 << 29);
     const long long wcap = prm.wait_clocks;
 
     if (tid == 0) {
@@ -1246,13 +1246,12 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
     if (tid == 0 && *abort_flag && prm.status) atomicAdd(prm.status + LLA_STATUS_TIMEOUT, 1);
 }
 
-// Pre-pass of the fp16 sweeps: writes an fp16 copy of k and clears *ok if an entry of k or q lies outside
-// the range in which that copy is faithful (magnitude above 60000; bf16 values below the fp16 subnormal
-// spacing simply round, an absolute change under 3e-8).  Eight elements per thread and step.
+// Pre-pass of the fp16 sweeps: writes an fp16 copy of k and the largest magnitudes of k and q, from which the sweeps
+// see whether that copy is faithful (fits_f16).  Eight elements per thread and step.
 __global__ void __launch_bounds__(256)
 f16_copy_kernel(const __nv_bfloat16* __restrict__ k, uint4* __restrict__ k16, int Hk, int n, int d, Strides sk,
-                const __nv_bfloat16* __restrict__ q, int H, int nq, Strides sq, int B, int* __restrict__ ok) {
-    bool bad = false;
+                const __nv_bfloat16* __restrict__ q, int H, int nq, Strides sq, int B, uint32_t* __restrict__ range) {
+    uint32_t k_max = 0, q_max = 0;
     const size_t stride = (size_t)gridDim.x * blockDim.x, t0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int vpr = d / 8;                                   // 16-byte groups per row
     const size_t k_vec = (size_t)B * Hk * n * vpr, q_vec = (size_t)B * H * nq * vpr;
@@ -1265,9 +1264,8 @@ f16_copy_kernel(const __nv_bfloat16* __restrict__ k, uint4* __restrict__ k16, in
         uint32_t h[4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-            const float a = __uint_as_float(w[e] << 16), b = __uint_as_float(w[e] & 0xFFFF0000u);
-            bad |= !(fabsf(a) <= 60000.f) || !(fabsf(b) <= 60000.f);
-            h[e] = pack_f16(a, b);
+            k_max = max_abs_bf16x2(k_max, w[e]);
+            h[e] = pack_f16(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xFFFF0000u));
         }
         k16[i] = make_uint4(h[0], h[1], h[2], h[3]);         // the copy is contiguous [B][Hk][n][d]
     }
@@ -1278,10 +1276,10 @@ f16_copy_kernel(const __nv_bfloat16* __restrict__ k, uint4* __restrict__ k16, in
         const uint4 raw = *reinterpret_cast<const uint4*>(q + sq.at(unit / H, unit % H, row) + 8 * c);
         const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            bad |= !(fabsf(__uint_as_float(w[e] << 16)) <= 60000.f) || !(fabsf(__uint_as_float(w[e] & 0xFFFF0000u)) <= 60000.f);
+        for (int e = 0; e < 4; ++e) q_max = max_abs_bf16x2(q_max, w[e]);
     }
-    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) *ok = 0;
+    publish_max_bf16(k_max, range);
+    publish_max_bf16(q_max, range + 1);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1382,7 +1380,7 @@ int launch_t(const ForwardArgs& a) {
     prm.rho = a.rho; prm.stats = a.stats; prm.iters = a.iters; prm.status = a.status;
     prm.scratch = nullptr;
     prm.scratch_slots = 0;
-    prm.f16_ok = nullptr;
+    prm.f16_range = nullptr;
     // the caller's workspace is cut into the D = 128 row-state slots (if it holds them) and the fp16 copy of k
     char* ws = static_cast<char*>(a.workspace);
     size_t ws_left = a.workspace ? a.workspace_bytes : 0;
@@ -1408,10 +1406,10 @@ int launch_t(const ForwardArgs& a) {
     }
     // fp16 sweeps: only with the copy of k that forward_tensor_prepass made; without it every sweep runs on
     // the bf16 inputs
-    if (a.k16 && a.f16_ok) {
+    if (a.k16 && a.f16_range) {
         const Strides c16 = contiguous_strides(Hk, a.n, D);
         if (!make_map_16bit_4d(&mk16, a.k16, a.B, Hk, a.n, D, c16.b, c16.h, c16.r, TC_BC, F16)) return LLA_ERR_CUDA;
-        prm.f16_ok = a.f16_ok;
+        prm.f16_range = a.f16_range;
     }
     bool precond = false;
     // preconditioned CG: only with the matrices that forward_tensor_prepass made ([units][blocks][D][D] fp16)
@@ -1476,7 +1474,7 @@ size_t forward_tensor_workspace_bytes(int B, int H, int n, int d) {
 // room for it, and records where it is in `a`; the head of the workspace is left to the D = 128 row state.
 int forward_tensor_prepass(ForwardArgs& a) {
     a.k16 = nullptr;
-    a.f16_ok = nullptr;
+    a.f16_range = nullptr;
     a.minv = nullptr;
     if (!forward_tensor_supported(a) || !a.workspace) return LLA_OK;
     if (std::min(a.precise_iters, a.precise_iters_early) >= (1 << 29)) return LLA_OK;
@@ -1485,18 +1483,18 @@ int forward_tensor_prepass(ForwardArgs& a) {
     if (a.workspace_bytes < head + f16_copy_bytes(k_elems)) return LLA_OK;
     char* ws = static_cast<char*>(a.workspace) + head;
     uint4* k16 = reinterpret_cast<uint4*>(ws);
-    int* okw = reinterpret_cast<int*>(ws + round256(k_elems * 2));
-    LLA_CUDA_TRY(cudaMemsetAsync(okw, 1, sizeof(int), a.stream));
+    uint32_t* range = reinterpret_cast<uint32_t*>(ws + round256(k_elems * 2));
+    LLA_CUDA_TRY(cudaMemsetAsync(range, 0, 2 * sizeof(uint32_t), a.stream));
     // with the preconditioner's matrices behind the copy (Gram scratch first), if enabled and there is room: one pass
     // over k makes all of it
     const int units = a.B * a.H / a.kv_group;
     const size_t used = head + f16_copy_bytes(k_elems);
     const size_t gram_b = precond_gram_bytes(units, a.n, a.d), minv_b = precond_minv_bytes(units, a.n, a.d);
     a.k16 = k16;
-    a.f16_ok = okw;
+    a.f16_range = range;
     if (a.precondition && a.workspace_bytes >= used + gram_b + minv_b) {
         char* gram = static_cast<char*>(a.workspace) + used;
-        const int rc = launch_precond(a, k16, okw, gram, gram + gram_b);
+        const int rc = launch_precond(a, k16, range, gram, gram + gram_b);
         if (rc != LLA_OK) return rc;
         a.minv = gram + gram_b;
         return LLA_OK;
@@ -1504,7 +1502,7 @@ int forward_tensor_prepass(ForwardArgs& a) {
     const size_t k_vec = k_elems / 8;
     const unsigned blocks = (unsigned)std::min<size_t>((k_vec + 255) / 256, 148 * 8);
     f16_copy_kernel<<<blocks, 256, 0, a.stream>>>(static_cast<const __nv_bfloat16*>(a.k), k16, a.H / a.kv_group, a.n, a.d, a.sk,
-                                                   static_cast<const __nv_bfloat16*>(a.q), a.H, a.nq, a.sq, a.B, okw);
+                                                   static_cast<const __nv_bfloat16*>(a.q), a.H, a.nq, a.sq, a.B, range);
     LLA_CUDA_TRY(cudaGetLastError());
     return LLA_OK;
 }

@@ -21,7 +21,7 @@
 // Three kernels, all on the caller's stream ahead of the forward kernel:
 //   precond_gram_kernel     a chunk of key blocks each: running sums of k_j k_j^T and k_j inside the chunk, one record per
 //                           block that is asked for.  It reads every key once, so it also makes the fp16 copy of k and
-//                           checks that k and q fit the fp16 range.  Bound by its loads; the products run on mma.sync,
+//                           finds the largest magnitudes of k and q.  Bound by its loads; the products run on mma.sync,
 //                           whose operands come straight from the tiles (ldmatrix.trans).  16 heads, n = 16384, d = 128:
 //                           85 us, where Gram sums on the CUDA cores, their scan over every block and a copy kernel took 430
 //   precond_scan_kernel     the sums of whole chunks (the records of their last blocks) become running sums over the sequence
@@ -37,7 +37,9 @@
 namespace lla {
 namespace {
 
+using sm100::max_abs_bf16x2;
 using sm100::pack_f16;
+using sm100::publish_max_bf16;
 using sm100::smem_u32;
 
 constexpr int PC_THREADS = 256;
@@ -49,7 +51,7 @@ struct PcParams {
     const __nv_bfloat16* q;
     float* gram;       // [units][blocks][D * D + D]
     uint4* k16;        // [units][n][D] fp16
-    int* f16_ok;       // cleared if an entry of k or q lies outside the fp16 range
+    uint32_t* range;   // the largest magnitudes of k and q (bf16 bit patterns)
     __half* minv;      // [units][blocks][D][D]; with a window the first [tiles] of a unit's are in use
     int n, nb, cb;     // keys; blocks; blocks per chunk
     int g0;            // first block that a query sees last; with a window the first query tile that is not solved directly
@@ -67,12 +69,6 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], uint32_t add
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// a pair of bf16 values as a pair of fp16 values; bad: one of them is beyond 60000 (or not a number)
-__device__ __forceinline__ uint32_t bf16x2_to_f16x2(uint32_t w, bool& bad) {
-    const float a = __uint_as_float(w << 16), b = __uint_as_float(w & 0xFFFF0000u);
-    bad |= !(fabsf(a) <= 60000.f) || !(fabsf(b) <= 60000.f);
-    return pack_f16(a, b);
 }
 
 template <int D>
@@ -97,7 +93,7 @@ precond_gram_kernel(const PcParams p) {
             raw[i] = j < p.n ? *reinterpret_cast<const uint4*>(src + (long long)j * p.sk.r) : make_uint4(0, 0, 0, 0);
         }
     };
-    bool bad = false;
+    uint32_t k_max = 0, q_max = 0;
     float s8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float acc[MT][NT][4] = {};
     const int m0 = (warp & 3) * 16 * MT, n0 = (warp >> 2) * 8 * NT;
@@ -113,9 +109,11 @@ precond_gram_kernel(const PcParams p) {
             uint32_t h[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                h[e] = bf16x2_to_f16x2(w[e], bad);
-                s8[2 * e] += __uint_as_float(w[e] << 16);
-                s8[2 * e + 1] += __uint_as_float(w[e] & 0xFFFF0000u);
+                const float x0 = __uint_as_float(w[e] << 16), x1 = __uint_as_float(w[e] & 0xFFFF0000u);
+                k_max = max_abs_bf16x2(k_max, w[e]);
+                h[e] = pack_f16(x0, x1);
+                s8[2 * e] += x0;
+                s8[2 * e + 1] += x1;
             }
             if (j < p.n) dst16[(size_t)j * CPR] = make_uint4(h[0], h[1], h[2], h[3]);
         }
@@ -162,7 +160,7 @@ precond_gram_kernel(const PcParams p) {
     const size_t nthr = (size_t)gridDim.x * gridDim.y * PC_THREADS, q_vec = (size_t)p.B * p.H * p.nq * CPR;
     const bool flat = p.sq.r == D && p.sq.h == (long long)p.nq * D && p.sq.b == (long long)p.H * p.nq * D;
     auto check = [&](const uint4& x) {
-        (void)bf16x2_to_f16x2(x.x, bad); (void)bf16x2_to_f16x2(x.y, bad); (void)bf16x2_to_f16x2(x.z, bad); (void)bf16x2_to_f16x2(x.w, bad);
+        q_max = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(q_max, x.x), x.y), x.z), x.w);
     };
     size_t i = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * PC_THREADS + tid;
     if (flat) {
@@ -182,7 +180,8 @@ precond_gram_kernel(const PcParams p) {
             check(*reinterpret_cast<const uint4*>(p.q + p.sq.at(unit / p.H, unit % p.H, row) + 8 * (int)(i % CPR)));
         }
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) *p.f16_ok = 0;
+    publish_max_bf16(k_max, p.range);
+    publish_max_bf16(q_max, p.range + 1);
 }
 
 // Records of the chunks' last blocks: running sums over the chunks, element by element (rec: floats of a record).
@@ -447,10 +446,10 @@ size_t precond_minv_bytes(int units, int n, int d) {
     return ((size_t)units * precond_blocks(n) * (size_t)d * d * sizeof(__half) + 255) & ~(size_t)255;
 }
 
-int launch_precond(const ForwardArgs& a, void* k16, int* f16_ok, void* gram, void* minv) {
+int launch_precond(const ForwardArgs& a, void* k16, uint32_t* range, void* gram, void* minv) {
     PcParams p = {};
     p.k = static_cast<const __nv_bfloat16*>(a.k); p.q = static_cast<const __nv_bfloat16*>(a.q);
-    p.gram = static_cast<float*>(gram); p.k16 = static_cast<uint4*>(k16); p.f16_ok = f16_ok; p.minv = static_cast<__half*>(minv);
+    p.gram = static_cast<float*>(gram); p.k16 = static_cast<uint4*>(k16); p.range = range; p.minv = static_cast<__half*>(minv);
     p.n = a.n; p.nb = precond_blocks(a.n);
     p.cb = (p.nb + PC_CHUNKS - 1) / PC_CHUNKS;
     p.B = a.B; p.Hk = a.H / a.kv_group; p.H = a.H; p.nq = a.nq;

@@ -218,6 +218,24 @@ __device__ __forceinline__ uint32_t split_f16x2(float a, float b, uint32_t& lo) 
     lo = pack_f16(a - ha, b - hb);
     return pack_f16(ha, hb);
 }
+// The larger magnitude of each half of two packed pairs of bf16 values, as bit patterns (not-a-number above infinity above all else).
+__device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t w) {
+    uint32_t r;
+    asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(m), "r"(w & 0x7FFF7FFFu));
+    return r;
+}
+// A warp's larger half into a word of global memory (zero before).
+__device__ __forceinline__ void publish_max_bf16(uint32_t m, uint32_t* word) {
+    const uint32_t v = __reduce_max_sync(0xffffffffu, max(m & 0xFFFFu, m >> 16));
+    if ((threadIdx.x & 31) == 0 && v != 0) atomicMax(word, v);
+}
+// Whether fp16 copies of k and q stand for the bf16 inputs, from the bit patterns of their largest magnitudes: below 60000,
+// and not so small that half the spacing of the fp16 subnormals, 2^-25, is more than 2^-16 of the largest entry.  (A tensor of
+// zeros is its own copy.)
+__device__ __forceinline__ bool fits_f16(uint32_t k_max, uint32_t q_max) {
+    auto fits = [](uint32_t m) { return m <= 0x476Au && (m >= 0x3B00u || m == 0u); };      // 59904, 2^-9
+    return fits(k_max) && fits(q_max);
+}
 // {hi16: bf16(a), lo16: bf16(b)}
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     uint32_t r;

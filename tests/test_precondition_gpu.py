@@ -254,3 +254,25 @@ def test_rows_of_few_keys_go_on_to_half_the_residual(d, n, nq, window):
             res.append(np.linalg.norm(b - cy) / np.linalg.norm(b))
     res = np.asarray(res)
     assert np.quantile(res, 0.5) <= 0.5e-4 and np.quantile(res, 0.9) <= 0.75e-4, np.sort(res)[::8]
+
+
+@pytest.mark.parametrize("d,size_q,size_k", [(64, 1e-4, 1e-4), (128, 1e-4, 1e-4), (64, 1.0, 3e-4), (64, 3e-4, 1.0), (64, 1e-3, 1e-3)])
+def test_small_inputs_keep_their_bits(d, size_q, size_k):
+    """Entries of q and k far below the fp16 range's middle: rho against float64 within the tolerance, whatever the solver.  (In fp16
+    an entry of 1e-5 is off by up to 0.3 %.)"""
+    n = 600
+    w, q, k, v = _case(d, n, n, 1, 1, 1.0, 1800 + d)
+    q, k = inputs.round_to_bf16(q * np.float32(size_q)), inputs.round_to_bf16(k * np.float32(size_k))
+    rows = np.linspace(d + d // 2, n - 1, 30).astype(int)
+    for lam in (1e-3, 1e-2 * size_k ** 2):
+        w = w.shrink(lam=lam)
+        K = k[0, 0].astype(np.float64)
+        for kw in ({"max_iters": 0}, {}):
+            rho = torch.zeros((1, 1, n, d), dtype=torch.float32, device="cuda")
+            _solve(w, q, k, v, n, 1, rho=rho, **kw)
+            for r in rows:
+                z = K[:r + 1] - q[0, 0, r]
+                s = w.scale * K[:r + 1] @ q[0, 0, r].astype(np.float64)
+                wt = np.exp(s - s.max())
+                ref = np.linalg.solve((wt[:, None] * z).T @ z + lam * np.exp(-s.max()) * np.eye(d), wt @ z)
+                assert np.linalg.norm(rho[0, 0, r].cpu().numpy() - ref) <= 4e-4 * np.linalg.norm(ref), (lam, kw, r)
