@@ -1349,10 +1349,10 @@ int launch_t(const ForwardArgs& a) {
     // can fill tiles together where a head's own rows leave its last tile partly empty (257 rows of four heads: nine
     // tiles instead of twelve).  Their rows must lie one behind the other in q, and none may be solved directly.
     const int group = a.kv_group;
-    // Nor with a narrow window and the preconditioner, whose matrix then is that of one head's tile: a row elsewhere in
-    // the sequence sees other keys, too few of them (fewer than 8 d) for their covariance to be much the same.
+    // Nor with the preconditioner where rows see fewer than 8 d keys, early in the sequence or under a narrow window: the matrix of a
+    // tile is that of one place in the sequence, and the covariance of so few keys differs much from place to place.
     const bool pack = group > 1 && hr == 0 && !a.block_mask && a.sq.h == (long long)a.nq * a.sq.r &&
-                      !(a.minv && a.causal && a.window > 0 && a.window < 8 * D) &&
+                      !(a.minv && a.causal && (a.n - a.nq < 8 * D || (a.window > 0 && a.window < 8 * D))) &&
                       (group * a.nq + TC_BR - 1) / TC_BR < group * tiles;
     const int units = pack ? a.B * Hk : a.B * a.H;          // unit: the rows that are cut into tiles together
     const int unit_rows = pack ? group * a.nq : a.nq;
