@@ -58,6 +58,7 @@ constexpr int TC_SLOT_MAX = 8;
 constexpr int TC_PRE = 4;            // key blocks fetched ahead of a sweep
 constexpr int TC_ORDER_MAX = 256;    // launch-order table size (query tiles)
 constexpr int TC_BLIST_MAX = 1024;   // key blocks a block-sparse tile can list (n <= 65536)
+constexpr float STAT_SCALE = 128.f;  // of the weights in an fp16 statistics sweep
 constexpr int TC_SPLIT_MAX = 4;      // sweeps of at most this many key blocks run in split mode (see the compute role)
 
 // SW_CG: a CG sweep on the bf16 inputs, P and U as bf16 hi + lo pairs.  SW_CG16, SW_CG16P: a CG sweep on the fp16 copies,
@@ -625,8 +626,8 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         float mx2 = -INFINITY, omega = 0.f, inv_omega = 0.f, ridge = 0.f, den = 0.f;
         float abar = 0.f;                                     // kbar.p (CG) or kbar.y (output)
         // fp16 sweeps: the search direction is stored as p * psc with psc a power of two that brings |p| to
-        // [1, 2.83) over the row's largest weight (where that is above one), so that its entries and u = w (a - abar) sit in
-        // the middle of the fp16 range whatever the scale of the right-hand side; pn2 tracks |p|^2 through the recurrence
+        // [1, 2.83) over the row's largest weight, so that its entries and u = w (a - abar) sit in
+        // the middle of the fp16 range whatever the scale of the right-hand side and of the weights; pn2 tracks |p|^2 through the recurrence
         // |p'|^2 = |r'|^2 + beta^2 |p|^2
         float pn2 = 0.f, psc = 1.f, ipsc = 1.f;               // (in the output sweep ipsc undoes the scale of y)
         int wexp = 0;                                         // largest weight of the row is at most 2^wexp
@@ -650,6 +651,9 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             const uint64_t c1c1 = pk2(c1, c1), nmx = pk2(-mx2, -mx2);
             const float ab_s = kind == SW_CG16 || kind == SW_CG16P ? abar * psc : abar;
             const uint64_t nab = pk2(-ab_s, -ab_s), oab = pk2(1.f + abar, 1.f + abar), neg1 = pk2(-ipsc, -ipsc);
+            // the statistics' weights as fp16 pairs: up to 2^8, they are scaled to the top of the range, so that the
+            // absolute error of a pair there, 2^-24, is 2^-31 of a weight of one
+            const uint64_t stat2 = pk2(STAT_SCALE, STAT_SCALE);
             uint64_t part2 = pk2(0.f, 0.f);
             const uint32_t a0 = ablk;
             if (kind != SW_STATS) ablk += nblk;
@@ -704,6 +708,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                             upk2(t2, t0, t1);
                             if (kind == SW_STATS) smax = fmaxf(smax, fmaxf(t0, t1));     // largest score, relative to the shift
                             uint64_t u2 = pk2(ex2f(t0), ex2f(t1));
+                            if (kind == SW_STATS && f16) u2 = mul2(u2, stat2);
                             if (kind == SW_CG || kind == SW_CG16P)
                                 u2 = mul2(u2, add2(pk2(__uint_as_float(av[2 * e2]), __uint_as_float(av[2 * e2 + 1])), nab));
                             if (kind == SW_OUT)
@@ -995,8 +1000,13 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         exchange(acc, u0, u1);
                     }
                     omega = pair_sum(part);
+                    if (f16_on) {
+                        omega *= 1.f / STAT_SCALE;
+#pragma unroll
+                        for (int e = 0; e < NCOL; ++e) acc[e] *= 1.f / STAT_SCALE;
+                    }
                 }
-                wexp = given ? 0 : (int)fminf(fmaxf(ceilf(tmax - mx2), 0.f), 8.f);
+                wexp = given ? 0 : (int)fminf(fmaxf(ceilf(tmax - mx2), -8.f), 8.f);
                 inv_omega = 1.f / omega;
                 const float lam_i = (prm.lambda_rows && row < nq) ? prm.lambda_rows[(size_t)bh * nq + row] : prm.lambda;
                 // ridge in the frame of the shift: lambda e^{-shift} by the definition; the printed algorithm adds

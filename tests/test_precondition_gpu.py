@@ -276,3 +276,27 @@ def test_small_inputs_keep_their_bits(d, size_q, size_k):
                 wt = np.exp(s - s.max())
                 ref = np.linalg.solve((wt[:, None] * z).T @ z + lam * np.exp(-s.max()) * np.eye(d), wt @ z)
                 assert np.linalg.norm(rho[0, 0, r].cpu().numpy() - ref) <= 4e-4 * np.linalg.norm(ref), (lam, kw, r)
+
+
+@pytest.mark.parametrize("d,n", [(64, 2500), (128, 2500)])
+def test_many_keys_of_small_weight(d, n):
+    """Eight keys of weight 2^-7.7 and thousands of about 2^-20, none larger (the weights are taken in the frame of a zero score where the
+    largest lies within 2^+-8): in fp16 the small ones are multiples of 2^-24.  The queries lie far from the keys, which makes the
+    systems sensitive to them; no larger an error than with bf16 operand pairs, whose bits are relative, and a quarter."""
+    w, q, k, v = _case(d, n, n, 1, 1, 1.0, 1900 + d)
+    rng = np.random.default_rng(11)
+    u = np.zeros(d, dtype=np.float32)
+    u[: d // 2] = (2.0 / d) ** 0.5
+    away = rng.standard_normal((n, d)) * 0.5
+    away -= np.outer(away @ u, u)
+    k = (away + np.outer(-13.9 / 6 + 0.05 * rng.standard_normal(n), u)).astype(np.float32)
+    k[:8] += (13.9 - 5.3) / 6 * u
+    q = np.broadcast_to(6 * d ** 0.5 * u, (n, d)) + 0.1 * rng.standard_normal((n, d)).astype(np.float32)
+    q, k = (inputs.round_to_bf16(x[None, None].astype(np.float32)) for x in (q, k))
+    rows = np.linspace(d + d // 2, n - 1, 40).astype(int)
+    ref = _exact(w, q, k, v, 0, 0, rows, n)
+    rms = []
+    for kw in ({"cg_precise_iters": L.LLA_CG_PRECISE_ALL}, {}, {"max_iters": 0}):
+        out, _, _ = _solve(w, q, k, v, n, 1, **kw)
+        rms.append(np.sqrt(np.mean(row_err(out[0, rows], ref) ** 2)))
+    assert max(rms[1:]) <= 1.25 * rms[0], rms
