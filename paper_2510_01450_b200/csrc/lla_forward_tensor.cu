@@ -1288,8 +1288,9 @@ f16_copy_kernel(const __nv_bfloat16* __restrict__ k, uint4* __restrict__ k16, in
 #pragma unroll
         for (int e = 0; e < 4; ++e) q_max = max_abs_bf16x2(q_max, w[e]);
     }
-    publish_max_bf16(k_max, range);
-    publish_max_bf16(q_max, range + 1);
+    __shared__ uint32_t s_max[2][8];
+    publish_max_bf16(k_max, range, s_max[0]);
+    publish_max_bf16(q_max, range + 1, s_max[1]);
 }
 
 // ------------------------------------------------------------------------------------------------

@@ -44,7 +44,8 @@ using sm100::smem_u32;
 
 constexpr int PC_THREADS = 256;
 constexpr int PC_BLOCK = 128;      // keys per Gram block
-constexpr int PC_CHUNKS = 8;       // at most
+constexpr int PC_CHUNKS = 32;      // at most
+constexpr int PC_QLOADS = 8;       // 16-byte loads in flight of a thread that looks at q
 
 struct PcParams {
     const __nv_bfloat16* k;
@@ -54,6 +55,7 @@ struct PcParams {
     uint32_t* range;   // the largest magnitudes of k and q (bf16 bit patterns)
     __half* minv;      // [units][blocks][D][D]; with a window the first [tiles] of a unit's are in use
     int n, nb, cb;     // keys; blocks; blocks per chunk
+    int chunks, k_blocks;   // chunks of a unit; thread blocks that read k
     int g0;            // first block that a query sees last; with a window the first query tile that is not solved directly
     int tiles;         // query tiles of 128 rows per head
     int B, Hk, H, nq;
@@ -80,9 +82,31 @@ precond_gram_kernel(const PcParams p) {
     extern __shared__ __align__(16) uint8_t pc_raw[];
     __nv_bfloat16* ks = reinterpret_cast<__nv_bfloat16*>(pc_raw);                     // [2][PC_BLOCK][LD]
     float* sums = reinterpret_cast<float*>(pc_raw + 2 * PC_BLOCK * LD * 2);           // [PC_THREADS][9]
-    const int u = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int b0 = blockIdx.x * p.cb, b1 = min(p.nb, b0 + p.cb);
+    __shared__ uint32_t s_max[PC_THREADS / 32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int col = tid % CPR, row0 = tid / CPR;
+    // The blocks behind those of k look at q, a tile of one head's rows at a time, whatever its strides.  (Shared out over the blocks
+    // of k instead, one load in flight a thread unless q was one piece, 32 heads over one with q as [B, n, H, d] took
+    // 0.6 ms longer at n = 4096, d = 128.)
+    if ((int)blockIdx.x >= p.k_blocks) {
+        constexpr int ROWS = PC_QLOADS * RPI;
+        const int tiles = (p.nq + ROWS - 1) / ROWS, all = p.B * p.H * tiles;
+        uint32_t q_max = 0;
+        for (int t = blockIdx.x - p.k_blocks; t < all; t += gridDim.x - p.k_blocks) {
+            const int head = t / tiles, r0 = (t - head * tiles) * ROWS + row0;
+            const __nv_bfloat16* src = p.q + p.sq.at(head / p.H, head % p.H, r0) + 8 * col;
+            uint4 x[PC_QLOADS];
+#pragma unroll
+            for (int i = 0; i < PC_QLOADS; ++i)
+                x[i] = r0 + i * RPI < p.nq ? *reinterpret_cast<const uint4*>(src + (long long)(i * RPI) * p.sq.r) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int i = 0; i < PC_QLOADS; ++i)
+                q_max = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(q_max, x[i].x), x[i].y), x[i].z), x[i].w);
+        }
+        publish_max_bf16(q_max, p.range + 1, s_max);
+        return;
+    }
+    const int u = blockIdx.x / p.chunks, b0 = (blockIdx.x - u * p.chunks) * p.cb, b1 = min(p.nb, b0 + p.cb);
     const __nv_bfloat16* src = p.k + p.sk.at(u / p.Hk, u % p.Hk, 0) + 8 * col;
     uint4* dst16 = p.k16 + (size_t)u * p.n * CPR + col;
     uint4 raw[NLD];
@@ -93,7 +117,7 @@ precond_gram_kernel(const PcParams p) {
             raw[i] = j < p.n ? *reinterpret_cast<const uint4*>(src + (long long)j * p.sk.r) : make_uint4(0, 0, 0, 0);
         }
     };
-    uint32_t k_max = 0, q_max = 0;
+    uint32_t k_max = 0;
     float s8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float acc[MT][NT][4] = {};
     const int m0 = (warp & 3) * 16 * MT, n0 = (warp >> 2) * 8 * NT;
@@ -156,32 +180,7 @@ precond_gram_kernel(const PcParams p) {
         }
         // (the next tile goes to the other buffer; the one after it is written behind the next barrier)
     }
-    // the range of q, shared out over the grid: eight loads in flight a thread where q is one piece
-    const size_t nthr = (size_t)gridDim.x * gridDim.y * PC_THREADS, q_vec = (size_t)p.B * p.H * p.nq * CPR;
-    const bool flat = p.sq.r == D && p.sq.h == (long long)p.nq * D && p.sq.b == (long long)p.H * p.nq * D;
-    auto check = [&](const uint4& x) {
-        q_max = max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(max_abs_bf16x2(q_max, x.x), x.y), x.z), x.w);
-    };
-    size_t i = ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * PC_THREADS + tid;
-    if (flat) {
-        const uint4* qv = reinterpret_cast<const uint4*>(p.q);
-        for (; i + 7 * nthr < q_vec; i += 8 * nthr) {
-            uint4 x[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) x[e] = qv[i + e * nthr];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) check(x[e]);
-        }
-        for (; i < q_vec; i += nthr) check(qv[i]);
-    } else {
-        for (; i < q_vec; i += nthr) {
-            const size_t rowi = i / CPR;
-            const int row = (int)(rowi % p.nq), unit = (int)(rowi / p.nq);
-            check(*reinterpret_cast<const uint4*>(p.q + p.sq.at(unit / p.H, unit % p.H, row) + 8 * (int)(i % CPR)));
-        }
-    }
-    publish_max_bf16(k_max, p.range);
-    publish_max_bf16(q_max, p.range + 1);
+    publish_max_bf16(k_max, p.range, s_max);
 }
 
 // Records of the chunks' last blocks: running sums over the chunks, element by element (rec: floats of a record).
@@ -190,18 +189,22 @@ precond_scan_kernel(float* __restrict__ gram, int nb, int cb, int rec) {
     cudaGridDependencySynchronize();
     const int e = blockIdx.x * PC_THREADS + threadIdx.x, chunks = (nb + cb - 1) / cb;
     if (4 * e >= rec) return;
+    constexpr int AHEAD = 8;
     float4* p = reinterpret_cast<float4*>(gram + (size_t)blockIdx.y * nb * rec) + e;
     auto at = [&](int c) { return (size_t)(min(nb, (c + 1) * cb) - 1) * (rec / 4); };
-    float4 x[PC_CHUNKS];
+    float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c0 = 0; c0 < chunks; c0 += AHEAD) {
+        float4 x[AHEAD];
 #pragma unroll
-    for (int c = 0; c < PC_CHUNKS; ++c)
-        if (c < chunks) x[c] = p[at(c)];
+        for (int c = 0; c < AHEAD; ++c)
+            if (c0 + c < chunks) x[c] = p[at(c0 + c)];
 #pragma unroll
-    for (int c = 1; c < PC_CHUNKS; ++c)
-        if (c < chunks) {
-            x[c].x += x[c - 1].x; x[c].y += x[c - 1].y; x[c].z += x[c - 1].z; x[c].w += x[c - 1].w;
-            p[at(c)] = x[c];
-        }
+        for (int c = 0; c < AHEAD; ++c)
+            if (c0 + c < chunks) {
+                sum.x += x[c].x; sum.y += x[c].y; sum.z += x[c].z; sum.w += x[c].w;
+                if (c0 + c > 0) p[at(c0 + c)] = sum;
+            }
+    }
 }
 
 // The integers t <= y of min(max(t, 0), len) added up.
@@ -410,11 +413,13 @@ precond_invert_kernel(const PcParams p) {
 }
 
 template <int D>
-int launch_t(const PcParams& p, cudaStream_t st) {
+int launch_t(const PcParams& p, int sms, cudaStream_t st) {
     const int units = p.B * p.Hk;
     const size_t smem = 2 * (size_t)PC_BLOCK * (D + 8) * 2 + sizeof(float) * PC_THREADS * 9;
     LLA_CUDA_TRY(cudaFuncSetAttribute(precond_gram_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    precond_gram_kernel<D><<<dim3((p.nb + p.cb - 1) / p.cb, units), PC_THREADS, smem, st>>>(p);
+    const int rows = PC_QLOADS * (PC_THREADS / (D / 8));
+    const long long q_tiles = (long long)p.B * p.H * ((p.nq + rows - 1) / rows);
+    precond_gram_kernel<D><<<p.k_blocks + (int)std::min<long long>(q_tiles, 4 * sms), PC_THREADS, smem, st>>>(p);
     LLA_CUDA_TRY(cudaGetLastError());
     // (the two small kernels are programmatic dependents: their launches overlap the kernel before)
     cudaLaunchConfig_t cfg = {};
@@ -451,15 +456,24 @@ int launch_precond(const ForwardArgs& a, void* k16, uint32_t* range, void* gram,
     p.k = static_cast<const __nv_bfloat16*>(a.k); p.q = static_cast<const __nv_bfloat16*>(a.q);
     p.gram = static_cast<float*>(gram); p.k16 = static_cast<uint4*>(k16); p.range = range; p.minv = static_cast<__half*>(minv);
     p.n = a.n; p.nb = precond_blocks(a.n);
-    p.cb = (p.nb + PC_CHUNKS - 1) / PC_CHUNKS;
     p.B = a.B; p.Hk = a.H / a.kv_group; p.H = a.H; p.nq = a.nq;
+    int dev = 0, sms = 0;
+    LLA_CUDA_TRY(cudaGetDevice(&dev));
+    LLA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    // chunks: two thread blocks an SM, whatever the number of heads (with eight per head, one key/value head had eight in all)
+    const int units = p.B * p.Hk;
+    const int most = std::min(std::max(2 * sms / units, 8), PC_CHUNKS);
+    p.cb = (p.nb + most - 1) / most;
+    if (p.cb > 1) p.cb += p.cb & 1;      // a chunk's last block is then one whose record is written anyway
+    p.chunks = (p.nb + p.cb - 1) / p.cb;
+    p.k_blocks = p.chunks * units;
     p.causal = a.causal; p.window = a.causal ? a.window : 0; p.head_rows = a.head_rows > 0 ? a.head_rows : 0;
     p.tiles = (a.nq + PC_BLOCK - 1) / PC_BLOCK;
     p.g0 = p.window > 0 ? head_rows_count(a) / PC_BLOCK          // (rows before are solved directly)
                         : std::max(a.n - a.nq, std::min(a.n, p.head_rows) - 1) / PC_BLOCK;
     p.lambda = a.lambda; p.sk = a.sk; p.sq = a.sq;
-    if (a.d == 64) return launch_t<64>(p, a.stream);
-    if (a.d == 128) return launch_t<128>(p, a.stream);
+    if (a.d == 64) return launch_t<64>(p, sms, a.stream);
+    if (a.d == 128) return launch_t<128>(p, sms, a.stream);
     return LLA_ERR_UNSUPPORTED;
 }
 

@@ -224,10 +224,17 @@ __device__ __forceinline__ uint32_t max_abs_bf16x2(uint32_t m, uint32_t w) {
     asm("max.u16x2 %0, %1, %2;" : "=r"(r) : "r"(m), "r"(w & 0x7FFF7FFFu));
     return r;
 }
-// A warp's larger half into a word of global memory (zero before).
-__device__ __forceinline__ void publish_max_bf16(uint32_t m, uint32_t* word) {
+// The largest half over a thread block into a word of global memory (zero before): one atomic operation a block.  All threads,
+// once per array of shared memory (one word a warp).
+__device__ __forceinline__ void publish_max_bf16(uint32_t m, uint32_t* word, uint32_t* s_max) {
     const uint32_t v = __reduce_max_sync(0xffffffffu, max(m & 0xFFFFu, m >> 16));
-    if ((threadIdx.x & 31) == 0 && v != 0) atomicMax(word, v);
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t x = 0;
+        for (unsigned i = 0; i < blockDim.x / 32; ++i) x = max(x, s_max[i]);
+        if (x != 0) atomicMax(word, x);
+    }
 }
 // Whether fp16 copies of k and q stand for the bf16 inputs, from the bit patterns of their largest magnitudes: below 60000,
 // and not so small that half the spacing of the fp16 subnormals, 2^-25, is more than 2^-16 of the largest entry.  (A tensor of

@@ -300,3 +300,40 @@ def test_many_keys_of_small_weight(d, n):
         out, _, _ = _solve(w, q, k, v, n, 1, **kw)
         rms.append(np.sqrt(np.mean(row_err(out[0, rows], ref) ** 2)))
     assert max(rms[1:]) <= 1.25 * rms[0], rms
+
+
+@pytest.mark.parametrize("d,B,n,nq,H,Hkv", [(64, 1, 300, 300, 4, 1), (128, 2, 4500, 1300, 4, 1), (64, 1, 5000, 1257, 8, 2), (128, 1, 700, 129, 2, 2)])
+def test_the_pre_pass_reads_any_layout_of_q_and_any_number_of_heads(d, B, n, nq, H, Hkv):
+    """Few key/value heads cut their keys into more chunks (one block of keys a chunk, two and more; 4500 keys: a last chunk of one
+    block), and q is looked at a tile of rows at a time: the same output bits for [B, H, nq, d] and [B, nq, H, d], and one entry
+    beyond the fp16 range in the last row of the last head turns the fp16 sweeps off either way."""
+    w = inputs.CONFIGS[2].shrink(B=B, H=H, n=n, d=d, dv=d, seed=2000 + n)
+    q, _, _ = inputs.make_prefill(w)
+    _, k, v = inputs.make_prefill(w.shrink(H=Hkv, seed=2001 + n))
+    q = np.ascontiguousarray(q[:, :, n - nq:])
+    nbytes = L.lla_forward_workspace_bytes(B, H, n, d, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    kd, vd = dev(k, "bf16"), dev(v, "bf16")
+    sums = []
+    for big in (False, True):
+        if big:
+            q[-1, -1, -1, -1] = 65536.0
+        outs = []
+        for strided in (False, True):
+            qd = dev(np.ascontiguousarray(q.transpose(0, 2, 1, 3)) if strided else q, "bf16")
+            out = torch.full((B, H, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+            status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+            L.lla_forward_ex(qd, kd, vd, out, B, H, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, q_rows=nq, kv_heads=Hkv,
+                             q_strides=(nq * H * d, d, H * d) if strided else None, device_status=status, workspace=ws,
+                             workspace_bytes=nbytes, cg_precondition=1, stream=stream_ptr())
+            torch.cuda.synchronize()
+            outs.append(out[:, :, :-1])
+            sums.append(status.cpu().tolist()[L.STATUS_ITER_SUM])
+        assert torch.isfinite(outs[0]).all()
+        # (packed rows of grouped heads need q in one piece; unpacked tiles end where other rows are)
+        assert row_err(outs[0].cpu().numpy(), outs[1].cpu().numpy().astype(np.float64)).max() <= 4e-4
+    assert max(sums[:2]) < min(sums[2:])
+    for h in (0, H - 1):
+        rows = np.linspace(max(0, d + d // 2 - (n - nq)), nq - 2, 12).astype(int)
+        ref = _exact(w, q[-1:], k[-1:], v[-1:], h, h * Hkv // H, rows, nq)
+        assert row_err(outs[0][-1, h].cpu().numpy()[rows], ref).max() <= TOL_BF16
