@@ -904,6 +904,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             tc_wait_st();
             tc_fence_before();
             named_sync_compute();
+            bool issued = false;
             if (warp == 0) {
                 if (!m_ready) m_ready = mbar_wait(bar(B_MFULL), 0, abort_flag, wcap);     // the matrix has landed (first use)
                 tc_fence_after();
@@ -913,9 +914,12 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         mma_ts_k64c(el0, tm_c + TC_Z_COL, tm_c + TC_R_COL + 32 * rb,
                                     make_desc(sb_c + Cfg::SM_M + rb * KBLK, Cfg::KSUB_BYTES), IDESC_TS16, rb > 0);
                     tc_commit_el(el0, bar(B_ACCFULL));
+                    issued = true;
                 }
             }
             acc_wait();
+            // (an aborted block: TMEM and shared memory stay until the product that this warp issued is done)
+            if (issued && !ok) (void)mbar_wait_landed(bar(B_ACCFULL), acc_uses & 1, wcap);
         };
         // f(e, z_e) for this thread's entries
         auto each_z = [&](auto&& fn) {

@@ -337,3 +337,27 @@ def test_the_pre_pass_reads_any_layout_of_q_and_any_number_of_heads(d, B, n, nq,
         rows = np.linspace(max(0, d + d // 2 - (n - nq)), nq - 2, 12).astype(int)
         ref = _exact(w, q[-1:], k[-1:], v[-1:], h, h * Hkv // H, rows, nq)
         assert row_err(outs[0][-1, h].cpu().numpy()[rows], ref).max() <= TOL_BF16
+
+
+@pytest.mark.parametrize("d,n,nq", [(64, 700, 700), (128, 1000, 300)])
+def test_a_preconditioned_block_whose_waits_run_out_leaves_cleanly(d, n, nq):
+    """No copy is issued, the matrix's neither, so every wait expires; the blocks leave, are counted, and the next call is right."""
+    w, q, k, v = _case(d, n, nq, 2, 2, 1.0, 2100 + n)
+    args = [dev(x, "bf16") for x in (q, k, v)]
+    nbytes = L.lla_forward_workspace_bytes(1, 2, n, d, d)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+
+    def run(**kw):
+        out = torch.full((1, 2, nq, d), float("nan"), dtype=torch.float32, device="cuda")
+        status = torch.zeros(L.LLA_STATUS_WORDS, dtype=torch.int32, device="cuda")
+        L.lla_forward_ex(*args, out, 1, 2, n, d, d, w.scale, w.lam, out_dtype=L.LLA_F32, q_rows=nq, device_status=status, workspace=ws,
+                         workspace_bytes=nbytes, cg_precondition=1, stream=stream_ptr(), **kw)
+        torch.cuda.synchronize()
+        return out, status.cpu().tolist()
+
+    good, st = run()
+    assert st[L.STATUS_TIMEOUT] == 0 and torch.isfinite(good).all()
+    _, st = run(debug_wait_clocks=1 << 20, debug_flags=L.LLA_DEBUG_NO_LOADS)
+    assert st[L.STATUS_TIMEOUT] > 0
+    again, st = run()
+    assert st[L.STATUS_TIMEOUT] == 0 and torch.equal(good, again)
