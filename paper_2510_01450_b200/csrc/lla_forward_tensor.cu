@@ -630,7 +630,11 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         // the middle of the fp16 range whatever the scale of the right-hand side and of the weights; pn2 tracks |p|^2 through the recurrence
         // |p'|^2 = |r'|^2 + beta^2 |p|^2
         float pn2 = 0.f, psc = 1.f, ipsc = 1.f;               // (in the output sweep ipsc undoes the scale of y)
-        int wexp = 0;                                         // largest weight of the row is at most 2^wexp
+        int wexp = 0;                                         // largest weight of the row: at most 2^wexp, and not far below
+        // ... but no larger than leaves U in the fp16 range: |u| <= 2^wtop |p| |k - kbar| with |k - kbar| < 2 sqrt(D) max |k| <
+        // 2^(6 + 1 + kexp), |p| < 2^1.5 and 2^wtop no less than the largest weight, so 2^-pdown |u| < 2^15 for this:
+        int pdown = 0;
+        const int kexp = f16_on ? (int)(prm.f16_range[0] >> 7) - 127 : 0;
         uint32_t ablk = 0;                                    // blocks with a product A so far (D = 128: slot = ablk % 2)
         float smax = -INFINITY;                               // statistics sweep: largest score of the row, relative to the shift
         uint32_t blk = 0;                                     // global block counter (buffer = blk & 1)
@@ -843,7 +847,7 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
         };
         auto write_p = [&]() {
             if (f16_on) {
-                scale_of(pn2, wexp);
+                scale_of(pn2, pdown);
                 write_operand16(p, psc, ipsc);
             } else {
                 write_operand(p);
@@ -1010,7 +1014,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
                         for (int e = 0; e < NCOL; ++e) acc[e] *= 1.f / STAT_SCALE;
                     }
                 }
-                wexp = given ? 0 : (int)fminf(fmaxf(ceilf(tmax - mx2), -8.f), 8.f);
+                // (statistics given: the largest weight is between the mean and the sum)
+                wexp = (int)fminf(fmaxf(ceilf(given ? fminf(__log2f(omega / (float)(L - jlo)), 0.f) : tmax - mx2), -8.f), 8.f);
+                const int wtop = given ? (int)fminf(fmaxf(ceilf(__log2f(omega)), -8.f), 8.f) : wexp;
+                pdown = max(wexp, wtop + kexp - 7);
                 inv_omega = 1.f / omega;
                 const float lam_i = (prm.lambda_rows && row < nq) ? prm.lambda_rows[(size_t)bh * nq + row] : prm.lambda;
                 // ridge in the frame of the shift: lambda e^{-shift} by the definition; the printed algorithm adds

@@ -401,3 +401,20 @@ def test_backward_preconditioned_solve_with_a_window(d, n, window):
         assert grad_err(a, b).max() <= TOL, name
     a, b = (t.cpu().numpy().ravel() for t in its)
     assert b[b >= 0].mean() < 0.9 * a[a >= 0].mean()
+
+
+@pytest.mark.parametrize("d,n,size", [(64, 420, 300.0), (128, 420, 300.0), (64, 420, 2000.0)])
+def test_backward_large_keys_and_weights(backward_oracle, d, n, size):
+    """Keys some thousands long under queries that keep the scores moderate, row maxima of about 2^5 in the frame of a zero score: U = w (a - abar)
+    of the extra solve must not leave the fp16 range."""
+    w = inputs.CONFIGS[2].shrink(B=1, H=2, n=n, d=d, dv=d, seed=330 + d, lam=100.0 * size ** 2)
+    q, k, v = inputs.make_prefill(w)
+    g = inputs.make_upstream_grad(w) * np.float32(size)      # (the keys' gradients shrink with their size)
+    s = np.float32(d ** 0.5)
+    k = inputs.round_to_bf16(k * s * np.float32(size))
+    q = inputs.round_to_bf16(q * s * np.float32(1.2 / size))
+    ref = backward_oracle.backward(q, k, v, g, w.scale, w.lam)
+    for kw in ({}, {"max_iters": 64}):
+        got = run_backward(w, q, k, v, g, **kw)
+        for name, a, b in zip(("dq", "dk", "dv"), got, ref):
+            assert grad_err(a, b).max() <= TOL, (name, kw)
