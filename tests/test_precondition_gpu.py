@@ -224,14 +224,17 @@ def test_a_block_mask_runs_plain_conjugate_gradients():
     assert np.array_equal(plain[0], default[0]) and np.array_equal(plain[1], default[1])
 
 
-@pytest.mark.parametrize("d,n,nq,window", [(64, 500, 460, 0), (64, 500, 439, 0), (128, 700, 580, 0), (64, 1500, 1500, 120), (128, 1500, 1500, 250)])
-def test_rows_of_few_keys_go_on_to_half_the_residual(d, n, nq, window):
+@pytest.mark.parametrize("d,n,nq,window,unit", [(64, 500, 460, 0, False), (64, 500, 439, 0, False), (128, 700, 580, 0, False),
+                                                (64, 1500, 1500, 120, False), (128, 1500, 1500, 250, False), (64, 500, 460, 0, True)])
+def test_rows_of_few_keys_go_on_to_half_the_residual(d, n, nq, window, unit):
     """Whatever tile a row of at most 2 d keys falls into: in a chunk whose tiles start elsewhere, and under a window.  The residual
     is that of the saved solution, in float64: y = rho / (1 - b . rho) solves C y = b to half of 1e-4; nine rows in ten
     within another quarter of the tolerance for what rounding adds to the solver's own residual (operand pairs in every iteration:
     of the order of 1e-5)."""
     H = 4
     w, q, k, v = _case(d, n, nq, H, H, 1.0, 1700 + nq)
+    if unit:      # scores of unit variance: weights far from uniform, such rows stop at the tolerance itself
+        q, k = (inputs.round_to_bf16(x * np.float32(d ** 0.5)) for x in (q, k))
     seen = np.arange(n - nq, n) + 1
     seen = np.minimum(seen, window) if window else seen
     rows = np.flatnonzero((seen >= d + d // 2) & (seen <= 2 * d))
@@ -253,7 +256,9 @@ def test_rows_of_few_keys_go_on_to_half_the_residual(d, n, nq, window):
             cy = (wt * ((kk - kb) @ y)) @ (kk - kb) / wt.sum() + w.lam * np.exp(-sc.max()) / wt.sum() * y
             res.append(np.linalg.norm(b - cy) / np.linalg.norm(b))
     res = np.asarray(res)
-    assert np.quantile(res, 0.5) <= 0.5e-4 and np.quantile(res, 0.9) <= 0.75e-4, np.sort(res)[::8]
+    stop = 1e-4 if unit else 0.5e-4
+    assert np.quantile(res, 0.5) <= stop and np.quantile(res, 0.9) <= stop + 0.25e-4, np.sort(res)[::8]
+    assert not unit or np.quantile(res, 0.5) > 0.5e-4, np.sort(res)[::8]
 
 
 @pytest.mark.parametrize("d,size_q,size_k", [(64, 1e-4, 1e-4), (128, 1e-4, 1e-4), (64, 1.0, 3e-4), (64, 3e-4, 1.0), (64, 1e-3, 1e-3)])
