@@ -240,6 +240,11 @@ int precond_blocks(int n);
 __host__ __device__ __forceinline__ int precond_block_used(int g, int nb) { return g < 16 ? g : (g | 1) < nb ? (g | 1) : nb - 1; }
 // ... and the first block of the group that ends with block g
 __host__ __device__ __forceinline__ int precond_group_start(int g) { return g < 16 ? g : g & ~1; }
+// With a sliding window there is a matrix per query tile instead, and two tiles share one where their rows see at least 2048 keys:
+// whether tile t of a head whose rows start at position off is such a tile.  Its group ends with the odd tile, or the last.
+__host__ __device__ __forceinline__ bool precond_tiles_paired(int t, int off, int window) {
+    return window >= 2048 && off + 128 * (t & ~1) >= 2048;
+}
 size_t precond_gram_bytes(int units, int n, int d);     // fp32 running Gram sums (scratch of the pre-pass)
 size_t precond_minv_bytes(int units, int n, int d);     // the fp16 matrices [units][blocks][d][d]
 // the pre-pass with the matrices: the fp16 copy of k and the largest magnitudes of k and q (range[2], zero before) as well

@@ -319,8 +319,10 @@ forward_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant
             auto load_m = [&]() {
                 if (Cfg::Q_IN_TMEM && !mbar_wait(bar(B_QREAD), 0, abort_flag, wcap)) return;
                 const int last = !prm.causal ? n - 1 : min(n - 1, off + (wraps ? prm.nq_pos : r0p + TC_BR) - 1);
-                // (with a window one per query tile of a head; for the tiles that grouped heads share, the one of the middle row)
-                const int gm = prm.window > 0 && prm.causal ? min(r0p + TC_BR / 2, prm.nq_pos - 1) / TC_BR : precond_block_used(last / 128, (n + 127) / 128);
+                // (with a window one per query tile of a head or two; for the tiles that grouped heads share, that of the middle row)
+                const int mid = min(r0p + TC_BR / 2, prm.nq_pos - 1) / TC_BR;
+                const int of_tile = precond_tiles_paired(mid, off, prm.window) ? min(mid | 1, (prm.nq_pos - 1) / TC_BR) : mid;
+                const int gm = prm.window > 0 && prm.causal ? of_tile : precond_block_used(last / 128, (n + 127) / 128);
                 m_issued = true;
                 mbar_expect_tx(bar(B_MFULL), D * D * 2);
                 for (int rb = 0; rb < D / 64; ++rb)

@@ -13,8 +13,8 @@
 // (With full weight the first row is off by a whole block: 15.8 instead of 12.1 iterations in the second tile at d = 64, 6.0
 // instead of 5.0 in the sixth, three instead of two past 14 K keys at d = 128.)
 //
-// A sliding window moves with the row, so there every query tile has a matrix of its own, in which each block of keys has the
-// weight of its mean share in the windows of the tile's rows: the block that the first rows see none of, and the one that
+// A sliding window moves with the row, so there every query tile has a matrix of its own (two share one where they see 2048 keys
+// and more), in which each block of keys has the weight of its mean share in the windows of the tile's rows: the block that the first rows see none of, and the one that
 // the last rows have left behind, count by the keys that a row of the tile sees of them on average.  The weights lie between
 // zero and one and add up to the mean number of visible keys, which is at least one: nothing here divides by zero.
 //
@@ -224,7 +224,7 @@ __device__ __forceinline__ float window_share(int first, int last, int window, i
 
 // One preconditioner per group of key blocks that tiles ask for (precond_block_used names the group's last block g): the keys
 // before the group, those of the group with the mean weight that the group's rows give them.  With a sliding window one per
-// query tile: every block of keys with its mean share in the windows of the tile's rows.
+// query tile or two: every block of keys with its mean share in the windows of the tile's rows.
 constexpr int PC_TERMS = 12;
 template <int D>
 __global__ void __launch_bounds__(PC_THREADS)
@@ -254,18 +254,35 @@ precond_invert_kernel(const PcParams p) {
     if (p.window > 0) {
         if (g >= p.tiles) return;
         const int off = p.n - p.nq;
+        const bool paired = precond_tiles_paired(g, off, p.window);
+        if (paired && !(g & 1) && g + 1 < p.tiles) return;      // the odd tile's serves both
         const int last = min(p.n - 1, off + PC_BLOCK * g + PC_BLOCK - 1);
-        const int first = min(max(off + PC_BLOCK * g, p.head_rows - 1), last);
-        auto share = [&](int b) { return window_share(first, last, p.window, b, p.n); };
-        // the mean number of visible keys
-        L = (float)(sum_clamped(last + 1, p.window) - sum_clamped(first, p.window)) / (float)(last - first + 1);
-        if (tid == 0) {
-            // sum_b share(b) block(b) in the running sums: the shares change at the two blocks that hold the first rows' and the
-            // last rows' first keys and at the two that hold the rows themselves
-            const int lo = max(0, first + 1 - p.window) / PC_BLOCK, hi = last / PC_BLOCK;
-            for (int b = lo - 1; b <= min(lo + 1, hi); ++b) sum_to(b, share(b) - share(b + 1));
-            for (int b = max(lo + 2, hi - 2); b <= hi; ++b) sum_to(b, share(b) - share(b + 1));
-            s_terms = terms;
+        const int first = min(max(off + PC_BLOCK * (paired ? g & ~1 : g), p.head_rows - 1), last);
+        const int hi = last / PC_BLOCK;
+        if (paired) {
+            // Wide windows: shares of the blocks that hold the rows, and the first keys cut at the nearest block to their mean, at most
+            // half a block of sixteen and more.  (With the shares of those blocks too an inversion reads up to 14 records: 2300 instead of
+            // 2260 us at n = 16384, 8 heads, d = 128, window 2500.)
+            const int start = max(0, (first + last) / 2 + 1 - p.window), b0 = (start + PC_BLOCK / 2) / PC_BLOCK;
+            L = 0.5f * (float)(first + last) + 1.f - (float)(PC_BLOCK * b0);
+            if (tid == 0) {
+                for (int b = hi - 3; b <= hi; ++b)
+                    sum_to(b, window_share(first, last, p.n, b, p.n) - window_share(first, last, p.n, b + 1, p.n));
+                sum_to(b0 - 1, -1.f);
+                s_terms = terms;
+            }
+        } else {
+            auto share = [&](int b) { return window_share(first, last, p.window, b, p.n); };
+            // the mean number of visible keys
+            L = (float)(sum_clamped(last + 1, p.window) - sum_clamped(first, p.window)) / (float)(last - first + 1);
+            if (tid == 0) {
+                // sum_b share(b) block(b) in the running sums: the shares change at the two blocks that hold the first rows' to the
+                // last rows' first keys and at the two that hold the rows themselves
+                const int lo = max(0, first + 1 - p.window) / PC_BLOCK;
+                for (int b = lo - 1; b <= min(lo + 1, hi); ++b) sum_to(b, share(b) - share(b + 1));
+                for (int b = max(lo + 2, hi - 2); b <= hi; ++b) sum_to(b, share(b) - share(b + 1));
+                s_terms = terms;
+            }
         }
     } else {
         if (p.causal && precond_block_used(g, p.nb) != g) return;        // no tile asks for this block's matrix

@@ -125,6 +125,8 @@ def _exact(w, q, k, v, h, hk, rows, nq, window=0):
     (128, 2637, 2637, 2, 2, 256, 1.0),
     (128, 2637, 2637, 2, 2, 224, 8 * 2 ** 0.5),      # scores of unit variance
     (64, 2500, 2500, 2, 2, 333, 8.0),
+    (64, 4900, 4900, 2, 2, 2100, 1.0),     # two tiles share a matrix past 2048 keys; the last one has its own
+    (64, 4900, 2300, 4, 2, 2050, 1.0),
 ])
 def test_the_matrices_of_a_window_are_made_of_the_keys_that_its_rows_see(d, n, nq, H, Hkv, window, spread):
     """Past 2048 keys and below it: fewer iterations than plain conjugate gradients in the first and in the second tile of every
