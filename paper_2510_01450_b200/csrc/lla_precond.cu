@@ -222,82 +222,98 @@ __device__ __forceinline__ float window_share(int first, int last, int window, i
     return (float)(seen - left) / (float)(len * (last - first + 1));
 }
 
+// The sums over keys that a matrix is made of, as records and their weights: what the records of blocks and of chunks before
+// them add up to.
+constexpr int PC_TERMS = 12;
+struct PcTerms {
+    int at[PC_TERMS];
+    float wt[PC_TERMS];
+    int count;
+    float keys;      // the weights of all keys
+    // the sums up to block b: its own record, and unless it is the last of its chunk that of the chunk before
+    __device__ __forceinline__ void sum_to(int b, float weight, int cb, int nb) {
+        if (b < 0 || weight == 0.f) return;
+        add(b, weight);
+        const int before = b / cb * cb - 1;
+        if (before >= 0 && b != before + cb && b != nb - 1) add(before, weight);
+    }
+    __device__ __forceinline__ void add(int record, float weight) {
+        for (int i = 0; i < count; ++i)
+            if (at[i] == record) { wt[i] += weight; return; }
+        at[count] = record;
+        wt[count++] = weight;
+    }
+};
+
+// With a sliding window: every block of keys with its mean share in the windows of the rows of tile g (of two tiles that share).
+// (Not inlined: in the kernel's instruction stream it cost the calls without a window 4 us of 237, one head, n = 4096, d = 64.)
+__device__ __noinline__ void window_terms(PcTerms* t, int g, int off, int n, int nb, int cb, int window, int head_rows) {
+    const bool paired = precond_tiles_paired(g, off, window);
+    const int last = min(n - 1, off + PC_BLOCK * g + PC_BLOCK - 1);
+    const int first = min(max(off + PC_BLOCK * (paired ? g & ~1 : g), head_rows - 1), last);
+    const int hi = last / PC_BLOCK;
+    // the shares change at the two blocks that hold the rows (three for two tiles) ...
+    const int lo = max(0, first + 1 - window) / PC_BLOCK;
+    int lead = max(lo + 2, hi - 2);
+    if (paired) {
+        // (wide windows: the first keys cut at the nearest block to their mean, at most half a block of sixteen and more.  With the
+        // shares of those blocks too an inversion reads up to 14 records: 2300 instead of 2260 us at n = 16384, 8 heads, d = 128,
+        // window 2500)
+        const int b0 = (max(0, (first + last) / 2 + 1 - window) + PC_BLOCK / 2) / PC_BLOCK;
+        t->keys = 0.5f * (float)(first + last) + 1.f - (float)(PC_BLOCK * b0);
+        t->sum_to(b0 - 1, -1.f, cb, nb);
+        lead = hi - 3;
+        window = n;
+    } else {
+        // ... and at the two that hold the first rows' to the last rows' first keys
+        t->keys = (float)(sum_clamped(last + 1, window) - sum_clamped(first, window)) / (float)(last - first + 1);
+        for (int b = lo - 1; b <= min(lo + 1, hi); ++b)
+            t->sum_to(b, window_share(first, last, window, b, n) - window_share(first, last, window, b + 1, n), cb, nb);
+    }
+    for (int b = lead; b <= hi; ++b)
+        t->sum_to(b, window_share(first, last, window, b, n) - window_share(first, last, window, b + 1, n), cb, nb);
+}
+
 // One preconditioner per group of key blocks that tiles ask for (precond_block_used names the group's last block g): the keys
 // before the group, those of the group with the mean weight that the group's rows give them.  With a sliding window one per
-// query tile or two: every block of keys with its mean share in the windows of the tile's rows.
-constexpr int PC_TERMS = 12;
+// query tile or two.
 template <int D>
 __global__ void __launch_bounds__(PC_THREADS)
 precond_invert_kernel(const PcParams p) {
     constexpr int TR = D / 16, V = D / 64;
     constexpr int rec = D * D + D;
     __shared__ float s_red[PC_THREADS / 32];
-    __shared__ int s_bad, s_at[PC_TERMS], s_terms;
+    __shared__ int s_bad;
+    __shared__ PcTerms s_terms;
     __shared__ __align__(16) float s_row[2][D], s_col[2][D];
-    __shared__ float sv[D], s_wt[PC_TERMS];
+    __shared__ float sv[D];
     const int u = blockIdx.y, tid = threadIdx.x;
     const int g = p.causal ? p.g0 + (int)blockIdx.x : p.nb - 1;      // the matrix's place; a query tile with a window
-    float L;
-    int terms = 0;
-    // the sums up to block b: its own record, and unless it is the last of its chunk that of the chunk before
-    auto add = [&](int at, float weight) {
-        for (int i = 0; i < terms; ++i)
-            if (s_at[i] == at) { s_wt[i] += weight; return; }
-        s_at[terms] = at;
-        s_wt[terms++] = weight;
-    };
-    auto sum_to = [&](int b, float weight) {
-        if (b < 0 || weight == 0.f) return;
-        add(b, weight);
-        if ((b + 1) % p.cb != 0 && b != p.nb - 1 && b >= p.cb) add(b / p.cb * p.cb - 1, weight);
-    };
     if (p.window > 0) {
         if (g >= p.tiles) return;
-        const int off = p.n - p.nq;
-        const bool paired = precond_tiles_paired(g, off, p.window);
-        if (paired && !(g & 1) && g + 1 < p.tiles) return;      // the odd tile's serves both
-        const int last = min(p.n - 1, off + PC_BLOCK * g + PC_BLOCK - 1);
-        const int first = min(max(off + PC_BLOCK * (paired ? g & ~1 : g), p.head_rows - 1), last);
-        const int hi = last / PC_BLOCK;
-        if (paired) {
-            // Wide windows: shares of the blocks that hold the rows, and the first keys cut at the nearest block to their mean, at most
-            // half a block of sixteen and more.  (With the shares of those blocks too an inversion reads up to 14 records: 2300 instead of
-            // 2260 us at n = 16384, 8 heads, d = 128, window 2500.)
-            const int start = max(0, (first + last) / 2 + 1 - p.window), b0 = (start + PC_BLOCK / 2) / PC_BLOCK;
-            L = 0.5f * (float)(first + last) + 1.f - (float)(PC_BLOCK * b0);
-            if (tid == 0) {
-                for (int b = hi - 3; b <= hi; ++b)
-                    sum_to(b, window_share(first, last, p.n, b, p.n) - window_share(first, last, p.n, b + 1, p.n));
-                sum_to(b0 - 1, -1.f);
-                s_terms = terms;
-            }
-        } else {
-            auto share = [&](int b) { return window_share(first, last, p.window, b, p.n); };
-            // the mean number of visible keys
-            L = (float)(sum_clamped(last + 1, p.window) - sum_clamped(first, p.window)) / (float)(last - first + 1);
-            if (tid == 0) {
-                // sum_b share(b) block(b) in the running sums: the shares change at the two blocks that hold the first rows' to the
-                // last rows' first keys and at the two that hold the rows themselves
-                const int lo = max(0, first + 1 - p.window) / PC_BLOCK;
-                for (int b = lo - 1; b <= min(lo + 1, hi); ++b) sum_to(b, share(b) - share(b + 1));
-                for (int b = max(lo + 2, hi - 2); b <= hi; ++b) sum_to(b, share(b) - share(b + 1));
-                s_terms = terms;
-            }
+        if (precond_tiles_paired(g, p.n - p.nq, p.window) && !(g & 1) && g + 1 < p.tiles) return;      // the odd tile's serves both
+        if (tid == 0) {
+            s_terms.count = 0;
+            window_terms(&s_terms, g, p.n - p.nq, p.n, p.nb, p.cb, p.window, p.head_rows);
         }
     } else {
         if (p.causal && precond_block_used(g, p.nb) != g) return;        // no tile asks for this block's matrix
-        const int start = precond_group_start(g), hi = min(p.n, PC_BLOCK * (g + 1));
-        const float len = (float)(hi - PC_BLOCK * start);
-        const float first = (float)max(p.head_rows - PC_BLOCK * start, 0);
-        const float w = p.causal ? fminf(fmaxf(0.5f * (first + len) / len, 0.5f), 1.f) : 1.f;
-        L = (float)(PC_BLOCK * start) + w * len;
         if (tid == 0) {
-            sum_to(g, w);
-            sum_to(start - 1, 1.f - w);
-            s_terms = terms;
+            const int start = precond_group_start(g), hi = min(p.n, PC_BLOCK * (g + 1));
+            const float len = (float)(hi - PC_BLOCK * start);
+            const float first = (float)max(p.head_rows - PC_BLOCK * start, 0);
+            const float w = p.causal ? fminf(fmaxf(0.5f * (first + len) / len, 0.5f), 1.f) : 1.f;
+            // (the records are those of blocks g and start - 1 and of the chunks before them, mostly one)
+            const int e = start - 1, cg = g / p.cb * p.cb - 1, ce = e < 0 ? -1 : e / p.cb * p.cb - 1;
+            const bool more_g = cg >= 0 && g != cg + p.cb && g != p.nb - 1, more_e = ce >= 0 && e != ce + p.cb;
+            s_terms.at[0] = g;           s_terms.wt[0] = w;
+            s_terms.at[1] = max(e, 0);   s_terms.wt[1] = e < 0 ? 0.f : 1.f - w;
+            s_terms.at[2] = max(cg, 0);  s_terms.wt[2] = (more_g ? w : 0.f) + (more_e && ce == cg ? 1.f - w : 0.f);
+            s_terms.at[3] = max(ce, 0);  s_terms.wt[3] = more_e && ce != cg ? 1.f - w : 0.f;
+            s_terms.count = 4;
+            s_terms.keys = (float)(PC_BLOCK * start) + w * len;
         }
     }
-    const float invL = 1.f / L;
     const float* base = p.gram + (size_t)u * p.nb * rec;
     if (tid == 0) s_bad = 0;
     // Thread (ty, tx) of the 16 x 16 grid keeps the entries (64 i + 4 ty + .., 64 j + 4 tx + ..) in registers.
@@ -305,10 +321,13 @@ precond_invert_kernel(const PcParams p) {
     float a[TR][TR] = {};
     float mine = 0.f;
     __syncthreads();
+    const float invL = 1.f / s_terms.keys;
+    const int terms = s_terms.count;
     cudaGridDependencySynchronize();
-    for (int c = 0; c < s_terms; ++c) {
-        const float wt = s_wt[c];
-        const float* r = base + (size_t)s_at[c] * rec;
+    for (int c = 0; c < terms; ++c) {
+        const float wt = s_terms.wt[c];
+        if (wt == 0.f) continue;
+        const float* r = base + (size_t)s_terms.at[c] * rec;
 #pragma unroll
         for (int i = 0; i < TR; ++i)
 #pragma unroll
@@ -477,9 +496,11 @@ int launch_precond(const ForwardArgs& a, void* k16, uint32_t* range, void* gram,
     int dev = 0, sms = 0;
     LLA_CUDA_TRY(cudaGetDevice(&dev));
     LLA_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // chunks: two thread blocks an SM, whatever the number of heads (with eight per head, one key/value head had eight in all)
+    // chunks: two thread blocks an SM at d = 64 and one at d = 128, where the registers hold no more, whatever the number of heads
+    // (with eight chunks always, one key/value head had eight blocks in all: 32 heads over one, n = 4096, d = 128: 70 us more).
+    // Many heads keep eight: with 16 chunks 16 heads of 16384 keys took 83 us instead of 78.
     const int units = p.B * p.Hk;
-    const int most = std::min(std::max(2 * sms / units, 8), PC_CHUNKS);
+    const int most = std::min(std::max((a.d == 64 ? 2 : 1) * sms / units, 8), PC_CHUNKS);
     p.cb = (p.nb + most - 1) / most;
     if (p.cb > 1) p.cb += p.cb & 1;      // a chunk's last block is then one whose record is written anyway
     p.chunks = (p.nb + p.cb - 1) / p.cb;
