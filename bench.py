@@ -34,11 +34,11 @@ LEGS = (2, 3)         # the other bf16 prefill workloads, reported as sub-object
 L2_BYTES = 126e6
 # DRAM bytes (read + write) per launch of the dominant kernel from the ncu captures summarised under
 # profiles/: (bytes, summary file).  Workload 4 was captured with 2 of its 16 heads and scaled by 8
-# (traffic is per head: Q, K, V once).
+# (traffic is per head: Q, the fp16 copy of K, V and the preconditioner's matrices once; without the pre-pass that makes those).
 NCU_TRAFFIC = {
-    2: (12.68e6, "profiles/forward_tc_kernel_cfg2.md"),
-    3: (4 * 17.06e6, "profiles/forward_tc_kernel_cfg3.md (8 of 32 units captured, x 4)"),
-    4: (8 * (33.67e6 + 2.58e6), "profiles/forward_tc_kernel_cfg4.md (2 of 16 heads captured, x 8)"),
+    2: (14.85e6, "profiles/forward_tc_kernel_cfg2.md"),
+    3: (4 * 14.33e6, "profiles/forward_tc_kernel_cfg3.md (8 of 32 units captured, x 4)"),
+    4: (8 * (30.04e6 + 1.92e6), "profiles/forward_tc_kernel_cfg4.md (2 of 16 heads captured, x 8)"),
 }
 NCU_DECODE_TRAFFIC = (1.188e9 + 25.2e6 + 34.3e6, "profiles/decode_tc_kernel_cfg5.md")   # streaming read + record write, solve read
 
@@ -439,7 +439,8 @@ def run_ours(args):
                 "ms_per_step": 1e3 * e2e_s / e2e_steps,
                 "note": "lla_forward_host on pinned buffers; the host link carries "
                         f"{(h2d + pout.numel() * 2) / 1e6:.0f} MB per step"},
-        # per step: the fp16 copy of k, the iterative-rows kernel, the direct-rows kernel
+        # per step: the three kernels of the preconditioner's pre-pass (the first makes the fp16 copy of k as well), the
+        # iterative-rows kernel, the direct-rows kernel
         "gpu_launches": 5 * args.steps,
     }
     line.update(legs)

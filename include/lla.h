@@ -190,8 +190,9 @@ typedef struct lla_forward_params {
                        error than the tolerance leaves.  The search direction P is rounded to fp16 before it is used at all, so
                        its products are exact.  The sweeps read an fp16 copy of k made by a pre-pass into `workspace`
                        (without room for it there, or with the largest magnitude in q or in k above 6e4 or, but for zeros,
-                       below 2^-9, they read the bf16 inputs, and every iteration uses bf16 pairs for both operands).  0 = default (1 iteration; 4 for the row
-                       tiles within the first 8 d positions, which converge more slowly); n > 0 = n
+                       below 2^-9, they read the bf16 inputs, and every iteration uses bf16 pairs for both operands).
+                       0 = default (1 iteration; 4 for the row tiles within the first 8 d positions, which converge
+                       more slowly); n > 0 = n
                        iterations for every tile; LLA_CG_PRECISE_ALL = every iteration with bf16 pairs;
                        LLA_CG_PRECISE_NONE = fp16 from the first iteration on */
     long long q_strides[3], k_strides[3], v_strides[3], out_strides[3];
@@ -210,15 +211,20 @@ typedef struct lla_forward_params {
                        dense.  n <= 65536.  Shapes the tensor-core kernel does not cover: LLA_ERR_UNSUPPORTED */
     long long block_mask_stride;     /* bytes from one (batch, head) unit's mask to the next; 0 = one mask for all */
     int cg_precondition;  /* tensor-core kernel only.  1 = conjugate gradients preconditioned with the inverse covariance of the
-                       visible keys: a d x d matrix per block of 128 keys, built by a pre-pass into `workspace` (plain CG
-                       without room for it there).  The system of a row is that covariance under the row's attention
-                       weights, so the closer the weights are to uniform the fewer iterations remain -- half and less
-                       on the synthetic workloads, four fifths with scores of unit variance.  The
-                       solution is the same within the tolerance; a row on which the rounded matrix turns out
-                       not to be positive definite carries on with plain CG.
+                       visible keys: a d x d matrix per block of 128 keys (per two past 2048 keys; with a window per
+                       query tile), built by a pre-pass into `workspace` (plain CG without room for it there, and
+                       where the sweeps read the bf16 inputs: see cg_precise_iters).  The system of a row is that
+                       covariance under the row's attention weights, so the closer the weights are to uniform the
+                       fewer iterations remain -- half and less on the synthetic workloads, four fifths with scores
+                       of unit variance, where calls of few heads and short sequences take up to a seventh longer
+                       than plain CG (with a hundredth of its rows at the iteration cap).  The solution is the same
+                       within the tolerance; a row on which the rounded matrix turns out not to be positive
+                       definite, and a causal row of fewer than 1.5 d keys, carries on with plain CG.
                        0 = default: with the other solver settings (max_iters, tol, cg_precise_iters, impl) at their
-                       defaults, head_rows at its default or above 1.5 d, no lambda_rows and the ridge of the definition, the library chooses, which at
-                       present means as with 1 unless there are fewer than n / 4 query rows or a block mask; otherwise plain conjugate gradients as in Algorithm 2 */
+                       defaults, head_rows at its default or above 1.5 d, no lambda_rows and the ridge of the definition, the library
+                       chooses, which at present means as with 1 unless there are fewer than n / 4 query rows or a block
+                       mask; otherwise plain conjugate gradients as in Algorithm 2 (so max_iters = 64, the default cap,
+                       given as such, asks for those) */
     long long debug_wait_clocks; /* tensor-core kernel only: cap, in SM clocks, of every bounded wait on a barrier
                        inside the kernel (0 = default, about 2^31).  A wait that runs out makes its thread block
                        stop: the block waits for the copies and MMAs it has issued itself, releases its tensor
@@ -339,10 +345,11 @@ int lla_decode_noalloc(const void *q, const void *kcache, const void *vcache, co
                        void *out, int B, int H, int Lmax, int d, int dv, int in_dtype,
                        int out_dtype, float scale, float lambda, int splits, void *stream);
 
-/* Scratch bytes lla_forward_ex can use for this problem (0 when none).  Only the d = 128 tensor-core
- * kernel has any (2 x SM count x 192 KiB: per-SM slots for the CG row vectors; the call queries the
- * current device's SM count).  It is optional: given a workspace of that size the call allocates
- * nothing (two calls that may run at the same time need separate workspaces); without one the
+/* Scratch bytes lla_forward_ex can use for this problem (0 when none).  Only the tensor-core kernel has any: the fp16
+ * copy of k, the preconditioner's records and matrices, and at d = 128 2 x SM count x 192 KiB of per-SM slots for the CG row
+ * vectors (the call queries the current device's SM count).  It is optional: given a workspace of that size the call allocates
+ * nothing (two calls that may run at the same time need separate workspaces); with less it runs without the matrices, or without
+ * the copy (plain conjugate gradients on bf16 operand pairs), and at d = 128 without room for the slots the
  * library keeps its own buffer per GPU, allocated with cudaMalloc by the first such call and shared
  * safely by all later ones (blocks address it by SM id and one block fills an SM). */
 size_t lla_forward_workspace_bytes(int B, int H, int n, int d, int dv, int in_dtype, int impl);

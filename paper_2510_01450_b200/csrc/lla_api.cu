@@ -70,8 +70,11 @@ HostPipe* host_pipe() {
 bool head_size_ok(int d, int dv) { return d == dv && (d == 16 || d == 64 || d == 128); }
 
 // The preconditioner's pre-pass reads every key, its gain is in the sweeps of the query tiles: whole sequences gain 15 % (32
-// heads, n = 1024, d = 64: 309 -> 266 us) to 30 % (16 heads, n = 16384, d = 128: 12.9 -> 9.0 ms), a chunk of 257 queries on 5003
-// keys with scores of unit variance loses (16 heads over 4, d = 128: 577 -> 633 us).
+// heads, n = 1024, d = 64: 309 -> 266 us) to 30 % (16 heads, n = 16384, d = 128: 12.9 -> 9.0 ms).  Chunks, preconditioned over plain
+// time at n = 2000, 5000 and 12000, 8 to 32 heads, both head sizes: 1/16 of the sequence 0.73 .. 1.06 with iid inputs and 0.92 .. 1.16 with
+// scores of unit variance, 1/8 0.77 .. 1.01 and 1.00 .. 1.14, 1/4 0.76 .. 0.95 and 0.96 .. 1.06, 1/2 0.73 .. 0.88 and 0.98 .. 1.07.  So
+// from a quarter on: what unit variance loses there, a few percent at most (with a tenth of the rows at the cap), is little beside
+// what nearly uniform weights gain, and below it is not.
 // Nor under a block mask: the matrices are those of all keys, and a row that attends some needs as many iterations with them as
 // without (8 heads, n = 8192, d = 64, 5 % of the blocks: 474 -> 546 us; d = 128, n = 4096, scores of unit variance: 1377 -> 1767 us).
 bool precondition_pays(int n, int nq, bool masked) { return 4ll * nq >= n && !masked; }
@@ -497,8 +500,8 @@ size_t lla_backward_workspace_bytes(int B, int H, int n, int d) {
 
 size_t lla_forward_workspace_bytes(int B, int H, int n, int d, int dv, int in_dtype, int impl) {
     if (B < 1 || H < 1 || n < 1) return 0;
-    // Only the tensor-core kernel uses any: the fp16 copy of k for its later CG sweeps and, for d = 128, one
-    // slot per SM id for the row vectors it keeps off chip (see lla_forward_tensor.cu).
+    // Only the tensor-core kernel uses any: the fp16 copy of k for its sweeps, the preconditioner's records and matrices and, for
+    // d = 128, one slot per SM id for the row vectors it keeps off chip (see lla_forward_tensor.cu).
     if (in_dtype == LLA_BF16 && (d == 64 || d == 128) && dv == d && impl != LLA_IMPL_SIMT)
         return lla::forward_tensor_workspace_bytes(B, H, n, d);
     return 0;

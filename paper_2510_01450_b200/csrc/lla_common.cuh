@@ -120,8 +120,8 @@ struct ForwardArgs {
     int precondition = 0;       // 1: preconditioned CG when the workspace has room for the matrices
     const void* k16 = nullptr;  // fp16 copy of k, and the largest magnitudes of k and q (bf16 bit patterns): set by
     const uint32_t* f16_range = nullptr;   // forward_tensor_prepass
-    int precise_iters = 1;      // tensor-core kernel: CG iterations run with bf16 hi + lo operand pairs before the
-    int precise_iters_early = 4;   // switch to single fp16 operands (see lla_forward_params.cg_precise_iters); the
+    int precise_iters = 1;      // tensor-core kernel: CG iterations run with U as fp16 hi + lo pairs before the switch
+    int precise_iters_early = 4;   // to single fp16 values (see lla_forward_params.cg_precise_iters); the
                                 // second value is for row tiles that end within the first 8 d positions
 };
 
@@ -230,10 +230,11 @@ int launch_head_rows(const ForwardArgs& a);
 int launch_forward_simt(const ForwardArgs& a);
 int launch_forward_tensor(const ForwardArgs& a);
 bool forward_tensor_supported(const ForwardArgs& a);
-int forward_tensor_prepass(ForwardArgs& a);    // fp16 copy of k into the workspace (no-op without room)
+int forward_tensor_prepass(ForwardArgs& a);    // fp16 copy of k, and the matrices, into the workspace (no-op without room)
 size_t forward_tensor_scratch_bytes();         // d = 128 row-state scratch (0 if the device cannot be queried)
-size_t forward_tensor_workspace_bytes(int B, int H, int n, int d);   // that scratch + the fp16 copy of k (upper bound: kv heads = H)
-// CG preconditioner of the tensor-core forward (lla_precond.cu): one d x d fp16 matrix per block of 128 keys
+size_t forward_tensor_workspace_bytes(int B, int H, int n, int d);   // that scratch, the fp16 copy of k, the Gram records and the
+                                                                     // matrices (upper bound: kv heads = H)
+// CG preconditioner of the tensor-core forward (lla_precond.cu): room for one d x d fp16 matrix per block of 128 keys
 int precond_blocks(int n);
 // Beyond the first 16 blocks (2048 keys) the covariance changes little from one block of 128 keys to the next: two blocks share
 // a matrix there.  The last block of the group that holds block g of nb, whose matrix the tiles of the group take ...

@@ -5,14 +5,14 @@
 //
 //   TMA            K block (and V block in the last sweep) -> 128B-swizzled shared memory
 //   MMA 1 (SS)     S = Q K^T                     [128 x 64] fp32 in TMEM
-//                  A = P_hi K^T + P_lo K^T       [128 x 64] fp32 in TMEM   (CG and output sweeps)
+//                  A = P K^T                     [128 x 64] fp32 in TMEM   (CG and output sweeps; bf16 P and the output
+//                                                sweep's y as hi + lo, two products)
 //   CUDA cores     one thread pair per query row reads S, A from TMEM, forms
-//                      max sweep     running row maximum m_i
 //                      stats sweep   w = exp(s - m),                 omega += w
 //                      CG sweep      u = w (a - kbar.p)              (Algorithm 2's W .* (P K^T))
 //                      output sweep  c = w (1 - (a - kbar.y)),       den += c
-//                  splits the result into bf16 hi + lo and stores both back into the TMEM columns S
-//                  came from (two 16-bit values per column)
+//                  and stores it as 16-bit hi + lo (a later CG sweep: one fp16 value) back into the TMEM
+//                  columns S came from (two values per column)
 //   MMA 2 (TS)     ACC += U_hi B + U_lo B, A operand straight from TMEM, B = the same K block read
 //                  MN-major (or the V block in the output sweep)
 //
@@ -25,7 +25,8 @@
 // warps 9 and 10 issue the two MMA streams.  The weights w and c and the solution y are carried as pairs hi + lo of 16-bit
 // values: a single bf16 rounding of those operands would leave a 2e-3..5e-3 error in the output, above the 2e-3 gate.  A search
 // direction P is rounded to one fp16 value per entry before it is used anywhere, so its products carry no rounding at all;
-// U is a pair in the first CG iterations and one fp16 value later.  Q, K, V are exact bf16 inputs.
+// U is a pair in the first CG iterations and one fp16 value later.  V is the bf16 input; Q and K are fp16 copies of theirs where those
+// keep the bits (fits_f16), else the inputs themselves.
 //
 // The mathematics is the centred form described in lla_forward_simt.cu (same CG, same freeze rule).
 // All waits on mbarriers are bounded; a wait that expires sets LLA_STATUS_TIMEOUT and the block
@@ -130,7 +131,7 @@ struct TcParams {
     int n, nq, causal, head_rows, max_iters, first_tile;   // n keys; nq query rows of a unit
     int nq_pos;          // query rows of a head, at positions n - nq_pos .. n - 1.  nq = nq_pos, or a multiple of it: the heads
                          // that share a key/value head as one unit, row r being row r % nq_pos of its head r / nq_pos
-    int precise_iters;   // CG iterations whose operands are bf16 hi + lo pairs; later ones use single fp16 operands
+    int precise_iters;   // CG iterations with U as an fp16 hi + lo pair; later ones use single fp16 values
     int precise_iters_early;   // the same for the row tiles that end within the first 8 D positions
     long long wait_clocks;   // cap of every bounded wait, in SM clocks
     int no_loads;        // test aid: the TMA warp issues no copy at all, so that every wait expires with nothing in flight

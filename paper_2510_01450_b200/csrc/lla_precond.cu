@@ -8,25 +8,30 @@
 // the synthetic workloads it takes away more than half of the iterations.  It never changes the solution, only the path to
 // it, so it is built in fp32 and stored in fp16; a block whose inversion breaks down gets the identity.
 //
-// The rows of a tile see between none and all of the tile's own keys, so those enter with the mean of that, half their
-// weight: a row's own covariance is then off by half a block's worth of keys at most, whichever row of the tile it is.
+// Without a window the rows of a tile see between none and all of the tile's own keys, so those enter with the mean of that, half
+// their weight: a row's own covariance is then off by half a block's worth of keys at most, whichever row of the tile it is, and by
+// half a group of two blocks past 2048 keys, where two tiles share a matrix.
 // (With full weight the first row is off by a whole block: 15.8 instead of 12.1 iterations in the second tile at d = 64, 6.0
-// instead of 5.0 in the sixth, three instead of two past 14 K keys at d = 128.)
+// instead of 5.0 in the sixth, three instead of two past 14 K keys at d = 128.)  A chunk of queries whose tiles do not start at a
+// block of keys takes the matrix of the block that its tile's last row sees last.
 //
 // A sliding window moves with the row, so there every query tile has a matrix of its own (two share one where they see 2048 keys
-// and more), in which each block of keys has the weight of its mean share in the windows of the tile's rows: the block that the first rows see none of, and the one that
-// the last rows have left behind, count by the keys that a row of the tile sees of them on average.  The weights lie between
-// zero and one and add up to the mean number of visible keys, which is at least one: nothing here divides by zero.
+// and more), in which each block of keys has the weight of its mean share in the windows of the tile's rows: the block that the
+// first rows see none of, and the one that the last rows have left behind, count by the keys that a row of the tile sees of
+// them on average.  The weights lie between zero and one and add up to the mean number of visible keys, which is at least one:
+// nothing here divides by zero.
 //
 // Three kernels, all on the caller's stream ahead of the forward kernel:
 //   precond_gram_kernel     a chunk of key blocks each: running sums of k_j k_j^T and k_j inside the chunk, one record per
 //                           block that is asked for.  It reads every key once, so it also makes the fp16 copy of k and
-//                           finds the largest magnitudes of k and q.  Bound by its loads; the products run on mma.sync,
-//                           whose operands come straight from the tiles (ldmatrix.trans).  16 heads, n = 16384, d = 128:
-//                           85 us, where Gram sums on the CUDA cores, their scan over every block and a copy kernel took 430
+//                           finds the largest magnitudes of k and q.  The products run on mma.sync, whose operands come
+//                           straight from the tiles (ldmatrix.trans).  16 heads, n = 16384, d = 128: 81 us, twice what
+//                           its 280 MB take at the copy bandwidth: eight warps an SM (165 registers a thread) hide a
+//                           part of the loads' latency, the top stall.  (Gram sums on the CUDA cores, their scan over
+//                           every block and a copy kernel took 430 us)
 //   precond_scan_kernel     the sums of whole chunks (the records of their last blocks) become running sums over the sequence
-//   precond_invert_kernel   M_g = (G / L - s s^T / L^2 + (lambda / L) I)^{-1}, G and s from the records of the block and of
-//                           the chunk before it, by Gauss-Jordan elimination in registers, scaled to a largest entry of one
+//   precond_invert_kernel   M_g = (G / L - s s^T / L^2 + ridge I)^{-1} with ridge = lambda / L or more, G and s from the records
+//                           of the block and of the chunk before it, by Gauss-Jordan elimination in registers, scaled to a largest entry of one
 //                           (conjugate gradients do not see the scale of a preconditioner), rounded to fp16.
 #include <cuda_fp16.h>
 

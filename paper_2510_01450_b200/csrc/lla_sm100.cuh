@@ -212,7 +212,8 @@ __device__ __forceinline__ uint32_t pack_f16(float a, float b) {
     return r;
 }
 // Split two fp32 values into fp16 hi + lo pairs: hi is the value cut to 11 significant bits, lo the rounded remainder, so
-// hi + lo keeps 22 bits down to an absolute error of 2^-25 (half the spacing of the fp16 subnormals).
+// hi + lo keeps 22 bits down to an absolute error of 2^-25 (half the spacing of the fp16 subnormals); 2^-24 for values below
+// 2^-14, whose hi the conversion rounds once more.
 __device__ __forceinline__ uint32_t split_f16x2(float a, float b, uint32_t& lo) {
     const float ha = __uint_as_float(__float_as_uint(a) & 0xFFFFE000u), hb = __uint_as_float(__float_as_uint(b) & 0xFFFFE000u);
     lo = pack_f16(a - ha, b - hb);
