@@ -189,8 +189,8 @@ typedef struct lla_forward_params {
                        which has fallen by then, so the coarser operands of the later iterations add less
                        error than the tolerance leaves.  The search direction P is rounded to fp16 before it is used at all, so
                        its products are exact.  The sweeps read an fp16 copy of k made by a pre-pass into `workspace`
-                       (without room for it there, or with the largest magnitude in q or in k above 6e4 or, but for zeros,
-                       below 2^-9, they read the bf16 inputs, and every iteration uses bf16 pairs for both operands).
+                       (without room for it there, or with the largest magnitude in q or in k above 6e4 or, but for zeros and
+                       for q under keys of 2^-2 and more, below 2^-9, they read the bf16 inputs, and every iteration uses bf16 pairs for both operands).
                        0 = default (1 iteration; 4 for the row tiles within the first 8 d positions, which converge
                        more slowly); n > 0 = n
                        iterations for every tile; LLA_CG_PRECISE_ALL = every iteration with bf16 pairs;

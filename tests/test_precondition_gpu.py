@@ -127,6 +127,8 @@ def _exact(w, q, k, v, h, hk, rows, nq, window=0):
     (64, 2500, 2500, 2, 2, 333, 8.0),
     (64, 4900, 4900, 2, 2, 2100, 1.0),     # two tiles share a matrix past 2048 keys; the last one has its own
     (64, 4900, 2300, 4, 2, 2050, 1.0),
+    (64, 2600, 700, 4, 2, 600, 1.0),       # grouped heads in common tiles: the matrix of the tile's middle row
+    (64, 5000, 1300, 4, 2, 2100, 1.0),
 ])
 def test_the_matrices_of_a_window_are_made_of_the_keys_that_its_rows_see(d, n, nq, H, Hkv, window, spread):
     """Past 2048 keys and below it: fewer iterations than plain conjugate gradients in the first and in the second tile of every
@@ -263,7 +265,8 @@ def test_rows_of_few_keys_go_on_to_half_the_residual(d, n, nq, window, unit):
     assert not unit or np.quantile(res, 0.5) > 0.5e-4, np.sort(res)[::8]
 
 
-@pytest.mark.parametrize("d,size_q,size_k", [(64, 1e-4, 1e-4), (128, 1e-4, 1e-4), (64, 1.0, 3e-4), (64, 3e-4, 1.0), (64, 1e-3, 1e-3)])
+@pytest.mark.parametrize("d,size_q,size_k", [(64, 1e-4, 1e-4), (128, 1e-4, 1e-4), (64, 1.0, 3e-4), (64, 3e-4, 1.0), (64, 1e-3, 1e-3),
+                                              (64, 3e-5, 2.0), (128, 1e-4, 100.0), (64, 1e-3, 0.3)])
 def test_small_inputs_keep_their_bits(d, size_q, size_k):
     """Entries of q and k far below the fp16 range's middle: rho against float64 within the tolerance, whatever the solver.  (In fp16
     an entry of 1e-5 is off by up to 0.3 %.)"""
